@@ -68,14 +68,6 @@ __device__ __forceinline__ double second_invariant(const Grad9& g) {
 
 // ----------------------------------------------------------------------------- reductions
 
-template <int M>
-__device__ __forceinline__ void warp_sum(double (&v)[M]) {
-#pragma unroll
-  for (int m = 0; m < M; ++m)
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v[m] += __shfl_down_sync(0xffffffffu, v[m], off);
-}
-
 // Larger of two non-negative doubles (+inf allowed). For such values the IEEE order is the order
 // of their bit patterns as integers, so the comparison runs on the integer units: GB300 issues
 // FP64 instructions at a small fraction of its integer rate. Every max-reduction here reduces
@@ -85,61 +77,90 @@ __device__ __forceinline__ double max_nonneg(double a, double b) {
   return __longlong_as_double(x > y ? x : y);
 }
 
-template <int M>
-__device__ __forceinline__ void warp_max(double (&v)[M]) {
-#pragma unroll
-  for (int m = 0; m < M; ++m)
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-      v[m] = max_nonneg(v[m], __shfl_down_sync(0xffffffffu, v[m], off));
+// What a reduction does with two values of its type V, and the double it ends in.
+struct SumD {
+  using V = double;
+  using Total = SumD;   // the operation on the doubles of the blocks
+  static __device__ __forceinline__ V zero() { return 0.0; }
+  static __device__ __forceinline__ V add(V a, V b) { return a + b; }
+  static __device__ __forceinline__ V shfl_xor(V a, int m) {
+    return __shfl_xor_sync(0xffffffffu, a, m);
+  }
+  static __device__ __forceinline__ double value(V a) { return a; }
+};
+struct MaxD : SumD {   // of non-negative values
+  using Total = MaxD;
+  static __device__ __forceinline__ V add(V a, V b) { return max_nonneg(a, b); }
+};
+
+__host__ __device__ constexpr int pow2_at_least(int m) {
+  return m <= 1 ? 1 : 2 * pow2_at_least((m + 1) / 2);
 }
 
-// Sum (or max, of non-negative values) of M values over the block; the result is valid in
-// thread 0. Fixed order, so the result is the same run to run for the same launch shape.
-// smem: >= 32*M doubles.
-template <int M, bool IsMax>
-__device__ __forceinline__ void block_reduce(double (&v)[M], double* smem) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nw = (blockDim.x + 31) >> 5;
-  if (IsMax) warp_max<M>(v); else warp_sum<M>(v);
-  if (lane == 0) {
+// Reduce Mp values (a power of two) over a warp by halving: at stage k a lane keeps one half of its
+// values and gives the other half to the lane that differs in bit k, so that Mp - 1 + log2(32/Mp)
+// additions take the place of 5 Mp. Every lane ends with the total of value fold_slot<Mp>(lane).
+// What this saves: GB300 issues an FP64 instruction of a warp in 16 cycles of the SM's one FP64
+// pipe, and a float-float addition is 10 float instructions, so the 20 to 40 additions per thread
+// of a plain shuffle tree of 4 to 8 values cost more than the stencil arithmetic they followed.
+// Measured per launch, with the ends of the Krylov kernels one thread a system (hosc_krylov4.cuh):
+// x/r at 41^3 mixed 20.4 -> 10.0 us, at 101^3 mixed 33.1 -> 21.4 us, at 91^3 FP64 128 -> 75 us; p/v
+// 13.7 -> 9.3, 45.2 -> 39.8 and 164 -> 138 us.
+template <class Op, int Mp>
+__device__ __forceinline__ typename Op::V warp_fold(typename Op::V (&v)[Mp]) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int m = 0; m < M; ++m) smem[wid * M + m] = v[m];
-  }
-  __syncthreads();
-  if (wid == 0) {
+  for (int k = 0; (Mp >> k) > 1; ++k) {
+    const int h = Mp >> (k + 1);
+    const bool up = (lane >> k) & 1;
 #pragma unroll
-    for (int m = 0; m < M; ++m) v[m] = (lane < nw) ? smem[lane * M + m] : (IsMax ? 0.0 : 0.0);
-    if (IsMax) warp_max<M>(v); else warp_sum<M>(v);
+    for (int q = 0; q < h; ++q) {
+      const typename Op::V give = up ? v[q] : v[q + h], keep = up ? v[q + h] : v[q];
+      v[q] = Op::add(keep, Op::shfl_xor(give, 1 << k));
+    }
   }
-  __syncthreads();
+  typename Op::V r = v[0];
+#pragma unroll
+  for (int off = Mp; off < 32; off <<= 1) r = Op::add(r, Op::shfl_xor(r, off));
+  return r;
+}
+template <int Mp>
+__device__ __forceinline__ int fold_slot(int lane) {
+  int m = 0;
+#pragma unroll
+  for (int k = 0; (Mp >> k) > 1; ++k) m |= ((lane >> k) & 1) ? Mp >> (k + 1) : 0;
+  return m;
 }
 
-// Block sum of M values whose per-thread terms are float: the warp stage adds in float, the
-// warp sums are widened to double for the cross-warp stage (and the grid stage that follows), so
-// each thread does no double arithmetic. The result is valid in thread 0.
-template <int M>
-__device__ __forceinline__ void block_sum_f32(const float (&vf)[M], double (&v)[M], double* smem) {
-  float w[M];
+// Warp 0: totals over the block's warps of s[warp * Mp + m]; lane m (m < Mp) gets value m.
+template <class Op, int Mp>
+__device__ __forceinline__ typename Op::V cross_warps(const typename Op::V* s) {
+  const int lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+  typename Op::V r = Op::zero();
+  for (int w = lane / Mp; w < nw; w += 32 / Mp) r = Op::add(r, s[w * Mp + lane % Mp]);
 #pragma unroll
-  for (int m = 0; m < M; ++m) {
-    w[m] = vf[m];
+  for (int off = Mp; off < 32; off <<= 1) r = Op::add(r, Op::shfl_xor(r, off));
+  return r;
+}
+
+constexpr int kMaxWarps = 16;   // warps of a block that reduces
+
+// Sum (or max, of non-negative values) of M values over the block; thread m < M returns value m.
+// Fixed order, so the result is the same run to run for the same launch shape.
+template <class Op, int M>
+__device__ __forceinline__ typename Op::V block_total(const typename Op::V (&v)[M]) {
+  using V = typename Op::V;
+  constexpr int Mp = pow2_at_least(M);
+  static_assert(Mp <= 32, "at most 32 values");
+  __shared__ V s_w[kMaxWarps * Mp];
+  V x[Mp];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) w[m] += __shfl_down_sync(0xffffffffu, w[m], off);
-  }
+  for (int m = 0; m < Mp; ++m) x[m] = m < M ? v[m < M ? m : 0] : Op::zero();
+  const V r = warp_fold<Op, Mp>(x);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nw = (blockDim.x + 31) >> 5;
-  if (lane == 0) {
-#pragma unroll
-    for (int m = 0; m < M; ++m) smem[wid * M + m] = (double)w[m];
-  }
+  if (lane < Mp) s_w[wid * Mp + fold_slot<Mp>(lane)] = r;
   __syncthreads();
-  if (wid == 0) {
-#pragma unroll
-    for (int m = 0; m < M; ++m) v[m] = (lane < nw) ? smem[lane * M + m] : 0.0;
-    warp_sum<M>(v);
-  }
-  __syncthreads();
+  return wid == 0 ? cross_warps<Op, Mp>(s_w) : Op::zero();
 }
 
 // Doubles per row of the partials buffer for M values per block: kRedSlots, 2 kRedSlots for
@@ -150,73 +171,58 @@ __host__ __device__ constexpr int row_stride() {
   return M > 2 * kRedSlots ? 4 * kRedSlots : (M > kRedSlots ? 2 * kRedSlots : kRedSlots);
 }
 
-// Publish the M partials of block b of nb (valid in thread 0) and report whether this block is
-// the last one to do so. No thread waits on another block: the last block to take a ticket does
-// the final reduction, every other block simply exits.
-template <int M>
-__device__ __forceinline__ bool publish_is_last(const double (&v)[M], double* red,
-                                                unsigned int* counter, unsigned int b,
-                                                unsigned int nb) {
+// Reduction over the grid of M values per thread. Block b of nb writes its totals to its row of
+// red and takes a ticket; the block that takes the last one (no block waits for another) sums
+// the rows in a fixed order and returns the totals in shared memory, valid for its every thread;
+// the other blocks return null. The ticket counter is left at zero for the next kernel.
+// In the last block, with Mp the power of two >= M, thread t reads slot t % Mp of rows t / Mp,
+// t / Mp + blockDim/Mp, ... (consecutive threads read consecutive doubles; four rows' loads in
+// flight at a time). blockDim.x must be a multiple of 32, at most 32 kMaxWarps.
+template <class Op, int M>
+__device__ __forceinline__ const double* grid_total(const typename Op::V (&v)[M], double* red,
+                                                    unsigned int* counter, unsigned int b,
+                                                    unsigned int nb) {
+  constexpr int Mp = pow2_at_least(M);
+  constexpr long S = row_stride<M>();
+  using T = typename Op::Total;
+  __shared__ double s_d[kMaxWarps * Mp];
+  __shared__ double s_tot[Mp];
   __shared__ int s_last;
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int m = 0; m < M; ++m) red[(long)b * row_stride<M>() + m] = v[m];
-    __threadfence();
-    const unsigned int ticket = atomicAdd(counter, 1u);
-    s_last = (ticket == nb - 1);
+  const typename Op::V mine = block_total<Op, M>(v);
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  if (wid == 0) {
+    if (lane < M) red[(long)b * S + lane] = Op::value(mine);
+    __syncwarp();
+    if (lane == 0) {
+      __threadfence();
+      s_last = atomicAdd(counter, 1u) == nb - 1;
+    }
   }
   __syncthreads();
-  return s_last != 0;
-}
-
-// The same for a one-dimensional grid.
-template <int M>
-__device__ __forceinline__ bool publish_is_last(const double (&v)[M], double* red,
-                                                unsigned int* counter) {
-  return publish_is_last<M>(v, red, counter, blockIdx.x, gridDim.x);
-}
-
-// In the last block: reduce the partials of all blocks in a fixed order (valid in thread 0) and
-// re-arm the ticket counter for the next kernel. With Mp the power of two >= M, thread t reads
-// slot t % Mp (if below M) of rows t / Mp, t / Mp + blockDim/Mp, ... (consecutive threads read
-// consecutive doubles; four rows' loads in flight at a time), then the threads of each slot
-// combine through shuffles and shared memory.
-// blockDim.x must be a multiple of 32 (and at least Mp); smem: >= 32*M doubles.
-template <int M, bool IsMax>
-__device__ __forceinline__ void reduce_partials(double (&tot)[M], const double* red, int nblocks,
-                                                unsigned int* counter, double* smem) {
-  static_assert(M >= 1 && M <= 32, "at most 32 values per block");
-  constexpr int Mp = M <= 1 ? 1 : M <= 2 ? 2 : M <= 4 ? 4 : M <= 8 ? 8 : M <= 16 ? 16 : 32;
-  constexpr long S = row_stride<M>();
+  if (!s_last) return nullptr;
   __threadfence();
-  const int t = threadIdx.x, bd = blockDim.x;
-  const int m = t % Mp, rstep = bd / Mp;
-  auto op = [](double a, double b) { return IsMax ? max_nonneg(a, b) : a + b; };
+  const int m = t % Mp, rstep = blockDim.x / Mp, nr = (int)nb;
   double acc = 0.0;
-  int r = m < M ? t / Mp : nblocks;   // lanes past the M values read nothing
-  for (; r + 3 * rstep < nblocks; r += 4 * rstep) {
+  int r = m < M ? t / Mp : nr;   // lanes past the M values read nothing
+  for (; r + 3 * rstep < nr; r += 4 * rstep) {
     const double a0 = __ldcg(red + r * S + m);
     const double a1 = __ldcg(red + (r + rstep) * S + m);
     const double a2 = __ldcg(red + (r + 2 * rstep) * S + m);
     const double a3 = __ldcg(red + (r + 3 * rstep) * S + m);
-    acc = op(op(op(op(acc, a0), a1), a2), a3);
+    acc = T::add(T::add(acc, T::add(a0, a1)), T::add(a2, a3));
   }
-  for (; r < nblocks; r += rstep) acc = op(acc, __ldcg(red + r * S + m));
+  for (; r < nr; r += rstep) acc = T::add(acc, __ldcg(red + r * S + m));
 #pragma unroll
-  for (int off = 16; off >= Mp; off >>= 1) acc = op(acc, __shfl_down_sync(0xffffffffu, acc, off));
-  const int lane = t & 31, wid = t >> 5, nw = bd >> 5;
-  if (lane < M) smem[wid * M + lane] = acc;
+  for (int off = Mp; off < 32; off <<= 1) acc = T::add(acc, T::shfl_xor(acc, off));
+  if (lane < Mp) s_d[wid * Mp + lane] = acc;
   __syncthreads();
-  if (t == 0) {
-#pragma unroll
-    for (int q = 0; q < M; ++q) {
-      double v = 0.0;
-      for (int w = 0; w < nw; ++w) v = op(v, smem[w * M + q]);
-      tot[q] = v;
-    }
-    *counter = 0u;
+  if (wid == 0) {
+    const double tot = cross_warps<T, Mp>(s_d);
+    if (lane < Mp) s_tot[lane] = tot;
+    if (lane == 0) *counter = 0u;
   }
   __syncthreads();
+  return s_tot;
 }
 
 }  // namespace hosc

@@ -42,7 +42,6 @@ __global__ void k_nu_local(DevParams P, const double* __restrict__ th, double* n
 // One block: Nu_avg(z) (Simpson in y), its maximum, and the Simpson surface means.
 __global__ void k_nu_reduce(DevParams P, const double* nu_hot, const double* nu_cold,
                             double* nu_avg, double* scal) {
-  __shared__ double smem[32 * 2];
   const int N = P.N;
   const double hy = P.Ly / (N - 1), hz = P.Lz / (N - 1);
   for (int k = threadIdx.x; k < N; k += blockDim.x) {
@@ -58,7 +57,9 @@ __global__ void k_nu_reduce(DevParams P, const double* nu_hot, const double* nu_
     acc[0] += simpson_w(k, N, hz) * nu_avg[k];
     acc[1] += simpson_w(k, N, hz) * sc;
   }
-  block_reduce<2, false>(acc, smem);
+  const double sum = block_total<SumD, 2>(acc);   // thread m: sum m
+  __shared__ double s_sum[2];
+  if (threadIdx.x < 2) s_sum[threadIdx.x] = sum;
   __syncthreads();   // every nu_avg read above precedes its scaling
   for (int k = threadIdx.x; k < N; k += blockDim.x) nu_avg[k] /= P.Ly;
   __syncthreads();
@@ -67,8 +68,8 @@ __global__ void k_nu_reduce(DevParams P, const double* nu_hot, const double* nu_
     for (int k = 0; k < N; ++k) mx = fmax(mx, nu_avg[k]);
     const double area = P.Ly * P.Lz;
     scal[0] = mx;
-    scal[1] = acc[0] / area;
-    scal[2] = acc[1] / area;
+    scal[1] = s_sum[0] / area;
+    scal[2] = s_sum[1] / area;
   }
 }
 
@@ -80,7 +81,6 @@ __global__ void __launch_bounds__(kThreads) k_entropy(DevParams P, const double*
                                                      int store, double* red,
                                                      unsigned int* counter, int nblocks,
                                                      double* scal) {
-  __shared__ double smem[32 * 2];
   const int N = P.N;
   const long n3 = (long)N * N * N;
   const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -119,14 +119,8 @@ __global__ void __launch_bounds__(kThreads) k_entropy(DevParams P, const double*
     acc[0] = wgt * eht;
     acc[1] = wgt * eff;
   }
-  block_reduce<2, false>(acc, smem);
-  if (publish_is_last<2>(acc, red, counter)) {
-    double tot[2];
-    reduce_partials<2, false>(tot, red, nblocks, counter, smem);
-    if (threadIdx.x == 0) {
-      scal[3] = tot[0];
-      scal[4] = tot[1];
-    }
+  if (const double* tot = grid_total<SumD, 2>(acc, red, counter, blockIdx.x, (unsigned)nblocks)) {
+    if (threadIdx.x < 2) scal[3 + threadIdx.x] = tot[threadIdx.x];
   }
 }
 

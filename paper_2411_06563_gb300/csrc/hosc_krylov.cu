@@ -62,22 +62,12 @@ __device__ __forceinline__ double launch_bytes(const DevParams& P, const int don
   return word_bytes * ni * ni * ni * words;
 }
 
-// Block partial of M dot-product terms a[m] * b[m] in double (valid in thread 0).
-template <int M>
-__device__ __forceinline__ void block_partial(const double (&a)[M], const double (&b)[M],
-                                              double (&out)[M], double* smem) {
-#pragma unroll
-  for (int m = 0; m < M; ++m) out[m] = a[m] * b[m];
-  block_reduce<M, false>(out, smem);
-}
-
 // r = r_0 = rhs, x = 0, p = v = 0; ||r_0||^2 per system.
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_bicg_init(DevParams P, Fields F, int nblocks) {
-  __shared__ double smem[32 * 4];
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   int c;
-  T da[4] = {T(0), T(0), T(0), T(0)}, db[4] = {T(0), T(0), T(0), T(0)};
+  double dot[4] = {};
   if (interior_index(P, t, c)) {
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
@@ -89,32 +79,11 @@ __global__ void __launch_bounds__(kThreads) k_bicg_init(DevParams P, Fields F, i
       vec<T>(F.vk[0][s])[c] = T(0);
       vec<T>(F.vk[1][s])[c] = T(0);
       if (P.solver == 1) vec<T>(F.u0[s])[c] = T(0);
-      da[s] = r;
-      db[s] = r;
+      dot[s] = r * r;
     }
   }
-  double part[4];
-  block_partial<4>(da, db, part, smem);
-  if (publish_is_last<4>(part, F.red, F.counter)) {
-    double tot[4];
-    reduce_partials<4, false>(tot, F.red, nblocks, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        k.r0norm = sqrt(tot[s]);
-        k.rnorm = k.r0norm;
-        k.rho = tot[s];   // BiCGSTAB(2): rho_0 after the first cycle's rho_0 = -omega rho_0, j = 0
-        k.alpha = P.solver == 1 ? 0.0 : 1.0;
-        k.omega = 1.0;
-        k.beta = 0.0;
-        k.g1 = k.g2 = 0.0;
-        k.iters = 0;
-        k.status = 0;
-        // an inner pressure pass solves the momentum systems only
-        k.done = (k.r0norm == 0.0 || *F.halt || (s == 3 && P.inner_pass)) ? 1 : 0;
-      }
-    }
-  }
+  if (const double* tot = grid_total<SumD, 4>(dot, F.red, F.counter, blockIdx.x, nblocks))
+    finish_init(P, F, tot);
 }
 
 // End of one pass of the captured BiCGSTAB loop body: continue while a system is iterating.
@@ -130,7 +99,6 @@ __global__ void k_loop_cond(const KrylovScalars* ks, cudaGraphConditionalHandle 
 // partial r0 . v_new; last block: alpha = rho / (r0 . v).
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_bicg_pv(DevParams P, Fields F, int pp, int nblocks) {
-  __shared__ double smem[32 * 4];
   __shared__ T s_beta[4], s_omega[4];
   __shared__ int s_done[4];
   if (threadIdx.x < 4) {
@@ -143,7 +111,7 @@ __global__ void __launch_bounds__(kThreads) k_bicg_pv(DevParams P, Fields F, int
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   const int sy = P.N, sz = P.N * P.N;
   int c;
-  T da[4] = {T(0), T(0), T(0), T(0)}, db[4] = {T(0), T(0), T(0), T(0)};
+  double dot[4] = {};
   if (interior_index(P, t, c)) {
 #pragma unroll 1
     for (int s = 0; s < 4; ++s) {
@@ -160,28 +128,12 @@ __global__ void __launch_bounds__(kThreads) k_bicg_pv(DevParams P, Fields F, int
       const T vn = apply7<T>(A, c, pn[0], pn[1], pn[2], pn[3], pn[4], pn[5], pn[6]);
       vec<T>(F.pk[1 - pp][s])[c] = pn[0];
       vec<T>(F.vk[1 - pp][s])[c] = vn;
-      da[s] = vec<T>(F.rhs[s])[c];
-      db[s] = vn;
+      dot[s] = vec<T>(F.rhs[s])[c] * vn;
     }
   }
-  double part[4];
-  block_partial<4>(da, db, part, smem);
-  if (publish_is_last<4>(part, F.red, F.counter)) {
-    double tot[4];
-    reduce_partials<4, false>(tot, F.red, nblocks, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        if (tot[s] == 0.0 || !isfinite(tot[s])) {
-          k.done = 1;
-          k.status = HOSC_ENOCONV;
-          continue;
-        }
-        k.alpha = k.rho / tot[s];
-      }
-      F.alg_bytes[HOSC_K_BICG_PV] += launch_bytes(P, s_done, 6.0, 7.0, sizeof(T));
-    }
+  if (const double* tot = grid_total<SumD, 4>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
+    finish_pv(F, tot);
+    count_bytes(F, HOSC_K_BICG_PV, launch_bytes(P, s_done, 6.0, 7.0, sizeof(T)));
   }
 }
 
@@ -189,7 +141,6 @@ __global__ void __launch_bounds__(kThreads) k_bicg_pv(DevParams P, Fields F, int
 // last block: omega = (t . s)/(t . t) (0 when t = 0).
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_bicg_st(DevParams P, Fields F, int pp, int nblocks) {
-  __shared__ double smem[32 * 8];
   __shared__ T s_alpha[4];
   __shared__ int s_done[4];
   if (threadIdx.x < 4) {
@@ -202,8 +153,7 @@ __global__ void __launch_bounds__(kThreads) k_bicg_st(DevParams P, Fields F, int
   const int sy = P.N, sz = P.N * P.N;
   const int np = 1 - pp;   // buffers written by k_bicg_pv of this iteration
   int c;
-  T da[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-  T db[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+  double dot[8] = {};
   if (interior_index(P, t, c)) {
 #pragma unroll 1
     for (int s = 0; s < 4; ++s) {
@@ -218,25 +168,13 @@ __global__ void __launch_bounds__(kThreads) k_bicg_st(DevParams P, Fields F, int
       const T* const* A = (s < 3) ? ops<T>(F.Am) : ops<T>(F.Ae);
       const T tv = apply7<T>(A, c, sv[0], sv[1], sv[2], sv[3], sv[4], sv[5], sv[6]);
       vec<T>(F.t[s])[c] = tv;
-      da[2 * s] = tv;
-      db[2 * s] = sv[0];
-      da[2 * s + 1] = tv;
-      db[2 * s + 1] = tv;
+      dot[s] = tv * sv[0];
+      dot[4 + s] = tv * tv;
     }
   }
-  double part[8];
-  block_partial<8>(da, db, part, smem);
-  if (publish_is_last<8>(part, F.red, F.counter)) {
-    double tot[8];
-    reduce_partials<8, false>(tot, F.red, nblocks, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        k.omega = tot[2 * s + 1] > 0.0 ? tot[2 * s] / tot[2 * s + 1] : 0.0;
-      }
-      F.alg_bytes[HOSC_K_BICG_ST] += launch_bytes(P, s_done, 3.0, 7.0, sizeof(T));
-    }
+  if (const double* tot = grid_total<SumD, 8>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
+    finish_st(F, tot);
+    count_bytes(F, HOSC_K_BICG_ST, launch_bytes(P, s_done, 3.0, 7.0, sizeof(T)));
   }
 }
 
@@ -244,7 +182,6 @@ __global__ void __launch_bounds__(kThreads) k_bicg_st(DevParams P, Fields F, int
 // last block: convergence test, breakdown test, beta and rho for the next iteration.
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_bicg_xr(DevParams P, Fields F, int pp, int nblocks) {
-  __shared__ double smem[32 * 8];
   __shared__ T s_alpha[4], s_omega[4];
   __shared__ int s_done[4];
   if (threadIdx.x < 4) {
@@ -257,8 +194,7 @@ __global__ void __launch_bounds__(kThreads) k_bicg_xr(DevParams P, Fields F, int
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   const int np = 1 - pp;
   int c;
-  T da[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-  T db[8] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+  double dot[8] = {};
   if (interior_index(P, t, c)) {
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
@@ -270,38 +206,13 @@ __global__ void __launch_bounds__(kThreads) k_bicg_xr(DevParams P, Fields F, int
       x[c] = x[c] + a * vec<T>(F.pk[np][s])[c] + om * sv;
       const T rn = sv - om * vec<T>(F.t[s])[c];
       r[c] = rn;
-      da[2 * s] = vec<T>(F.rhs[s])[c];
-      db[2 * s] = rn;
-      da[2 * s + 1] = rn;
-      db[2 * s + 1] = rn;
+      dot[s] = vec<T>(F.rhs[s])[c] * rn;
+      dot[4 + s] = rn * rn;
     }
   }
-  double part[8];
-  block_partial<8>(da, db, part, smem);
-  if (publish_is_last<8>(part, F.red, F.counter)) {
-    double tot[8];
-    reduce_partials<8, false>(tot, F.red, nblocks, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        const double rho_new = tot[2 * s];
-        k.rnorm = sqrt(tot[2 * s + 1]);
-        k.iters += 1;
-        if (k.rnorm <= P.tol_lin * k.r0norm) {
-          k.done = 1;
-          k.status = 0;
-        } else if (!isfinite(k.rnorm) || k.iters >= P.max_lin_iter || rho_new == 0.0 ||
-                   k.omega == 0.0) {
-          k.done = 1;
-          k.status = HOSC_ENOCONV;
-        } else {
-          k.beta = (rho_new / k.rho) * (k.alpha / k.omega);
-          k.rho = rho_new;
-        }
-      }
-      F.alg_bytes[HOSC_K_BICG_XR] += launch_bytes(P, s_done, 8.0, 0.0, sizeof(T));
-    }
+  if (const double* tot = grid_total<SumD, 8>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
+    finish_xr(P, F, tot);
+    count_bytes(F, HOSC_K_BICG_XR, launch_bytes(P, s_done, 8.0, 0.0, sizeof(T)));
   }
 }
 
@@ -360,19 +271,29 @@ __device__ __forceinline__ void b2_fail(KrylovScalars& k) {
   k.status = HOSC_ENOCONV;
 }
 
+// rt . u (slots 0..3): alpha = rho / (rt . u).
+__device__ __forceinline__ void b2_finish_alpha(const Fields& F, const double* tot) {
+  if (threadIdx.x >= 4) return;
+  KrylovScalars& k = F.ks[threadIdx.x];
+  const int done = k.done;
+  const double rho = k.rho, d = tot[threadIdx.x];
+  if (done) return;
+  if (d == 0.0 || !isfinite(d)) b2_fail(k);
+  else k.alpha = rho / d;
+}
+
 __device__ __forceinline__ const double* const* b2_op(const Fields& F, int s) {
   return (s < 3) ? ops<double>(F.Am) : ops<double>(F.Ae);
 }
 
 // B1
 __global__ void __launch_bounds__(kThreads) k_b2_u1(DevParams P, Fields F, int cp, int nblocks) {
-  __shared__ double smem[32 * 4];
   __shared__ B2Shared sh;
   if (b2_load(F, sh)) return;
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   const int sy = P.N, sz = P.N * P.N;
   int c;
-  double da[4] = {0, 0, 0, 0}, db[4] = {0, 0, 0, 0};
+  double dot[4] = {};
   if (interior_index(P, t, c)) {
     int nb[7];
     nbrs7(c, sy, sz, nb);
@@ -388,39 +309,23 @@ __global__ void __launch_bounds__(kThreads) k_b2_u1(DevParams P, Fields F, int c
       const double u1 = apply7<double>(b2_op(F, s), c, un[0], un[1], un[2], un[3], un[4], un[5],
                                        un[6]);
       F.vk[0][s][c] = u1;
-      da[s] = F.rhs[s][c];
-      db[s] = u1;
+      dot[s] = F.rhs[s][c] * u1;
     }
   }
-  double part[4];
-  block_partial<4>(da, db, part, smem);
-  if (publish_is_last<4>(part, F.red, F.counter)) {
-    double tot[4];
-    reduce_partials<4, false>(tot, F.red, nblocks, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        if (tot[s] == 0.0 || !isfinite(tot[s])) {
-          b2_fail(k);
-          continue;
-        }
-        k.alpha = k.rho / tot[s];
-      }
-      F.alg_bytes[HOSC_K_BICG_PV] += launch_bytes(P, sh.done, 4.0, 7.0, sizeof(double));
-    }
+  if (const double* tot = grid_total<SumD, 4>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
+    b2_finish_alpha(F, tot);
+    count_bytes(F, HOSC_K_BICG_PV, launch_bytes(P, sh.done, 4.0, 7.0, sizeof(double)));
   }
 }
 
 // B2
 __global__ void __launch_bounds__(kThreads) k_b2_r1(DevParams P, Fields F, int cp, int nblocks) {
-  __shared__ double smem[32 * 4];
   __shared__ B2Shared sh;
   if (b2_load(F, sh)) return;
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   const int sy = P.N, sz = P.N * P.N;
   int c;
-  double da[4] = {0, 0, 0, 0}, db[4] = {0, 0, 0, 0};
+  double dot[4] = {};
   if (interior_index(P, t, c)) {
     int nb[7];
     nbrs7(c, sy, sz, nb);
@@ -441,40 +346,34 @@ __global__ void __launch_bounds__(kThreads) k_b2_r1(DevParams P, Fields F, int c
       const double u0 = r0[c] - b * F.u0[s][c];
       F.u0[s][c] = u0;
       F.x[s][c] += a * u0;
-      da[s] = F.rhs[s][c];
-      db[s] = r1;
+      dot[s] = F.rhs[s][c] * r1;
     }
   }
-  double part[4];
-  block_partial<4>(da, db, part, smem);
-  if (publish_is_last<4>(part, F.red, F.counter)) {
-    double tot[4];
-    reduce_partials<4, false>(tot, F.red, nblocks, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        if (k.rho == 0.0 || !isfinite(tot[s])) {
+  if (const double* tot = grid_total<SumD, 4>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
+    if (threadIdx.x < 4) {
+      KrylovScalars& k = F.ks[threadIdx.x];
+      const double rho1 = tot[threadIdx.x];
+      if (!k.done) {
+        if (k.rho == 0.0 || !isfinite(rho1)) {
           b2_fail(k);
-          continue;
+        } else {
+          k.beta = k.alpha * rho1 / k.rho;
+          k.rho = rho1;
         }
-        k.beta = k.alpha * tot[s] / k.rho;
-        k.rho = tot[s];
       }
-      F.alg_bytes[HOSC_K_BICG_ST] += launch_bytes(P, sh.done, 9.0, 7.0, sizeof(double));
     }
+    count_bytes(F, HOSC_K_BICG_ST, launch_bytes(P, sh.done, 9.0, 7.0, sizeof(double)));
   }
 }
 
 // B3
 __global__ void __launch_bounds__(kThreads) k_b2_u2(DevParams P, Fields F, int cp, int nblocks) {
-  __shared__ double smem[32 * 4];
   __shared__ B2Shared sh;
   if (b2_load(F, sh)) return;
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   const int sy = P.N, sz = P.N * P.N;
   int c;
-  double da[4] = {0, 0, 0, 0}, db[4] = {0, 0, 0, 0};
+  double dot[4] = {};
   if (interior_index(P, t, c)) {
     int nb[7];
     nbrs7(c, sy, sz, nb);
@@ -493,46 +392,28 @@ __global__ void __launch_bounds__(kThreads) k_b2_u2(DevParams P, Fields F, int c
                                        un[6]);
       F.vk[1][s][c] = un[0];
       F.u2[s][c] = u2;
-      da[s] = F.rhs[s][c];
-      db[s] = u2;
+      dot[s] = F.rhs[s][c] * u2;
     }
   }
-  double part[4];
-  block_partial<4>(da, db, part, smem);
-  if (publish_is_last<4>(part, F.red, F.counter)) {
-    double tot[4];
-    reduce_partials<4, false>(tot, F.red, nblocks, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        if (tot[s] == 0.0 || !isfinite(tot[s])) {
-          b2_fail(k);
-          continue;
-        }
-        k.alpha = k.rho / tot[s];
-      }
-      F.alg_bytes[HOSC_K_BICG_PV] += launch_bytes(P, sh.done, 8.0, 7.0, sizeof(double));
-    }
+  if (const double* tot = grid_total<SumD, 4>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
+    b2_finish_alpha(F, tot);
+    count_bytes(F, HOSC_K_BICG_PV, launch_bytes(P, sh.done, 8.0, 7.0, sizeof(double)));
   }
 }
 
 // B4
 __global__ void __launch_bounds__(kThreads) k_b2_r2(DevParams P, Fields F, int cp, int nblocks) {
-  __shared__ double smem[32 * 20];
   __shared__ B2Shared sh;
   if (b2_load(F, sh)) return;
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   const int sy = P.N, sz = P.N * P.N;
   int c;
   // per system: r1.r1, r1.r2, r2.r2, r0.r1, r0.r2
-  double da[20], db[20];
-#pragma unroll
-  for (int m = 0; m < 20; ++m) da[m] = db[m] = 0.0;
+  double dot[20] = {};
   if (interior_index(P, t, c)) {
     int nb[7];
     nbrs7(c, sy, sz, nb);
-#pragma unroll 1
+#pragma unroll   // dot[] is indexed by the system: unrolled, it stays in registers
     for (int s = 0; s < 4; ++s) {
       if (sh.done[s]) continue;
       double* r0 = cp ? F.r[s] : F.t[s];
@@ -549,49 +430,42 @@ __global__ void __launch_bounds__(kThreads) k_b2_r2(DevParams P, Fields F, int c
       F.pk[1][s][c] = rn[0];
       F.r2[s][c] = r2;
       F.x[s][c] += a * F.u0[s][c];
-      const double d0[5] = {rn[0], rn[0], r2, r0c, r0c}, d1[5] = {rn[0], r2, r2, rn[0], r2};
-#pragma unroll
-      for (int m = 0; m < 5; ++m) {
-        da[5 * s + m] = d0[m];
-        db[5 * s + m] = d1[m];
-      }
+      dot[5 * s] = rn[0] * rn[0];
+      dot[5 * s + 1] = rn[0] * r2;
+      dot[5 * s + 2] = r2 * r2;
+      dot[5 * s + 3] = r0c * rn[0];
+      dot[5 * s + 4] = r0c * r2;
     }
   }
-  double part[20];
-  block_partial<20>(da, db, part, smem);
-  if (publish_is_last<20>(part, F.red, F.counter)) {
-    double tot[20];
-    reduce_partials<20, false>(tot, F.red, nblocks, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        const double* d = tot + 5 * s;   // r1.r1, r1.r2, r2.r2, r0.r1, r0.r2
-        const double sig1 = d[0];
-        const double tau = sig1 > 0.0 ? d[1] / sig1 : 0.0;
-        const double sig2 = d[2] - tau * d[1];   // |r_2 - tau r_1|^2
+  if (const double* tot = grid_total<SumD, 20>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
+    if (threadIdx.x < 4) {
+      KrylovScalars& k = F.ks[threadIdx.x];
+      const double* d = tot + 5 * threadIdx.x;   // r1.r1, r1.r2, r2.r2, r0.r1, r0.r2
+      const double sig1 = d[0];
+      const double tau = sig1 > 0.0 ? d[1] / sig1 : 0.0;
+      const double sig2 = d[2] - tau * d[1];   // |r_2 - tau r_1|^2
+      if (!k.done) {
         if (!(sig1 > 0.0) || !(sig2 > 0.0) || !isfinite(sig2)) {
           b2_fail(k);
-          continue;
+        } else {
+          const double gp1 = d[3] / sig1, g2 = (d[4] - tau * d[3]) / sig2;
+          k.g2 = g2;
+          k.g1 = gp1 - tau * g2;
+          k.omega = g2;
         }
-        const double gp1 = d[3] / sig1, g2 = (d[4] - tau * d[3]) / sig2;
-        k.g2 = g2;
-        k.g1 = gp1 - tau * g2;
-        k.omega = g2;
       }
-      F.alg_bytes[HOSC_K_BICG_ST] += launch_bytes(P, sh.done, 10.0, 7.0, sizeof(double));
     }
+    count_bytes(F, HOSC_K_BICG_ST, launch_bytes(P, sh.done, 10.0, 7.0, sizeof(double)));
   }
 }
 
 // B5
 __global__ void __launch_bounds__(kThreads) k_b2_mr(DevParams P, Fields F, int cp, int nblocks) {
-  __shared__ double smem[32 * 8];
   __shared__ B2Shared sh;
   if (b2_load(F, sh)) return;
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
   int c;
-  double da[8] = {0, 0, 0, 0, 0, 0, 0, 0}, db[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  double dot[8] = {};
   if (interior_index(P, t, c)) {
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
@@ -603,37 +477,30 @@ __global__ void __launch_bounds__(kThreads) k_b2_mr(DevParams P, Fields F, int c
       const double rn = r0c - g1 * r1 - g2 * r2;
       r0[c] = rn;
       F.u0[s][c] -= g1 * F.vk[1][s][c] + g2 * F.u2[s][c];
-      da[2 * s] = F.rhs[s][c];
-      db[2 * s] = rn;
-      da[2 * s + 1] = rn;
-      db[2 * s + 1] = rn;
+      dot[s] = F.rhs[s][c] * rn;
+      dot[4 + s] = rn * rn;
     }
   }
-  double part[8];
-  block_partial<8>(da, db, part, smem);
-  if (publish_is_last<8>(part, F.red, F.counter)) {
-    double tot[8];
-    reduce_partials<8, false>(tot, F.red, nblocks, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        const double rho1 = tot[2 * s];
-        k.rnorm = sqrt(tot[2 * s + 1]);
+  if (const double* tot = grid_total<SumD, 8>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
+    if (threadIdx.x < 4) {
+      KrylovScalars& k = F.ks[threadIdx.x];
+      if (!k.done) {
+        const double rho1 = tot[threadIdx.x], rnorm = sqrt(tot[4 + threadIdx.x]);
+        k.rnorm = rnorm;
         k.iters += 2;
         const double rho0 = -k.omega * k.rho;
-        if (k.rnorm <= P.tol_lin * k.r0norm) {
+        if (rnorm <= P.tol_lin * k.r0norm) {
           k.done = 1;
           k.status = 0;
-        } else if (!isfinite(k.rnorm) || k.iters >= P.max_lin_iter || rho0 == 0.0) {
+        } else if (!isfinite(rnorm) || k.iters >= P.max_lin_iter || rho0 == 0.0) {
           b2_fail(k);
         } else {
           k.beta = k.alpha * rho1 / rho0;
           k.rho = rho1;
         }
       }
-      F.alg_bytes[HOSC_K_BICG_XR] += launch_bytes(P, sh.done, 11.0, 0.0, sizeof(double));
     }
+    count_bytes(F, HOSC_K_BICG_XR, launch_bytes(P, sh.done, 11.0, 0.0, sizeof(double)));
   }
 }
 
@@ -650,7 +517,6 @@ __global__ void __launch_bounds__(kThreads) k_b2_mr(DevParams P, Fields F, int c
 // (kr, kr1) since k6_a reads it at the neighbours while writing it.
 
 __global__ void __launch_bounds__(kThreads) k6_init(DevParams P, Fields F) {
-  __shared__ double smem[32 * 4];
   const int N = P.N;
   const int n3 = N * N * N;
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -670,33 +536,12 @@ __global__ void __launch_bounds__(kThreads) k6_init(DevParams P, Fields F) {
     F.kv[1][c] = z;
     ff_dot4(acc, r, r);
   }
-  double part[4];
-  block_ff<4>(acc, part, smem);
-  if (publish_is_last<4>(part, F.red, F.counter)) {
-    double tot[4];
-    reduce_partials<4, false>(tot, F.red, gridDim.x, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        k.r0norm = sqrt(tot[s]);
-        k.rnorm = k.r0norm;
-        k.rho = tot[s];
-        k.alpha = 0.0;   // the first k6_a then leaves x = 0, r = r_0 and sets p = r_0
-        k.omega = 0.0;
-        k.beta = 0.0;
-        k.iters = 0;
-        k.pad = 0;       // no x, r update applied yet
-        k.status = 0;
-        // an inner pressure pass solves the momentum systems only
-        k.done = (k.r0norm == 0.0 || *F.halt || (s == 3 && P.inner_pass)) ? 1 : 0;
-      }
-    }
-  }
+  if (const double* tot = grid_total<SumFF, 4>(acc, F.red, F.counter, blockIdx.x, gridDim.x))
+    finish_init(P, F, tot);
 }
 
 template <int MinB>
 __global__ void __launch_bounds__(256, MinB) k6_a(DevParams P, Fields F, int pp) {
-  __shared__ double smem[32 * 8];
   __shared__ Scal4 sc;
   load_scalars(F.ks, sc);
   if (sc.all_done) return;   // uniform over the grid
@@ -738,41 +583,35 @@ __global__ void __launch_bounds__(256, MinB) k6_a(DevParams P, Fields F, int pp)
       pc = pz;
     }
   }
-  double part[12];
-  block_ff<12>(acc, part, smem);
-  if (publish_is_last<12>(part, F.red, F.counter, block_id(), block_count())) {
-    double tot[12];
-    reduce_partials<12, false>(tot, F.red, block_count(), F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
+  if (const double* tot =
+          grid_total<SumFF, 12>(acc, F.red, F.counter, block_id(), block_count())) {
+    if (threadIdx.x < 4) {
+      const int s = threadIdx.x;
+      KrylovScalars& k = F.ks[s];
+      if (!k.done) {
         k.rnorm = sqrt(tot[4 + s]);
         if (k.pad) k.iters += 1;
         k.pad = 1;
         if (k.rnorm <= P.tol_lin * k.r0norm) {
           k.done = 1;
           k.status = 0;
-          continue;
-        }
-        if (!isfinite(k.rnorm) || k.iters >= P.max_lin_iter || tot[s] == 0.0 ||
-            !isfinite(tot[s])) {
+        } else if (!isfinite(k.rnorm) || k.iters >= P.max_lin_iter || tot[s] == 0.0 ||
+                   !isfinite(tot[s])) {
           k.done = 1;
           k.status = HOSC_ENOCONV;
-          continue;
+        } else {
+          k.rho = tot[8 + s];   // rho_i = r_0 . r_i from the stored r_i
+          k.alpha = k.rho / tot[s];
         }
-        k.rho = tot[8 + s];   // rho_i = r_0 . r_i from the stored r_i
-        k.alpha = k.rho / tot[s];
       }
-      // r p v t x r0 in, x r p v out, the compact operators
-      F.alg_bytes[HOSC_K_BICG_PV] += bytes4(P, 10.0 + op_words(ene));
     }
+    // r p v t x r0 in, x r p v out, the compact operators
+    count_bytes(F, HOSC_K_BICG_PV, bytes4(P, 10.0 + op_words(ene)));
   }
 }
 
 template <int MinB>
 __global__ void __launch_bounds__(256, MinB) k6_b(DevParams P, Fields F, int pp) {
-  __shared__ double smem[32 * 8];
   __shared__ Scal4 sc;
   load_scalars(F.ks, sc);
   if (sc.all_done) return;
@@ -802,30 +641,27 @@ __global__ void __launch_bounds__(256, MinB) k6_b(DevParams P, Fields F, int pp)
       sc0 = sz;
     }
   }
-  double part[16];
-  block_ff<16>(acc, part, smem);
-  if (publish_is_last<16>(part, F.red, F.counter, block_id(), block_count())) {
-    double tot[16];
-    reduce_partials<16, false>(tot, F.red, block_count(), F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        const double ts = tot[s], tt = tot[4 + s], r0s = tot[8 + s], r0t = tot[12 + s];
-        const double om = tt > 0.0 ? ts / tt : 0.0;
-        const double rho_next = r0s - om * r0t;   // r_0 . (s - omega t) = r_0 . r_{i+1}
+  if (const double* tot =
+          grid_total<SumFF, 16>(acc, F.red, F.counter, block_id(), block_count())) {
+    if (threadIdx.x < 4) {
+      const int s = threadIdx.x;
+      KrylovScalars& k = F.ks[s];
+      const double ts = tot[s], tt = tot[4 + s], r0s = tot[8 + s], r0t = tot[12 + s];
+      const double om = tt > 0.0 ? ts / tt : 0.0;
+      const double rho_next = r0s - om * r0t;   // r_0 . (s - omega t) = r_0 . r_{i+1}
+      if (!k.done) {
         if (om == 0.0 || rho_next == 0.0 || !isfinite(rho_next)) {
           k.done = 1;
           k.status = HOSC_ENOCONV;
-          continue;
+        } else {
+          // k6_a recomputes rho_{i+1} from the stored r_{i+1}; this value only sets beta
+          k.beta = (rho_next / k.rho) * (k.alpha / om);
+          k.omega = om;
         }
-        // k6_a recomputes rho_{i+1} from the stored r_{i+1}; this value only sets beta
-        k.beta = (rho_next / k.rho) * (k.alpha / om);
-        k.omega = om;
       }
-      // r v r0 in, t out, the compact operators
-      F.alg_bytes[HOSC_K_BICG_ST] += bytes4(P, 4.0 + op_words(ene));
     }
+    // r v r0 in, t out, the compact operators
+    count_bytes(F, HOSC_K_BICG_ST, bytes4(P, 4.0 + op_words(ene)));
   }
 }
 
@@ -923,7 +759,6 @@ __device__ __forceinline__ Op4 staged_op(const float4* sq, const StageLayout& L,
 // Staged p/v kernel (same arithmetic as k4_pv).
 __global__ void __launch_bounds__(256) k5_pv(DevParams P, Fields F, int pp) {
   extern __shared__ float4 ring[];
-  __shared__ double smem[32 * 4];
   __shared__ Scal4 sc;
   load_scalars(F.ks, sc);
   if (sc.all_done) return;
@@ -967,33 +802,17 @@ __global__ void __launch_bounds__(256) k5_pv(DevParams P, Fields F, int pp) {
     pc = pz;
     __syncthreads();   // the stage of plane k is free for plane k+4
   }
-  double part[4];
-  block_ff<4>(acc, part, smem);
   const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
   const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
-  if (publish_is_last<4>(part, F.red, F.counter, bid, nb)) {
-    double tot[4];
-    reduce_partials<4, false>(tot, F.red, nb, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        if (tot[s] == 0.0 || !isfinite(tot[s])) {
-          k.done = 1;
-          k.status = HOSC_ENOCONV;
-          continue;
-        }
-        k.alpha = k.rho / tot[s];
-      }
-      F.alg_bytes[HOSC_K_BICG_PV] += bytes4(P, 6.0 + op_words(ene));
-    }
+  if (const double* tot = grid_total<SumFF, 4>(acc, F.red, F.counter, bid, nb)) {
+    finish_pv(F, tot);
+    count_bytes(F, HOSC_K_BICG_PV, bytes4(P, 6.0 + op_words(ene)));
   }
 }
 
 // Staged s/t kernel (same arithmetic as k4_st).
 __global__ void __launch_bounds__(256) k5_st(DevParams P, Fields F, int pp) {
   extern __shared__ float4 ring[];
-  __shared__ double smem[32 * 8];
   __shared__ Scal4 sc;
   load_scalars(F.ks, sc);
   if (sc.all_done) return;
@@ -1034,21 +853,11 @@ __global__ void __launch_bounds__(256) k5_st(DevParams P, Fields F, int pp) {
     sc0 = sz;
     __syncthreads();
   }
-  double part[8];
-  block_ff<8>(acc, part, smem);
   const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
   const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
-  if (publish_is_last<8>(part, F.red, F.counter, bid, nb)) {
-    double tot[8];
-    reduce_partials<8, false>(tot, F.red, nb, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        k.omega = tot[4 + s] > 0.0 ? tot[s] / tot[4 + s] : 0.0;
-      }
-      F.alg_bytes[HOSC_K_BICG_ST] += bytes4(P, 3.0 + op_words(ene));
-    }
+  if (const double* tot = grid_total<SumFF, 8>(acc, F.red, F.counter, bid, nb)) {
+    finish_st(F, tot);
+    count_bytes(F, HOSC_K_BICG_ST, bytes4(P, 3.0 + op_words(ene)));
   }
 }
 
@@ -1112,7 +921,6 @@ void launch_bicg_init(const DevParams& P, const Fields& F, cudaStream_t s) {
 // flight. Same arithmetic and float-float partials as k4_xr; one block partial per block.
 template <int U>
 __global__ void __launch_bounds__(256) k8_xr(DevParams P, Fields F, int pp) {
-  __shared__ double smem[32 * 8];
   __shared__ Scal4 sc;
   pdl_wait_and_release();
   load_scalars(F.ks, sc);
@@ -1160,10 +968,10 @@ __global__ void __launch_bounds__(256) k8_xr(DevParams P, Fields F, int pp) {
     ff_dot4(acc, __ldg(R0 + c), rn);
     ff_dot4(acc + 4, rn, rn);
   }
-  double part[8];
-  block_ff<8>(acc, part, smem);
-  if (publish_is_last<8>(part, F.red, F.counter, blockIdx.x, gridDim.x))
-    xr_finish(P, F, gridDim.x, smem);
+  if (const double* tot = grid_total<SumFF, 8>(acc, F.red, F.counter, blockIdx.x, gridDim.x)) {
+    finish_xr(P, F, tot);
+    count_bytes(F, HOSC_K_BICG_XR, bytes4(P, 8.0));   // r v p x t r0 in, x r out
+  }
 }
 
 // Blocks of the flat x/r kernel: resident blocks of one wave.

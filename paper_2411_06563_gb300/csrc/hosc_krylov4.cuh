@@ -45,40 +45,17 @@ __device__ __forceinline__ FF ff_add(FF a, FF b) {
   return r;
 }
 
-__device__ __forceinline__ FF ff_shfl_down(FF a, int off) {
-  FF r;
-  r.hi = __shfl_down_sync(0xffffffffu, a.hi, off);
-  r.lo = __shfl_down_sync(0xffffffffu, a.lo, off);
-  return r;
-}
-
-// Block sum of M per-thread float-float accumulators; thread 0 receives the totals in double.
-template <int M>
-__device__ __forceinline__ void block_ff(FF (&acc)[M], double (&out)[M], double* smem) {
-  FF* fs = reinterpret_cast<FF*>(smem);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nw = (blockDim.x + 31) >> 5;
-#pragma unroll
-  for (int m = 0; m < M; ++m) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc[m] = ff_add(acc[m], ff_shfl_down(acc[m], off));
+// Sums of float-float values; the blocks' totals are added in double.
+struct SumFF {
+  using V = FF;
+  using Total = SumD;
+  static __device__ __forceinline__ V zero() { return FF{0.0f, 0.0f}; }
+  static __device__ __forceinline__ V add(V a, V b) { return ff_add(a, b); }
+  static __device__ __forceinline__ V shfl_xor(V a, int m) {
+    return FF{__shfl_xor_sync(0xffffffffu, a.hi, m), __shfl_xor_sync(0xffffffffu, a.lo, m)};
   }
-  if (lane == 0) {
-#pragma unroll
-    for (int m = 0; m < M; ++m) fs[wid * M + m] = acc[m];
-  }
-  __syncthreads();
-  if (wid == 0) {
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-      FF x = (lane < nw) ? fs[lane * M + m] : FF{0.0f, 0.0f};
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) x = ff_add(x, ff_shfl_down(x, off));
-      out[m] = (double)x.hi + (double)x.lo;
-    }
-  }
-  __syncthreads();
-}
+  static __device__ __forceinline__ double value(V a) { return (double)a.hi + (double)a.lo; }
+};
 
 // ------------------------------------------------------------------ interleaved FP32 solve
 
@@ -188,24 +165,101 @@ struct Scal4 {
   int all_done;
 };
 
+// The first warp reads the four systems' scalars, one lane a system.
 __device__ __forceinline__ void load_scalars(const KrylovScalars* ks, Scal4& sc) {
-  if (threadIdx.x == 0) {
-    float a[4], b[4], om[4];
-    int all = 1;
-    for (int s = 0; s < 4; ++s) {
-      const int d = ks[s].done;
+  if (threadIdx.x < 32) {
+    const int s = threadIdx.x;
+    int d = 1;
+    if (s < 4) {
+      const double a = ks[s].alpha, b = ks[s].beta, om = ks[s].omega;
+      d = ks[s].done;
       sc.done[s] = d;
-      all &= d;
-      a[s] = d ? 0.f : (float)ks[s].alpha;
-      b[s] = d ? 0.f : (float)ks[s].beta;
-      om[s] = d ? 0.f : (float)ks[s].omega;
+      (&sc.a.x)[s] = d ? 0.f : (float)a;
+      (&sc.b.x)[s] = d ? 0.f : (float)b;
+      (&sc.om.x)[s] = d ? 0.f : (float)om;
     }
-    sc.a = make_float4(a[0], a[1], a[2], a[3]);
-    sc.b = make_float4(b[0], b[1], b[2], b[3]);
-    sc.om = make_float4(om[0], om[1], om[2], om[3]);
-    sc.all_done = all;
+    const int all = __all_sync(0xffffffffu, d != 0);
+    if (s == 0) sc.all_done = all;
   }
   __syncthreads();
+}
+
+// ---- ends of the Krylov kernels: the last block of a launch sets the scalars the next kernel
+// needs from the launch's totals, one thread a system (each an FP64 divide or square root and a few
+// dependent reads: one after another they took 4 us of a 20 us launch on a 41^3 grid).
+
+// r_0 . r_0 of each system: the solve starts.
+__device__ __forceinline__ void finish_init(const DevParams& P, const Fields& F, const double* tot) {
+  if (threadIdx.x >= 4) return;
+  const int s = threadIdx.x;
+  KrylovScalars& k = F.ks[s];
+  const int halt = *F.halt;
+  const double norm = sqrt(tot[s]);
+  k.r0norm = norm;
+  k.rnorm = norm;
+  k.rho = tot[s];   // BiCGSTAB(2): rho_0 after the first cycle's rho_0 = -omega rho_0, j = 0
+  // the first kernel of the merged form then leaves x = 0, r = r_0 and sets p = r_0
+  k.alpha = (P.krylov_fp32 ? P.merged : P.solver) ? 0.0 : 1.0;
+  k.omega = (P.krylov_fp32 && P.merged) ? 0.0 : 1.0;
+  k.beta = 0.0;
+  k.g1 = k.g2 = 0.0;
+  k.iters = 0;
+  k.pad = 0;
+  k.status = 0;
+  // an inner pressure pass solves the momentum systems only
+  k.done = (norm == 0.0 || halt || (s == 3 && P.inner_pass)) ? 1 : 0;
+}
+
+// r_0 . v of each system: alpha = rho / (r_0 . v).
+__device__ __forceinline__ void finish_pv(const Fields& F, const double* tot) {
+  if (threadIdx.x >= 4) return;
+  KrylovScalars& k = F.ks[threadIdx.x];
+  const int done = k.done;
+  const double rho = k.rho, d = tot[threadIdx.x];
+  if (done) return;
+  if (d == 0.0 || !isfinite(d)) {
+    k.done = 1;
+    k.status = HOSC_ENOCONV;
+  } else {
+    k.alpha = rho / d;
+  }
+}
+
+// t . s (slots 0..3) and t . t (4..7): omega = (t . s) / (t . t), 0 when t = 0.
+__device__ __forceinline__ void finish_st(const Fields& F, const double* tot) {
+  if (threadIdx.x >= 4) return;
+  KrylovScalars& k = F.ks[threadIdx.x];
+  if (k.done) return;
+  const double ts = tot[threadIdx.x], tt = tot[4 + threadIdx.x];
+  k.omega = tt > 0.0 ? ts / tt : 0.0;
+}
+
+// r_0 . r (slots 0..3) and r . r (4..7): the convergence and breakdown tests, beta and rho of the
+// next iteration.
+__device__ __forceinline__ void finish_xr(const DevParams& P, const Fields& F, const double* tot) {
+  if (threadIdx.x >= 4) return;
+  KrylovScalars& k = F.ks[threadIdx.x];
+  const int done = k.done, iters = k.iters + 1;
+  const double rho = k.rho, alpha = k.alpha, omega = k.omega, r0norm = k.r0norm;
+  if (done) return;
+  const double rho_new = tot[threadIdx.x], rnorm = sqrt(tot[4 + threadIdx.x]);
+  k.rnorm = rnorm;
+  k.iters = iters;
+  if (rnorm <= P.tol_lin * r0norm) {
+    k.done = 1;
+    k.status = 0;
+  } else if (!isfinite(rnorm) || iters >= P.max_lin_iter || rho_new == 0.0 || omega == 0.0) {
+    k.done = 1;
+    k.status = HOSC_ENOCONV;
+  } else {
+    k.beta = (rho_new / rho) * (alpha / omega);
+    k.rho = rho_new;
+  }
+}
+
+// Add a launch's algorithmic bytes (a thread that takes no part in the ends above).
+__device__ __forceinline__ void count_bytes(const Fields& F, int kid, double bytes) {
+  if (threadIdx.x == blockDim.x - 1) atomicAdd(F.alg_bytes + kid, bytes);
 }
 
 // Algorithmic bytes of one interleaved launch: words (float4 per interior node) moved.
@@ -228,7 +282,6 @@ __device__ __forceinline__ void pdl_wait_and_release() {
 // Returns true in the block that finished the launch's reduction (its scalars are then final).
 __device__ __forceinline__ bool k4_init_body(const DevParams& P, const Fields& F, unsigned vbx,
                                              unsigned vnb) {
-  __shared__ double smem[32 * 4];
   const unsigned N = P.N;
   const unsigned n3 = N * N * N;
   FF acc[4] = {};
@@ -248,28 +301,9 @@ __device__ __forceinline__ bool k4_init_body(const DevParams& P, const Fields& F
     F.kv[1][c] = z;
     ff_dot4(acc, r, r);
   }
-  double part[4];
-  block_ff<4>(acc, part, smem);
-  if (!publish_is_last<4>(part, F.red, F.counter, vbx, vnb)) return false;
-  {
-    double tot[4];
-    reduce_partials<4, false>(tot, F.red, vnb, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        k.r0norm = sqrt(tot[s]);
-        k.rnorm = k.r0norm;
-        k.rho = tot[s];
-        k.alpha = 1.0;
-        k.omega = 1.0;
-        k.beta = 0.0;
-        k.iters = 0;
-        k.status = 0;
-        // an inner pressure pass solves the momentum systems only
-        k.done = (k.r0norm == 0.0 || *F.halt || (s == 3 && P.inner_pass)) ? 1 : 0;
-      }
-    }
-  }
+  const double* tot = grid_total<SumFF, 4>(acc, F.red, F.counter, vbx, vnb);
+  if (!tot) return false;
+  finish_init(P, F, tot);
   return true;
 }
 
@@ -281,7 +315,6 @@ __global__ void __launch_bounds__(kThreads) k4_init(DevParams P, Fields F) {
 // r_0 . v_new; last block: alpha = rho / (r_0 . v_new).
 __device__ __forceinline__ void k4_pv_body(const DevParams& P, const Fields& F, int pp,
                                             const VGrid& vg) {
-  __shared__ double smem[32 * 4];
   __shared__ Scal4 sc;
   load_scalars(F.ks, sc);
   if (sc.all_done) return;   // uniform over the grid
@@ -314,25 +347,11 @@ __device__ __forceinline__ void k4_pv_body(const DevParams& P, const Fields& F, 
       pc = pz;
     }
   }
-  double part[4];
-  block_ff<4>(acc, part, smem);
-  if (publish_is_last<4>(part, F.red, F.counter, block_id(vg), block_count(vg))) {
-    double tot[4];
-    reduce_partials<4, false>(tot, F.red, block_count(vg), F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        if (tot[s] == 0.0 || !isfinite(tot[s])) {
-          k.done = 1;
-          k.status = HOSC_ENOCONV;
-          continue;
-        }
-        k.alpha = k.rho / tot[s];
-      }
-      // r p v r0 in, p v out, the compact operators
-      F.alg_bytes[HOSC_K_BICG_PV] += bytes4(P, 6.0 + op_words(ene));
-    }
+  if (const double* tot =
+          grid_total<SumFF, 4>(acc, F.red, F.counter, block_id(vg), block_count(vg))) {
+    finish_pv(F, tot);
+    // r p v r0 in, p v out, the compact operators
+    count_bytes(F, HOSC_K_BICG_PV, bytes4(P, 6.0 + op_words(ene)));
   }
 }
 
@@ -347,7 +366,6 @@ __global__ void __launch_bounds__(MinB == 2 ? 384 : 256, MinB)
 // omega = (t . s) / (t . t) (0 when t = 0).
 __device__ __forceinline__ void k4_st_body(const DevParams& P, const Fields& F, int pp,
                                             const VGrid& vg) {
-  __shared__ double smem[32 * 8];
   __shared__ Scal4 sc;
   load_scalars(F.ks, sc);
   if (sc.all_done) return;
@@ -376,20 +394,11 @@ __device__ __forceinline__ void k4_st_body(const DevParams& P, const Fields& F, 
       sc0 = sz;
     }
   }
-  double part[8];
-  block_ff<8>(acc, part, smem);
-  if (publish_is_last<8>(part, F.red, F.counter, block_id(vg), block_count(vg))) {
-    double tot[8];
-    reduce_partials<8, false>(tot, F.red, block_count(vg), F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        k.omega = tot[4 + s] > 0.0 ? tot[s] / tot[4 + s] : 0.0;
-      }
-      // r v in, t out, the compact operators
-      F.alg_bytes[HOSC_K_BICG_ST] += bytes4(P, 3.0 + op_words(ene));
-    }
+  if (const double* tot =
+          grid_total<SumFF, 8>(acc, F.red, F.counter, block_id(vg), block_count(vg))) {
+    finish_st(F, tot);
+    // r v in, t out, the compact operators
+    count_bytes(F, HOSC_K_BICG_ST, bytes4(P, 3.0 + op_words(ene)));
   }
 }
 
@@ -400,41 +409,11 @@ __global__ void __launch_bounds__(MinB == 2 ? 384 : 256, MinB)
   k4_st_body(P, F, pp, hw_grid());
 }
 
-// The last block of an x/r launch: totals of (r_0 . r, r . r) per system, then the convergence and
-// breakdown tests, beta and rho of the next iteration.
-__device__ __forceinline__ void xr_finish(const DevParams& P, const Fields& F, unsigned nblocks,
-                                          double* smem) {
-  double tot[8];
-  reduce_partials<8, false>(tot, F.red, nblocks, F.counter, smem);
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < 4; ++s) {
-      KrylovScalars& k = F.ks[s];
-      if (k.done) continue;
-      const double rho_new = tot[s];
-      k.rnorm = sqrt(tot[4 + s]);
-      k.iters += 1;
-      if (k.rnorm <= P.tol_lin * k.r0norm) {
-        k.done = 1;
-        k.status = 0;
-      } else if (!isfinite(k.rnorm) || k.iters >= P.max_lin_iter || rho_new == 0.0 ||
-                 k.omega == 0.0) {
-        k.done = 1;
-        k.status = HOSC_ENOCONV;
-      } else {
-        k.beta = (rho_new / k.rho) * (k.alpha / k.omega);
-        k.rho = rho_new;
-      }
-    }
-    F.alg_bytes[HOSC_K_BICG_XR] += bytes4(P, 8.0);   // r v p x t r0 in, x r out
-  }
-}
-
 // s = r - alpha v; x += alpha p + omega s; r = s - omega t; partials (r_0 . r, r . r); last block:
 // convergence and breakdown tests, beta and rho of the next iteration.
 // Returns true in the block that finished the launch's reduction (convergence decided).
 __device__ __forceinline__ bool k4_xr_body(const DevParams& P, const Fields& F, int pp,
                                             const VGrid& vg) {
-  __shared__ double smem[32 * 8];
   __shared__ Scal4 sc;
   load_scalars(F.ks, sc);
   if (sc.all_done) return false;
@@ -456,10 +435,11 @@ __device__ __forceinline__ bool k4_xr_body(const DevParams& P, const Fields& F, 
       ff_dot4(acc + 4, rn, rn);
     }
   }
-  double part[8];
-  block_ff<8>(acc, part, smem);
-  if (!publish_is_last<8>(part, F.red, F.counter, block_id(vg), block_count(vg))) return false;
-  xr_finish(P, F, block_count(vg), smem);
+  const double* tot =
+      grid_total<SumFF, 8>(acc, F.red, F.counter, block_id(vg), block_count(vg));
+  if (!tot) return false;
+  finish_xr(P, F, tot);
+  count_bytes(F, HOSC_K_BICG_XR, bytes4(P, 8.0));   // r v p x t r0 in, x r out
   return true;
 }
 

@@ -494,7 +494,6 @@ __global__ void __launch_bounds__(kThreads, sizeof(Tc) == sizeof(float) ? 3 : 0)
 template <class Ts>
 __device__ __forceinline__ void k_apply_increment_body(const DevParams& P, const Fields& F,
                                                        int cur, int nblocks, unsigned vbx) {
-  __shared__ double smem[64];
   if (*F.halt) return;
   const unsigned N = P.N;
   const unsigned n3 = N * N * N;
@@ -533,10 +532,7 @@ __device__ __forceinline__ void k_apply_increment_body(const DevParams& P, const
       F.w[1 - cur][t] = F.w[cur][t];
     }
   }
-  block_reduce<2, true>(m, smem);
-  if (publish_is_last<2>(m, F.red, F.counter, vbx, nblocks)) {
-    double tot[2];
-    reduce_partials<2, true>(tot, F.red, nblocks, F.counter, smem);
+  if (const double* tot = grid_total<MaxD, 2>(m, F.red, F.counter, vbx, nblocks)) {
     if (threadIdx.x == 0) {
       // an inner pressure pass changes u, v, w only: theta's change stays that of the first pass
       if (!P.inner_pass) F.rec->res_theta = tot[1];
@@ -608,7 +604,6 @@ __device__ __forceinline__ int wall_weights(int a, int N, int idx[2], double wt[
 // walls keep theta = 1 and theta = 0. Max |change| joins the step record.
 __device__ __forceinline__ void k_theta_walls_body(const DevParams& P, const Fields& F,
                                                    int nblocks, unsigned vbx) {
-  __shared__ double smem[32];
   if (*F.halt) return;
   const int N = P.N, ni = N - 2;
   const int t = vbx * blockDim.x + threadIdx.x;
@@ -629,10 +624,7 @@ __device__ __forceinline__ void k_theta_walls_body(const DevParams& P, const Fie
     m[0] = absfin(s - F.th[c]);
     F.th[c] = s;
   }
-  block_reduce<1, true>(m, smem);
-  if (publish_is_last<1>(m, F.red, F.counter, vbx, nblocks)) {
-    double tot[1];
-    reduce_partials<1, true>(tot, F.red, nblocks, F.counter, smem);
+  if (const double* tot = grid_total<MaxD, 1>(m, F.red, F.counter, vbx, nblocks)) {
     if (threadIdx.x == 0) {
       F.rec->res = fmax(F.rec->res, tot[0]);
       if (!P.inner_pass) F.rec->res_theta = fmax(F.rec->res_theta, tot[0]);
@@ -647,7 +639,6 @@ __global__ void __launch_bounds__(kThreads) k_theta_walls(DevParams P, Fields F,
 // Central div V^{n+1} at interior nodes and its maximum.
 __device__ __forceinline__ void k_divergence_body(const DevParams& P, const Fields& F, int nxt,
                                                   int nblocks, unsigned vbx) {
-  __shared__ double smem[32];
   if (*F.halt) return;
   const int N = P.N, ni = N - 2;
   const int cnt = ni * ni * ni;
@@ -664,10 +655,7 @@ __device__ __forceinline__ void k_divergence_body(const DevParams& P, const Fiel
     F.div[c] = d;
     m[0] = absfin(d);
   }
-  block_reduce<1, true>(m, smem);
-  if (publish_is_last<1>(m, F.red, F.counter, vbx, nblocks)) {
-    double tot[1];
-    reduce_partials<1, true>(tot, F.red, nblocks, F.counter, smem);
+  if (const double* tot = grid_total<MaxD, 1>(m, F.red, F.counter, vbx, nblocks)) {
     if (threadIdx.x == 0) F.rec->div_max = tot[0];
   }
 }

@@ -152,7 +152,6 @@ __global__ void __launch_bounds__(kTmaMaxThreads)
     k7_stencil(DevParams P, Fields F, int pp, const __grid_constant__ TmaMaps tm) {
   constexpr int M = PV ? 4 : 8;
   extern __shared__ unsigned char tdyn[];
-  __shared__ double smem[32 * 8];
   __shared__ Scal4 sc;
   __shared__ __align__(8) unsigned long long full[S];
   __shared__ __align__(8) unsigned long long empty[S];
@@ -283,33 +282,18 @@ __global__ void __launch_bounds__(kTmaMaxThreads)
     }
     if (!ok) failed = 1;
   }
-  double part[M];
-  block_ff<M>(acc, part, smem);   // synchronises the block: failed is final here
   const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
   const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
+  // synchronises the block: failed is final after it
+  const double* tot = grid_total<SumFF, M>(acc, F.red, F.counter, bid, nb);
   const bool bad = failed != 0;
-  if (publish_is_last<M>(part, F.red, F.counter, bid, nb)) {
-    double tot[M];
-    reduce_partials<M, false>(tot, F.red, nb, F.counter, smem);
-    if (threadIdx.x == 0) {
-      for (int s = 0; s < 4; ++s) {
-        KrylovScalars& k = F.ks[s];
-        if (k.done) continue;
-        if (PV) {
-          if (tot[s] == 0.0 || !isfinite(tot[s])) {
-            k.done = 1;
-            k.status = HOSC_ENOCONV;
-            continue;
-          }
-          k.alpha = k.rho / tot[s];
-        } else {
-          k.omega = tot[4 + s] > 0.0 ? tot[s] / tot[4 + s] : 0.0;
-        }
-      }
-      // p/v: r p v r0 in, p v out; s/t: r v in, t out; the compact operators
-      if (PV) F.alg_bytes[HOSC_K_BICG_PV] += bytes4(P, 6.0 + op_words(ene));
-      else F.alg_bytes[HOSC_K_BICG_ST] += bytes4(P, 3.0 + op_words(ene));
-    }
+  if (tot) {
+    if (PV) finish_pv(F, tot);
+    else finish_st(F, tot);
+    // p/v: r p v r0 in, p v out; s/t: r v in, t out; the compact operators
+    count_bytes(F, PV ? HOSC_K_BICG_PV : HOSC_K_BICG_ST,
+                bytes4(P, (PV ? 6.0 : 3.0) + op_words(ene)));
+    __syncthreads();   // a failed block's marks below come after these
   }
   if (bad && threadIdx.x == 0) {
     for (int s = 0; s < 4; ++s) {
