@@ -200,32 +200,50 @@ DevParams device_params(const hosc_params& p, int have_prev, int phase) {
   d.Ly = p.Ly > 0.0 ? p.Ly : 1.0;
   d.Lz = p.Lz > 0.0 ? p.Lz : 1.0;
   const double sp[3] = {d.h, d.Ly / (p.N - 1), d.Lz / (p.N - 1)};
-  double sq[3];
+  RhsC<double>& rc = d.rc;
+  double sum_isq = 0.0;
   for (int a = 0; a < 3; ++a) {
-    sq[a] = sp[a] * sp[a];
-    d.inv2[a] = 0.5 / sp[a];
-    d.isq[a] = 1.0 / sq[a];
-    d.sq12[a] = sq[a] / 12.0;
-    d.ih[a] = 1.0 / sp[a];
+    const double sq = sp[a] * sp[a];
+    d.inv2[a] = rc.i2[a] = 0.5 / sp[a];
+    rc.isq[a] = 1.0 / sq;
+    rc.s12[a] = sq / 12.0;
+    rc.h12[a] = sp[a] / 12.0;
+    rc.h24[a] = sp[a] / 24.0;
+    rc.cs[a] = -0.5 * p.dt * rc.isq[a];
+    sum_isq += rc.isq[a];
   }
-  for (int a = 0; a < 3; ++a) {   // the (a, a+1) edge group and the weights of p1, q1, r1
-    const int b = (a + 1) % 3;
-    d.grp[a] = d.sq12[a] + d.sq12[b];
-    d.pw[2 * a] = 2.0 * sq[b] / (sq[a] + sq[b]);
-    d.pw[2 * a + 1] = 2.0 * sq[a] / (sq[a] + sq[b]);
+  for (int q = 0; q < 3; ++q) {   // the pair (a, b)
+    const double ha = sp[q], hb = sp[(q + 1) % 3];
+    const double s2 = ha * ha + hb * hb, g = s2 / 12.0;
+    rc.e0[q] = g / (ha * ha * hb * hb);
+    rc.ea[q] = 0.5 * g / (ha * hb * hb);
+    rc.eb[q] = 0.5 * g / (ha * ha * hb);
+    rc.ec[q] = 0.25 * g / (ha * hb);
+    rc.xa[q] = hb / s2;
+    rc.xb[q] = ha / s2;
   }
   for (int a = 0; a < 3; ++a) {
-    d.inv2f[a] = (float)d.inv2[a];
-    d.isqf[a] = (float)d.isq[a];
-    d.sq12f[a] = (float)d.sq12[a];
-    d.ihf[a] = (float)d.ih[a];
-    d.grpf[a] = (float)d.grp[a];
+    const int o = (a + 2) % 3;   // the pair with direction a in second place
+    rc.face[a] = 2.0 * (rc.e0[a] + rc.e0[o]);
+    rc.kd[a] = 2.0 * (rc.ea[a] + rc.eb[o]);
   }
-  for (int q = 0; q < 6; ++q) d.pwf[q] = (float)d.pw[q];
-  for (int a = 0; a < 3; ++a) d.csf[a] = (float)(-0.5 * p.dt * d.isq[a]);
-  d.s3 = (d.isq[0] + d.isq[1] + d.isq[2]) / 3.0;
-  d.s3f = (float)d.s3;
+  rc.dt = p.dt;
+  rc.hdt = -0.5 * p.dt;
+  rc.dtq = p.dt * sum_isq;
+  rc.s3 = sum_isq / 3.0;
+  static_assert(sizeof(RhsC<double>) == 2 * sizeof(RhsC<float>), "two arrays of one type each");
+  for (size_t q = 0; q < sizeof(RhsC<float>) / sizeof(float); ++q)
+    ((float*)&d.rcf)[q] = (float)((const double*)&rc)[q];
+  for (int a = 0; a < 3; ++a) {
+    d.inv2f[a] = d.rcf.i2[a];
+    d.csf[a] = d.rcf.cs[a];
+  }
   d.eta_exp = 0.5 * (p.n - 1.0);
+  {
+    const double m = d.eta_exp != 0.0 ? rint(1.0 / fabs(d.eta_exp)) : 0.0;
+    // equal to the rounding of n - 1: the power then differs by less than its last place
+    if (m >= 2.0 && m <= 64.0 && fabs(fabs(d.eta_exp) * m - 1.0) < 1e-15) d.eta_root = (int)m;
+  }
   d.dtf = (float)p.dt;
   d.Prf = (float)p.Pr;
   d.iPr = 1.0 / p.Pr;

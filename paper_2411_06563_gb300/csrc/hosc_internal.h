@@ -11,7 +11,24 @@
 namespace hosc {
 
 constexpr int kThreads = 256;     // threads per block of the grid-stride stencil kernels
+// Threads per block of the FP64 sweeps. One warp fills an SM's FP64 pipe (16 cycles an instruction),
+// so what counts on the small grids is that the warps spread over the SMs: 21^3 nodes in blocks of 256
+// occupied 27 of the 152.
+constexpr int kFp64Threads = 64;
 constexpr int kRedSlots = 8;      // doubles of partial sums written per block
+
+// Spacing constants of the right-hand sides and operators of Eq. (5) in the arithmetic type of the
+// sweep. Directions d = x, y, z with spacings h_d; pairs p = 0, 1, 2 are (a, b) = (x, y), (y, z),
+// (z, x), with the edge-group factor g = (h_a^2 + h_b^2)/12.
+template <class T>
+struct RhsC {
+  T i2[3], isq[3], s12[3], h12[3], h24[3];   // 1/(2h), 1/h^2, h^2/12, h/12, h/24
+  T e0[3], ea[3], eb[3], ec[3];   // g/(h_a h_b)^2, g/(2 h_a h_b^2), g/(2 h_a^2 h_b), g/(4 h_a h_b)
+  T xa[3], xb[3];                 // h_b^2/((h_a^2 + h_b^2) h_b), h_a^2/((h_a^2 + h_b^2) h_a)
+  T face[3], kd[3];               // 2 (e0 of the pairs with d), 2 (ea, eb of the pairs with d)
+  T cs[3];                        // -dt/(2 h_d^2)
+  T dt, hdt, dtq, s3;             // dt, -dt/2, dt (1/h^2 + 1/k^2 + 1/l^2), a third of that sum / dt
+};
 
 // Scalars that kernels take by value.
 struct DevParams {
@@ -39,16 +56,14 @@ struct DevParams {
   double h, h2;      // grid spacing along x and its square
   double Ly, Lz;     // box 1 x Ly x Lz: lengths along y and z (1 for the cube)
   // Spacing constants of the directions d = x, y, z (spacings h, k, l = h, Ly h, Lz h), in double
-  // and in float (the float sweeps read them as operands): 1/(2 h_d), 1/h_d^2, h_d^2/12, 1/h_d;
-  // the edge-group factors (h^2+k^2)/12, (k^2+l^2)/12, (l^2+h^2)/12; the weights of the
-  // first-derivative terms of p1, q1, r1: 2k^2/(h^2+k^2), 2h^2/(h^2+k^2), 2l^2/(k^2+l^2),
-  // 2k^2/(k^2+l^2), 2h^2/(l^2+h^2), 2l^2/(l^2+h^2) (all 1 when h = k = l)
-  double inv2[3], isq[3], sq12[3], ih[3], grp[3], pw[6];
-  float inv2f[3], isqf[3], sq12f[3], ihf[3], grpf[3], pwf[6];
+  // and in float (the float sweeps read them as operands): 1/(2 h_d), and the constants of the
+  // right-hand sides
+  double inv2[3];
+  float inv2f[3];
   float csf[3];      // -dt/(2 h_d^2): the dt part of the symmetric weights of the compact operators
-  double s3;         // (1/h^2 + 1/k^2 + 1/l^2)/3: threshold of the pseudo-time mass (1/h^2 when
-                     // h = k = l)
-  float s3f;
+  RhsC<double> rc;
+  RhsC<float> rcf;
+  int eta_root;      // m when (n - 1)/2 = -1/m or 1/m for an integer m in 2..64, else 0
   double eta_exp;    // (n - 1)/2, the exponent of the regularised viscosity
   // float copies of the scalars the float sweeps use (converted once on the host)
   float dtf, Prf, Raf, theta_reff, I2_epsf, eta_expf, a_limitf, a_boostf;
@@ -158,7 +173,7 @@ struct Fields {
 // Bytes of a context's device workspace (the BiCGSTAB(2) vectors included when bicgstab2);
 // fills f when base != 0.
 size_t workspace_layout(int N, int bicgstab2, Fields* f, char* base);
-int red_blocks(long count);
+int red_blocks(long count, int threads = kThreads);
 // Rows of the per-block partials buffer of an N^3 context: enough for any launch shape the
 // validation accepts (at least 32 threads per block, one plane per thread).
 inline long red_rows(long n3) { return n3 / 16 + 1024; }

@@ -94,10 +94,11 @@ __device__ __noinline__ void visc_item(const RoundMember& M, int cur, int tile) 
   const Fields& F = M.F;
   if (P.sweep_fp32)
     k_viscosity_body<float>(P, F.us[cur], F.vs[cur], F.ws[cur], reinterpret_cast<float*>(F.eta),
-                            reinterpret_cast<float*>(F.L[cur]), F.halt, (unsigned)tile);
+                            reinterpret_cast<float*>(F.L[cur]), F.halt, (unsigned)tile,
+                            (unsigned)M.interior);
   else
     k_viscosity_body<double>(P, F.u[cur], F.v[cur], F.w[cur], F.eta, F.L[cur], F.halt,
-                             (unsigned)tile);
+                             (unsigned)tile, (unsigned)M.interior);
 }
 
 __device__ __noinline__ void sources_item(const RoundMember& M, int cur, int tile) {
@@ -108,10 +109,10 @@ __device__ __noinline__ void sources_item(const RoundMember& M, int cur, int til
                           reinterpret_cast<const float*>(F.eta),
                           reinterpret_cast<float*>(F.Eu[cur]),
                           reinterpret_cast<float*>(F.Ev[cur]), reinterpret_cast<float*>(F.Ew[cur]),
-                          F.halt, (unsigned)tile);
+                          F.halt, (unsigned)tile, (unsigned)M.interior);
   else
     k_sources_body<double>(P, F.u[cur], F.v[cur], F.w[cur], F.th, F.p, F.eta, F.Eu[cur],
-                           F.Ev[cur], F.Ew[cur], F.halt, (unsigned)tile);
+                           F.Ev[cur], F.Ew[cur], F.halt, (unsigned)tile, (unsigned)M.interior);
 }
 
 __device__ __noinline__ bool init_item(const RoundMember& M, int tile) {
@@ -175,12 +176,13 @@ struct FlowDev {
 __device__ __forceinline__ int flow_tiles(const RoundMember& M, int ph) {
   switch (ph) {
     case PH_RHS: case PH_DIV: case PH_PCORR: return M.interior;
+    case PH_VISC: case PH_SOURCES: return M.interior + M.pressure_walls;
     case PH_INIT: return M.init;
     case PH_PV: case PH_ST: case PH_XR: return M.kx * M.ky;
     case PH_TWALLS: return M.theta_walls;
     case PH_PWALLS: return M.pressure_walls;
     case PH_FINISH: return 1;
-    default: return M.nodes;   // shadows, viscosity, sources, increments
+    default: return M.nodes;   // shadows, increments
   }
 }
 
@@ -380,7 +382,7 @@ hosc_status launch_flow(RoundState* S, const std::vector<RoundMember>& members, 
   long most = 0;
   for (const RoundMember& M : members) {
     long m = M.nodes;
-    if (M.interior > m) m = M.interior;
+    if (M.interior + M.pressure_walls > m) m = M.interior + M.pressure_walls;
     if ((long)M.kx * M.ky > m) m = (long)M.kx * M.ky;
     most += m;
   }

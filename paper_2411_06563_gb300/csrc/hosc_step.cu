@@ -2,7 +2,7 @@
 // Sec. 2.2): viscosity (S1), momentum sources (S2), compact right-hand sides and level-(n+1)
 // operator weights (S3/S4), increments, wall conditions, divergence and the modified
 // artificial-compressibility pressure correction (S6-S8). The device code is in
-// hosc_step_dev.cuh; one block of kThreads threads per 256 nodes.
+// hosc_step_dev.cuh; one thread per node.
 
 #include <math.h>
 
@@ -14,7 +14,7 @@ void launch_arm(const Fields& F, int stop_steady, cudaStream_t s) {
   k_arm<<<1, 32, 0, s>>>(F.halt, F.ring_pos, F.steady_stop, stop_steady);
 }
 
-int red_blocks(long count) { return (int)((count + kThreads - 1) / kThreads); }
+int red_blocks(long count, int threads) { return (int)((count + threads - 1) / threads); }
 
 
 void launch_shadow(const DevParams& P, const Fields& F, int cur, int both, cudaStream_t s) {
@@ -29,28 +29,42 @@ void launch_shadow(const DevParams& P, const Fields& F, int cur, int both, cudaS
   }
 }
 
+// Grid of a sweep over all nodes: the interior nodes' blocks, then the boundary nodes'.
+struct SweepGrid {
+  int threads;
+  unsigned nbi, nb;
+};
+static SweepGrid sweep_grid(const DevParams& P) {
+  const long n3 = (long)P.N * P.N * P.N, ni = P.N - 2, ni3 = ni * ni * ni;
+  SweepGrid g;
+  g.threads = P.sweep_fp32 ? kThreads : kFp64Threads;
+  g.nbi = red_blocks(ni3, g.threads);
+  g.nb = g.nbi + red_blocks(n3 - ni3, g.threads);
+  return g;
+}
+
 void launch_viscosity(const DevParams& P, const Fields& F, int cur, cudaStream_t s) {
-  const long n3 = (long)P.N * P.N * P.N;
+  const SweepGrid g = sweep_grid(P);
   if (P.sweep_fp32)
-    k_viscosity<float><<<red_blocks(n3), kThreads, 0, s>>>(
+    k_viscosity<float><<<g.nb, g.threads, 0, s>>>(
         P, F.us[cur], F.vs[cur], F.ws[cur], reinterpret_cast<float*>(F.eta),
-        reinterpret_cast<float*>(F.L[cur]), F.halt);
+        reinterpret_cast<float*>(F.L[cur]), F.halt, g.nbi);
   else
-    k_viscosity<double><<<red_blocks(n3), kThreads, 0, s>>>(P, F.u[cur], F.v[cur], F.w[cur],
-                                                            F.eta, F.L[cur], F.halt);
+    k_viscosity<double><<<g.nb, g.threads, 0, s>>>(P, F.u[cur], F.v[cur], F.w[cur], F.eta,
+                                                   F.L[cur], F.halt, g.nbi);
 }
 
 void launch_sources(const DevParams& P, const Fields& F, int cur, cudaStream_t s) {
-  const long n3 = (long)P.N * P.N * P.N;
+  const SweepGrid g = sweep_grid(P);
   if (P.sweep_fp32)
-    k_sources<float><<<red_blocks(n3), kThreads, 0, s>>>(
+    k_sources<float><<<g.nb, g.threads, 0, s>>>(
         P, F.us[cur], F.vs[cur], F.ws[cur], F.ths, F.ps, reinterpret_cast<const float*>(F.eta),
         reinterpret_cast<float*>(F.Eu[cur]), reinterpret_cast<float*>(F.Ev[cur]),
-        reinterpret_cast<float*>(F.Ew[cur]), F.halt);
+        reinterpret_cast<float*>(F.Ew[cur]), F.halt, g.nbi);
   else
-    k_sources<double><<<red_blocks(n3), kThreads, 0, s>>>(P, F.u[cur], F.v[cur], F.w[cur], F.th,
-                                                          F.p, F.eta, F.Eu[cur], F.Ev[cur],
-                                                          F.Ew[cur], F.halt);
+    k_sources<double><<<g.nb, g.threads, 0, s>>>(P, F.u[cur], F.v[cur], F.w[cur], F.th, F.p,
+                                                 F.eta, F.Eu[cur], F.Ev[cur], F.Ew[cur], F.halt,
+                                                 g.nbi);
 }
 
 template <class Tc, class Ts>
@@ -69,7 +83,8 @@ static void rhs_t(const DevParams& P, const Fields& F, int cur, cudaStream_t s) 
     th = (const Tc*)F.th;
     up = (const Tc*)F.u[o]; vp = (const Tc*)F.v[o]; wp = (const Tc*)F.w[o];
   }
-  k_rhs<Tc, Ts><<<red_blocks(ni * ni * ni), kThreads, 0, s>>>(
+  const int threads = sizeof(Tc) == sizeof(float) ? kThreads : kFp64Threads;
+  k_rhs<Tc, Ts><<<red_blocks(ni * ni * ni, threads), threads, 0, s>>>(
       P, u, v, w, th, T(F.L[cur]), T(F.Eu[cur]), T(F.Ev[cur]), T(F.Ew[cur]), T(F.L[o]), up, vp,
       wp, T(F.Eu[o]), T(F.Ev[o]), T(F.Ew[o]), F);
 }

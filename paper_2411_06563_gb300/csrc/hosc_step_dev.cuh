@@ -11,6 +11,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "hosc_device.cuh"
 #include "hosc_internal.h"
 
@@ -46,12 +48,41 @@ __device__ __forceinline__ T par(double d, float f) {
   else return d;
 }
 
-template <class T, class S>
-__device__ __forceinline__ T grad_axis_t(const S* HOSC_RESTRICT f, long c, int a, int N, long st,
-                                         T inv2h) {
-  if (a == 0) return (T(-3) * (T)f[c] + T(4) * (T)f[c + st] - (T)f[c + 2 * st]) * inv2h;
-  if (a == N - 1) return (T(3) * (T)f[c] - T(4) * (T)f[c - st] + (T)f[c - 2 * st]) * inv2h;
-  return ((T)f[c + st] - (T)f[c - st]) * inv2h;
+__device__ __forceinline__ int node32(int i, int j, int k, int N) { return i + N * (j + N * k); }
+
+// Node number t of the y faces (x interior, all z), then of the z faces (x, y interior):
+// 0 <= t < 2 (N-2) N + 2 (N-2)^2, x fastest.
+__device__ __forceinline__ void boundary_yz(int t, int N, int& i, int& j, int& k) {
+  const int ni = N - 2;
+  if (t < 2 * ni * N) {
+    const int side = t / (ni * N), r = t - side * ni * N;
+    const int q = r / ni;
+    i = 1 + (r - q * ni);
+    k = q;
+    j = side ? N - 1 : 0;
+  } else {
+    const int u = t - 2 * ni * N;
+    const int side = u / (ni * ni), r = u - side * ni * ni;
+    const int q = r / ni;
+    i = 1 + (r - q * ni);
+    j = 1 + q;
+    k = side ? N - 1 : 0;
+  }
+}
+
+// Node number t of the cube's boundary, 0 <= t < N^3 - (N-2)^3: the x faces, then the y and z
+// faces as in boundary_yz.
+__device__ __forceinline__ void boundary_node(int t, int N, int& i, int& j, int& k) {
+  const int N2 = N * N;
+  if (t < 2 * N2) {
+    const int side = t / N2, r = t - side * N2;
+    const int q = r / N;
+    j = r - q * N;
+    k = q;
+    i = side ? N - 1 : 0;
+  } else {
+    boundary_yz(t - 2 * N2, N, i, j, k);
+  }
 }
 
 template <class T>
@@ -59,94 +90,142 @@ struct Grad9T {
   T ux, uy, uz, vx, vy, vz, wx, wy, wz;
 };
 
-// Spacing constants of the directions x, y, z in the arithmetic type T (spacings h, k, l of a
-// box 1 x Ly x Lz; all equal in the cube): 1/(2 h_d), 1/h_d^2, h_d^2/12, 1/h_d, the edge-group
-// factors and the weights of p1, q1, r1 (DevParams).
+// 1/(2 h_d) of the directions in the arithmetic type T.
 template <class T>
-struct Spc {
-  T i2[3], isq[3], s12[3], ih[3], grp[3], pw[6], s3;
+struct Inv2h {
+  T x, y, z;
 };
-
 template <class T>
-__device__ __forceinline__ Spc<T> spacing(const DevParams& P) {
-  Spc<T> s;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    if constexpr (sizeof(T) == sizeof(float)) {
-      s.i2[a] = P.inv2f[a];
-      s.isq[a] = P.isqf[a];
-      s.s12[a] = P.sq12f[a];
-      s.ih[a] = P.ihf[a];
-      s.grp[a] = P.grpf[a];
-    } else {
-      s.i2[a] = P.inv2[a];
-      s.isq[a] = P.isq[a];
-      s.s12[a] = P.sq12[a];
-      s.ih[a] = P.ih[a];
-      s.grp[a] = P.grp[a];
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < 6; ++q) {
-    if constexpr (sizeof(T) == sizeof(float)) s.pw[q] = P.pwf[q];
-    else s.pw[q] = P.pw[q];
-  }
-  if constexpr (sizeof(T) == sizeof(float)) s.s3 = P.s3f;
-  else s.s3 = P.s3;
-  return s;
+__device__ __forceinline__ Inv2h<T> inv2h(const DevParams& P) {
+  if constexpr (sizeof(T) == sizeof(float)) return {P.inv2f[0], P.inv2f[1], P.inv2f[2]};
+  else return {P.inv2[0], P.inv2[1], P.inv2[2]};
+}
+// The constants of the right-hand sides in the arithmetic type T.
+template <class T>
+__device__ __forceinline__ const RhsC<T>& rhs_constants(const DevParams& P) {
+  if constexpr (sizeof(T) == sizeof(float)) return P.rcf;
+  else return P.rc;
 }
 
-template <class T, class S>
-__device__ __forceinline__ Grad9T<T> velocity_gradients_t(const S* HOSC_RESTRICT u,
-                                                          const S* HOSC_RESTRICT v,
-                                                          const S* HOSC_RESTRICT w, int i,
-                                                          int j, int k, int N,
-                                                          const T i2[3]) {
-  const long c = node(i, j, k, N);
-  const long sy = N, sz = (long)N * N;
+// Derivative along an axis with memory stride st at a node of coordinate a along it. WALL: the node
+// may lie on a wall of that axis (second-order one-sided there); otherwise central.
+template <bool WALL, class T>
+__device__ __forceinline__ T grad_axis_t(const T* HOSC_RESTRICT f, int c, int a, int N, int st,
+                                         T inv2h) {
+  if constexpr (WALL) {
+    if (a == 0) return (T(-3) * f[c] + T(4) * f[c + st] - f[c + 2 * st]) * inv2h;
+    if (a == N - 1) return (T(3) * f[c] - T(4) * f[c - st] + f[c - 2 * st]) * inv2h;
+  }
+  return (f[c + st] - f[c - st]) * inv2h;
+}
+
+template <bool WALL, class T>
+__device__ __forceinline__ Grad9T<T> velocity_gradients_t(const T* HOSC_RESTRICT u,
+                                                          const T* HOSC_RESTRICT v,
+                                                          const T* HOSC_RESTRICT w, int i, int j,
+                                                          int k, int N, const Inv2h<T>& i2) {
+  const int sy = N, sz = N * N, c = node32(i, j, k, N);
   Grad9T<T> g;
-  g.ux = grad_axis_t<T>(u, c, i, N, 1, i2[0]);
-  g.uy = grad_axis_t<T>(u, c, j, N, sy, i2[1]);
-  g.uz = grad_axis_t<T>(u, c, k, N, sz, i2[2]);
-  g.vx = grad_axis_t<T>(v, c, i, N, 1, i2[0]);
-  g.vy = grad_axis_t<T>(v, c, j, N, sy, i2[1]);
-  g.vz = grad_axis_t<T>(v, c, k, N, sz, i2[2]);
-  g.wx = grad_axis_t<T>(w, c, i, N, 1, i2[0]);
-  g.wy = grad_axis_t<T>(w, c, j, N, sy, i2[1]);
-  g.wz = grad_axis_t<T>(w, c, k, N, sz, i2[2]);
+  g.ux = grad_axis_t<WALL>(u, c, i, N, 1, i2.x);
+  g.uy = grad_axis_t<WALL>(u, c, j, N, sy, i2.y);
+  g.uz = grad_axis_t<WALL>(u, c, k, N, sz, i2.z);
+  g.vx = grad_axis_t<WALL>(v, c, i, N, 1, i2.x);
+  g.vy = grad_axis_t<WALL>(v, c, j, N, sy, i2.y);
+  g.vz = grad_axis_t<WALL>(v, c, k, N, sz, i2.z);
+  g.wx = grad_axis_t<WALL>(w, c, i, N, 1, i2.x);
+  g.wy = grad_axis_t<WALL>(w, c, j, N, sy, i2.y);
+  g.wz = grad_axis_t<WALL>(w, c, k, N, sz, i2.z);
   return g;
+}
+
+// The sweeps over all nodes (S1, S2) run the interior nodes in their first nbi blocks and the
+// boundary nodes in the others: with both in one warp (an x row has a wall node at either end)
+// every third warp went through the one-sided forms of each derivative beside the central ones.
+// Measured with the split: S1 in float 249 -> 146 us at 257^3 and 17.2 -> 14.4 us at 101^3, S2 in
+// float 354 -> 198 and 20.9 -> 16.6 us, S2 in double 236 -> 123 us at 101^3.
+// Calls f(WALL, i, j, k) for this thread's node.
+template <class Fn>
+__device__ __forceinline__ void sweep_node(int N, unsigned vbx, unsigned nbi, Fn f) {
+  const int ni = N - 2;
+  if (vbx < nbi) {
+    const int t = (int)(vbx * blockDim.x + threadIdx.x);
+    if (t >= ni * ni * ni) return;
+    const int q = t / ni;
+    f(std::false_type(), 1 + t - q * ni, 1 + q % ni, 1 + q / ni);
+  } else {
+    const int t = (int)((vbx - nbi) * blockDim.x + threadIdx.x);
+    if (t >= N * N * N - ni * ni * ni) return;
+    int i, j, k;
+    boundary_node(t, N, i, j, k);
+    f(std::true_type(), i, j, k);
+  }
 }
 
 // ------------------------------------------------------------------------------------ S1
 
+// x^(-1/m) for an integer m in 2..64: a float estimate y of 1e-6 and one third-order step of
+// Newton's iteration on y^-m = x, y (1 - r)^(-1/m) to r^2 with r = 1 - x y^m (the r^3 term is below
+// 1e-16 of y); y^m by squaring. Largest error found against 200-bit arithmetic over 20 000 x in
+// [1e-12, 1e12]: 0.75 units in the last place (m = 8), 0.79 (m = 64); about 15 FP64 instructions
+// against some 130 of pow().
+__device__ __forceinline__ double inverse_root(double x, int m) {
+  const float a = 1.0f / (float)m;
+  const double y = (double)exp2f(-a * log2f((float)x));
+  double p = 1.0, b = y;
+  for (int e = m;;) {   // m is the same for every thread
+    if (e & 1) p *= b;
+    if ((e >>= 1) == 0) break;
+    b *= b;
+  }
+  const double r = fma(-x, p, 1.0);
+  const float c2 = 0.5f * a * (1.0f + a);
+  return fma(y, r * fma((double)c2, r, 1.0 / (double)m), y);
+}
+
 // eta = (I2 + eps)^((n-1)/2) (Eqs. 7-8), eta == 1 for n == 1; L = 1/(Pr eta) (Sec. 2.2 momentum
 // coefficients). On cube edges and corners, where the one-sided strain rates of two or three
 // no-slip walls vanish identically, I2 is taken at the node one step inward along each of those
-// wall normals.
+// wall normals. In double, where 2/|n-1| is an integer m (n = 0.75 and 1.25: 8), the power is
+// inverse_root: 303 -> 120 us per sweep at 101^3 with the split of sweep_node (FP64-bound); pow()
+// for other indices and outside [1e-30, 1e30].
 template <class T>
 __device__ __forceinline__ void k_viscosity_body(const DevParams& P, const T* HOSC_RESTRICT u,
                                                  const T* HOSC_RESTRICT v, const T* HOSC_RESTRICT w,
                                                  T* HOSC_RESTRICT eta, T* HOSC_RESTRICT L,
-                                                 const int* HOSC_RESTRICT halt, unsigned vbx) {
-  const unsigned N = P.N;
-  const unsigned t = vbx * blockDim.x + threadIdx.x;
-  if (t >= N * N * N || *halt) return;
-  const unsigned q = t / N;
-  int i = (int)(t - q * N), j = (int)(q % N), k = (int)(q / N);
-  T e = T(1);
-  if (!P.newtonian) {
-    if (on_wall(i, (int)N) + on_wall(j, (int)N) + on_wall(k, (int)N) >= 2) {
-      i = inward(i, (int)N);
-      j = inward(j, (int)N);
-      k = inward(k, (int)N);
+                                                 const int* HOSC_RESTRICT halt, unsigned vbx,
+                                                 unsigned nbi) {
+  if (*halt) return;
+  const int N = P.N;
+  sweep_node(N, vbx, nbi, [&](auto wall, int i, int j, int k) {
+    constexpr bool WALL = decltype(wall)::value;
+    const int t = node32(i, j, k, N);
+    if (P.newtonian) {
+      eta[t] = T(1);
+      L[t] = T(1) / par<T>(P.Pr, P.Prf);
+      return;
     }
-    const Grad9T<T> g = velocity_gradients_t<T, T>(u, v, w, i, j, k, N, spacing<T>(P).i2);
+    if (WALL && on_wall(i, N) + on_wall(j, N) + on_wall(k, N) >= 2) {
+      i = inward(i, N);
+      j = inward(j, N);
+      k = inward(k, N);
+    }
+    const Grad9T<T> g = velocity_gradients_t<WALL, T>(u, v, w, i, j, k, N, inv2h<T>(P));
     const T a = g.uz + g.wx, b = g.uy + g.vx, c = g.vz + g.wy;
     const T I2 = T(2) * (g.ux * g.ux + g.vy * g.vy + g.wz * g.wz) + a * a + b * b + c * c;
-    e = tpow<T>(I2 + par<T>(P.I2_eps, P.I2_epsf), par<T>(P.eta_exp, P.eta_expf));
-  }
-  eta[t] = e;
-  L[t] = T(1) / (par<T>(P.Pr, P.Prf) * e);
+    const T x = I2 + par<T>(P.I2_eps, P.I2_epsf);
+    if constexpr (sizeof(T) == sizeof(double)) {
+      if (P.eta_root && x >= 1e-30 && x <= 1e30) {
+        const double z = inverse_root(x, P.eta_root);
+        const bool thin = P.eta_exp < 0.0;   // the same for every thread
+        eta[t] = thin ? z : 1.0 / z;
+        L[t] = thin ? 1.0 / (P.Pr * z) : P.iPr * z;
+        return;
+      }
+    }
+    const T e = tpow<T>(x, par<T>(P.eta_exp, P.eta_expf));
+    eta[t] = e;
+    L[t] = T(1) / (par<T>(P.Pr, P.Prf) * e);
+  });
 }
 
 template <class T>
@@ -154,8 +233,9 @@ __global__ void __launch_bounds__(kThreads) k_viscosity(DevParams P, const T* HO
                                                         const T* HOSC_RESTRICT v,
                                                         const T* HOSC_RESTRICT w,
                                                         T* HOSC_RESTRICT eta, T* HOSC_RESTRICT L,
-                                                        const int* HOSC_RESTRICT halt) {
-  k_viscosity_body(P, u, v, w, eta, L, halt, blockIdx.x);
+                                                        const int* HOSC_RESTRICT halt,
+                                                        unsigned nbi) {
+  k_viscosity_body(P, u, v, w, eta, L, halt, blockIdx.x, nbi);
 }
 
 // ------------------------------------------------------------------------------------ S2
@@ -172,29 +252,33 @@ __device__ __forceinline__ void k_sources_body(const DevParams& P, const T* HOSC
                                                const T* HOSC_RESTRICT th, const T* HOSC_RESTRICT p,
                                                const T* HOSC_RESTRICT eta, T* HOSC_RESTRICT Eu,
                                                T* HOSC_RESTRICT Ev, T* HOSC_RESTRICT Ew,
-                                               const int* HOSC_RESTRICT halt, unsigned vbx) {
+                                               const int* HOSC_RESTRICT halt, unsigned vbx,
+                                               unsigned nbi) {
+  if (*halt) return;
   const int N = P.N;
-  const unsigned t = vbx * blockDim.x + threadIdx.x;
-  if (t >= (unsigned)N * N * N || *halt) return;
-  const unsigned q = t / (unsigned)N;
-  const int i = (int)(t - q * (unsigned)N), j = (int)(q % (unsigned)N), k = (int)(q / (unsigned)N);
-  const Spc<T> sp = spacing<T>(P);
-  const long sy = N, sz = (long)N * N;
-  const Grad9T<T> g = velocity_gradients_t<T, T>(u, v, w, i, j, k, N, sp.i2);
-  const T ex = grad_axis_t<T>(eta, t, i, N, 1, sp.i2[0]);
-  const T ey = grad_axis_t<T>(eta, t, j, N, sy, sp.i2[1]);
-  const T ez = grad_axis_t<T>(eta, t, k, N, sz, sp.i2[2]);
-  const T px = grad_axis_t<T>(p, t, i, N, 1, sp.i2[0]);
-  const T py = grad_axis_t<T>(p, t, j, N, sy, sp.i2[1]);
-  const T pz = grad_axis_t<T>(p, t, k, N, sz, sp.i2[2]);
-  const T e = eta[t];
-  const T exy = T(0.5) * (g.uy + g.vx), exz = T(0.5) * (g.uz + g.wx), eyz = T(0.5) * (g.vz + g.wy);
-  const T ie = T(1) / e;   // one division per node
-  const T a = ie * par<T>(P.iPr, P.iPrf), b = T(2) * ie;
-  Eu[t] = -px * a + b * (g.ux * ex + exy * ey + exz * ez);
-  Ev[t] = -py * a + b * (exy * ex + g.vy * ey + eyz * ez) +
-          par<T>(P.Ra, P.Raf) * ((T)th[t] - par<T>(P.theta_ref, P.theta_reff)) / e;
-  Ew[t] = -pz * a + b * (exz * ex + eyz * ey + g.wz * ez);
+  sweep_node(N, vbx, nbi, [&](auto wall, int i, int j, int k) {
+    constexpr bool WALL = decltype(wall)::value;
+    const Inv2h<T> i2 = inv2h<T>(P);
+    const int sy = N, sz = N * N, t = node32(i, j, k, N);
+    const Grad9T<T> g = velocity_gradients_t<WALL, T>(u, v, w, i, j, k, N, i2);
+    const T ex = grad_axis_t<WALL>(eta, t, i, N, 1, i2.x);
+    const T ey = grad_axis_t<WALL>(eta, t, j, N, sy, i2.y);
+    const T ez = grad_axis_t<WALL>(eta, t, k, N, sz, i2.z);
+    const T px = grad_axis_t<WALL>(p, t, i, N, 1, i2.x);
+    const T py = grad_axis_t<WALL>(p, t, j, N, sy, i2.y);
+    const T pz = grad_axis_t<WALL>(p, t, k, N, sz, i2.z);
+    const T e = eta[t];
+    const T exy = T(0.5) * (g.uy + g.vx), exz = T(0.5) * (g.uz + g.wx),
+            eyz = T(0.5) * (g.vz + g.wy);
+    const T ie = T(1) / e;
+    const T a = ie * par<T>(P.iPr, P.iPrf), b = T(2) * ie;
+    const T buoy = par<T>(P.Ra, P.Raf) * (th[t] - par<T>(P.theta_ref, P.theta_reff));
+    Eu[t] = -px * a + b * (g.ux * ex + exy * ey + exz * ez);
+    // an FP64 division is some 15 instructions of the pipe that bounds the double form
+    Ev[t] = -py * a + b * (exy * ex + g.vy * ey + eyz * ez) +
+            (sizeof(T) == sizeof(double) ? buoy * ie : buoy / e);
+    Ew[t] = -pz * a + b * (exz * ex + eyz * ey + g.wz * ez);
+  });
 }
 
 template <class T>
@@ -206,30 +290,13 @@ __global__ void __launch_bounds__(kThreads) k_sources(DevParams P, const T* HOSC
                                                      const T* HOSC_RESTRICT eta,
                                                      T* HOSC_RESTRICT Eu, T* HOSC_RESTRICT Ev,
                                                      T* HOSC_RESTRICT Ew,
-                                                     const int* HOSC_RESTRICT halt) {
-  k_sources_body(P, u, v, w, th, p, eta, Eu, Ev, Ew, halt, blockIdx.x);
+                                                     const int* HOSC_RESTRICT halt, unsigned nbi) {
+  k_sources_body(P, u, v, w, th, p, eta, Eu, Ev, Ew, halt, blockIdx.x, nbi);
 }
 
 // ------------------------------------------------------------------------------------ S3/S4
 
 // 7-point neighbourhood order: centre, x+, x-, y+, y-, z+, z-.
-template <class T>
-struct D7 {
-  T dx, dy, dz, dxx, dyy, dzz;
-};
-
-template <class T>
-__device__ __forceinline__ D7<T> diffs7(const T f[7], const Spc<T>& s) {
-  D7<T> d;
-  d.dx = (f[1] - f[2]) * s.i2[0];
-  d.dy = (f[3] - f[4]) * s.i2[1];
-  d.dz = (f[5] - f[6]) * s.i2[2];
-  d.dxx = (f[1] - T(2) * f[0] + f[2]) * s.isq[0];
-  d.dyy = (f[3] - T(2) * f[0] + f[4]) * s.isq[1];
-  d.dzz = (f[5] - T(2) * f[0] + f[6]) * s.isq[2];
-  return d;
-}
-
 template <class T, class S>
 __device__ __forceinline__ void load7(const S* HOSC_RESTRICT a, long c, long sy, long sz, T f[7]) {
   f[0] = (T)a[c];
@@ -262,69 +329,87 @@ __device__ __forceinline__ void load19(const T* HOSC_RESTRICT a, long c, long sy
   f[18] = (T)a[c - sz - 1];
 }
 
-// One edge group of Eq. (5), directions (a, b) with inverse spacings ia, ib:
-//   da^2 db^2 chi - Vb da^2 db chi - Va da db^2 chi - c1 da db chi
-// from F[pp], F[0p], F[mp], F[p0], F[00], F[m0], F[pm], F[0m], F[mm] (first index along a).
+// What a 7-point neighbourhood gives to Eq. (5): its centre, the sum of its second differences
+// times h_d^2, and f_{+d} - f_{-d} of each direction.
 template <class T>
-__device__ __forceinline__ T edge_group(T Fpp, T F0p, T Fmp, T Fp0, T F00, T Fm0, T Fpm, T F0m,
-                                        T Fmm, T Va, T Vb, T c1, T ia, T ib) {
-  const T ia2 = ia * ia, ib2 = ib * ib;
-  const T d22 = (Fpp + Fmp + Fpm + Fmm - T(2) * (F0p + F0m + Fp0 + Fm0) + T(4) * F00) * ia2 * ib2;
-  const T d21 = ((Fpp - T(2) * F0p + Fmp) - (Fpm - T(2) * F0m + Fmm)) * (T(0.5) * ia2 * ib);
-  const T d12 = ((Fpp - T(2) * Fp0 + Fpm) - (Fmp - T(2) * Fm0 + Fmm)) * (T(0.5) * ia * ib2);
-  const T d11 = (Fpp - Fmp - Fpm + Fmm) * (T(0.25) * ia * ib);
-  return d22 - Vb * d21 - Va * d12 - c1 * d11;
-}
-
-// Coefficients of Eq. (5) shared by the systems with the same G*, H*, I* (K* = 0).
-template <class T>
-struct Eq5 {
-  T G, H, I, al, be, ga, M1, M2, M3, p1, q1, r1;
+struct Star {
+  T c, lap, b[3];
 };
 
-// [1 + (dx^2 - G dx) h^2/12 + (dy^2 - H dy) k^2/12 + (dz^2 - I dz) l^2/12 + (dt/2) dt^-] f
 template <class T>
-__device__ __forceinline__ T bracket(const D7<T>& d, T f0, T f_prev, const Eq5<T>& c,
-                                     const Spc<T>& s) {
-  return f0 + s.s12[0] * (d.dxx - c.G * d.dx) + s.s12[1] * (d.dyy - c.H * d.dy) +
-         s.s12[2] * (d.dzz - c.I * d.dz) + T(0.5) * (f0 - f_prev);
+__device__ __forceinline__ Star<T> star(const T f[7]) {
+  Star<T> s;
+  s.c = f[0];
+  s.b[0] = f[1] - f[2];
+  s.b[1] = f[3] - f[4];
+  s.b[2] = f[5] - f[6];
+  s.lap = ((f[1] + f[2]) + (f[3] + f[4]) + (f[5] + f[6])) - T(6) * f[0];
+  return s;
 }
 
+// [(dx^2 - G dx) h^2/12 + (dy^2 - H dy) k^2/12 + (dz^2 - I dz) l^2/12] f, with v24 = (G h, H k,
+// I l)/24
 template <class T>
-__device__ __forceinline__ Eq5<T> eq5_coefficients(const T G7[7], const T H7[7], const T I7[7],
-                                                   T Gp, T Hp, T Ip, const Spc<T>& s) {
-  Eq5<T> c;
-  c.G = G7[0];
-  c.H = H7[0];
-  c.I = I7[0];
-  const D7<T> dG = diffs7<T>(G7, s), dH = diffs7<T>(H7, s), dI = diffs7<T>(I7, s);
-  c.al = T(1) + s.s12[0] * (c.G * c.G - T(2) * dG.dx);
-  c.be = T(1) + s.s12[1] * (c.H * c.H - T(2) * dH.dy);
-  c.ga = T(1) + s.s12[2] * (c.I * c.I - T(2) * dI.dz);
-  c.M1 = bracket<T>(dG, G7[0], Gp, c, s);
-  c.M2 = bracket<T>(dH, H7[0], Hp, c, s);
-  c.M3 = bracket<T>(dI, I7[0], Ip, c, s);
-  // p1 = -G H + 2/(h^2+k^2) (k^2 dy G + h^2 dx H), and cyclically
-  c.p1 = -c.G * c.H + s.pw[0] * dG.dy + s.pw[1] * dH.dx;
-  c.q1 = -c.H * c.I + s.pw[2] * dH.dz + s.pw[3] * dI.dy;
-  c.r1 = -c.I * c.G + s.pw[4] * dI.dx + s.pw[5] * dG.dz;
-  return c;
+__device__ __forceinline__ T compact_terms(const Star<T>& s, const T v24[3]) {
+  return T(1.0 / 12.0) * s.lap - v24[0] * s.b[0] - v24[1] * s.b[1] - v24[2] * s.b[2];
 }
 
-// The level-n operator of Eq. (5) applied to chi (19 points):
+// The level-n operator of Eq. (5),
 //  -al dx^2 - be dy^2 - ga dz^2 + M1 dx + M2 dy + M3 dz
-//  - (h^2+k^2)/12 [xy group] - (k^2+l^2)/12 [yz group] - (l^2+h^2)/12 [zx group]
+//  - (h^2+k^2)/12 [dx^2 dy^2 - H dx^2 dy - G dx dy^2 - p1 dx dy] - (yz group) - (zx group),
+// as weights of the 18 neighbours (the centre's is minus their sum, since no term acts on a
+// constant), for the systems with the same G*, H*, I* (K* = 0). One set of weights serves u, v and
+// w: 18 differences and 18 fused multiply-adds a system in place of some 110 operations when each
+// system evaluates the difference operators. Applied to f_i - f_0 (exact for neighbours within a
+// factor of two), so that nothing of the size |f|/h^2 cancels.
 template <class T>
-__device__ __forceinline__ T applyB(const Eq5<T>& c, const T f[19], const Spc<T>& s) {
-  const D7<T> d = diffs7<T>(f, s);
-  const T gxy = edge_group<T>(f[7], f[3], f[8], f[1], f[0], f[2], f[9], f[4], f[10], c.G, c.H,
-                              c.p1, s.ih[0], s.ih[1]);
-  const T gyz = edge_group<T>(f[11], f[5], f[12], f[3], f[0], f[4], f[13], f[6], f[14], c.H, c.I,
-                              c.q1, s.ih[1], s.ih[2]);
-  const T gzx = edge_group<T>(f[15], f[1], f[16], f[5], f[0], f[6], f[17], f[2], f[18], c.I, c.G,
-                              c.r1, s.ih[2], s.ih[0]);
-  return -c.al * d.dxx - c.be * d.dyy - c.ga * d.dzz + c.M1 * d.dx + c.M2 * d.dy + c.M3 * d.dz -
-         s.grp[1] * gyz - s.grp[0] * gxy - s.grp[2] * gzx;
+struct LevelN {
+  T V[3], v24[3];
+  T w[18];   // x+, x-, y+, y-, z+, z-, then the edges in load19's order
+};
+
+// V: G*, H*, I* at the 7 points (as stars), Vp: at level n-1 (used when hist).
+template <class T>
+__device__ __forceinline__ LevelN<T> level_n(const Star<T> (&V)[3], const T (&Vp)[3], bool hist,
+                                             const RhsC<T>& k) {
+  LevelN<T> o;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    o.V[d] = V[d].c;
+    o.v24[d] = V[d].c * k.h24[d];
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    // al = 1 + h^2/12 (G^2 - 2 dx G); M1 = [1 + compact terms + (dt/2) dt^-] G
+    const T al = T(1) + (k.s12[d] * V[d].c) * V[d].c - k.h12[d] * V[d].b[d];
+    T M = V[d].c + compact_terms(V[d], o.v24);
+    if (hist) M += T(0.5) * (V[d].c - Vp[d]);
+    const T S = k.face[d] - al * k.isq[d];
+    const T D = M * k.i2[d] - V[d].c * k.kd[d];
+    o.w[2 * d] = S + D;
+    o.w[2 * d + 1] = S - D;
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {   // the pair (a, b)
+    const int a = q, b = (q + 1) % 3;
+    // p1 = -G H + 2/(h^2+k^2) (k^2 dy G + h^2 dx H), and cyclically
+    const T p1 = k.xa[q] * V[a].b[b] + k.xb[q] * V[b].b[a] - V[a].c * V[b].c;
+    const T Ea = k.ea[q] * V[a].c, Eb = k.eb[q] * V[b].c, Ec = k.ec[q] * p1;
+    const T hi = Eb - k.e0[q], lo = -k.e0[q] - Eb, up = Ea + Ec, dn = Ea - Ec;
+    o.w[6 + 4 * q] = hi + up;       // a+ b+
+    o.w[6 + 4 * q + 1] = hi - up;   // a- b+
+    o.w[6 + 4 * q + 2] = lo + dn;   // a+ b-
+    o.w[6 + 4 * q + 3] = lo - dn;   // a- b-
+  }
+  return o;
+}
+
+template <class T>
+__device__ __forceinline__ T apply_level_n(const LevelN<T>& o, const T f[19]) {
+  T s = T(0);
+#pragma unroll
+  for (int q = 0; q < 18; ++q) s += o.w[q] * (f[q + 1] - f[0]);
+  return s;
 }
 
 // Diagonal pseudo-time mass where the cell Reynolds number is high: the level-n operator carries
@@ -335,16 +420,26 @@ __device__ __forceinline__ T applyB(const Eq5<T>& c, const T f[19], const Spc<T>
 template <class T>
 __device__ __forceinline__ T pseudo_time_mass(T G, T H, T I, T L, T dt, T s3, T kappa) {
   const T g2 = G * G + H * H + I * I;
-  const T s = fmax(T(0), fmax(dt * (g2 / T(6) - s3), dt * g2 / T(6) - T(2) * L / T(3)));
+  const T g6 = g2 * T(1.0 / 6.0);
+  const T s = fmax(T(0), fmax(dt * (g6 - s3), dt * g6 - T(2.0 / 3.0) * L));
   return kappa * s;
 }
 
 // Right-hand sides of the increment form of Eq. (6),  A (chi^{n+1} - chi^n) = dt (R - B chi^n),
-// for u, v, w, theta at interior nodes, and the seven level-(n+1) weights L1..L7 of the momentum
-// and energy systems. Tc: arithmetic and the type of L, E*; Ts: type of the outputs.
+// for u, v, w, theta at interior nodes, and the level-(n+1) operators of the momentum and energy
+// systems. Tc: arithmetic and the type of L, E*; Ts: type of the outputs.
+//
+// Along direction d the +d and -d neighbours of the level-(n+1) operator weigh S_d - B_d and
+// S_d + B_d. Of Eq. (6)'s L (M_d/h_d^2 -+ (M_d V_d - M_{14+d})/(2 h_d)) with M_d = -dt/(2L) +
+// h_d^2/12 and M_{14+d} = h_d^2/(6L) d_d L, multiplying L through leaves no division:
+// S_d = -dt/(2 h_d^2) + L/12, B_d = ((-dt/2 + h_d^2 L/12) V_d - (h_d/12)(L_+ - L_-))/(2 h_d), and
+// the diagonal is L/2 + dt (1/h^2 + 1/k^2 + 1/l^2) + M18 + the pseudo-time mass.
+//
+// The FP64 pipe bounds the double forms (a warp's FP64 instruction takes 16 cycles of its SM): about
+// 500 FP64 instructions a node against 1100 when each system evaluated the difference operators:
+// 1742 -> 926 us at 101^3, 72 -> 21 us at 21^3 (there with the smaller blocks of kFp64Threads). The
+// float form is bound by issue slots: 51.3 -> 39.1 us at 101^3, 823 -> 661 us at 257^3.
 template <class Tc, class Ts>
-// The float build is bounded to 80 registers (three 256-thread blocks per SM); the double builds
-// keep the compiler's choice.
 __device__ __forceinline__ void k_rhs_body(const DevParams& P, const Tc* HOSC_RESTRICT u,
                                            const Tc* HOSC_RESTRICT v, const Tc* HOSC_RESTRICT w,
                                            const Tc* HOSC_RESTRICT th, const Tc* HOSC_RESTRICT L,
@@ -362,121 +457,123 @@ __device__ __forceinline__ void k_rhs_body(const DevParams& P, const Tc* HOSC_RE
   const int i = 1 + (int)(t - q * ni), j = 1 + (int)(q % ni), k = 1 + (int)(q / ni);
   const long sy = N, sz = (long)N * N;
   const long c = node(i, j, k, N);
-  const Spc<Tc> sp = spacing<Tc>(P);
-  const Tc tdt = par<Tc>(P.dt, P.dtf);
-  Tc rv[4], Am[7], Ae[7];   // right-hand sides and weights, stored at the end
-
-  Tc L7[7], u7[7], v7[7], w7[7];
-  load7<Tc, Tc>(L, c, sy, sz, L7);
-  load7<Tc, Tc>(u, c, sy, sz, u7);
-  load7<Tc, Tc>(v, c, sy, sz, v7);
-  load7<Tc, Tc>(w, c, sy, sz, w7);
-  const Tc Lc = L7[0];
-  const Tc Lpc = P.have_prev ? Lp[c] : Lc;
-  const Tc upc = P.have_prev ? (Tc)up[c] : u7[0];
-  const Tc vpc = P.have_prev ? (Tc)vp[c] : v7[0];
-  const Tc wpc = P.have_prev ? (Tc)wp[c] : w7[0];
+  const RhsC<Tc>& rc = rhs_constants<Tc>(P);
+  const bool hist = P.have_prev != 0;
+  const Tc kap = par<Tc>(P.a_boost, P.a_boostf);
+  Tc rv[4], Bm[3], Be[3], Dm, De, Lc;   // right-hand sides and compact operators, stored at the end
 
   // ---------------- momentum: L = 1/(Pr eta), G* = u L, H* = v L, I* = w L, K* = 0
   {
-    Tc G7[7], H7[7], I7[7];
+    Tc L7[7], f7[7];
+    load7<Tc, Tc>(L, c, sy, sz, L7);
+    Lc = L7[0];
+    const Tc Lpc = hist ? Lp[c] : Lc;
+    Star<Tc> V[3];
+    Tc Vp[3] = {Tc(0), Tc(0), Tc(0)};
+    const Tc* const vel[3] = {u, v, w};
+    const Tc* const old[3] = {up, vp, wp};
 #pragma unroll
-    for (int q = 0; q < 7; ++q) {
-      G7[q] = u7[q] * L7[q];
-      H7[q] = v7[q] * L7[q];
-      I7[q] = w7[q] * L7[q];
+    for (int d = 0; d < 3; ++d) {
+      load7<Tc, Tc>(vel[d], c, sy, sz, f7);
+#pragma unroll
+      for (int s = 0; s < 7; ++s) f7[s] *= L7[s];
+      V[d] = star(f7);
+      if (hist) Vp[d] = old[d][c] * Lpc;
     }
-    const Eq5<Tc> cm = eq5_coefficients<Tc>(G7, H7, I7, upc * Lpc, vpc * Lpc, wpc * Lpc, sp);
+    const LevelN<Tc> op = level_n<Tc>(V, Vp, hist, rc);
     // one momentum system: source E (level n, and n-1 when kept) and the field X
     auto system = [&](const Tc* HOSC_RESTRICT E, const Tc* HOSC_RESTRICT Ep,
                       const Tc* HOSC_RESTRICT X) {
       Tc E7[7], f19[19];
       load7<Tc, Tc>(E, c, sy, sz, E7);
-      const Tc Epc = P.have_prev ? Ep[c] : E7[0];
-      const Tc R = bracket<Tc>(diffs7<Tc>(E7, sp), E7[0], Epc, cm, sp);
+      Tc R = E7[0] + compact_terms(star(E7), op.v24);
+      if (hist) R += Tc(0.5) * (E7[0] - Ep[c]);
       load19<Tc>(X, c, sy, sz, f19);
-      return tdt * (R - applyB<Tc>(cm, f19, sp));
+      return rc.dt * (R - apply_level_n(op, f19));
     };
     rv[0] = system(Eu, Eup, u);
     rv[1] = system(Ev, Evp, v);
     rv[2] = system(Ew, Ewp, w);
-    // level-(n+1) weights (Eq. 6): M_d = -dt/(2L) + h_d^2/12, M15 = (h^2/(6L)) dx L, ...
-    const D7<Tc> dL = diffs7<Tc>(L7, sp);
-    const Tc iL = Tc(1) / Lc;   // one division per node
-    const Tc m0 = Tc(-0.5) * tdt * iL, inv6L = Tc(2) * iL;   // h_d^2/(6L) = (h_d^2/12) (2/L)
-    const Tc Mx = m0 + sp.s12[0], My = m0 + sp.s12[1], Mz = m0 + sp.s12[2];
-    const Tc m15 = sp.s12[0] * inv6L * dL.dx, m16 = sp.s12[1] * inv6L * dL.dy,
-             m17 = sp.s12[2] * inv6L * dL.dz;
-    Tc M18 = Tc(0.5) * (Lc - Lpc) + sp.s12[0] * (dL.dxx - cm.G * dL.dx) +
-             sp.s12[1] * (dL.dyy - cm.H * dL.dy) + sp.s12[2] * (dL.dzz - cm.I * dL.dz);
+    const Star<Tc> sL = star(L7);
+    Tc M18 = compact_terms(sL, op.v24);
+    if (hist) M18 += Tc(0.5) * (Lc - Lpc);
     // keep the extrapolated mass positive where L changes fast (the steady state is unaffected)
-    const Tc alim = par<Tc>(P.a_limit, P.a_limitf), kap = par<Tc>(P.a_boost, P.a_boostf);
+    const Tc alim = par<Tc>(P.a_limit, P.a_limitf);
     if (alim > Tc(0)) M18 = fmax(M18, -alim * Lc);
-    const Tc sig_m =
-        kap > Tc(0) ? pseudo_time_mass<Tc>(cm.G, cm.H, cm.I, Lc, tdt, sp.s3, kap) : Tc(0);
-    const Tc ax = Mx * sp.isq[0], ay = My * sp.isq[1], az = Mz * sp.isq[2];
-    Am[0] = Lc * (Tc(1) - Tc(2) * (ax + ay + az)) + M18 + sig_m;
-    Am[1] = Lc * (ax - Mx * cm.G * sp.i2[0] + m15 * sp.i2[0]);
-    Am[2] = Lc * (ax + Mx * cm.G * sp.i2[0] - m15 * sp.i2[0]);
-    Am[3] = Lc * (ay - My * cm.H * sp.i2[1] + m16 * sp.i2[1]);
-    Am[4] = Lc * (ay + My * cm.H * sp.i2[1] - m16 * sp.i2[1]);
-    Am[5] = Lc * (az - Mz * cm.I * sp.i2[2] + m17 * sp.i2[2]);
-    Am[6] = Lc * (az + Mz * cm.I * sp.i2[2] - m17 * sp.i2[2]);
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      Bm[d] = ((rc.hdt + rc.s12[d] * Lc) * op.V[d] - rc.h12[d] * sL.b[d]) * rc.i2[d];
+    Dm = (Tc(0.5) * Lc + rc.dtq) + M18;
+    if (kap > Tc(0))
+      Dm += pseudo_time_mass<Tc>(op.V[0], op.V[1], op.V[2], Lc, rc.dt, rc.s3, kap);
   }
   // ---------------- energy: L = 1, G* = u, H* = v, I* = w, K* = E* = 0
   {
-    const Eq5<Tc> ce = eq5_coefficients<Tc>(u7, v7, w7, upc, vpc, wpc, sp);
-    Tc f19[19];
+    Tc f7[7], f19[19];
+    Star<Tc> V[3];
+    Tc Vp[3] = {Tc(0), Tc(0), Tc(0)};
+    const Tc* const vel[3] = {u, v, w};
+    const Tc* const old[3] = {up, vp, wp};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      load7<Tc, Tc>(vel[d], c, sy, sz, f7);
+      V[d] = star(f7);
+      if (hist) Vp[d] = old[d][c];
+    }
+    const LevelN<Tc> op = level_n<Tc>(V, Vp, hist, rc);
     load19<Tc>(th, c, sy, sz, f19);
-    rv[3] = -tdt * applyB<Tc>(ce, f19, sp);
-    const Tc m0 = Tc(-0.5) * tdt;
-    const Tc Mx = m0 + sp.s12[0], My = m0 + sp.s12[1], Mz = m0 + sp.s12[2];
-    const Tc ax = Mx * sp.isq[0], ay = My * sp.isq[1], az = Mz * sp.isq[2];
-    const Tc kap = par<Tc>(P.a_boost, P.a_boostf);
-    const Tc sig_e =
-        kap > Tc(0) ? pseudo_time_mass<Tc>(ce.G, ce.H, ce.I, Tc(1), tdt, sp.s3, kap) : Tc(0);
-    Ae[0] = Tc(1) - Tc(2) * (ax + ay + az) + sig_e;
-    Ae[1] = ax - Mx * ce.G * sp.i2[0];
-    Ae[2] = ax + Mx * ce.G * sp.i2[0];
-    Ae[3] = ay - My * ce.H * sp.i2[1];
-    Ae[4] = ay + My * ce.H * sp.i2[1];
-    Ae[5] = az - Mz * ce.I * sp.i2[2];
-    Ae[6] = az + Mz * ce.I * sp.i2[2];
+    rv[3] = -rc.dt * apply_level_n(op, f19);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) Be[d] = ((rc.hdt + rc.s12[d]) * rc.i2[d]) * op.V[d];
+    De = Tc(0.5) + rc.dtq;
+    if (kap > Tc(0))
+      De += pseudo_time_mass<Tc>(op.V[0], op.V[1], op.V[2], Tc(1), rc.dt, rc.s3, kap);
   }
+  const Tc dm = Dm != Tc(0) ? Dm : Tc(1), de = De != Tc(0) ? De : Tc(1);
   if (P.precond) {   // Jacobi row scaling: each right-hand side over its row's diagonal
-    const Tc dm = Am[0] != Tc(0) ? Am[0] : Tc(1), de = Ae[0] != Tc(0) ? Ae[0] : Tc(1);
 #pragma unroll
     for (int s = 0; s < 3; ++s) rv[s] /= dm;
     rv[3] /= de;
-    if constexpr (sizeof(Ts) != sizeof(float)) {   // the planar weights too (the compact float
-#pragma unroll                                      // operators divide by D when applied)
-      for (int q = 0; q < 7; ++q) {
-        Am[q] /= dm;
-        Ae[q] /= de;
-      }
-    }
   }
-  if constexpr (sizeof(Ts) == sizeof(float)) {   // interleaved float storage
+  if constexpr (sizeof(Ts) == sizeof(float)) {   // interleaved float storage, compact operators
     F.kr0[c] = make_float4((float)rv[0], (float)rv[1], (float)rv[2], (float)rv[3]);
-    // compact operators: the antisymmetric halves (W_{-d} - W_{+d})/2 and the diagonal
-    F.kwm[c] = make_float4((float)(Tc(0.5) * (Am[2] - Am[1])), (float)(Tc(0.5) * (Am[4] - Am[3])),
-                           (float)(Tc(0.5) * (Am[6] - Am[5])), (float)Am[0]);
-    F.kwe[c] = make_float4((float)(Tc(0.5) * (Ae[2] - Ae[1])), (float)(Tc(0.5) * (Ae[4] - Ae[3])),
-                           (float)(Tc(0.5) * (Ae[6] - Ae[5])), (float)Ae[0]);
+    F.kwm[c] = make_float4((float)Bm[0], (float)Bm[1], (float)Bm[2], (float)Dm);
+    F.kwe[c] = make_float4((float)Be[0], (float)Be[1], (float)Be[2], (float)De);
     F.kL[c] = (float)Lc;
   } else {                                         // planar double storage
 #pragma unroll
     for (int s = 0; s < 4; ++s) F.rhs[s][c] = (double)rv[s];
+    Tc Am[7], Ae[7];
+    Am[0] = Dm;
+    Ae[0] = De;
 #pragma unroll
-    for (int q = 0; q < 7; ++q) {
-      F.Am[q][c] = (double)Am[q];
-      F.Ae[q][c] = (double)Ae[q];
+    for (int d = 0; d < 3; ++d) {
+      const Tc Sm = rc.cs[d] + Tc(1.0 / 12.0) * Lc, Se = rc.cs[d] + Tc(1.0 / 12.0);
+      Am[1 + 2 * d] = Sm - Bm[d];
+      Am[2 + 2 * d] = Sm + Bm[d];
+      Ae[1 + 2 * d] = Se - Be[d];
+      Ae[2 + 2 * d] = Se + Be[d];
+    }
+    if (P.precond) {   // the weights too (the compact float operators divide by D when applied)
+#pragma unroll
+      for (int s = 0; s < 7; ++s) {
+        Am[s] /= dm;
+        Ae[s] /= de;
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < 7; ++s) {
+      F.Am[s][c] = (double)Am[s];
+      F.Ae[s][c] = (double)Ae[s];
     }
   }
 }
 
+// The float build is bounded to 80 registers (three 256-thread blocks per SM), the double builds to
+// 168 (six blocks of kFp64Threads).
 template <class Tc, class Ts>
-__global__ void __launch_bounds__(kThreads, sizeof(Tc) == sizeof(float) ? 3 : 0) k_rhs(
+__global__ void __launch_bounds__(sizeof(Tc) == sizeof(float) ? kThreads : kFp64Threads,
+                                  sizeof(Tc) == sizeof(float) ? 3 : 6) k_rhs(
     DevParams P, const Tc* HOSC_RESTRICT u, const Tc* HOSC_RESTRICT v,
     const Tc* HOSC_RESTRICT w, const Tc* HOSC_RESTRICT th, const Tc* HOSC_RESTRICT L,
     const Tc* HOSC_RESTRICT Eu, const Tc* HOSC_RESTRICT Ev, const Tc* HOSC_RESTRICT Ew,
@@ -545,43 +642,6 @@ template <class Ts>
 __global__ void __launch_bounds__(kThreads) k_apply_increment(DevParams P, Fields F, int cur,
                                                               int nblocks) {
   k_apply_increment_body<Ts>(P, F, cur, nblocks, blockIdx.x);
-}
-
-__device__ __forceinline__ int node32(int i, int j, int k, int N) { return i + N * (j + N * k); }
-
-// Node number t of the y faces (x interior, all z), then of the z faces (x, y interior):
-// 0 <= t < 2 (N-2) N + 2 (N-2)^2, x fastest.
-__device__ __forceinline__ void boundary_yz(int t, int N, int& i, int& j, int& k) {
-  const int ni = N - 2;
-  if (t < 2 * ni * N) {
-    const int side = t / (ni * N), r = t - side * ni * N;
-    const int q = r / ni;
-    i = 1 + (r - q * ni);
-    k = q;
-    j = side ? N - 1 : 0;
-  } else {
-    const int u = t - 2 * ni * N;
-    const int side = u / (ni * ni), r = u - side * ni * ni;
-    const int q = r / ni;
-    i = 1 + (r - q * ni);
-    j = 1 + q;
-    k = side ? N - 1 : 0;
-  }
-}
-
-// Node number t of the cube's boundary, 0 <= t < N^3 - (N-2)^3: the x faces, then the y and z
-// faces as in boundary_yz.
-__device__ __forceinline__ void boundary_node(int t, int N, int& i, int& j, int& k) {
-  const int N2 = N * N;
-  if (t < 2 * N2) {
-    const int side = t / N2, r = t - side * N2;
-    const int q = r / N;
-    j = r - q * N;
-    k = q;
-    i = side ? N - 1 : 0;
-  } else {
-    boundary_yz(t - 2 * N2, N, i, j, k);
-  }
 }
 
 // Extrapolation weights along one axis for a wall condition of zero normal derivative:
