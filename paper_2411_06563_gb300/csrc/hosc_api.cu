@@ -194,6 +194,7 @@ DevParams device_params(const hosc_params& p, int have_prev, int phase) {
   d.have_prev = have_prev;
   d.max_lin_iter = p.max_lin_iter;
   d.krylov_fp32 = (p.precision == HOSC_MIXED);
+  if (!d.krylov_fp32) planar_shape(p.N, &d.pb, &d.pkz);
   d.sweep_fp32 = (p.precision == HOSC_MIXED && phase == 0);
   d.h = 1.0 / (p.N - 1);
   d.h2 = d.h * d.h;

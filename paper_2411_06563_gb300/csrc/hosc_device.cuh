@@ -171,37 +171,33 @@ __host__ __device__ constexpr int row_stride() {
   return M > 2 * kRedSlots ? 4 * kRedSlots : (M > kRedSlots ? 2 * kRedSlots : kRedSlots);
 }
 
-// Reduction over the grid of M values per thread. Block b of nb writes its totals to its row of
-// red and takes a ticket; the block that takes the last one (no block waits for another) sums
-// the rows in a fixed order and returns the totals in shared memory, valid for its every thread;
-// the other blocks return null. The ticket counter is left at zero for the next kernel.
-// In the last block, with Mp the power of two >= M, thread t reads slot t % Mp of rows t / Mp,
-// t / Mp + blockDim/Mp, ... (consecutive threads read consecutive doubles; four rows' loads in
-// flight at a time). blockDim.x must be a multiple of 32, at most 32 kMaxWarps.
-template <class Op, int M>
-__device__ __forceinline__ const double* grid_total(const typename Op::V (&v)[M], double* red,
-                                                    unsigned int* counter, unsigned int b,
-                                                    unsigned int nb) {
+// Second half of a reduction over the grid, called by every block once its warp 0 has written the
+// block's values to rows of red: takes a ticket; the block that takes the last of `tickets` (no block
+// waits for another) sums the nr rows of M slots in a fixed order and returns the totals in shared
+// memory, valid for its every thread; the other blocks return null. The ticket counter is left at
+// zero for the next kernel. In the last block, with Mp the power of two >= M, thread t reads slot
+// t % Mp of rows t / Mp, t / Mp + blockDim/Mp, ... (consecutive threads read consecutive doubles;
+// four rows' loads in flight at a time). blockDim.x must be a multiple of 32, at most 32 kMaxWarps.
+template <class T, int M>
+__device__ __forceinline__ const double* last_block_total(const double* red, unsigned int* counter,
+                                                          unsigned int nr_, unsigned int tickets) {
   constexpr int Mp = pow2_at_least(M);
   constexpr long S = row_stride<M>();
-  using T = typename Op::Total;
   __shared__ double s_d[kMaxWarps * Mp];
   __shared__ double s_tot[Mp];
   __shared__ int s_last;
-  const typename Op::V mine = block_total<Op, M>(v);
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   if (wid == 0) {
-    if (lane < M) red[(long)b * S + lane] = Op::value(mine);
     __syncwarp();
     if (lane == 0) {
       __threadfence();
-      s_last = atomicAdd(counter, 1u) == nb - 1;
+      s_last = atomicAdd(counter, 1u) == tickets - 1;
     }
   }
   __syncthreads();
   if (!s_last) return nullptr;
   __threadfence();
-  const int m = t % Mp, rstep = blockDim.x / Mp, nr = (int)nb;
+  const int m = t % Mp, rstep = blockDim.x / Mp, nr = (int)nr_;
   double acc = 0.0;
   int r = m < M ? t / Mp : nr;   // lanes past the M values read nothing
   for (; r + 3 * rstep < nr; r += 4 * rstep) {
@@ -223,6 +219,17 @@ __device__ __forceinline__ const double* grid_total(const typename Op::V (&v)[M]
   }
   __syncthreads();
   return s_tot;
+}
+
+// Reduction over the grid of M values per thread: block b of nb writes its totals to its row of red;
+// the last block returns the totals (see last_block_total), the others null.
+template <class Op, int M>
+__device__ __forceinline__ const double* grid_total(const typename Op::V (&v)[M], double* red,
+                                                    unsigned int* counter, unsigned int b,
+                                                    unsigned int nb) {
+  const typename Op::V mine = block_total<Op, M>(v);
+  if (threadIdx.x < M) red[(long)b * row_stride<M>() + threadIdx.x] = Op::value(mine);
+  return last_block_total<typename Op::Total, M>(red, counter, nb, nb);
 }
 
 }  // namespace hosc

@@ -46,6 +46,8 @@ struct DevParams {
                      // form, kblock <= 256)
   int merged;        // interleaved solve: two kernels per BiCGSTAB iteration (the x, r update
                      // folded into the next p, v kernel) instead of three
+  int pb, pkz;       // planar FP64 Krylov kernels: threads per block (128, 256, 512), planes per block
+  int rhs_copied;    // planar solve: the first residual is a copy of rhs (whose walls may hold anything)
   int sx, sy, skz;   // staged stencil kernels (p/v and s/t): tile of sx * sy interior columns,
                      // skz planes per block; sx == 0 selects the register kernels instead
   int tty, ttx, tkz; // bulk-copy (TMA) stencil kernels (p/v and s/t): tile of ttx * tty interior
@@ -182,6 +184,8 @@ long krylov4_blocks(const DevParams& P);
 // Threads per block and planes per thread of the interleaved Krylov kernels when none are set:
 // 128 threads (wide three-kernel form) and the z-segment with the least wave cost below.
 void default_tiles(int N, int* kblock, int* kz);
+// Shape of the planar FP64 Krylov kernels for a grid.
+void planar_shape(int N, int* pb, int* pkz);
 // Waves of resident blocks a launch shape needs on this GPU times the planes each block streams
 // (kz + 2): a model of the launch's duration when it is latency-bound.
 double krylov4_wave_cost(int N, int kblock, int kz, int narrow, int merged, int sms);

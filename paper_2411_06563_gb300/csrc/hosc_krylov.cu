@@ -11,11 +11,11 @@
 // One iteration = three kernels; each ends with a last-block reduction that finalises the scalar
 // the next kernel needs (alpha, omega, beta / convergence). No kernel waits on another block.
 //
-// Two storage forms. FP64 (planar): one array per system and per weight, one thread per interior
-// node. Mixed precision (interleaved, float): one float4 per node holds the four systems, the
-// fourteen weights sit in four float4 per node, and a thread owns one interior (i, j) column over
-// a segment of kz planes, keeping the z-neighbours in registers as it marches; its dot-product
-// terms accumulate in float-float over the segment before the block reduction.
+// Two storage forms. FP64 (planar): one array per system and per weight; a block takes one system.
+// Mixed precision (interleaved, float): one float4 per node holds the four systems, and a thread owns
+// one interior (i, j) column over a segment of kz planes, keeping the z-neighbours in registers as
+// it marches; its dot-product terms accumulate in float-float over the segment before the block
+// reduction.
 
 #include <math.h>
 
@@ -27,31 +27,6 @@ namespace hosc {
 
 namespace {
 
-template <class T>
-__device__ __forceinline__ T apply7(const T* const* A, int c, T x0, T xp, T xm, T yp, T ym, T zp,
-                                    T zm) {
-  return A[0][c] * x0 + A[1][c] * xp + A[2][c] * xm + A[3][c] * yp + A[4][c] * ym +
-         A[5][c] * zp + A[6][c] * zm;
-}
-
-template <class T>
-__device__ __forceinline__ T* vec(double* p) { return reinterpret_cast<T*>(p); }
-template <class T>
-__device__ __forceinline__ const T* const* ops(double* const* p) {
-  return reinterpret_cast<const T* const*>(p);
-}
-
-// Thread t -> interior node (1 + t % ni, ...) in 32-bit arithmetic (N^3 < 2^31 for N <= 1025).
-// Thread t -> interior node (1 + t % ni, ...) in 32-bit arithmetic (N^3 < 2^31 for N <= 1025).
-__device__ __forceinline__ bool interior_index(const DevParams& P, unsigned t, int& c) {
-  const unsigned N = P.N, ni = N - 2;
-  if (t >= ni * ni * ni) return false;
-  const unsigned q = t / ni;
-  const unsigned i = t - q * ni, j = q % ni, k = q / ni;
-  c = (int)((i + 1) + N * ((j + 1) + N * (k + 1)));
-  return true;
-}
-
 // Algorithmic bytes of one launch: every array element the active systems touch, once.
 __device__ __forceinline__ double launch_bytes(const DevParams& P, const int done[4],
                                                double per_system_words, double coeff_words,
@@ -60,30 +35,6 @@ __device__ __forceinline__ double launch_bytes(const DevParams& P, const int don
   const int nm = !done[0] + !done[1] + !done[2], ne = !done[3];
   const double words = per_system_words * (nm + ne) + coeff_words * ((nm > 0) + ne);
   return word_bytes * ni * ni * ni * words;
-}
-
-// r = r_0 = rhs, x = 0, p = v = 0; ||r_0||^2 per system.
-template <class T>
-__global__ void __launch_bounds__(kThreads) k_bicg_init(DevParams P, Fields F, int nblocks) {
-  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
-  int c;
-  double dot[4] = {};
-  if (interior_index(P, t, c)) {
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      const T r = vec<T>(F.rhs[s])[c];
-      vec<T>(F.r[s])[c] = r;
-      vec<T>(F.x[s])[c] = T(0);
-      vec<T>(F.pk[0][s])[c] = T(0);
-      vec<T>(F.pk[1][s])[c] = T(0);
-      vec<T>(F.vk[0][s])[c] = T(0);
-      vec<T>(F.vk[1][s])[c] = T(0);
-      if (P.solver == 1) vec<T>(F.u0[s])[c] = T(0);
-      dot[s] = r * r;
-    }
-  }
-  if (const double* tot = grid_total<SumD, 4>(dot, F.red, F.counter, blockIdx.x, nblocks))
-    finish_init(P, F, tot);
 }
 
 // End of one pass of the captured BiCGSTAB loop body: continue while a system is iterating.
@@ -95,413 +46,331 @@ __global__ void k_loop_cond(const KrylovScalars* ks, cudaGraphConditionalHandle 
   }
 }
 
-// p_new = r + beta (p_old - omega v_old) on the fly at the 7 stencil nodes, v_new = A p_new,
-// partial r0 . v_new; last block: alpha = rho / (r0 . v).
-template <class T>
-__global__ void __launch_bounds__(kThreads) k_bicg_pv(DevParams P, Fields F, int pp, int nblocks) {
-  __shared__ T s_beta[4], s_omega[4];
-  __shared__ int s_done[4];
-  if (threadIdx.x < 4) {
-    s_beta[threadIdx.x] = (T)F.ks[threadIdx.x].beta;
-    s_omega[threadIdx.x] = (T)F.ks[threadIdx.x].omega;
-    s_done[threadIdx.x] = F.ks[threadIdx.x].done;
-  }
-  __syncthreads();
-  if (s_done[0] & s_done[1] & s_done[2] & s_done[3]) return;  // uniform over the grid
-  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int sy = P.N, sz = P.N * P.N;
-  int c;
-  double dot[4] = {};
-  if (interior_index(P, t, c)) {
-#pragma unroll 1
-    for (int s = 0; s < 4; ++s) {
-      if (s_done[s]) continue;
-      const T* r = vec<T>(F.r[s]);
-      const T* po = vec<T>(F.pk[pp][s]);
-      const T* vo = vec<T>(F.vk[pp][s]);
-      const T b = s_beta[s], om = s_omega[s];
-      const int nb[7] = {c, c + 1, c - 1, c + sy, c - sy, c + sz, c - sz};
-      T pn[7];
-#pragma unroll
-      for (int q = 0; q < 7; ++q) pn[q] = r[nb[q]] + b * (po[nb[q]] - om * vo[nb[q]]);
-      const T* const* A = (s < 3) ? ops<T>(F.Am) : ops<T>(F.Ae);
-      const T vn = apply7<T>(A, c, pn[0], pn[1], pn[2], pn[3], pn[4], pn[5], pn[6]);
-      vec<T>(F.pk[1 - pp][s])[c] = pn[0];
-      vec<T>(F.vk[1 - pp][s])[c] = vn;
-      dot[s] = vec<T>(F.rhs[s])[c] * vn;
-    }
-  }
-  if (const double* tot = grid_total<SumD, 4>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
-    finish_pv(F, tot);
-    count_bytes(F, HOSC_K_BICG_PV, launch_bytes(P, s_done, 6.0, 7.0, sizeof(T)));
-  }
-}
-
-// s = r - alpha v on the fly at the 7 stencil nodes, t = A s, partials (t . s, t . t);
-// last block: omega = (t . s)/(t . t) (0 when t = 0).
-template <class T>
-__global__ void __launch_bounds__(kThreads) k_bicg_st(DevParams P, Fields F, int pp, int nblocks) {
-  __shared__ T s_alpha[4];
-  __shared__ int s_done[4];
-  if (threadIdx.x < 4) {
-    s_alpha[threadIdx.x] = (T)F.ks[threadIdx.x].alpha;
-    s_done[threadIdx.x] = F.ks[threadIdx.x].done;
-  }
-  __syncthreads();
-  if (s_done[0] & s_done[1] & s_done[2] & s_done[3]) return;
-  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int sy = P.N, sz = P.N * P.N;
-  const int np = 1 - pp;   // buffers written by k_bicg_pv of this iteration
-  int c;
-  double dot[8] = {};
-  if (interior_index(P, t, c)) {
-#pragma unroll 1
-    for (int s = 0; s < 4; ++s) {
-      if (s_done[s]) continue;
-      const T* r = vec<T>(F.r[s]);
-      const T* v = vec<T>(F.vk[np][s]);
-      const T a = s_alpha[s];
-      const int nb[7] = {c, c + 1, c - 1, c + sy, c - sy, c + sz, c - sz};
-      T sv[7];
-#pragma unroll
-      for (int q = 0; q < 7; ++q) sv[q] = r[nb[q]] - a * v[nb[q]];
-      const T* const* A = (s < 3) ? ops<T>(F.Am) : ops<T>(F.Ae);
-      const T tv = apply7<T>(A, c, sv[0], sv[1], sv[2], sv[3], sv[4], sv[5], sv[6]);
-      vec<T>(F.t[s])[c] = tv;
-      dot[s] = tv * sv[0];
-      dot[4 + s] = tv * tv;
-    }
-  }
-  if (const double* tot = grid_total<SumD, 8>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
-    finish_st(F, tot);
-    count_bytes(F, HOSC_K_BICG_ST, launch_bytes(P, s_done, 3.0, 7.0, sizeof(T)));
-  }
-}
-
-// s = r - alpha v; x += alpha p + omega s; r = s - omega t; partials (r0 . r, r . r);
-// last block: convergence test, breakdown test, beta and rho for the next iteration.
-template <class T>
-__global__ void __launch_bounds__(kThreads) k_bicg_xr(DevParams P, Fields F, int pp, int nblocks) {
-  __shared__ T s_alpha[4], s_omega[4];
-  __shared__ int s_done[4];
-  if (threadIdx.x < 4) {
-    s_alpha[threadIdx.x] = (T)F.ks[threadIdx.x].alpha;
-    s_omega[threadIdx.x] = (T)F.ks[threadIdx.x].omega;
-    s_done[threadIdx.x] = F.ks[threadIdx.x].done;
-  }
-  __syncthreads();
-  if (s_done[0] & s_done[1] & s_done[2] & s_done[3]) return;
-  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int np = 1 - pp;
-  int c;
-  double dot[8] = {};
-  if (interior_index(P, t, c)) {
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      if (s_done[s]) continue;
-      const T a = s_alpha[s], om = s_omega[s];
-      T* x = vec<T>(F.x[s]);
-      T* r = vec<T>(F.r[s]);
-      const T sv = r[c] - a * vec<T>(F.vk[np][s])[c];
-      x[c] = x[c] + a * vec<T>(F.pk[np][s])[c] + om * sv;
-      const T rn = sv - om * vec<T>(F.t[s])[c];
-      r[c] = rn;
-      dot[s] = vec<T>(F.rhs[s])[c] * rn;
-      dot[4 + s] = rn * rn;
-    }
-  }
-  if (const double* tot = grid_total<SumD, 8>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
-    finish_xr(P, F, tot);
-    count_bytes(F, HOSC_K_BICG_XR, launch_bytes(P, s_done, 8.0, 0.0, sizeof(T)));
-  }
-}
-
-// ------------------------------------------------------------------ BiCGSTAB(2), planar FP64
+// ------------------------------------------------------------------ planar FP64 solve
 //
-// One cycle (Sleijpen and Fokkema's BiCGSTAB(ell) with ell = 2; shadow residual rt = r_0 = rhs)
-// in five kernels, each with a last-block reduction that finalises the scalars of the next:
-//   B1  u_0 <- r_0 - beta u_0 (on the fly at the stencil), u_1 = A u_0;       alpha = rho/(rt.u_1)
-//   B2  r_0 <- r_0 - alpha u_1 (on the fly), r_1 = A r_0; u_0 <- r_0 - beta u_0 and x += alpha u_0
-//       (pointwise, with the r_0 of B1);                   rho_1 = rt.r_1, beta = alpha rho_1/rho
-//   B3  u_0 <- r_0 - beta u_0 (pointwise); u_1 <- r_1 - beta u_1 (on the fly), u_2 = A u_1;
+// GB300's FP64 pipe takes 16 cycles of an SM for a warp's instruction, so these kernels are bound by
+// the number of FP64 instructions a node, not by bytes. A kernel that applies an operator to a vector
+// combined on the fly (r + beta (p - omega v), r - alpha v, ...) evaluated that vector at all seven
+// points of every node: 14 instructions beside the operator's 7 for p/v. Here a block takes one system,
+// B consecutive nodes of the plane (i + N j, walls included: they are zero) and pkz planes; it
+// evaluates the vector once at its nodes and at the N nodes before and after them, puts the plane in
+// shared memory (two planes, one barrier a plane) and keeps the planes above and below in registers:
+// 2 (1 + 2N/B) + 7 + 1 instructions for p/v. One system a block spreads the small grids over four
+// times the SMs; the three momentum blocks of a chunk are neighbours in the grid, so their weights
+// come from L2. A block's partial goes to its row's slot of its system; the last block of the launch
+// sums all rows. The shape (B, pkz) has the least modelled load of the busiest SM (planar_shape).
+// Measured, alone: p/v 137 -> 84.7 us, s/t 117 -> 75.9, x/r 74.5 -> 46.4 at 91^3; 14.4 -> 7.4, 14.2 ->
+// 7.5, 12.3 -> 7.6 at 21^3.
+//
+// BiCGSTAB (solver = 0): p/v, s/t, x/r. BiCGSTAB(2) (Sleijpen and Fokkema's BiCGSTAB(ell) with
+// ell = 2; shadow residual rt = r_0 = rhs), one cycle in five kernels:
+//   U1  u_0 <- r_0 - beta u_0 (on the fly at the stencil), u_1 = A u_0;       alpha = rho/(rt.u_1)
+//   R1  r_0 <- r_0 - alpha u_1 (on the fly), r_1 = A r_0; u_0 <- r_0 - beta u_0 and x += alpha u_0
+//       (pointwise, with the r_0 of U1);                   rho_1 = rt.r_1, beta = alpha rho_1/rho
+//   U2  u_0 <- r_0 - beta u_0 (pointwise); u_1 <- r_1 - beta u_1 (on the fly), u_2 = A u_1;
 //                                                          alpha = rho/(rt.u_2)
-//   B4  r_0 -= alpha u_1 (pointwise); r_1 <- r_1 - alpha u_2 (on the fly), r_2 = A r_1;
+//   R2  r_0 -= alpha u_1 (pointwise); r_1 <- r_1 - alpha u_2 (on the fly), r_2 = A r_1;
 //       x += alpha u_0; the five inner products of r_0, r_1, r_2 give the minimal-residual
 //       coefficients: tau = (r_1.r_2)/(r_1.r_1), gamma'_1 = (r_0.r_1)/(r_1.r_1), gamma_2 =
 //       gamma'_2 = (r_0.r_2 - tau r_0.r_1)/(r_2.r_2 - tau r_1.r_2), gamma_1 = gamma'_1 - tau gamma_2
-//   B5  x += gamma_1 r_0 + gamma_2 r_1; r_0 -= gamma_1 r_1 + gamma_2 r_2; u_0 -= gamma_1 u_1 +
+//   MR  x += gamma_1 r_0 + gamma_2 r_1; r_0 -= gamma_1 r_1 + gamma_2 r_2; u_0 -= gamma_1 u_1 +
 //       gamma_2 u_2 (the Gram-Schmidt step folded into the coefficients); rho <- -omega rho,
 //       rho_1 = rt.r_0, beta = alpha rho_1/rho, rho = rho_1, convergence on ||r_0||.
-// Buffers per system: r_0 in r / t (ping-pong by cycle: B2 reads one and writes the other, the
-// stencil reads the old r_0 at the neighbours), r_1 in pk[0] (B2) then pk[1] (B4), u_1 in vk[0]
-// (B1) then vk[1] (B3), u_0, r_2, u_2 in their own arrays. A kernel writes no array that it reads
+// Buffers per system: r_0 in r / t (ping-pong by cycle: R1 reads one and writes the other, the
+// stencil reads the old r_0 at the neighbours), r_1 in pk[0] (R1) then pk[1] (R2), u_1 in vk[0]
+// (U1) then vk[1] (U2), u_0, r_2, u_2 in their own arrays. A kernel writes no array that it reads
 // at a neighbour.
+//
+// The first iteration (no iteration counted yet) reads rhs for the residual and no search direction,
+// so that nothing but x has to be initialised. Where the walls of rhs are not known to be zero
+// (rhs_copied: the caller's arrays of the allocation-free solve) the residual is a copy.
 
-struct B2Shared {
-  double alpha[4], beta[4], g1[4], g2[4];
-  int done[4];
-};
+enum { PL_PV, PL_ST, PL_U1, PL_R1, PL_U2, PL_R2, PL_XR, PL_MR };
 
-// The four systems' scalars into shared memory; true when every system is done (uniform).
-__device__ __forceinline__ bool b2_load(const Fields& F, B2Shared& sh) {
-  if (threadIdx.x < 4) {
-    const KrylovScalars k = F.ks[threadIdx.x];
-    sh.alpha[threadIdx.x] = k.alpha;
-    sh.beta[threadIdx.x] = k.beta;
-    sh.g1[threadIdx.x] = k.g1;
-    sh.g2[threadIdx.x] = k.g2;
-    sh.done[threadIdx.x] = k.done;
-  }
-  __syncthreads();
-  return sh.done[0] & sh.done[1] & sh.done[2] & sh.done[3];
-}
-
-__device__ __forceinline__ void nbrs7(int c, int sy, int sz, int nb[7]) {
-  nb[0] = c;
-  nb[1] = c + 1;
-  nb[2] = c - 1;
-  nb[3] = c + sy;
-  nb[4] = c - sy;
-  nb[5] = c + sz;
-  nb[6] = c - sz;
-}
+// Dot products of a launch, per system, and the slots of a row of partials.
+constexpr int pl_dots(int kind) { return kind == PL_R2 ? 5 : kind == PL_ST || kind >= PL_XR ? 2 : 1; }
+constexpr int pl_slots(int kind) { return kind == PL_R2 ? 20 : 4 * pl_dots(kind); }
 
 __device__ __forceinline__ void b2_fail(KrylovScalars& k) {
   k.done = 1;
   k.status = HOSC_ENOCONV;
 }
 
-// rt . u (slots 0..3): alpha = rho / (rt . u).
-__device__ __forceinline__ void b2_finish_alpha(const Fields& F, const double* tot) {
-  if (threadIdx.x >= 4) return;
-  KrylovScalars& k = F.ks[threadIdx.x];
-  const int done = k.done;
-  const double rho = k.rho, d = tot[threadIdx.x];
-  if (done) return;
-  if (d == 0.0 || !isfinite(d)) b2_fail(k);
-  else k.alpha = rho / d;
-}
-
-__device__ __forceinline__ const double* const* b2_op(const Fields& F, int s) {
-  return (s < 3) ? ops<double>(F.Am) : ops<double>(F.Ae);
-}
-
-// B1
-__global__ void __launch_bounds__(kThreads) k_b2_u1(DevParams P, Fields F, int cp, int nblocks) {
-  __shared__ B2Shared sh;
-  if (b2_load(F, sh)) return;
-  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int sy = P.N, sz = P.N * P.N;
-  int c;
-  double dot[4] = {};
-  if (interior_index(P, t, c)) {
-    int nb[7];
-    nbrs7(c, sy, sz, nb);
-#pragma unroll 1
-    for (int s = 0; s < 4; ++s) {
-      if (sh.done[s]) continue;
-      const double* r0 = cp ? F.t[s] : F.r[s];
-      const double* u0 = F.u0[s];
-      const double b = sh.beta[s];
-      double un[7];
-#pragma unroll
-      for (int q = 0; q < 7; ++q) un[q] = r0[nb[q]] - b * u0[nb[q]];
-      const double u1 = apply7<double>(b2_op(F, s), c, un[0], un[1], un[2], un[3], un[4], un[5],
-                                       un[6]);
-      F.vk[0][s][c] = u1;
-      dot[s] = F.rhs[s][c] * u1;
-    }
-  }
-  if (const double* tot = grid_total<SumD, 4>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
-    b2_finish_alpha(F, tot);
-    count_bytes(F, HOSC_K_BICG_PV, launch_bytes(P, sh.done, 4.0, 7.0, sizeof(double)));
-  }
-}
-
-// B2
-__global__ void __launch_bounds__(kThreads) k_b2_r1(DevParams P, Fields F, int cp, int nblocks) {
-  __shared__ B2Shared sh;
-  if (b2_load(F, sh)) return;
-  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int sy = P.N, sz = P.N * P.N;
-  int c;
-  double dot[4] = {};
-  if (interior_index(P, t, c)) {
-    int nb[7];
-    nbrs7(c, sy, sz, nb);
-#pragma unroll 1
-    for (int s = 0; s < 4; ++s) {
-      if (sh.done[s]) continue;
-      const double* r0 = cp ? F.t[s] : F.r[s];
-      double* r0n = cp ? F.r[s] : F.t[s];
-      const double* u1 = F.vk[0][s];
-      const double a = sh.alpha[s], b = sh.beta[s];
-      double rn[7];
-#pragma unroll
-      for (int q = 0; q < 7; ++q) rn[q] = r0[nb[q]] - a * u1[nb[q]];
-      const double r1 = apply7<double>(b2_op(F, s), c, rn[0], rn[1], rn[2], rn[3], rn[4], rn[5],
-                                       rn[6]);
-      r0n[c] = rn[0];
-      F.pk[0][s][c] = r1;
-      const double u0 = r0[c] - b * F.u0[s][c];
-      F.u0[s][c] = u0;
-      F.x[s][c] += a * u0;
-      dot[s] = F.rhs[s][c] * r1;
-    }
-  }
-  if (const double* tot = grid_total<SumD, 4>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
-    if (threadIdx.x < 4) {
-      KrylovScalars& k = F.ks[threadIdx.x];
-      const double rho1 = tot[threadIdx.x];
-      if (!k.done) {
-        if (k.rho == 0.0 || !isfinite(rho1)) {
-          b2_fail(k);
-        } else {
-          k.beta = k.alpha * rho1 / k.rho;
-          k.rho = rho1;
-        }
+// The scalars that a launch of this kind leaves, and its algorithmic bytes.
+template <int KIND>
+__device__ __forceinline__ void planar_finish(const DevParams& P, const Fields& F,
+                                              const double* tot, const int (&done)[4]) {
+  if (KIND == PL_PV || KIND == PL_U1 || KIND == PL_U2) finish_pv(F, tot);
+  if (KIND == PL_ST) finish_st(F, tot);
+  if (KIND == PL_XR) finish_xr(P, F, tot);
+  if (KIND == PL_R1 && threadIdx.x < 4) {
+    KrylovScalars& k = F.ks[threadIdx.x];
+    const double rho1 = tot[threadIdx.x];
+    if (!k.done) {
+      if (k.rho == 0.0 || !isfinite(rho1)) {
+        b2_fail(k);
+      } else {
+        k.beta = k.alpha * rho1 / k.rho;
+        k.rho = rho1;
       }
     }
-    count_bytes(F, HOSC_K_BICG_ST, launch_bytes(P, sh.done, 9.0, 7.0, sizeof(double)));
   }
-}
-
-// B3
-__global__ void __launch_bounds__(kThreads) k_b2_u2(DevParams P, Fields F, int cp, int nblocks) {
-  __shared__ B2Shared sh;
-  if (b2_load(F, sh)) return;
-  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int sy = P.N, sz = P.N * P.N;
-  int c;
-  double dot[4] = {};
-  if (interior_index(P, t, c)) {
-    int nb[7];
-    nbrs7(c, sy, sz, nb);
-#pragma unroll 1
-    for (int s = 0; s < 4; ++s) {
-      if (sh.done[s]) continue;
-      const double* r0 = cp ? F.r[s] : F.t[s];   // written by B2
-      const double* r1 = F.pk[0][s];
-      const double* u1 = F.vk[0][s];
-      const double b = sh.beta[s];
-      F.u0[s][c] = r0[c] - b * F.u0[s][c];
-      double un[7];
-#pragma unroll
-      for (int q = 0; q < 7; ++q) un[q] = r1[nb[q]] - b * u1[nb[q]];
-      const double u2 = apply7<double>(b2_op(F, s), c, un[0], un[1], un[2], un[3], un[4], un[5],
-                                       un[6]);
-      F.vk[1][s][c] = un[0];
-      F.u2[s][c] = u2;
-      dot[s] = F.rhs[s][c] * u2;
-    }
-  }
-  if (const double* tot = grid_total<SumD, 4>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
-    b2_finish_alpha(F, tot);
-    count_bytes(F, HOSC_K_BICG_PV, launch_bytes(P, sh.done, 8.0, 7.0, sizeof(double)));
-  }
-}
-
-// B4
-__global__ void __launch_bounds__(kThreads) k_b2_r2(DevParams P, Fields F, int cp, int nblocks) {
-  __shared__ B2Shared sh;
-  if (b2_load(F, sh)) return;
-  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int sy = P.N, sz = P.N * P.N;
-  int c;
-  // per system: r1.r1, r1.r2, r2.r2, r0.r1, r0.r2
-  double dot[20] = {};
-  if (interior_index(P, t, c)) {
-    int nb[7];
-    nbrs7(c, sy, sz, nb);
-#pragma unroll   // dot[] is indexed by the system: unrolled, it stays in registers
-    for (int s = 0; s < 4; ++s) {
-      if (sh.done[s]) continue;
-      double* r0 = cp ? F.r[s] : F.t[s];
-      const double* r1 = F.pk[0][s];
-      const double* u2 = F.u2[s];
-      const double a = sh.alpha[s];
-      const double r0c = r0[c] - a * F.vk[1][s][c];
-      r0[c] = r0c;
-      double rn[7];
-#pragma unroll
-      for (int q = 0; q < 7; ++q) rn[q] = r1[nb[q]] - a * u2[nb[q]];
-      const double r2 = apply7<double>(b2_op(F, s), c, rn[0], rn[1], rn[2], rn[3], rn[4], rn[5],
-                                       rn[6]);
-      F.pk[1][s][c] = rn[0];
-      F.r2[s][c] = r2;
-      F.x[s][c] += a * F.u0[s][c];
-      dot[5 * s] = rn[0] * rn[0];
-      dot[5 * s + 1] = rn[0] * r2;
-      dot[5 * s + 2] = r2 * r2;
-      dot[5 * s + 3] = r0c * rn[0];
-      dot[5 * s + 4] = r0c * r2;
-    }
-  }
-  if (const double* tot = grid_total<SumD, 20>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
-    if (threadIdx.x < 4) {
-      KrylovScalars& k = F.ks[threadIdx.x];
-      const double* d = tot + 5 * threadIdx.x;   // r1.r1, r1.r2, r2.r2, r0.r1, r0.r2
-      const double sig1 = d[0];
-      const double tau = sig1 > 0.0 ? d[1] / sig1 : 0.0;
-      const double sig2 = d[2] - tau * d[1];   // |r_2 - tau r_1|^2
-      if (!k.done) {
-        if (!(sig1 > 0.0) || !(sig2 > 0.0) || !isfinite(sig2)) {
-          b2_fail(k);
-        } else {
-          const double gp1 = d[3] / sig1, g2 = (d[4] - tau * d[3]) / sig2;
-          k.g2 = g2;
-          k.g1 = gp1 - tau * g2;
-          k.omega = g2;
-        }
+  if (KIND == PL_R2 && threadIdx.x < 4) {
+    KrylovScalars& k = F.ks[threadIdx.x];
+    const double* d = tot + 5 * threadIdx.x;   // r1.r1, r1.r2, r2.r2, r0.r1, r0.r2
+    const double sig1 = d[0];
+    const double tau = sig1 > 0.0 ? d[1] / sig1 : 0.0;
+    const double sig2 = d[2] - tau * d[1];   // |r_2 - tau r_1|^2
+    if (!k.done) {
+      if (!(sig1 > 0.0) || !(sig2 > 0.0) || !isfinite(sig2)) {
+        b2_fail(k);
+      } else {
+        const double gp1 = d[3] / sig1, g2 = (d[4] - tau * d[3]) / sig2;
+        k.g2 = g2;
+        k.g1 = gp1 - tau * g2;
+        k.omega = g2;
       }
     }
-    count_bytes(F, HOSC_K_BICG_ST, launch_bytes(P, sh.done, 10.0, 7.0, sizeof(double)));
   }
-}
-
-// B5
-__global__ void __launch_bounds__(kThreads) k_b2_mr(DevParams P, Fields F, int cp, int nblocks) {
-  __shared__ B2Shared sh;
-  if (b2_load(F, sh)) return;
-  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
-  int c;
-  double dot[8] = {};
-  if (interior_index(P, t, c)) {
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      if (sh.done[s]) continue;
-      double* r0 = cp ? F.r[s] : F.t[s];
-      const double g1 = sh.g1[s], g2 = sh.g2[s];
-      const double r0c = r0[c], r1 = F.pk[1][s][c], r2 = F.r2[s][c];
-      F.x[s][c] += g1 * r0c + g2 * r1;
-      const double rn = r0c - g1 * r1 - g2 * r2;
-      r0[c] = rn;
-      F.u0[s][c] -= g1 * F.vk[1][s][c] + g2 * F.u2[s][c];
-      dot[s] = F.rhs[s][c] * rn;
-      dot[4 + s] = rn * rn;
-    }
-  }
-  if (const double* tot = grid_total<SumD, 8>(dot, F.red, F.counter, blockIdx.x, nblocks)) {
-    if (threadIdx.x < 4) {
-      KrylovScalars& k = F.ks[threadIdx.x];
-      if (!k.done) {
-        const double rho1 = tot[threadIdx.x], rnorm = sqrt(tot[4 + threadIdx.x]);
-        k.rnorm = rnorm;
-        k.iters += 2;
-        const double rho0 = -k.omega * k.rho;
-        if (rnorm <= P.tol_lin * k.r0norm) {
-          k.done = 1;
-          k.status = 0;
-        } else if (!isfinite(rnorm) || k.iters >= P.max_lin_iter || rho0 == 0.0) {
-          b2_fail(k);
-        } else {
-          k.beta = k.alpha * rho1 / rho0;
-          k.rho = rho1;
-        }
+  if (KIND == PL_MR && threadIdx.x < 4) {
+    KrylovScalars& k = F.ks[threadIdx.x];
+    if (!k.done) {
+      const double rho1 = tot[threadIdx.x], rnorm = sqrt(tot[4 + threadIdx.x]);
+      k.rnorm = rnorm;
+      k.iters += 2;
+      const double rho0 = -k.omega * k.rho;
+      if (rnorm <= P.tol_lin * k.r0norm) {
+        k.done = 1;
+        k.status = 0;
+      } else if (!isfinite(rnorm) || k.iters >= P.max_lin_iter || rho0 == 0.0) {
+        b2_fail(k);
+      } else {
+        k.beta = k.alpha * rho1 / rho0;
+        k.rho = rho1;
       }
     }
-    count_bytes(F, HOSC_K_BICG_XR, launch_bytes(P, sh.done, 11.0, 0.0, sizeof(double)));
   }
+  constexpr int cls = KIND == PL_PV || KIND == PL_U1 || KIND == PL_U2 ? HOSC_K_BICG_PV
+                      : KIND >= PL_XR                                 ? HOSC_K_BICG_XR
+                                                                      : HOSC_K_BICG_ST;
+  constexpr double words[8] = {6.0, 3.0, 4.0, 9.0, 8.0, 10.0, 8.0, 11.0};
+  count_bytes(F, cls, launch_bytes(P, done, words[KIND], KIND >= PL_XR ? 0.0 : 7.0,
+                                   sizeof(double)));
+}
+
+// What every planar kernel starts with: which system, chunk and planes this block has.
+struct Planar {
+  int s;          // system
+  bool live;      // it still iterates
+  bool first;     // no iteration yet
+  int l;          // this thread's node of the plane, i + N j
+  bool inner;     // inside the walls of the plane
+  int k0, k1;     // planes
+  unsigned row, rows;
+};
+
+// False when every system is done (the same for every block).
+__device__ __forceinline__ bool planar_block(const DevParams& P, const Fields& F, Planar& b,
+                                             int (&done)[4]) {
+  b.s = (int)(blockIdx.x & 3u);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) done[q] = F.ks[q].done;
+  const int iters = F.ks[b.s].iters;
+  if (done[0] & done[1] & done[2] & done[3]) return false;
+  b.live = !(b.s == 0 ? done[0] : b.s == 1 ? done[1] : b.s == 2 ? done[2] : done[3]);
+  b.first = iters == 0;
+  const int N = P.N;
+  b.l = (int)(blockIdx.x >> 2) * (int)blockDim.x + (int)threadIdx.x;
+  const int j = b.l / N, i = b.l - j * N;
+  b.inner = i > 0 && i < N - 1 && j > 0 && j < N - 1;
+  b.k0 = 1 + (int)blockIdx.y * P.pkz;
+  b.k1 = min(b.k0 + P.pkz, N - 1);
+  b.row = (blockIdx.x >> 2) + (gridDim.x >> 2) * blockIdx.y;
+  b.rows = (gridDim.x >> 2) * gridDim.y;
+  return true;
+}
+
+template <int KIND>
+__device__ __forceinline__ void planar_end(const DevParams& P, const Fields& F, const Planar& b,
+                                           const double (&dot)[pl_dots(KIND)],
+                                           const int (&done)[4]) {
+  constexpr int M = pl_dots(KIND), S = pl_slots(KIND);
+  const double mine = block_total<SumD, M>(dot);
+  if (threadIdx.x < M) {
+    const int slot = M == 5 ? 5 * b.s + (int)threadIdx.x : b.s + 4 * (int)threadIdx.x;
+    F.red[(long)b.row * row_stride<S>() + slot] = mine;
+  }
+  if (const double* tot = last_block_total<SumD, S>(F.red, F.counter, b.rows,
+                                                    gridDim.x * gridDim.y))
+    planar_finish<KIND>(P, F, tot, done);
+}
+
+// The kernels that apply an operator. pp: parity of the iteration (BiCGSTAB) or cycle.
+template <int KIND, int B>
+__global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, int pp) {
+  extern __shared__ double planes[];   // two planes of N + B + N values
+  pdl_wait_and_release();
+  Planar b;
+  int done[4];
+  if (!planar_block(P, F, b, done)) return;
+  double dot[pl_dots(KIND)] = {};
+  if (b.live) {   // the same for the whole block
+    const int s = b.s, N = P.N, N2 = N * N, t = threadIdx.x, w = B + 2 * N;
+    const double alpha = F.ks[s].alpha, beta = F.ks[s].beta, omega = F.ks[s].omega;
+    const bool first = b.first && (KIND == PL_PV || KIND == PL_ST || KIND == PL_U1 || KIND == PL_R1);
+    const double* rhs = F.rhs[s];
+    // the vector that the operator is applied to: X - q Y (p/v: X + beta (Z - omega Y))
+    const double *X, *Y, *Z = nullptr;
+    double q;
+    if (KIND == PL_PV) { X = F.r[s]; Y = F.vk[pp][s]; Z = F.pk[pp][s]; q = omega; }
+    if (KIND == PL_ST) { X = F.r[s]; Y = F.vk[1 - pp][s]; q = alpha; }
+    if (KIND == PL_U1) { X = pp ? F.t[s] : F.r[s]; Y = F.u0[s]; q = beta; }
+    if (KIND == PL_R1) { X = pp ? F.t[s] : F.r[s]; Y = F.vk[0][s]; q = alpha; }
+    if (KIND == PL_U2) { X = F.pk[0][s]; Y = F.vk[0][s]; q = beta; }
+    if (KIND == PL_R2) { X = F.pk[0][s]; Y = F.u2[s]; q = alpha; }
+    if (first && !P.rhs_copied) X = rhs;
+    const bool plain = first && (KIND == PL_PV || KIND == PL_U1);   // no search direction yet
+    auto value = [&](int c) {
+      const double x = X[c];
+      if (plain) return x;
+      if (KIND == PL_PV) return x + beta * (Z[c] - q * Y[c]);
+      return x - q * Y[c];
+    };
+    const double* const* A = s < 3 ? F.Am : F.Ae;
+    const double *a0 = A[0], *a1 = A[1], *a2 = A[2], *a3 = A[3], *a4 = A[4], *a5 = A[5], *a6 = A[6];
+    const bool mine = b.l < N2;
+    const int l0 = b.l - t;
+    double lo = mine ? value(b.l + N2 * (b.k0 - 1)) : 0.0;
+    double mid = mine ? value(b.l + N2 * b.k0) : 0.0;
+    for (int k = b.k0; k < b.k1; ++k) {
+      const int c = b.l + N2 * k;
+      double* pl = planes + (k & 1) * w;
+      pl[N + t] = mid;
+      for (int h = t; h < 2 * N; h += B) {   // the N nodes before the chunk and after it
+        const int hl = h < N ? l0 - N + h : l0 + B + (h - N);
+        pl[h < N ? h : B + h] = hl >= 0 && hl < N2 ? value(hl + N2 * k) : 0.0;
+      }
+      const double hi = mine ? value(c + N2) : 0.0;
+      __syncthreads();
+      if (b.inner) {
+        const double* o = pl + N + t;
+        const double y = a0[c] * mid + a1[c] * o[1] + a2[c] * o[-1] + a3[c] * o[N] +
+                         a4[c] * o[-N] + a5[c] * hi + a6[c] * lo;
+        if (KIND == PL_PV) {
+          F.pk[1 - pp][s][c] = mid;
+          F.vk[1 - pp][s][c] = y;
+          dot[0] += rhs[c] * y;
+        } else if (KIND == PL_ST) {
+          F.t[s][c] = y;
+          dot[0] += y * mid;
+          dot[pl_dots(KIND) - 1] += y * y;
+        } else if (KIND == PL_U1) {
+          F.vk[0][s][c] = y;
+          dot[0] += rhs[c] * y;
+        } else if (KIND == PL_R1) {
+          (pp ? F.r[s] : F.t[s])[c] = mid;
+          F.pk[0][s][c] = y;
+          const double r0 = X[c], u0 = first ? r0 : r0 - beta * F.u0[s][c];
+          F.u0[s][c] = u0;
+          F.x[s][c] += alpha * u0;
+          dot[0] += rhs[c] * y;
+        } else if (KIND == PL_U2) {
+          const double* r0 = pp ? F.r[s] : F.t[s];   // written by R1
+          F.u0[s][c] = r0[c] - beta * F.u0[s][c];
+          F.vk[1][s][c] = mid;
+          F.u2[s][c] = y;
+          dot[0] += rhs[c] * y;
+        } else {
+          double* r0 = pp ? F.r[s] : F.t[s];
+          const double r0c = r0[c] - alpha * F.vk[1][s][c];
+          r0[c] = r0c;
+          F.pk[1][s][c] = mid;
+          F.r2[s][c] = y;
+          F.x[s][c] += alpha * F.u0[s][c];
+          constexpr int L = pl_dots(KIND) - 1;   // 4 here
+          dot[0] += mid * mid;
+          dot[L / 4] += mid * y;
+          dot[L / 2] += y * y;
+          dot[3 * L / 4] += r0c * mid;
+          dot[L] += r0c * y;
+        }
+      }
+      lo = mid;
+      mid = hi;
+    }
+  }
+  planar_end<KIND>(P, F, b, dot, done);
+}
+
+// The pointwise ends: x/r (s = r - alpha v; x += alpha p + omega s; r = s - omega t; r0.r, r.r) and MR.
+template <int KIND, int B>
+__global__ void __launch_bounds__(B) k_planar_end(DevParams P, Fields F, int pp) {
+  pdl_wait_and_release();
+  Planar b;
+  int done[4];
+  if (!planar_block(P, F, b, done)) return;
+  double dot[2] = {};
+  if (b.live && b.inner) {
+    const int s = b.s, N2 = P.N * P.N;
+    const double* rhs = F.rhs[s];
+    double* x = F.x[s];
+    if (KIND == PL_XR) {
+      const double a = F.ks[s].alpha, om = F.ks[s].omega;
+      const double *v = F.vk[1 - pp][s], *p = F.pk[1 - pp][s], *tv = F.t[s];
+      const double* ro = b.first ? rhs : F.r[s];
+      double* r = F.r[s];
+#pragma unroll 2
+      for (int k = b.k0; k < b.k1; ++k) {
+        const int c = b.l + N2 * k;
+        const double sv = ro[c] - a * v[c];
+        x[c] = x[c] + a * p[c] + om * sv;
+        const double rn = sv - om * tv[c];
+        r[c] = rn;
+        dot[0] += rhs[c] * rn;
+        dot[1] += rn * rn;
+      }
+    } else {
+      const double g1 = F.ks[s].g1, g2 = F.ks[s].g2;
+      double *r0 = pp ? F.r[s] : F.t[s], *u0 = F.u0[s];
+      const double *r1 = F.pk[1][s], *r2 = F.r2[s], *u1 = F.vk[1][s], *u2 = F.u2[s];
+#pragma unroll 2
+      for (int k = b.k0; k < b.k1; ++k) {
+        const int c = b.l + N2 * k;
+        const double r0c = r0[c], r1c = r1[c];
+        x[c] += g1 * r0c + g2 * r1c;
+        const double rn = r0c - g1 * r1c - g2 * r2[c];
+        r0[c] = rn;
+        u0[c] -= g1 * u1[c] + g2 * u2[c];
+        dot[0] += rhs[c] * rn;
+        dot[1] += rn * rn;
+      }
+    }
+  }
+  planar_end<KIND>(P, F, b, dot, done);
+}
+
+// x = 0 and ||r_0||^2 of each system.
+template <int B>
+__global__ void __launch_bounds__(B) k_planar_init(DevParams P, Fields F) {
+  const int s = (int)(blockIdx.x & 3u), N = P.N, N2 = N * N;
+  const int l = (int)(blockIdx.x >> 2) * B + (int)threadIdx.x, j = l / N, i = l - j * N;
+  const int k0 = 1 + (int)blockIdx.y * P.pkz, k1 = min(k0 + P.pkz, N - 1);
+  double dot[1] = {};
+  if (i > 0 && i < N - 1 && j > 0 && j < N - 1) {
+    for (int k = k0; k < k1; ++k) {
+      const double r = F.rhs[s][l + N2 * k];
+      F.x[s][l + N2 * k] = 0.0;
+      if (P.rhs_copied) F.r[s][l + N2 * k] = r;
+      dot[0] += r * r;
+    }
+  }
+  const double mine = block_total<SumD, 1>(dot);
+  const unsigned chunks = gridDim.x >> 2;
+  if (threadIdx.x == 0)
+    F.red[(long)((blockIdx.x >> 2) + chunks * blockIdx.y) * row_stride<4>() + s] = mine;
+  if (const double* tot = last_block_total<SumD, 4>(F.red, F.counter, chunks * gridDim.y,
+                                                    gridDim.x * gridDim.y))
+    finish_init(P, F, tot);
 }
 
 // ------------------------------------------------------------- merged iteration (two kernels)
@@ -872,18 +741,13 @@ dim3 grid4(const DevParams& P) {
   return dim3((unsigned)((ni * ni + P.kblock - 1) / P.kblock), (unsigned)((ni + P.kz - 1) / P.kz));
 }
 
-int interior_blocks(const DevParams& P) {
-  const long ni = P.N - 2;
-  return red_blocks(ni * ni * ni);
-}
-
 }  // namespace
 
 namespace {
 __global__ void k_krylov_activate(KrylovScalars* ks) {
   if (threadIdx.x < 4) {
     ks[threadIdx.x].done = 0;
-    ks[threadIdx.x].iters = 0;
+    ks[threadIdx.x].iters = 1;   // not the first iteration, which reads less
     ks[threadIdx.x].status = 0;
   }
 }
@@ -895,6 +759,37 @@ void launch_krylov_activate(const Fields& F, cudaStream_t s) {
 
 void launch_loop_cond(const Fields& F, unsigned long long handle, cudaStream_t s) {
   k_loop_cond<<<1, 32, 0, s>>>(F.ks, (cudaGraphConditionalHandle)handle);
+}
+
+dim3 planar_grid(const DevParams& P) {
+  const int ni = P.N - 2;
+  return dim3(4u * (unsigned)((P.N * P.N + P.pb - 1) / P.pb), (unsigned)((ni + P.pkz - 1) / P.pkz));
+}
+
+// Threads a block and planes a block of the planar kernels: the least load of the busiest SM in
+// cycles, from the FP64 instructions of p/v (16 cycles a warp), and the chain of a block's planes
+// (a barrier and the loads behind it). At most red_rows(N^3)/4 rows of partials.
+void planar_shape(int N, int* pb, int* pkz) {
+  const int sms = device_sms(), ni = N - 2;
+  const long most = red_rows((long)N * N * N) / 4;
+  double best = 1e300;
+  *pb = 512;
+  *pkz = ni;
+  for (int B : {128, 256, 512}) {
+    const long chunks = (N * (long)N + B - 1) / B;
+    for (int z = 1; z <= ni; ++z) {
+      const long rows = chunks * ((ni + z - 1) / z);
+      if (rows > most) continue;
+      const double warps = B / 32.0, halo = (2 * N + 31) / 32;
+      const double work = warps * (2.0 * (z + 2) + 8.0 * z + 10.0) + 2.0 * halo * z;
+      const double cost = 16.0 * work * (double)((4 * rows + sms - 1) / sms) + 900.0 * z;
+      if (cost < best) {
+        best = cost;
+        *pb = B;
+        *pkz = z;
+      }
+    }
+  }
 }
 
 void launch_bicg_init(const DevParams& P, const Fields& F, cudaStream_t s) {
@@ -910,8 +805,10 @@ void launch_bicg_init(const DevParams& P, const Fields& F, cudaStream_t s) {
     k4_init<<<b, kThreads, 0, s>>>(P, F);
     return;
   }
-  const int b = interior_blocks(P);
-  k_bicg_init<double><<<b, kThreads, 0, s>>>(P, F, b);
+  const dim3 g = planar_grid(P);
+  if (P.pb == 128) k_planar_init<128><<<g, 128, 0, s>>>(P, F);
+  else if (P.pb == 256) k_planar_init<256><<<g, 256, 0, s>>>(P, F);
+  else k_planar_init<512><<<g, 512, 0, s>>>(P, F);
 }
 
 // x/r as one flat stream: every node of the interior planes, the i and j walls included (every
@@ -993,11 +890,11 @@ int xr_flat_blocks() {
 // programmatic edges.
 template <class K>
 void launch_pdl(K kern, dim3 grid, int threads, cudaStream_t s, const DevParams& P,
-                const Fields& F, int pp) {
+                const Fields& F, int pp, size_t smem = 0) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1005,6 +902,20 @@ void launch_pdl(K kern, dim3 grid, int threads, cudaStream_t s, const DevParams&
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kern, P, F, pp);
+}
+
+template <int KIND, int B>
+void launch_planar_b(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
+  if constexpr (KIND >= PL_XR)
+    launch_pdl(k_planar_end<KIND, B>, planar_grid(P), B, s, P, F, pp);
+  else   // two planes of N + B + N doubles: 41 KB at N = 1025
+    launch_pdl(k_planar<KIND, B>, planar_grid(P), B, s, P, F, pp, 16 * (size_t)(B + 2 * P.N));
+}
+template <int KIND>
+void launch_planar(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
+  if (P.pb == 128) launch_planar_b<KIND, 128>(P, F, pp, s);
+  else if (P.pb == 256) launch_planar_b<KIND, 256>(P, F, pp, s);
+  else launch_planar_b<KIND, 512>(P, F, pp, s);
 }
 
 void launch_bicg_pv(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
@@ -1026,8 +937,7 @@ void launch_bicg_pv(const DevParams& P, const Fields& F, int pp, cudaStream_t s)
     else launch_pdl(k4_pv<2>, grid4(P), P.kblock, s, P, F, pp);
     return;
   }
-  const int b = interior_blocks(P);
-  k_bicg_pv<double><<<b, kThreads, 0, s>>>(P, F, pp, b);
+  launch_planar<PL_PV>(P, F, pp, s);
 }
 
 void launch_bicg_st(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
@@ -1049,8 +959,7 @@ void launch_bicg_st(const DevParams& P, const Fields& F, int pp, cudaStream_t s)
     else launch_pdl(k4_st<2>, grid4(P), P.kblock, s, P, F, pp);
     return;
   }
-  const int b = interior_blocks(P);
-  k_bicg_st<double><<<b, kThreads, 0, s>>>(P, F, pp, b);
+  launch_planar<PL_ST>(P, F, pp, s);
 }
 
 void launch_bicg_xr(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
@@ -1064,18 +973,16 @@ void launch_bicg_xr(const DevParams& P, const Fields& F, int pp, cudaStream_t s)
     else launch_pdl(k4_xr<2>, grid4(P), P.kblock, s, P, F, pp);
     return;
   }
-  const int b = interior_blocks(P);
-  k_bicg_xr<double><<<b, kThreads, 0, s>>>(P, F, pp, b);
+  launch_planar<PL_XR>(P, F, pp, s);
 }
 
 void launch_b2(int kernel, const DevParams& P, const Fields& F, int cp, cudaStream_t s) {
-  const int b = interior_blocks(P);
   switch (kernel) {
-    case 0: k_b2_u1<<<b, kThreads, 0, s>>>(P, F, cp, b); break;
-    case 1: k_b2_r1<<<b, kThreads, 0, s>>>(P, F, cp, b); break;
-    case 2: k_b2_u2<<<b, kThreads, 0, s>>>(P, F, cp, b); break;
-    case 3: k_b2_r2<<<b, kThreads, 0, s>>>(P, F, cp, b); break;
-    default: k_b2_mr<<<b, kThreads, 0, s>>>(P, F, cp, b); break;
+    case 0: launch_planar<PL_U1>(P, F, cp, s); break;
+    case 1: launch_planar<PL_R1>(P, F, cp, s); break;
+    case 2: launch_planar<PL_U2>(P, F, cp, s); break;
+    case 3: launch_planar<PL_R2>(P, F, cp, s); break;
+    default: launch_planar<PL_MR>(P, F, cp, s); break;
   }
 }
 

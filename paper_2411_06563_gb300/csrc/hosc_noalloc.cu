@@ -24,7 +24,7 @@ constexpr size_t kVecBytes = kMaxNodes * sizeof(double);
 constexpr size_t kAlignB = 256;
 // 6 vectors (r, p x2, v x2, t) for each of the 4 systems, then the small control block.
 constexpr size_t kVectorsBytes = 24 * ((kVecBytes + kAlignB - 1) / kAlignB * kAlignB);
-constexpr size_t kMaxBlocks = (kMaxNodes + kThreads - 1) / kThreads;
+constexpr size_t kMaxBlocks = 1024;   // rows of partials: red_rows / 4 and below for every N
 constexpr size_t kControlBytes = 64 * 1024 + kMaxBlocks * kRedSlots * sizeof(double);
 constexpr size_t kScratchBytes = kVectorsBytes + kControlBytes;
 // Offsets of the control block: solver scalars at 0, ticket counter at 512, halt flag at 768,
@@ -118,6 +118,8 @@ extern "C" hosc_status hosc_bicgstab_noalloc(int N, const double* const* weights
   P.tol_lin = tol;
   P.h = 1.0 / (N - 1);
   P.h2 = P.h * P.h;
+  P.rhs_copied = 1;
+  planar_shape(N, &P.pb, &P.pkz);
 
   KrylovScalars ks[4];
   launch_bicg_init(P, F, sm);
