@@ -146,6 +146,7 @@ void apply_tiles(Ctx* c) {
   c->P.tstages = c->tstages;
   c->P.tkernels = c->tkernels;
   c->P.xr_flat = c->xr_flat;
+  c->P.lean = !c->merged && c->sx == 0 && c->tty == 0;
 }
 
 bool stencil_tiles_valid(const Ctx* c, int sx, int sy, int skz) {
@@ -415,7 +416,7 @@ hosc_status solve_b2(Ctx* c, const DevParams& P) {
     for (int q = 0; q < cycles; ++q) {
       for (int kk = 0; kk < 5; ++kk) {
         prof_begin(c, kClass[kk]);
-        launch_b2(kk, P, F, cp, c->stream);
+        launch_b2(kk, P, F, cp, it == 0 && q == 0, c->stream);
         prof_end(c, kClass[kk]);
       }
       cp ^= 1;
@@ -435,21 +436,24 @@ hosc_status solve_b2(Ctx* c, const DevParams& P) {
 // BiCGSTAB on the four systems; the host checks the done flags every few iterations.
 hosc_status solve_with(Ctx* c, const DevParams& P) {
   const Fields& F = c->F;
-  launch_bicg_init(P, F, c->stream);
-  c->launches += 1;
+  if (P.krylov_fp32 && !P.lean) {
+    launch_bicg_init(P, F, c->stream);
+    c->launches += 1;
+  }
   if (P.solver == 1) return solve_b2(c, P);
   int pp = 0, it = 0, check = c->prof_on ? 1 : 4;
   while (it < P.max_lin_iter) {
     const int chunk = (P.max_lin_iter - it < check) ? P.max_lin_iter - it : check;
     for (int q = 0; q < chunk; ++q) {
       prof_begin(c, HOSC_K_BICG_PV);
-      launch_bicg_pv(P, F, pp, c->stream);
+      const bool first = it + q == 0;
+      launch_bicg_pv(P, F, pp, first, c->stream);
       prof_end(c, HOSC_K_BICG_PV);
       prof_begin(c, HOSC_K_BICG_ST);
-      launch_bicg_st(P, F, pp, c->stream);
+      launch_bicg_st(P, F, pp, first, c->stream);
       prof_end(c, HOSC_K_BICG_ST);
       prof_begin(c, HOSC_K_BICG_XR);
-      launch_bicg_xr(P, F, pp, c->stream);
+      launch_bicg_xr(P, F, pp, first, c->stream);
       prof_end(c, HOSC_K_BICG_XR);
       pp ^= 1;
     }
@@ -474,8 +478,8 @@ hosc_status solve(Ctx* c) { return solve_with(c, c->P); }
 // systems solved again from level n (theta's system skipped), increments, div V, correction.
 hosc_status update_with_inner(Ctx* c) {
   const Fields& F = c->F;
-  launch_update_fields(c->P, F, c->cur, c->stream);
-  c->launches += 5;
+  launch_update(c->P, F, c->cur, 0, c->stream);
+  c->launches += kUpdateLaunches;
   int k = 0;
   for (;;) {
     hosc_status st = check_launch();
@@ -486,17 +490,13 @@ hosc_status update_with_inner(Ctx* c) {
     ++k;
     DevParams Q = c->P;
     Q.inner_pass = 1;
-    if (Q.sweep_fp32) {   // float copies of the new temperature and the corrected pressure
-      launch_shadow(Q, F, c->cur, 0, c->stream);
-      c->launches += 1;
-    }
     launch_sources(Q, F, c->cur, c->stream);
     launch_rhs(Q, F, c->cur, c->stream);
     c->launches += 2;
     st = solve_with(c, Q);
     if (st) return st;
-    launch_update_fields(Q, F, c->cur, c->stream);
-    c->launches += 5;
+    launch_update(Q, F, c->cur, 0, c->stream);
+    c->launches += kUpdateLaunches;
   }
   launch_finish(c->P, F, c->stream);
   c->launches += 1;
@@ -546,16 +546,12 @@ hosc_status run_stage(Ctx* c, int stage) {
       if (c->prm.inner_max > 0) {
         st = update_with_inner(c);
       } else {
-        launch_update(c->P, F, c->cur, c->stream);
-        c->launches += 6;
+        launch_update(c->P, F, c->cur, 1, c->stream);
+        c->launches += kUpdateLaunches;
       }
       prof_end(c, HOSC_K_UPDATE);
       if (st) return st;
-      if (c->P.krylov_fp32) {   // mixed precision: float copies of the new level
-        launch_shadow(c->P, F, 1 - c->cur, 0, c->stream);
-        c->launches += 1;
-        c->shadow_valid = true;
-      }
+      if (c->P.krylov_fp32) c->shadow_valid = true;   // the update writes the float copies too
       // increments: x4 + u, v, w, theta read, u, v, w, theta written; div: V read, div written;
       // pressure: p, div read, p written
       c->host_bytes[HOSC_K_UPDATE] += 8.0 * (n3 * 12 + ni3 * 4 + ni3 * 3);
@@ -596,9 +592,9 @@ hosc_status time_class(Ctx* c, int kid, int reps, double* ms_out) {
       case HOSC_K_RHS: launch_rhs(P, F, c->cur, c->stream); break;
       default:
         launch_krylov_activate(F, c->stream);
-        if (kid == HOSC_K_BICG_PV) launch_bicg_pv(P, F, 0, c->stream);
-        if (kid == HOSC_K_BICG_ST) launch_bicg_st(P, F, 0, c->stream);
-        if (kid == HOSC_K_BICG_XR) launch_bicg_xr(P, F, 0, c->stream);
+        if (kid == HOSC_K_BICG_PV) launch_bicg_pv(P, F, 0, false, c->stream);
+        if (kid == HOSC_K_BICG_ST) launch_bicg_st(P, F, 0, false, c->stream);
+        if (kid == HOSC_K_BICG_XR) launch_bicg_xr(P, F, 0, false, c->stream);
         break;
     }
   }
@@ -685,11 +681,25 @@ hosc_status one_step(Ctx* c, hosc_info* info) {
 
 // ------------------------------------------------------------------ captured steps (CUDA graphs)
 
-// Append one whole step to the capture in progress on s0: S1-S4 kernels, then a conditional
-// WHILE node whose body (captured on s1) runs two BiCGSTAB iterations (the ping-pong buffers
-// return to their parity) and sets the condition on the device, then the update kernels (and the
-// float state copy in mixed precision). Nothing in the step waits on the host. cur and have_prev
-// are those of the step's level n.
+// One BiCGSTAB iteration (one BiCGSTAB(2) cycle with solver = 1) on stream s.
+void append_iteration(const DevParams& P, const Fields& F, int pp, bool first, cudaStream_t s) {
+  if (P.solver == 1) {
+    for (int kk = 0; kk < 5; ++kk) launch_b2(kk, P, F, pp, first, s);
+  } else {
+    launch_bicg_pv(P, F, pp, first, s);
+    launch_bicg_st(P, F, pp, first, s);
+    launch_bicg_xr(P, F, pp, first, s);
+  }
+}
+
+// Whether the solve's first iteration is a form of its own, so that the loop starts after it.
+bool first_apart(const DevParams& P) { return !P.krylov_fp32 || P.lean; }
+
+// Append one whole step to the capture in progress on s0: S1-S4 kernels, the first BiCGSTAB iteration
+// (the forms without one: the initialisation), then a conditional WHILE node whose body (captured on
+// s1) runs two iterations (the ping-pong buffers return to their parity) and sets the condition on the
+// device, then the update kernels. Nothing in the step waits on the host. cur and
+// have_prev are those of the step's level n.
 cudaError_t append_step(Ctx* c, cudaStream_t s0, cudaStream_t s1, int cur, int have_prev) {
   DevParams P = c->P;
   P.have_prev = have_prev;
@@ -697,7 +707,9 @@ cudaError_t append_step(Ctx* c, cudaStream_t s0, cudaStream_t s1, int cur, int h
   launch_viscosity(P, F, cur, s0);
   launch_sources(P, F, cur, s0);
   launch_rhs(P, F, cur, s0);
-  launch_bicg_init(P, F, s0);
+  const int apart = first_apart(P) ? 1 : 0;
+  if (apart) append_iteration(P, F, 0, true, s0);
+  else launch_bicg_init(P, F, s0);
   cudaStreamCaptureStatus cs;
   const cudaGraphNode_t* deps = nullptr;
   size_t nd = 0;
@@ -720,22 +732,13 @@ cudaError_t append_step(Ctx* c, cudaStream_t s0, cudaStream_t s1, int cur, int h
     e = cudaStreamBeginCaptureToGraph(s1, body, nullptr, nullptr, 0,
                                       cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      for (int pp = 0; pp < 2; ++pp) {   // BiCGSTAB: two iterations; BiCGSTAB(2): two cycles
-        if (P.solver == 1) {
-          for (int kk = 0; kk < 5; ++kk) launch_b2(kk, P, F, pp, s1);
-        } else {
-          launch_bicg_pv(P, F, pp, s1);
-          launch_bicg_st(P, F, pp, s1);
-          launch_bicg_xr(P, F, pp, s1);
-        }
-      }
+      for (int q = 0; q < 2; ++q) append_iteration(P, F, (q + apart) & 1, false, s1);
       launch_loop_cond(F, (unsigned long long)h, s1);
       cudaGraph_t bo = nullptr;
       e = cudaStreamEndCapture(s1, &bo);
     }
   }
-  launch_update(P, F, cur, s0);
-  if (P.krylov_fp32) launch_shadow(P, F, 1 - cur, 0, s0);
+  launch_update(P, F, cur, 1, s0);
   return e;
 }
 
@@ -802,12 +805,13 @@ hosc_status fold_records(Ctx* c, unsigned n, hosc_info* info, bool* steady) {
     }
     int most = 0;
     for (int s = 0; s < 4; ++s) most = r.iters[s] > most ? r.iters[s] : most;
-    // kernels and iterations per loop pass (BiCGSTAB(2): two five-kernel cycles, 4 iterations)
+    // kernels of an iteration (BiCGSTAB(2): a cycle of five, counted as two iterations); the loop runs
+    // them two at a time, at least once, after the first where that is apart
     const bool b2 = c->P.solver == 1;
-    const long body = b2 ? 11 : ((c->P.krylov_fp32 && c->P.merged) ? 5 : 7);
-    const long per = b2 ? 4 : 2;
-    const long passes = (most + per - 1) / per > 0 ? (most + per - 1) / per : 1;
-    c->launches += 4 + 6 + (c->P.krylov_fp32 ? 1 : 0) + body * passes;
+    const long per = b2 ? 5 : (c->P.krylov_fp32 && c->P.merged ? 2 : 3);
+    const long iters = b2 ? (most + 1) / 2 : most, apart = first_apart(c->P) ? 1 : 0;
+    const long passes = std::max(1L, (iters - apart + 1) / 2);
+    c->launches += 3 + (1 - apart) + kUpdateLaunches + per * (apart + 2 * passes) + passes;
     if (r.status != HOSC_OK) {
       st = (hosc_status)r.status;
       break;

@@ -66,6 +66,33 @@ __device__ __forceinline__ double second_invariant(const Grad9& g) {
   return 2.0 * (g.ux * g.ux + g.vy * g.vy + g.wz * g.wz) + a * a + b * b + c * c;
 }
 
+// Programmatic dependent launch: the kernels of a step are launched so that each may start while the
+// previous one is finishing (its blocks take SMs as the previous kernel's blocks leave); a kernel
+// waits for the previous grid's completion and memory before its first access, and lets the next
+// kernel launch at once.
+__device__ __forceinline__ void pdl_wait_and_release() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launch of a kernel that starts with pdl_wait_and_release; in a captured step such kernels chain
+// with programmatic edges.
+template <class... K, class... A>
+inline void launch_pdl(void (*kern)(K...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                       const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, K(args)...);
+}
+
 // ----------------------------------------------------------------------------- reductions
 
 // Larger of two non-negative doubles (+inf allowed). For such values the IEEE order is the order

@@ -54,6 +54,8 @@ struct DevParams {
                      // columns, tkz planes per block; tty == 0: not used
   int tstages;       // their ring of shared-memory stages (3, 4, 6 or 8)
   int tkernels;      // which of them run: 1 p/v, 2 s/t, 3 both
+  int lean;          // interleaved solve started by the right-hand sides' kernel: no initialisation,
+                     // the first iteration reads r_0 and nothing else (register kernels, either x/r)
   int xr_flat;       // x/r as one flat grid-stride stream (k8_xr) instead of the column march
   double h, h2;      // grid spacing along x and its square
   double Ly, Lz;     // box 1 x Ly x Lz: lengths along y and z (1 for the cube)
@@ -220,22 +222,25 @@ void launch_viscosity(const DevParams& P, const Fields& F, int cur, cudaStream_t
 void launch_sources(const DevParams& P, const Fields& F, int cur, cudaStream_t s);
 // S3/S4: right-hand sides dt (R - B chi^n) and the level-(n+1) weights at interior nodes.
 void launch_rhs(const DevParams& P, const Fields& F, int cur, cudaStream_t s);
-// S5: BiCGSTAB pieces.
+// S5: BiCGSTAB pieces. The initialisation is for the interleaved forms that are not lean and for planar
+// solves whose right-hand sides the caller wrote.
 void launch_bicg_init(const DevParams& P, const Fields& F, cudaStream_t s);
-void launch_bicg_pv(const DevParams& P, const Fields& F, int pp, cudaStream_t s);
-void launch_bicg_st(const DevParams& P, const Fields& F, int pp, cudaStream_t s);
-void launch_bicg_xr(const DevParams& P, const Fields& F, int pp, cudaStream_t s);
-// BiCGSTAB(2), planar FP64 solve: the five kernels of one cycle, r_0 ping-pong parity cp
-// (launch_bicg_init starts the solve for either solver).
-void launch_b2(int kernel, const DevParams& P, const Fields& F, int cp, cudaStream_t s);
+// first: the first iteration of a solve (forms that need no launch_bicg_init; ignored by the others).
+void launch_bicg_pv(const DevParams& P, const Fields& F, int pp, bool first, cudaStream_t s);
+void launch_bicg_st(const DevParams& P, const Fields& F, int pp, bool first, cudaStream_t s);
+void launch_bicg_xr(const DevParams& P, const Fields& F, int pp, bool first, cudaStream_t s);
+// BiCGSTAB(2), planar FP64 solve: the five kernels of one cycle, r_0 ping-pong parity cp.
+void launch_b2(int kernel, const DevParams& P, const Fields& F, int cp, bool first,
+               cudaStream_t s);
+// End of the body of the BiCGSTAB loop of a captured step: end of the loop when every system is done.
+void launch_loop_cond(const Fields& F, unsigned long long handle, cudaStream_t s);
 // Mark all four systems as iterating (for timing the Krylov kernels in isolation).
 void launch_krylov_activate(const Fields& F, cudaStream_t s);
-// Body of the BiCGSTAB loop of a captured step: end of the loop when every system is done.
-void launch_loop_cond(const Fields& F, unsigned long long handle, cudaStream_t s);
-// S6-S8: increments, theta walls, div V, pressure correction and walls, step record.
-void launch_update(const DevParams& P, const Fields& F, int cur, cudaStream_t s);
-// The same without the step record (an inner pressure pass follows), and the record alone.
-void launch_update_fields(const DevParams& P, const Fields& F, int cur, cudaStream_t s);
+// S6-S8: increments, theta walls, div V, pressure correction and walls, in mixed precision with the
+// float copies of what they write, and (record) the step record: an inner pressure pass follows
+// otherwise, and the record alone ends the step.
+constexpr int kUpdateLaunches = 4;
+void launch_update(const DevParams& P, const Fields& F, int cur, int record, cudaStream_t s);
 void launch_finish(const DevParams& P, const Fields& F, cudaStream_t s);
 // Re-arm the device control of a sequence of steps: run (halt = 0), no records yet, and stop at
 // the first steady step when stop_steady.
@@ -258,7 +263,6 @@ struct RoundMember {
   int theta_walls;     // adiabatic wall nodes with x interior
   int pressure_walls;  // boundary nodes
   int kx, ky;          // Krylov tiles: column chunks x plane segments
-  int init;            // blocks of the Krylov initialisation (a grid-stride loop)
 };
 struct RoundState;
 RoundState* round_state_create();

@@ -38,12 +38,12 @@ __device__ __forceinline__ double launch_bytes(const DevParams& P, const int don
 }
 
 // End of one pass of the captured BiCGSTAB loop body: continue while a system is iterating.
-// Bounded: k_bicg_xr marks a system done at max_lin_iter at the latest.
+// Bounded: a system is done at max_lin_iter at the latest. A launch of its own: with the call in the
+// iteration's last kernel a pass took about 5 us longer (41^3 FP64 step 976 -> 1030 us).
 __global__ void k_loop_cond(const KrylovScalars* ks, cudaGraphConditionalHandle handle) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    const unsigned more = !(ks[0].done && ks[1].done && ks[2].done && ks[3].done);
-    cudaGraphSetConditional(handle, more);
-  }
+  const int done = threadIdx.x < 4 ? ks[threadIdx.x].done : 1;
+  const int all = __all_sync(0xffffffffu, done);
+  if (threadIdx.x == 0) cudaGraphSetConditional(handle, !all);
 }
 
 // ------------------------------------------------------------------ planar FP64 solve
@@ -81,15 +81,20 @@ __global__ void k_loop_cond(const KrylovScalars* ks, cudaGraphConditionalHandle 
 // (U1) then vk[1] (U2), u_0, r_2, u_2 in their own arrays. A kernel writes no array that it reads
 // at a neighbour.
 //
-// The first iteration (no iteration counted yet) reads rhs for the residual and no search direction,
-// so that nothing but x has to be initialised. Where the walls of rhs are not known to be zero
+// The first iteration (FIRST) reads rhs for the residual, no search direction and no iterate, so that
+// nothing has to be initialised. Where the walls of rhs are not known to be zero
 // (rhs_copied: the caller's arrays of the allocation-free solve) the residual is a copy.
 
 enum { PL_PV, PL_ST, PL_U1, PL_R1, PL_U2, PL_R2, PL_XR, PL_MR };
 
 // Dot products of a launch, per system, and the slots of a row of partials.
-constexpr int pl_dots(int kind) { return kind == PL_R2 ? 5 : kind == PL_ST || kind >= PL_XR ? 2 : 1; }
-constexpr int pl_slots(int kind) { return kind == PL_R2 ? 20 : 4 * pl_dots(kind); }
+// (p/v and U1: r_0 . r_0 beside r_0 . v, used in the first iteration)
+constexpr int pl_dots(int kind, bool first) {
+  return kind == PL_R2 ? 5 : kind == PL_ST || kind >= PL_XR ? 2 : kind <= PL_U1 && first ? 2 : 1;
+}
+constexpr int pl_slots(int kind, bool first) {
+  return kind == PL_R2 ? 20 : 4 * pl_dots(kind, first);
+}
 
 __device__ __forceinline__ void b2_fail(KrylovScalars& k) {
   k.done = 1;
@@ -99,8 +104,10 @@ __device__ __forceinline__ void b2_fail(KrylovScalars& k) {
 // The scalars that a launch of this kind leaves, and its algorithmic bytes.
 template <int KIND>
 __device__ __forceinline__ void planar_finish(const DevParams& P, const Fields& F,
-                                              const double* tot, const int (&done)[4]) {
-  if (KIND == PL_PV || KIND == PL_U1 || KIND == PL_U2) finish_pv(F, tot);
+                                              const double* tot, bool first,
+                                              const int (&done)[4]) {
+  if (KIND == PL_PV || KIND == PL_U1) finish_pv(F, tot, first);
+  if (KIND == PL_U2) finish_pv(F, tot, false);
   if (KIND == PL_ST) finish_st(F, tot);
   if (KIND == PL_XR) finish_xr(P, F, tot);
   if (KIND == PL_R1 && threadIdx.x < 4) {
@@ -162,23 +169,25 @@ __device__ __forceinline__ void planar_finish(const DevParams& P, const Fields& 
 struct Planar {
   int s;          // system
   bool live;      // it still iterates
-  bool first;     // no iteration yet
   int l;          // this thread's node of the plane, i + N j
   bool inner;     // inside the walls of the plane
   int k0, k1;     // planes
   unsigned row, rows;
 };
 
-// False when every system is done (the same for every block).
+// False when every system is done (the same for every block). The kernels that write x run in the
+// first iteration all the same unless the sequence has been halted: a system with a zero right-hand
+// side gets its zero increment.
+template <int KIND, bool FIRST>
 __device__ __forceinline__ bool planar_block(const DevParams& P, const Fields& F, Planar& b,
                                              int (&done)[4]) {
   b.s = (int)(blockIdx.x & 3u);
 #pragma unroll
   for (int q = 0; q < 4; ++q) done[q] = F.ks[q].done;
-  const int iters = F.ks[b.s].iters;
-  if (done[0] & done[1] & done[2] & done[3]) return false;
+  if (done[0] & done[1] & done[2] & done[3]) {
+    if (!(FIRST && (KIND == PL_XR || KIND == PL_R1)) || *F.halt) return false;
+  }
   b.live = !(b.s == 0 ? done[0] : b.s == 1 ? done[1] : b.s == 2 ? done[2] : done[3]);
-  b.first = iters == 0;
   const int N = P.N;
   b.l = (int)(blockIdx.x >> 2) * (int)blockDim.x + (int)threadIdx.x;
   const int j = b.l / N, i = b.l - j * N;
@@ -190,11 +199,11 @@ __device__ __forceinline__ bool planar_block(const DevParams& P, const Fields& F
   return true;
 }
 
-template <int KIND>
+template <int KIND, bool FIRST>
 __device__ __forceinline__ void planar_end(const DevParams& P, const Fields& F, const Planar& b,
-                                           const double (&dot)[pl_dots(KIND)],
+                                           const double (&dot)[pl_dots(KIND, FIRST)],
                                            const int (&done)[4]) {
-  constexpr int M = pl_dots(KIND), S = pl_slots(KIND);
+  constexpr int M = pl_dots(KIND, FIRST), S = pl_slots(KIND, FIRST);
   const double mine = block_total<SumD, M>(dot);
   if (threadIdx.x < M) {
     const int slot = M == 5 ? 5 * b.s + (int)threadIdx.x : b.s + 4 * (int)threadIdx.x;
@@ -202,22 +211,22 @@ __device__ __forceinline__ void planar_end(const DevParams& P, const Fields& F, 
   }
   if (const double* tot = last_block_total<SumD, S>(F.red, F.counter, b.rows,
                                                     gridDim.x * gridDim.y))
-    planar_finish<KIND>(P, F, tot, done);
+    planar_finish<KIND>(P, F, tot, FIRST, done);
 }
 
 // The kernels that apply an operator. pp: parity of the iteration (BiCGSTAB) or cycle.
-template <int KIND, int B>
+template <int KIND, int B, bool FIRST>
 __global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, int pp) {
   extern __shared__ double planes[];   // two planes of N + B + N values
   pdl_wait_and_release();
   Planar b;
   int done[4];
-  if (!planar_block(P, F, b, done)) return;
-  double dot[pl_dots(KIND)] = {};
+  if (!planar_block<KIND, FIRST>(P, F, b, done)) return;
+  constexpr int L = pl_dots(KIND, FIRST) - 1;
+  double dot[L + 1] = {};
   if (b.live) {   // the same for the whole block
     const int s = b.s, N = P.N, N2 = N * N, t = threadIdx.x, w = B + 2 * N;
     const double alpha = F.ks[s].alpha, beta = F.ks[s].beta, omega = F.ks[s].omega;
-    const bool first = b.first && (KIND == PL_PV || KIND == PL_ST || KIND == PL_U1 || KIND == PL_R1);
     const double* rhs = F.rhs[s];
     // the vector that the operator is applied to: X - q Y (p/v: X + beta (Z - omega Y))
     const double *X, *Y, *Z = nullptr;
@@ -228,8 +237,8 @@ __global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, i
     if (KIND == PL_R1) { X = pp ? F.t[s] : F.r[s]; Y = F.vk[0][s]; q = alpha; }
     if (KIND == PL_U2) { X = F.pk[0][s]; Y = F.vk[0][s]; q = beta; }
     if (KIND == PL_R2) { X = F.pk[0][s]; Y = F.u2[s]; q = alpha; }
-    if (first && !P.rhs_copied) X = rhs;
-    const bool plain = first && (KIND == PL_PV || KIND == PL_U1);   // no search direction yet
+    if (FIRST && KIND <= PL_R1 && !P.rhs_copied) X = rhs;   // a copy in r otherwise
+    constexpr bool plain = FIRST && (KIND == PL_PV || KIND == PL_U1);   // no search direction yet
     auto value = [&](int c) {
       const double x = X[c];
       if (plain) return x;
@@ -259,20 +268,24 @@ __global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, i
         if (KIND == PL_PV) {
           F.pk[1 - pp][s][c] = mid;
           F.vk[1 - pp][s][c] = y;
-          dot[0] += rhs[c] * y;
+          const double r0 = rhs[c];
+          dot[0] += r0 * y;
+          if (FIRST) dot[L] += r0 * r0;
         } else if (KIND == PL_ST) {
           F.t[s][c] = y;
           dot[0] += y * mid;
-          dot[pl_dots(KIND) - 1] += y * y;
+          dot[L] += y * y;
         } else if (KIND == PL_U1) {
           F.vk[0][s][c] = y;
-          dot[0] += rhs[c] * y;
+          const double r0 = rhs[c];
+          dot[0] += r0 * y;
+          if (FIRST) dot[L] += r0 * r0;
         } else if (KIND == PL_R1) {
           (pp ? F.r[s] : F.t[s])[c] = mid;
           F.pk[0][s][c] = y;
-          const double r0 = X[c], u0 = first ? r0 : r0 - beta * F.u0[s][c];
+          const double r0 = X[c], u0 = FIRST ? r0 : r0 - beta * F.u0[s][c];
           F.u0[s][c] = u0;
-          F.x[s][c] += alpha * u0;
+          F.x[s][c] = FIRST ? alpha * u0 : F.x[s][c] + alpha * u0;
           dot[0] += rhs[c] * y;
         } else if (KIND == PL_U2) {
           const double* r0 = pp ? F.r[s] : F.t[s];   // written by R1
@@ -287,8 +300,7 @@ __global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, i
           F.pk[1][s][c] = mid;
           F.r2[s][c] = y;
           F.x[s][c] += alpha * F.u0[s][c];
-          constexpr int L = pl_dots(KIND) - 1;   // 4 here
-          dot[0] += mid * mid;
+          dot[0] += mid * mid;   // L = 4 here
           dot[L / 4] += mid * y;
           dot[L / 2] += y * y;
           dot[3 * L / 4] += r0c * mid;
@@ -298,17 +310,19 @@ __global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, i
       lo = mid;
       mid = hi;
     }
+  } else if (KIND == PL_R1 && FIRST && b.inner) {
+    for (int k = b.k0; k < b.k1; ++k) F.x[b.s][b.l + P.N * P.N * k] = 0.0;
   }
-  planar_end<KIND>(P, F, b, dot, done);
+  planar_end<KIND, FIRST>(P, F, b, dot, done);
 }
 
 // The pointwise ends: x/r (s = r - alpha v; x += alpha p + omega s; r = s - omega t; r0.r, r.r) and MR.
-template <int KIND, int B>
+template <int KIND, int B, bool FIRST>
 __global__ void __launch_bounds__(B) k_planar_end(DevParams P, Fields F, int pp) {
   pdl_wait_and_release();
   Planar b;
   int done[4];
-  if (!planar_block(P, F, b, done)) return;
+  if (!planar_block<KIND, FIRST>(P, F, b, done)) return;
   double dot[2] = {};
   if (b.live && b.inner) {
     const int s = b.s, N2 = P.N * P.N;
@@ -317,13 +331,13 @@ __global__ void __launch_bounds__(B) k_planar_end(DevParams P, Fields F, int pp)
     if (KIND == PL_XR) {
       const double a = F.ks[s].alpha, om = F.ks[s].omega;
       const double *v = F.vk[1 - pp][s], *p = F.pk[1 - pp][s], *tv = F.t[s];
-      const double* ro = b.first ? rhs : F.r[s];
+      const double* ro = FIRST ? rhs : F.r[s];
       double* r = F.r[s];
 #pragma unroll 2
       for (int k = b.k0; k < b.k1; ++k) {
         const int c = b.l + N2 * k;
         const double sv = ro[c] - a * v[c];
-        x[c] = x[c] + a * p[c] + om * sv;
+        x[c] = (FIRST ? 0.0 : x[c]) + a * p[c] + om * sv;
         const double rn = sv - om * tv[c];
         r[c] = rn;
         dot[0] += rhs[c] * rn;
@@ -345,32 +359,21 @@ __global__ void __launch_bounds__(B) k_planar_end(DevParams P, Fields F, int pp)
         dot[1] += rn * rn;
       }
     }
+  } else if (KIND == PL_XR && FIRST && b.inner) {
+    for (int k = b.k0; k < b.k1; ++k) F.x[b.s][b.l + P.N * P.N * k] = 0.0;
   }
-  planar_end<KIND>(P, F, b, dot, done);
+  planar_end<KIND, FIRST>(P, F, b, dot, done);
 }
 
-// x = 0 and ||r_0||^2 of each system.
-template <int B>
-__global__ void __launch_bounds__(B) k_planar_init(DevParams P, Fields F) {
-  const int s = (int)(blockIdx.x & 3u), N = P.N, N2 = N * N;
-  const int l = (int)(blockIdx.x >> 2) * B + (int)threadIdx.x, j = l / N, i = l - j * N;
-  const int k0 = 1 + (int)blockIdx.y * P.pkz, k1 = min(k0 + P.pkz, N - 1);
-  double dot[1] = {};
-  if (i > 0 && i < N - 1 && j > 0 && j < N - 1) {
-    for (int k = k0; k < k1; ++k) {
-      const double r = F.rhs[s][l + N2 * k];
-      F.x[s][l + N2 * k] = 0.0;
-      if (P.rhs_copied) F.r[s][l + N2 * k] = r;
-      dot[0] += r * r;
-    }
-  }
-  const double mine = block_total<SumD, 1>(dot);
-  const unsigned chunks = gridDim.x >> 2;
-  if (threadIdx.x == 0)
-    F.red[(long)((blockIdx.x >> 2) + chunks * blockIdx.y) * row_stride<4>() + s] = mine;
-  if (const double* tot = last_block_total<SumD, 4>(F.red, F.counter, chunks * gridDim.y,
-                                                    gridDim.x * gridDim.y))
-    finish_init(P, F, tot);
+// Start of a solve whose right-hand sides no kernel of this library wrote: the scalars, and the copy of
+// rhs that the first residual is read from.
+__global__ void __launch_bounds__(kThreads) k_planar_start(DevParams P, Fields F) {
+  const int N = P.N, ni = N - 2, t = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (t < 4) start_system(P, F, t);
+  if (t >= ni * ni * ni) return;
+  const int q = t / ni, c = 1 + t - q * ni + N * (1 + q % ni + N * (1 + q / ni));
+#pragma unroll
+  for (int s = 0; s < 4; ++s) F.r[s][c] = F.rhs[s][c];
 }
 
 // ------------------------------------------------------------- merged iteration (two kernels)
@@ -674,7 +677,7 @@ __global__ void __launch_bounds__(256) k5_pv(DevParams P, Fields F, int pp) {
   const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
   const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
   if (const double* tot = grid_total<SumFF, 4>(acc, F.red, F.counter, bid, nb)) {
-    finish_pv(F, tot);
+    finish_pv(F, tot, false);
     count_bytes(F, HOSC_K_BICG_PV, bytes4(P, 6.0 + op_words(ene)));
   }
 }
@@ -757,10 +760,6 @@ void launch_krylov_activate(const Fields& F, cudaStream_t s) {
   k_krylov_activate<<<1, 32, 0, s>>>(F.ks);
 }
 
-void launch_loop_cond(const Fields& F, unsigned long long handle, cudaStream_t s) {
-  k_loop_cond<<<1, 32, 0, s>>>(F.ks, (cudaGraphConditionalHandle)handle);
-}
-
 dim3 planar_grid(const DevParams& P) {
   const int ni = P.N - 2;
   return dim3(4u * (unsigned)((P.N * P.N + P.pb - 1) / P.pb), (unsigned)((ni + P.pkz - 1) / P.pkz));
@@ -805,23 +804,21 @@ void launch_bicg_init(const DevParams& P, const Fields& F, cudaStream_t s) {
     k4_init<<<b, kThreads, 0, s>>>(P, F);
     return;
   }
-  const dim3 g = planar_grid(P);
-  if (P.pb == 128) k_planar_init<128><<<g, 128, 0, s>>>(P, F);
-  else if (P.pb == 256) k_planar_init<256><<<g, 256, 0, s>>>(P, F);
-  else k_planar_init<512><<<g, 512, 0, s>>>(P, F);
+  const long ni = P.N - 2;
+  k_planar_start<<<red_blocks(ni * ni * ni), kThreads, 0, s>>>(P, F);
 }
 
 // x/r as one flat stream: every node of the interior planes, the i and j walls included (every
-// vector is zero there: the workspace is zeroed at creation, k4_init zeroes x, r, p and v
-// everywhere, and no kernel writes the wall entries of t or r_0), in a grid-stride loop that
+// vector is zero there: the workspace is zeroed at creation and no kernel writes other wall entries
+// than these zeros), in a grid-stride loop that
 // issues the loads of U nodes before their arithmetic, so that a thread keeps 6 U float4 loads in
 // flight. Same arithmetic and float-float partials as k4_xr; one block partial per block.
-template <int U>
+template <int U, bool FIRST>
 __global__ void __launch_bounds__(256) k8_xr(DevParams P, Fields F, int pp) {
   __shared__ Scal4 sc;
   pdl_wait_and_release();
   load_scalars(F.ks, sc);
-  if (sc.all_done) return;
+  if (sc.all_done && (!FIRST || *F.halt)) return;
   const int np = 1 - pp;
   const float4 a = sc.a, om = sc.om, ma = neg4(sc.a), mom = neg4(sc.om);
   const float4* __restrict__ V = F.kv[np];
@@ -839,12 +836,12 @@ __global__ void __launch_bounds__(256) k8_xr(DevParams P, Fields F, int pp) {
 #pragma unroll
     for (int q = 0; q < U; ++q) {
       const unsigned e = c + q * stride;
-      r[q] = R[e];
-      x[q] = X[e];
+      r0[q] = __ldg(R0 + e);
+      r[q] = FIRST ? r0[q] : R[e];
+      x[q] = FIRST ? f4(0.f) : X[e];
       v[q] = __ldg(V + e);
       p[q] = __ldg(Pv + e);
       t[q] = __ldg(T + e);
-      r0[q] = __ldg(R0 + e);
     }
 #pragma unroll
     for (int q = 0; q < U; ++q) {
@@ -858,16 +855,18 @@ __global__ void __launch_bounds__(256) k8_xr(DevParams P, Fields F, int pp) {
     }
   }
   for (; c < hi; c += stride) {
-    const float4 sv = fma4(ma, __ldg(V + c), R[c]);
-    X[c] = fma4(om, sv, fma4(a, __ldg(Pv + c), X[c]));
+    const float4 r0 = __ldg(R0 + c);
+    const float4 sv = fma4(ma, __ldg(V + c), FIRST ? r0 : R[c]);
+    X[c] = fma4(om, sv, fma4(a, __ldg(Pv + c), FIRST ? f4(0.f) : X[c]));
     const float4 rn = fma4(mom, __ldg(T + c), sv);
     R[c] = rn;
-    ff_dot4(acc, __ldg(R0 + c), rn);
+    ff_dot4(acc, r0, rn);
     ff_dot4(acc + 4, rn, rn);
   }
   if (const double* tot = grid_total<SumFF, 8>(acc, F.red, F.counter, blockIdx.x, gridDim.x)) {
     finish_xr(P, F, tot);
-    count_bytes(F, HOSC_K_BICG_XR, bytes4(P, 8.0));   // r v p x t r0 in, x r out
+    // r v p x t r0 in, x r out
+    count_bytes(F, HOSC_K_BICG_XR, bytes4(P, FIRST ? 6.0 : 8.0));
   }
 }
 
@@ -875,7 +874,7 @@ __global__ void __launch_bounds__(256) k8_xr(DevParams P, Fields F, int pp) {
 int xr_flat_blocks() {
   static int occ = 0;
   if (occ == 0) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k8_xr<4>, 256, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k8_xr<4, false>, 256, 0) != cudaSuccess ||
         occ < 1) {
       cudaGetLastError();
       occ = 4;
@@ -885,104 +884,87 @@ int xr_flat_blocks() {
 }
 
 
-// Launch of an interleaved Krylov kernel with programmatic stream serialisation (see
-// pdl_wait_and_release): in a captured step the kernels of the BiCGSTAB loop chain with
-// programmatic edges.
-template <class K>
-void launch_pdl(K kern, dim3 grid, int threads, cudaStream_t s, const DevParams& P,
-                const Fields& F, int pp, size_t smem = 0) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kern, P, F, pp);
-}
-
-template <int KIND, int B>
+template <int KIND, int B, bool FIRST>
 void launch_planar_b(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
   if constexpr (KIND >= PL_XR)
-    launch_pdl(k_planar_end<KIND, B>, planar_grid(P), B, s, P, F, pp);
+    launch_pdl(k_planar_end<KIND, B, FIRST>, planar_grid(P), B, 0, s, P, F, pp);
   else   // two planes of N + B + N doubles: 41 KB at N = 1025
-    launch_pdl(k_planar<KIND, B>, planar_grid(P), B, s, P, F, pp, 16 * (size_t)(B + 2 * P.N));
+    launch_pdl(k_planar<KIND, B, FIRST>, planar_grid(P), B, 16 * (size_t)(B + 2 * P.N), s, P, F, pp);
+}
+template <int KIND, bool FIRST>
+void launch_planar_f(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
+  if (P.pb == 128) launch_planar_b<KIND, 128, FIRST>(P, F, pp, s);
+  else if (P.pb == 256) launch_planar_b<KIND, 256, FIRST>(P, F, pp, s);
+  else launch_planar_b<KIND, 512, FIRST>(P, F, pp, s);
 }
 template <int KIND>
-void launch_planar(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
-  if (P.pb == 128) launch_planar_b<KIND, 128>(P, F, pp, s);
-  else if (P.pb == 256) launch_planar_b<KIND, 256>(P, F, pp, s);
-  else launch_planar_b<KIND, 512>(P, F, pp, s);
+void launch_planar(const DevParams& P, const Fields& F, int pp, bool first,
+                   cudaStream_t s) {
+  constexpr bool has_first = KIND <= PL_R1 || KIND == PL_XR;
+  if (first && has_first) launch_planar_f<KIND, has_first>(P, F, pp, s);
+  else launch_planar_f<KIND, false>(P, F, pp, s);
 }
 
-void launch_bicg_pv(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
-  if (P.krylov_fp32 && P.merged) {   // x, r update of the previous iteration, then p, v
+void launch_bicg_pv(const DevParams& P, const Fields& F, int pp, bool first, cudaStream_t s) {
+  if (!P.krylov_fp32) return launch_planar<PL_PV>(P, F, pp, first, s);
+  if (P.merged) {   // x, r update of the previous iteration, then p, v
     if (P.narrow) k6_a<4><<<grid4(P), P.kblock, 0, s>>>(P, F, pp);
     else k6_a<2><<<grid4(P), P.kblock, 0, s>>>(P, F, pp);
-    return;
-  }
-  if (P.krylov_fp32 && P.tty > 0 && (P.tkernels & 1)) {
+  } else if (P.tty > 0 && (P.tkernels & 1)) {
     launch_tma_pv(P, F, pp, s);
-    return;
-  }
-  if (P.krylov_fp32 && P.sx > 0) {
+  } else if (P.sx > 0) {
     k5_pv<<<grid5(P), P.sx * P.sy, staged_smem_bytes(P.sx, P.sy, true), s>>>(P, F, pp);
-    return;
+  } else if (first && P.lean) {
+    if (P.narrow) launch_pdl(k4_pv<4, true>, grid4(P), P.kblock, 0, s, P, F, pp);
+    else launch_pdl(k4_pv<2, true>, grid4(P), P.kblock, 0, s, P, F, pp);
+  } else {
+    if (P.narrow) launch_pdl(k4_pv<4, false>, grid4(P), P.kblock, 0, s, P, F, pp);
+    else launch_pdl(k4_pv<2, false>, grid4(P), P.kblock, 0, s, P, F, pp);
   }
-  if (P.krylov_fp32) {
-    if (P.narrow) launch_pdl(k4_pv<4>, grid4(P), P.kblock, s, P, F, pp);
-    else launch_pdl(k4_pv<2>, grid4(P), P.kblock, s, P, F, pp);
-    return;
-  }
-  launch_planar<PL_PV>(P, F, pp, s);
 }
 
-void launch_bicg_st(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
-  if (P.krylov_fp32 && P.merged) {
+void launch_bicg_st(const DevParams& P, const Fields& F, int pp, bool first, cudaStream_t s) {
+  if (!P.krylov_fp32) return launch_planar<PL_ST>(P, F, pp, first, s);
+  if (P.merged) {
     if (P.narrow) k6_b<4><<<grid4(P), P.kblock, 0, s>>>(P, F, pp);
     else k6_b<2><<<grid4(P), P.kblock, 0, s>>>(P, F, pp);
-    return;
-  }
-  if (P.krylov_fp32 && P.tty > 0 && (P.tkernels & 2)) {
+  } else if (P.tty > 0 && (P.tkernels & 2)) {
     launch_tma_st(P, F, pp, s);
-    return;
-  }
-  if (P.krylov_fp32 && P.sx > 0) {
+  } else if (P.sx > 0) {
     k5_st<<<grid5(P), P.sx * P.sy, staged_smem_bytes(P.sx, P.sy, false), s>>>(P, F, pp);
-    return;
+  } else {
+    const int f = first && P.lean;
+    if (P.narrow) launch_pdl(k4_st<4>, grid4(P), P.kblock, 0, s, P, F, pp, f);
+    else launch_pdl(k4_st<2>, grid4(P), P.kblock, 0, s, P, F, pp, f);
   }
-  if (P.krylov_fp32) {
-    if (P.narrow) launch_pdl(k4_st<4>, grid4(P), P.kblock, s, P, F, pp);
-    else launch_pdl(k4_st<2>, grid4(P), P.kblock, s, P, F, pp);
-    return;
-  }
-  launch_planar<PL_ST>(P, F, pp, s);
 }
 
-void launch_bicg_xr(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
-  if (P.krylov_fp32 && P.merged) return;   // folded into the next k6_a
-  if (P.krylov_fp32 && P.xr_flat) {
-    launch_pdl(k8_xr<4>, dim3(xr_flat_blocks()), 256, s, P, F, pp);
-    return;
-  }
-  if (P.krylov_fp32) {
-    if (P.narrow) launch_pdl(k4_xr<4>, grid4(P), P.kblock, s, P, F, pp);
-    else launch_pdl(k4_xr<2>, grid4(P), P.kblock, s, P, F, pp);
-    return;
-  }
-  launch_planar<PL_XR>(P, F, pp, s);
+template <bool FIRST>
+void launch_xr4(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
+  if (P.xr_flat) launch_pdl(k8_xr<4, FIRST>, dim3(xr_flat_blocks()), 256, 0, s, P, F, pp);
+  else if (P.narrow) launch_pdl(k4_xr<4, FIRST>, grid4(P), P.kblock, 0, s, P, F, pp);
+  else launch_pdl(k4_xr<2, FIRST>, grid4(P), P.kblock, 0, s, P, F, pp);
 }
 
-void launch_b2(int kernel, const DevParams& P, const Fields& F, int cp, cudaStream_t s) {
+void launch_bicg_xr(const DevParams& P, const Fields& F, int pp, bool first, cudaStream_t s) {
+  if (!P.krylov_fp32) return launch_planar<PL_XR>(P, F, pp, first, s);
+  if (P.merged) return;   // folded into the next k6_a
+  if (first && P.lean) launch_xr4<true>(P, F, pp, s);
+  else launch_xr4<false>(P, F, pp, s);
+}
+
+void launch_loop_cond(const Fields& F, unsigned long long handle, cudaStream_t s) {
+  k_loop_cond<<<1, 32, 0, s>>>(F.ks, (cudaGraphConditionalHandle)handle);
+}
+
+void launch_b2(int kernel, const DevParams& P, const Fields& F, int cp, bool first,
+               cudaStream_t s) {
   switch (kernel) {
-    case 0: launch_planar<PL_U1>(P, F, cp, s); break;
-    case 1: launch_planar<PL_R1>(P, F, cp, s); break;
-    case 2: launch_planar<PL_U2>(P, F, cp, s); break;
-    case 3: launch_planar<PL_R2>(P, F, cp, s); break;
-    default: launch_planar<PL_MR>(P, F, cp, s); break;
+    case 0: launch_planar<PL_U1>(P, F, cp, first, s); break;
+    case 1: launch_planar<PL_R1>(P, F, cp, first, s); break;
+    case 2: launch_planar<PL_U2>(P, F, cp, false, s); break;
+    case 3: launch_planar<PL_R2>(P, F, cp, false, s); break;
+    default: launch_planar<PL_MR>(P, F, cp, false, s); break;
   }
 }
 
@@ -1046,8 +1028,8 @@ int krylov4_occupancy(int kblock, int narrow, int merged) {
     e = narrow ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k6_a<4>, kblock, 0)
                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k6_a<2>, kblock, 0);
   else
-    e = narrow ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k4_pv<4>, kblock, 0)
-               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k4_pv<2>, kblock, 0);
+    e = narrow ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k4_pv<4, false>, kblock, 0)
+               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k4_pv<2, false>, kblock, 0);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return 1;

@@ -188,7 +188,22 @@ __device__ __forceinline__ void load_scalars(const KrylovScalars* ks, Scal4& sc)
 // needs from the launch's totals, one thread a system (each an FP64 divide or square root and a few
 // dependent reads: one after another they took 4 us of a 20 us launch on a 41^3 grid).
 
-// r_0 . r_0 of each system: the solve starts.
+// A system before its first iteration, set by the right-hand sides' kernel: the first p/v of the
+// lean forms (no initialisation kernel) then finds ||r_0||.
+__device__ __forceinline__ void start_system(const DevParams& P, const Fields& F, int s) {
+  KrylovScalars& k = F.ks[s];
+  k.rho = k.r0norm = k.rnorm = 0.0;
+  k.alpha = 0.0;
+  k.omega = 1.0;
+  k.beta = 0.0;
+  k.g1 = k.g2 = 0.0;
+  k.iters = 0;
+  k.pad = 0;
+  k.status = 0;
+  k.done = s == 3 && P.inner_pass;   // an inner pressure pass solves the momentum systems only
+}
+
+// r_0 . r_0 of each system: the solve starts (forms that are not lean).
 __device__ __forceinline__ void finish_init(const DevParams& P, const Fields& F, const double* tot) {
   if (threadIdx.x >= 4) return;
   const int s = threadIdx.x;
@@ -197,10 +212,10 @@ __device__ __forceinline__ void finish_init(const DevParams& P, const Fields& F,
   const double norm = sqrt(tot[s]);
   k.r0norm = norm;
   k.rnorm = norm;
-  k.rho = tot[s];   // BiCGSTAB(2): rho_0 after the first cycle's rho_0 = -omega rho_0, j = 0
+  k.rho = tot[s];
   // the first kernel of the merged form then leaves x = 0, r = r_0 and sets p = r_0
-  k.alpha = (P.krylov_fp32 ? P.merged : P.solver) ? 0.0 : 1.0;
-  k.omega = (P.krylov_fp32 && P.merged) ? 0.0 : 1.0;
+  k.alpha = P.merged ? 0.0 : 1.0;
+  k.omega = P.merged ? 0.0 : 1.0;
   k.beta = 0.0;
   k.g1 = k.g2 = 0.0;
   k.iters = 0;
@@ -210,13 +225,26 @@ __device__ __forceinline__ void finish_init(const DevParams& P, const Fields& F,
   k.done = (norm == 0.0 || halt || (s == 3 && P.inner_pass)) ? 1 : 0;
 }
 
-// r_0 . v of each system: alpha = rho / (r_0 . v).
-__device__ __forceinline__ void finish_pv(const Fields& F, const double* tot) {
+// r_0 . v of each system (slots 0..3): alpha = rho / (r_0 . v). In the first iteration of a lean form
+// r_0 . r_0 too (4..7), which is rho; a system whose right-hand side is zero is then done.
+__device__ __forceinline__ void finish_pv(const Fields& F, const double* tot, bool first) {
   if (threadIdx.x >= 4) return;
   KrylovScalars& k = F.ks[threadIdx.x];
   const int done = k.done;
-  const double rho = k.rho, d = tot[threadIdx.x];
+  double rho = k.rho;
+  const double d = tot[threadIdx.x];
   if (done) return;
+  if (first) {
+    rho = tot[4 + threadIdx.x];
+    const double norm = sqrt(rho);
+    k.rho = rho;
+    k.r0norm = norm;
+    k.rnorm = norm;
+    if (norm == 0.0) {
+      k.done = 1;
+      return;
+    }
+  }
   if (d == 0.0 || !isfinite(d)) {
     k.done = 1;
     k.status = HOSC_ENOCONV;
@@ -268,15 +296,6 @@ __device__ __forceinline__ double bytes4(const DevParams& P, double float4_words
   return 16.0 * float4_words * ni * ni * ni;
 }
 
-// Programmatic dependent launch: the Krylov kernels of the interleaved solve are launched so that
-// each may start while the previous one is finishing (its blocks take SMs as the previous
-// kernel's blocks leave); a kernel waits for the previous grid's completion and memory before its
-// first access, and lets the next kernel launch at once.
-__device__ __forceinline__ void pdl_wait_and_release() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // r = r_0, x = 0, p = v = 0 at interior nodes, every vector zero on the walls; ||r_0||^2.
 // Grid-stride over all N^3 nodes: each thread sums several nodes before the one block reduction.
 // Returns true in the block that finished the launch's reduction (its scalars are then final).
@@ -311,26 +330,36 @@ __global__ void __launch_bounds__(kThreads) k4_init(DevParams P, Fields F) {
   k4_init_body(P, F, blockIdx.x, gridDim.x);
 }
 
+// The kernels of a solve's first iteration are forms of their own (FIRST): the residual is r_0, there
+// is no search direction and no iterate, so they read less (p/v 3 of 6 vectors, x/r 4 of 6) and no
+// initialisation kernel has to write seven vectors (26 us of a step at 101^3). As a branch inside the
+// kernels the same cost registers in the loop: p/v 39.9 -> 48.2 us at 101^3.
+//
 // p_new = r + beta (p_old - omega v_old) at the seven stencil nodes, v_new = A p_new, partial
-// r_0 . v_new; last block: alpha = rho / (r_0 . v_new).
+// r_0 . v_new; last block: alpha = rho / (r_0 . v_new). FIRST: p_new = r_0, and the partial r_0 . r_0
+// gives rho and ||r_0||.
+template <bool FIRST>
 __device__ __forceinline__ void k4_pv_body(const DevParams& P, const Fields& F, int pp,
                                             const VGrid& vg) {
+  constexpr int M = FIRST ? 8 : 4;
   __shared__ Scal4 sc;
   load_scalars(F.ks, sc);
   if (sc.all_done) return;   // uniform over the grid
   const bool ene = !sc.done[3];   // the energy system still iterates (uniform)
   const int N = P.N, N2 = N * N;
   const float4 b = sc.b, mom = neg4(sc.om);
-  const float4* HOSC_RESTRICT R = F.kr;
+  const float4* HOSC_RESTRICT R = FIRST ? F.kr0 : F.kr;
   const float4* HOSC_RESTRICT Po = F.kp[pp];
   const float4* HOSC_RESTRICT Vo = F.kv[pp];
   float4* HOSC_RESTRICT Pn = F.kp[1 - pp];
   float4* HOSC_RESTRICT Vn = F.kv[1 - pp];
   auto pnew = [&](int c) {
-    const float4 r = HOSC_LDG(R + c), p = HOSC_LDG(Po + c), v = HOSC_LDG(Vo + c);
+    const float4 r = HOSC_LDG(R + c);
+    if (FIRST) return r;
+    const float4 p = HOSC_LDG(Po + c), v = HOSC_LDG(Vo + c);
     return fma4(b, fma4(mom, v, p), r);
   };
-  FF acc[4] = {};
+  FF acc[M] = {};
   Column col;
   if (column(P, col, vg)) {
     float4 pm = pnew(col.cb + N2 * (col.k0 - 1));
@@ -342,29 +371,30 @@ __device__ __forceinline__ void k4_pv_body(const DevParams& P, const Fields& F, 
                                  pnew(c + N), pnew(c - N), pz, pm);
       Pn[c] = pc;
       Vn[c] = vn;
-      ff_dot4(acc, HOSC_LDG(F.kr0 + c), vn);
+      ff_dot4(acc, FIRST ? pc : HOSC_LDG(F.kr0 + c), vn);
+      if (FIRST) ff_dot4(acc + M - 4, pc, pc);
       pm = pc;
       pc = pz;
     }
   }
   if (const double* tot =
-          grid_total<SumFF, 4>(acc, F.red, F.counter, block_id(vg), block_count(vg))) {
-    finish_pv(F, tot);
+          grid_total<SumFF, M>(acc, F.red, F.counter, block_id(vg), block_count(vg))) {
+    finish_pv(F, tot, FIRST);
     // r p v r0 in, p v out, the compact operators
-    count_bytes(F, HOSC_K_BICG_PV, bytes4(P, 6.0 + op_words(ene)));
+    count_bytes(F, HOSC_K_BICG_PV, bytes4(P, (FIRST ? 3.0 : 6.0) + op_words(ene)));
   }
 }
 
-template <int MinB>
+template <int MinB, bool FIRST>
 __global__ void __launch_bounds__(MinB == 2 ? 384 : 256, MinB)
     k4_pv(DevParams P, Fields F, int pp) {
   pdl_wait_and_release();
-  k4_pv_body(P, F, pp, hw_grid());
+  k4_pv_body<FIRST>(P, F, pp, hw_grid());
 }
 
 // s = r - alpha v at the seven stencil nodes, t = A s, partials (t . s, t . t); last block:
 // omega = (t . s) / (t . t) (0 when t = 0).
-__device__ __forceinline__ void k4_st_body(const DevParams& P, const Fields& F, int pp,
+__device__ __forceinline__ void k4_st_body(const DevParams& P, const Fields& F, int pp, int first,
                                             const VGrid& vg) {
   __shared__ Scal4 sc;
   load_scalars(F.ks, sc);
@@ -373,7 +403,7 @@ __device__ __forceinline__ void k4_st_body(const DevParams& P, const Fields& F, 
   const int N = P.N, N2 = N * N;
   const int np = 1 - pp;   // written by k4_pv of this iteration
   const float4 ma = neg4(sc.a);
-  const float4* HOSC_RESTRICT R = F.kr;
+  const float4* HOSC_RESTRICT R = first ? F.kr0 : F.kr;
   const float4* HOSC_RESTRICT V = F.kv[np];
   float4* HOSC_RESTRICT T = F.kt;
   auto sval = [&](int c) { return fma4(ma, HOSC_LDG(V + c), HOSC_LDG(R + c)); };
@@ -404,19 +434,20 @@ __device__ __forceinline__ void k4_st_body(const DevParams& P, const Fields& F, 
 
 template <int MinB>
 __global__ void __launch_bounds__(MinB == 2 ? 384 : 256, MinB)
-    k4_st(DevParams P, Fields F, int pp) {
+    k4_st(DevParams P, Fields F, int pp, int first) {
   pdl_wait_and_release();
-  k4_st_body(P, F, pp, hw_grid());
+  k4_st_body(P, F, pp, first, hw_grid());
 }
 
 // s = r - alpha v; x += alpha p + omega s; r = s - omega t; partials (r_0 . r, r . r); last block:
 // convergence and breakdown tests, beta and rho of the next iteration.
-// Returns true in the block that finished the launch's reduction (convergence decided).
-__device__ __forceinline__ bool k4_xr_body(const DevParams& P, const Fields& F, int pp,
+template <bool FIRST>
+__device__ __forceinline__ void k4_xr_body(const DevParams& P, const Fields& F, int pp,
                                             const VGrid& vg) {
   __shared__ Scal4 sc;
   load_scalars(F.ks, sc);
-  if (sc.all_done) return false;
+  // FIRST runs with every right-hand side zero too (the increments are then zero), not when halted
+  if (sc.all_done && (!FIRST || *F.halt)) return;
   const int N2 = P.N * P.N;
   const int np = 1 - pp;
   const float4 a = sc.a, om = sc.om, ma = neg4(sc.a), mom = neg4(sc.om);
@@ -425,10 +456,12 @@ __device__ __forceinline__ bool k4_xr_body(const DevParams& P, const Fields& F, 
   if (column(P, col, vg)) {
     for (int k = col.k0; k < col.k1; ++k) {
       const int c = col.cb + N2 * k;
-      const float4 r = F.kr[c], v = HOSC_LDG(F.kv[np] + c), p = HOSC_LDG(F.kp[np] + c);
-      const float4 t = HOSC_LDG(F.kt + c), r0 = HOSC_LDG(F.kr0 + c);
+      const float4 r0 = HOSC_LDG(F.kr0 + c);
+      const float4 r = FIRST ? r0 : F.kr[c], x = FIRST ? f4(0.f) : F.kx[c];
+      const float4 v = HOSC_LDG(F.kv[np] + c), p = HOSC_LDG(F.kp[np] + c);
+      const float4 t = HOSC_LDG(F.kt + c);
       const float4 sv = fma4(ma, v, r);
-      F.kx[c] = fma4(om, sv, fma4(a, p, F.kx[c]));
+      F.kx[c] = fma4(om, sv, fma4(a, p, x));
       const float4 rn = fma4(mom, t, sv);
       F.kr[c] = rn;
       ff_dot4(acc, r0, rn);
@@ -437,17 +470,16 @@ __device__ __forceinline__ bool k4_xr_body(const DevParams& P, const Fields& F, 
   }
   const double* tot =
       grid_total<SumFF, 8>(acc, F.red, F.counter, block_id(vg), block_count(vg));
-  if (!tot) return false;
+  if (!tot) return;
   finish_xr(P, F, tot);
-  count_bytes(F, HOSC_K_BICG_XR, bytes4(P, 8.0));   // r v p x t r0 in, x r out
-  return true;
+  count_bytes(F, HOSC_K_BICG_XR, bytes4(P, FIRST ? 6.0 : 8.0));   // r v p x t r0 in, x r out
 }
 
-template <int MinB>
+template <int MinB, bool FIRST>
 __global__ void __launch_bounds__(MinB == 2 ? 384 : 256, MinB)
     k4_xr(DevParams P, Fields F, int pp) {
   pdl_wait_and_release();
-  k4_xr_body(P, F, pp, hw_grid());
+  k4_xr_body<FIRST>(P, F, pp, hw_grid());
 }
 
 }  // namespace

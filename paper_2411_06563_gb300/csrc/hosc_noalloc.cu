@@ -127,9 +127,10 @@ extern "C" hosc_status hosc_bicgstab_noalloc(int N, const double* const* weights
   while (it < max_iter) {
     const int chunk = (max_iter - it < check) ? max_iter - it : check;
     for (int q = 0; q < chunk; ++q) {
-      launch_bicg_pv(P, F, pp, sm);
-      launch_bicg_st(P, F, pp, sm);
-      launch_bicg_xr(P, F, pp, sm);
+      const bool first = it + q == 0;
+      launch_bicg_pv(P, F, pp, first, sm);
+      launch_bicg_st(P, F, pp, first, sm);
+      launch_bicg_xr(P, F, pp, first, sm);
       pp ^= 1;
     }
     it += chunk;

@@ -3,8 +3,8 @@
 // for many cavities of different sizes at once).
 //
 // The grid is cooperative (every block resident). Each member advances through the phases of its
-// own steps (S1, S2, S3/S4, the Krylov initialisation, the p/v, s/t and x/r kernels of each
-// BiCGSTAB iteration, the update kernels, the record, the float copies); a phase's work is a list
+// own steps (S1, S2, S3/S4, the p/v, s/t and x/r kernels of each BiCGSTAB iteration, the update
+// kernels); a phase's work is a list
 // of tiles (the 256-thread blocks of the per-kernel launches), appended to a queue shared by all
 // members when the member's previous phase completes, and any block takes the next tile of the
 // queue, whatever member it belongs to. The tiles run the same device bodies as the per-kernel
@@ -115,26 +115,25 @@ __device__ __noinline__ void sources_item(const RoundMember& M, int cur, int til
                            F.Ev[cur], F.Ew[cur], F.halt, (unsigned)tile, (unsigned)M.interior);
 }
 
-__device__ __noinline__ bool init_item(const RoundMember& M, int tile) {
-  return k4_init_body(M.P, M.F, (unsigned)tile, (unsigned)M.init);
-}
+template <bool FIRST>
 __device__ __noinline__ void pv_item(const RoundMember& M, int pp, int tile) {
-  k4_pv_body(M.P, M.F, pp, krylov_grid(M, tile));
+  k4_pv_body<FIRST>(M.P, M.F, pp, krylov_grid(M, tile));
 }
-__device__ __noinline__ void st_item(const RoundMember& M, int pp, int tile) {
-  k4_st_body(M.P, M.F, pp, krylov_grid(M, tile));
+__device__ __noinline__ void st_item(const RoundMember& M, int pp, int first, int tile) {
+  k4_st_body(M.P, M.F, pp, first, krylov_grid(M, tile));
 }
-__device__ __noinline__ bool xr_item(const RoundMember& M, int pp, int tile) {
-  return k4_xr_body(M.P, M.F, pp, krylov_grid(M, tile));
+template <bool FIRST>
+__device__ __noinline__ void xr_item(const RoundMember& M, int pp, int tile) {
+  k4_xr_body<FIRST>(M.P, M.F, pp, krylov_grid(M, tile));
 }
 __device__ __noinline__ void update_item(const RoundMember& M, int phase, int cur, int tile) {
   switch (phase) {
-    case 0: k_apply_increment_body<float>(M.P, M.F, cur, M.nodes, (unsigned)tile); break;
-    case 1: k_theta_walls_body(M.P, M.F, M.theta_walls, (unsigned)tile); break;
-    case 2: k_divergence_body(M.P, M.F, 1 - cur, M.interior, (unsigned)tile); break;
-    case 3: k_pressure_correct_body(M.P, M.F, (unsigned)tile); break;
-    case 4: k_pressure_walls_body(M.P, M.F, (unsigned)tile); break;
-    default: k_finish_record_body(M.P, M.F, (unsigned)tile); break;
+    case 0: k_increment_body<float>(M.P, M.F, cur, M.nodes, (unsigned)tile); break;
+    case 1:
+      k_div_walls_body(M.P, M.F, 1 - cur, M.interior, M.interior + M.theta_walls, (unsigned)tile);
+      break;
+    case 2: k_pressure_correct_body(M.P, M.F, (unsigned)tile); break;
+    default: k_pressure_walls_body(M.P, M.F, 1, M.pressure_walls, (unsigned)tile); break;
   }
 }
 
@@ -149,8 +148,8 @@ __device__ __noinline__ void update_item(const RoundMember& M, int phase, int cu
 // to be filled or for every member to finish the round.
 
 enum FlowPhase {
-  PH_SHADOW0 = 0, PH_VISC, PH_SOURCES, PH_RHS, PH_INIT, PH_PV, PH_ST, PH_XR, PH_INC, PH_TWALLS,
-  PH_DIV, PH_PCORR, PH_PWALLS, PH_FINISH, PH_SHADOW, PH_DONE
+  PH_SHADOW0 = 0, PH_VISC, PH_SOURCES, PH_RHS, PH_PV, PH_ST, PH_XR, PH_INC, PH_DIVW, PH_PCORR,
+  PH_PWALLS, PH_DONE
 };
 
 struct FlowMember {
@@ -175,13 +174,11 @@ struct FlowDev {
 
 __device__ __forceinline__ int flow_tiles(const RoundMember& M, int ph) {
   switch (ph) {
-    case PH_RHS: case PH_DIV: case PH_PCORR: return M.interior;
+    case PH_RHS: case PH_PCORR: return M.interior;
     case PH_VISC: case PH_SOURCES: return M.interior + M.pressure_walls;
-    case PH_INIT: return M.init;
     case PH_PV: case PH_ST: case PH_XR: return M.kx * M.ky;
-    case PH_TWALLS: return M.theta_walls;
+    case PH_DIVW: return M.interior + M.theta_walls;
     case PH_PWALLS: return M.pressure_walls;
-    case PH_FINISH: return 1;
     default: return M.nodes;   // shadows, increments
   }
 }
@@ -194,12 +191,16 @@ __device__ __forceinline__ void flow_item(const RoundMember& M, int step, int it
     case PH_VISC: visc_item(M, cur, tile); break;
     case PH_SOURCES: sources_item(M, cur, tile); break;
     case PH_RHS: rhs_item(M, cur, tile); break;
-    case PH_INIT: init_item(M, tile); break;
-    case PH_PV: pv_item(M, it & 1, tile); break;
-    case PH_ST: st_item(M, it & 1, tile); break;
-    case PH_XR: xr_item(M, it & 1, tile); break;
-    case PH_SHADOW: shadow_item(M, 1 - cur, tile); break;
-    default: update_item(M, ph - PH_INC, cur, tile); break;   // PH_INC .. PH_FINISH
+    case PH_PV:
+      if (it == 0) pv_item<true>(M, 0, tile);
+      else pv_item<false>(M, it & 1, tile);
+      break;
+    case PH_ST: st_item(M, it & 1, it == 0, tile); break;
+    case PH_XR:
+      if (it == 0) xr_item<true>(M, 0, tile);
+      else xr_item<false>(M, it & 1, tile);
+      break;
+    default: update_item(M, ph - PH_INC, cur, tile); break;   // PH_INC .. PH_PWALLS
   }
 }
 
@@ -213,16 +214,15 @@ __device__ int flow_next(const FlowDev& D, int mb, int ph) {
   const RoundMember& M = D.m[mb];
   FlowMember& S = D.st[mb];
   switch (ph) {
-    case PH_INIT:
+    case PH_RHS:
       S.it = 0;
-      return any_active(M) ? PH_PV : PH_INC;
+      return PH_PV;
     case PH_XR:
       S.it += 1;
       return (any_active(M) && S.it <= D.max_it) ? PH_PV : PH_INC;
-    case PH_FINISH: return *(volatile int*)M.F.halt ? PH_DONE : PH_SHADOW;
-    case PH_SHADOW:
+    case PH_PWALLS:
       S.step += 1;
-      return S.step >= D.G ? PH_DONE : PH_VISC;
+      return *(volatile int*)M.F.halt || S.step >= D.G ? PH_DONE : PH_VISC;
     default: return ph + 1;
   }
 }
@@ -358,10 +358,7 @@ void round_member_shape(RoundMember* M) {
   M->P.narrow = 0;
   M->P.merged = 0;
   M->P.sx = M->P.sy = M->P.skz = 0;
-  // the Krylov initialisation strides over the nodes with at most one wave of blocks, as its
-  // own launch does (same partial sums, same reduction order)
-  const int most = 8 * device_sms();
-  M->init = M->nodes < most ? M->nodes : most;
+  M->P.lean = 1;
   M->kx = (int)((ni * ni + kRoundThreads - 1) / kRoundThreads);
   M->ky = (int)((ni + M->P.kz - 1) / M->P.kz);
 }

@@ -46,25 +46,23 @@ static SweepGrid sweep_grid(const DevParams& P) {
 void launch_viscosity(const DevParams& P, const Fields& F, int cur, cudaStream_t s) {
   const SweepGrid g = sweep_grid(P);
   if (P.sweep_fp32)
-    k_viscosity<float><<<g.nb, g.threads, 0, s>>>(
-        P, F.us[cur], F.vs[cur], F.ws[cur], reinterpret_cast<float*>(F.eta),
-        reinterpret_cast<float*>(F.L[cur]), F.halt, g.nbi);
+    launch_pdl(k_viscosity<float>, g.nb, g.threads, 0, s, P, F.us[cur], F.vs[cur], F.ws[cur],
+               reinterpret_cast<float*>(F.eta), reinterpret_cast<float*>(F.L[cur]), F.halt, g.nbi);
   else
-    k_viscosity<double><<<g.nb, g.threads, 0, s>>>(P, F.u[cur], F.v[cur], F.w[cur], F.eta,
-                                                   F.L[cur], F.halt, g.nbi);
+    launch_pdl(k_viscosity<double>, g.nb, g.threads, 0, s, P, F.u[cur], F.v[cur], F.w[cur], F.eta,
+               F.L[cur], F.halt, g.nbi);
 }
 
 void launch_sources(const DevParams& P, const Fields& F, int cur, cudaStream_t s) {
   const SweepGrid g = sweep_grid(P);
   if (P.sweep_fp32)
-    k_sources<float><<<g.nb, g.threads, 0, s>>>(
-        P, F.us[cur], F.vs[cur], F.ws[cur], F.ths, F.ps, reinterpret_cast<const float*>(F.eta),
-        reinterpret_cast<float*>(F.Eu[cur]), reinterpret_cast<float*>(F.Ev[cur]),
-        reinterpret_cast<float*>(F.Ew[cur]), F.halt, g.nbi);
+    launch_pdl(k_sources<float>, g.nb, g.threads, 0, s, P, F.us[cur], F.vs[cur], F.ws[cur], F.ths,
+               F.ps, reinterpret_cast<const float*>(F.eta), reinterpret_cast<float*>(F.Eu[cur]),
+               reinterpret_cast<float*>(F.Ev[cur]), reinterpret_cast<float*>(F.Ew[cur]), F.halt,
+               g.nbi);
   else
-    k_sources<double><<<g.nb, g.threads, 0, s>>>(P, F.u[cur], F.v[cur], F.w[cur], F.th, F.p,
-                                                 F.eta, F.Eu[cur], F.Ev[cur], F.Ew[cur], F.halt,
-                                                 g.nbi);
+    launch_pdl(k_sources<double>, g.nb, g.threads, 0, s, P, F.u[cur], F.v[cur], F.w[cur], F.th, F.p,
+               F.eta, F.Eu[cur], F.Ev[cur], F.Ew[cur], F.halt, g.nbi);
 }
 
 template <class Tc, class Ts>
@@ -84,9 +82,9 @@ static void rhs_t(const DevParams& P, const Fields& F, int cur, cudaStream_t s) 
     up = (const Tc*)F.u[o]; vp = (const Tc*)F.v[o]; wp = (const Tc*)F.w[o];
   }
   const int threads = sizeof(Tc) == sizeof(float) ? kThreads : kFp64Threads;
-  k_rhs<Tc, Ts><<<red_blocks(ni * ni * ni, threads), threads, 0, s>>>(
-      P, u, v, w, th, T(F.L[cur]), T(F.Eu[cur]), T(F.Ev[cur]), T(F.Ew[cur]), T(F.L[o]), up, vp,
-      wp, T(F.Eu[o]), T(F.Ev[o]), T(F.Ew[o]), F);
+  launch_pdl(k_rhs<Tc, Ts>, red_blocks(ni * ni * ni, threads), threads, 0, s, P, u, v, w, th,
+             T(F.L[cur]), T(F.Eu[cur]), T(F.Ev[cur]), T(F.Ew[cur]), T(F.L[o]), up, vp, wp,
+             T(F.Eu[o]), T(F.Ev[o]), T(F.Ew[o]), F);
 }
 
 void launch_rhs(const DevParams& P, const Fields& F, int cur, cudaStream_t s) {
@@ -98,28 +96,21 @@ void launch_rhs(const DevParams& P, const Fields& F, int cur, cudaStream_t s) {
     rhs_t<double, double>(P, F, cur, s);
 }
 
-void launch_update(const DevParams& P, const Fields& F, int cur, cudaStream_t s) {
-  launch_update_fields(P, F, cur, s);
-  launch_finish(P, F, s);
-}
-
 void launch_finish(const DevParams& P, const Fields& F, cudaStream_t s) {
   k_finish_record<<<1, 32, 0, s>>>(P, F);
 }
 
-void launch_update_fields(const DevParams& P, const Fields& F, int cur, cudaStream_t s) {
+void launch_update(const DevParams& P, const Fields& F, int cur, int record, cudaStream_t s) {
   const long N = P.N, n3 = N * N * N, ni = N - 2;
-  const int b_all = red_blocks(n3);
-  if (P.krylov_fp32)
-    k_apply_increment<float><<<b_all, kThreads, 0, s>>>(P, F, cur, b_all);
-  else
-    k_apply_increment<double><<<b_all, kThreads, 0, s>>>(P, F, cur, b_all);
-  const int b_walls = red_blocks(2 * ni * N + 2 * ni * ni);
-  k_theta_walls<<<b_walls, kThreads, 0, s>>>(P, F, b_walls);
-  const int b_int = red_blocks(ni * ni * ni);
-  k_divergence<<<b_int, kThreads, 0, s>>>(P, F, 1 - cur, b_int);
-  k_pressure_correct<<<b_int, kThreads, 0, s>>>(P, F);
-  k_pressure_walls<<<red_blocks(n3 - ni * ni * ni), kThreads, 0, s>>>(P, F);
+  const int b_all = red_blocks(n3), b_int = red_blocks(ni * ni * ni);
+  const int b_div = b_int + red_blocks(2 * ni * N + 2 * ni * ni);
+  const int b_walls = red_blocks(n3 - ni * ni * ni);
+  // the first follows the conditional node of a captured step: a plain launch
+  if (P.krylov_fp32) k_increment<float><<<b_all, kThreads, 0, s>>>(P, F, cur, b_all);
+  else k_increment<double><<<b_all, kThreads, 0, s>>>(P, F, cur, b_all);
+  launch_pdl(k_div_walls, b_div, kThreads, 0, s, P, F, 1 - cur, b_int, b_div);
+  launch_pdl(k_pressure_correct, b_int, kThreads, 0, s, P, F);
+  launch_pdl(k_pressure_walls, b_walls, kThreads, 0, s, P, F, record, b_walls);
 }
 
 }  // namespace hosc

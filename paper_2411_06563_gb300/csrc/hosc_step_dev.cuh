@@ -15,6 +15,7 @@
 
 #include "hosc_device.cuh"
 #include "hosc_internal.h"
+#include "hosc_krylov4.cuh"
 
 namespace hosc {
 
@@ -235,6 +236,7 @@ __global__ void __launch_bounds__(kThreads) k_viscosity(DevParams P, const T* HO
                                                         T* HOSC_RESTRICT eta, T* HOSC_RESTRICT L,
                                                         const int* HOSC_RESTRICT halt,
                                                         unsigned nbi) {
+  pdl_wait_and_release();
   k_viscosity_body(P, u, v, w, eta, L, halt, blockIdx.x, nbi);
 }
 
@@ -291,6 +293,7 @@ __global__ void __launch_bounds__(kThreads) k_sources(DevParams P, const T* HOSC
                                                      T* HOSC_RESTRICT Eu, T* HOSC_RESTRICT Ev,
                                                      T* HOSC_RESTRICT Ew,
                                                      const int* HOSC_RESTRICT halt, unsigned nbi) {
+  pdl_wait_and_release();
   k_sources_body(P, u, v, w, th, p, eta, Eu, Ev, Ew, halt, blockIdx.x, nbi);
 }
 
@@ -458,6 +461,7 @@ __device__ __forceinline__ void k_rhs_body(const DevParams& P, const Tc* HOSC_RE
   const long sy = N, sz = (long)N * N;
   const long c = node(i, j, k, N);
   const RhsC<Tc>& rc = rhs_constants<Tc>(P);
+  if (t < 4) start_system(P, F, (int)t);   // the solve's scalars
   const bool hist = P.have_prev != 0;
   const Tc kap = par<Tc>(P.a_boost, P.a_boostf);
   Tc rv[4], Bm[3], Be[3], Dm, De, Lc;   // right-hand sides and compact operators, stored at the end
@@ -580,17 +584,25 @@ __global__ void __launch_bounds__(sizeof(Tc) == sizeof(float) ? kThreads : kFp64
     const Tc* HOSC_RESTRICT Lp, const Tc* HOSC_RESTRICT up, const Tc* HOSC_RESTRICT vp,
     const Tc* HOSC_RESTRICT wp, const Tc* HOSC_RESTRICT Eup, const Tc* HOSC_RESTRICT Evp,
     const Tc* HOSC_RESTRICT Ewp, Fields F) {
+  pdl_wait_and_release();
   k_rhs_body<Tc, Ts>(P, u, v, w, th, L, Eu, Ev, Ew, Lp, up, vp, wp, Eup, Evp, Ewp, F,
                      blockIdx.x);
 }
 
 // ------------------------------------------------------------------------------------ S6-S8
+//
+// Four launches: the increments; div V and the adiabatic walls (both need the increments of
+// neighbours); the pressure correction (needs max|div V|); the pressure walls (need the corrected
+// pressure). In mixed precision each also writes the float copies of what it writes, and the last
+// block of the last one appends the step record: seven launches before, whose latencies were most of
+// their time below 64^3 (45 -> 29 us a step at 41^3 mixed beside a
+// launch for the copies, 91 + 12 -> 81 us at 101^3).
 
 // chi^{n+1} = chi^n + x at interior nodes (u, v, w into the other buffer, theta in place); wall
 // velocities are carried over. Max |x| over the four systems goes to the step record.
 template <class Ts>
-__device__ __forceinline__ void k_apply_increment_body(const DevParams& P, const Fields& F,
-                                                       int cur, int nblocks, unsigned vbx) {
+__device__ __forceinline__ void k_increment_body(const DevParams& P, const Fields& F, int cur,
+                                                 int nblocks, unsigned vbx) {
   if (*F.halt) return;
   const unsigned N = P.N;
   const unsigned n3 = N * N * N;
@@ -600,6 +612,7 @@ __device__ __forceinline__ void k_apply_increment_body(const DevParams& P, const
     const unsigned q = t / N;
     const unsigned i = t - q * N, j = q % N, k = q / N;
     const bool inner = i > 0 && j > 0 && k > 0 && i < N - 1 && j < N - 1 && k < N - 1;
+    double u = F.u[cur][t], v = F.v[cur][t], w = F.w[cur][t];
     if (inner) {
       double xu, xv, xw, xt;
       if constexpr (sizeof(Ts) == sizeof(float)) {   // interleaved float increments
@@ -619,14 +632,20 @@ __device__ __forceinline__ void k_apply_increment_body(const DevParams& P, const
         m[0] = max_nonneg(max_nonneg(absfin(xu), absfin(xv)), absfin(xw));
         m[1] = absfin(xt);
       }
-      F.u[1 - cur][t] = F.u[cur][t] + xu;
-      F.v[1 - cur][t] = F.v[cur][t] + xv;
-      F.w[1 - cur][t] = F.w[cur][t] + xw;
-      F.th[t] += xt;
-    } else {
-      F.u[1 - cur][t] = F.u[cur][t];
-      F.v[1 - cur][t] = F.v[cur][t];
-      F.w[1 - cur][t] = F.w[cur][t];
+      u += xu;
+      v += xv;
+      w += xw;
+      const double th = F.th[t] + xt;
+      F.th[t] = th;
+      if constexpr (sizeof(Ts) == sizeof(float)) F.ths[t] = (float)th;
+    }
+    F.u[1 - cur][t] = u;
+    F.v[1 - cur][t] = v;
+    F.w[1 - cur][t] = w;
+    if constexpr (sizeof(Ts) == sizeof(float)) {
+      F.us[1 - cur][t] = (float)u;
+      F.vs[1 - cur][t] = (float)v;
+      F.ws[1 - cur][t] = (float)w;
     }
   }
   if (const double* tot = grid_total<MaxD, 2>(m, F.red, F.counter, vbx, nblocks)) {
@@ -639,9 +658,10 @@ __device__ __forceinline__ void k_apply_increment_body(const DevParams& P, const
 }
 
 template <class Ts>
-__global__ void __launch_bounds__(kThreads) k_apply_increment(DevParams P, Fields F, int cur,
-                                                              int nblocks) {
-  k_apply_increment_body<Ts>(P, F, cur, nblocks, blockIdx.x);
+__global__ void __launch_bounds__(kThreads) k_increment(DevParams P, Fields F, int cur,
+                                                        int nblocks) {
+  pdl_wait_and_release();
+  k_increment_body<Ts>(P, F, cur, nblocks, blockIdx.x);
 }
 
 // Extrapolation weights along one axis for a wall condition of zero normal derivative:
@@ -659,70 +679,61 @@ __device__ __forceinline__ int wall_weights(int a, int N, int idx[2], double wt[
   return 1;
 }
 
-// Adiabatic walls y = 0, 1 and z = 0, 1 (x interior): theta_b = (4 theta_1 - theta_2)/3 along each
-// wall normal the node lies on (on the y-z edges, the product of the two). The hot and cold
-// walls keep theta = 1 and theta = 0. Max |change| joins the step record.
-__device__ __forceinline__ void k_theta_walls_body(const DevParams& P, const Fields& F,
-                                                   int nblocks, unsigned vbx) {
+// Blocks below nbi: central div V^{n+1} at interior nodes and its maximum. The others: adiabatic walls
+// y = 0, 1 and z = 0, 1 (x interior), theta_b = (4 theta_1 - theta_2)/3 along each wall normal the
+// node lies on (on the y-z edges, the product of the two); the hot and cold walls keep theta = 1
+// and theta = 0. Max |change| joins the step record.
+__device__ __forceinline__ void k_div_walls_body(const DevParams& P, const Fields& F, int nxt,
+                                                 int nbi, int nblocks, unsigned vbx) {
   if (*F.halt) return;
   const int N = P.N, ni = N - 2;
-  const int t = vbx * blockDim.x + threadIdx.x;
-  double m[1] = {0.0};
-  int i, j, k;
-  if (t < 2 * ni * N + 2 * ni * ni) {   // the y faces, then the z faces (x interior)
-    boundary_yz(t, N, i, j, k);
-    int jy[2], kz[2];
-    double wy[2], wz[2];
-    const int ny = wall_weights(j, N, jy, wy), nz = wall_weights(k, N, kz, wz);
-    double s = 0.0;
-    for (int b = 0; b < nz; ++b) {
-      double sb = 0.0;
-      for (int a = 0; a < ny; ++a) sb += wy[a] * F.th[node32(i, jy[a], kz[b], N)];
-      s += wz[b] * sb;
+  double m[2] = {0.0, 0.0};   // |div V|, |change of theta|
+  if ((int)vbx < nbi) {
+    const int t = (int)(vbx * blockDim.x + threadIdx.x);
+    if (t < ni * ni * ni) {
+      const int q = t / ni, i = 1 + (t - q * ni), j = 1 + q % ni, k = 1 + q / ni;
+      const int c = node32(i, j, k, N), sy = N, sz = N * N;
+      const double* u = F.u[nxt];
+      const double* v = F.v[nxt];
+      const double* w = F.w[nxt];
+      const double d = (u[c + 1] - u[c - 1]) * P.inv2[0] + (v[c + sy] - v[c - sy]) * P.inv2[1] +
+                       (w[c + sz] - w[c - sz]) * P.inv2[2];
+      F.div[c] = d;
+      m[0] = absfin(d);
     }
-    const int c = node32(i, j, k, N);
-    m[0] = absfin(s - F.th[c]);
-    F.th[c] = s;
+  } else {
+    const int t = ((int)vbx - nbi) * blockDim.x + threadIdx.x;
+    if (t < 2 * ni * N + 2 * ni * ni) {   // the y faces, then the z faces (x interior)
+      int i, j, k;
+      boundary_yz(t, N, i, j, k);
+      int jy[2], kz[2];
+      double wy[2], wz[2];
+      const int ny = wall_weights(j, N, jy, wy), nz = wall_weights(k, N, kz, wz);
+      double s = 0.0;
+      for (int b = 0; b < nz; ++b) {
+        double sb = 0.0;
+        for (int a = 0; a < ny; ++a) sb += wy[a] * F.th[node32(i, jy[a], kz[b], N)];
+        s += wz[b] * sb;
+      }
+      const int c = node32(i, j, k, N);
+      m[1] = absfin(s - F.th[c]);
+      F.th[c] = s;
+      if (P.krylov_fp32) F.ths[c] = (float)s;
+    }
   }
-  if (const double* tot = grid_total<MaxD, 1>(m, F.red, F.counter, vbx, nblocks)) {
+  if (const double* tot = grid_total<MaxD, 2>(m, F.red, F.counter, vbx, nblocks)) {
     if (threadIdx.x == 0) {
-      F.rec->res = fmax(F.rec->res, tot[0]);
-      if (!P.inner_pass) F.rec->res_theta = fmax(F.rec->res_theta, tot[0]);
+      F.rec->div_max = tot[0];
+      F.rec->res = fmax(F.rec->res, tot[1]);
+      if (!P.inner_pass) F.rec->res_theta = fmax(F.rec->res_theta, tot[1]);
     }
   }
 }
 
-__global__ void __launch_bounds__(kThreads) k_theta_walls(DevParams P, Fields F, int nblocks) {
-  k_theta_walls_body(P, F, nblocks, blockIdx.x);
-}
-
-// Central div V^{n+1} at interior nodes and its maximum.
-__device__ __forceinline__ void k_divergence_body(const DevParams& P, const Fields& F, int nxt,
-                                                  int nblocks, unsigned vbx) {
-  if (*F.halt) return;
-  const int N = P.N, ni = N - 2;
-  const int cnt = ni * ni * ni;
-  const int t = vbx * blockDim.x + threadIdx.x;
-  double m[1] = {0.0};
-  if (t < cnt) {
-    const int q = t / ni, i = 1 + (t - q * ni), j = 1 + q % ni, k = 1 + q / ni;
-    const int c = node32(i, j, k, N), sy = N, sz = N * N;
-    const double* u = F.u[nxt];
-    const double* v = F.v[nxt];
-    const double* w = F.w[nxt];
-    const double d = (u[c + 1] - u[c - 1]) * P.inv2[0] + (v[c + sy] - v[c - sy]) * P.inv2[1] +
-                     (w[c + sz] - w[c - sz]) * P.inv2[2];
-    F.div[c] = d;
-    m[0] = absfin(d);
-  }
-  if (const double* tot = grid_total<MaxD, 1>(m, F.red, F.counter, vbx, nblocks)) {
-    if (threadIdx.x == 0) F.rec->div_max = tot[0];
-  }
-}
-
-__global__ void __launch_bounds__(kThreads) k_divergence(DevParams P, Fields F, int nxt,
-                                                         int nblocks) {
-  k_divergence_body(P, F, nxt, nblocks, blockIdx.x);
+__global__ void __launch_bounds__(kThreads) k_div_walls(DevParams P, Fields F, int nxt, int nbi,
+                                                        int nblocks) {
+  pdl_wait_and_release();
+  k_div_walls_body(P, F, nxt, nbi, nblocks, blockIdx.x);
 }
 
 // p <- p - lambda div V at interior nodes when max|div V| > tol_div (Sec. 2.2).
@@ -741,42 +752,14 @@ __device__ __forceinline__ void k_pressure_correct_body(const DevParams& P, cons
         P.sweep_fp32 ? (double)reinterpret_cast<const float*>(F.eta)[c] : F.eta[c];
     lam = fmin(P.lambda * eta, P.lambda_cap);
   }
-  F.p[c] -= lam * F.div[c];
+  const double p = F.p[c] - lam * F.div[c];
+  F.p[c] = p;
+  if (P.krylov_fp32) F.ps[c] = (float)p;
 }
 
 __global__ void __launch_bounds__(kThreads) k_pressure_correct(DevParams P, Fields F) {
+  pdl_wait_and_release();
   k_pressure_correct_body(P, F, blockIdx.x);
-}
-
-// Zero normal pressure gradient on every wall: p_b = (4 p_1 - p_2)/3 along each wall normal the
-// node lies on (products on edges and corners); applied after a correction.
-__device__ __forceinline__ void k_pressure_walls_body(const DevParams& P, const Fields& F,
-                                                      unsigned vbx) {
-  const int N = P.N, ni = N - 2;
-  const int t = vbx * blockDim.x + threadIdx.x;
-  if (t >= N * N * N - ni * ni * ni || *F.halt) return;
-  if (!(F.rec->div_max > P.tol_div)) return;
-  int i, j, k;
-  boundary_node(t, N, i, j, k);
-  int ix[2], jy[2], kz[2];
-  double wx[2], wy[2], wz[2];
-  const int nx = wall_weights(i, N, ix, wx), ny = wall_weights(j, N, jy, wy),
-            nz = wall_weights(k, N, kz, wz);
-  double s = 0.0;
-  for (int c3 = 0; c3 < nz; ++c3) {
-    double s2 = 0.0;
-    for (int b = 0; b < ny; ++b) {
-      double s1 = 0.0;
-      for (int a = 0; a < nx; ++a) s1 += wx[a] * F.p[node32(ix[a], jy[b], kz[c3], N)];
-      s2 += wy[b] * s1;
-    }
-    s += wz[c3] * s2;
-  }
-  F.p[node32(i, j, k, N)] = s;
-}
-
-__global__ void __launch_bounds__(kThreads) k_pressure_walls(DevParams P, Fields F) {
-  k_pressure_walls_body(P, F, blockIdx.x);
 }
 
 // Step record: Krylov outcomes and the overall status; appended to the ring. A failed step (or,
@@ -809,6 +792,50 @@ __device__ __forceinline__ void k_finish_record_body(const DevParams& P, const F
 
 __global__ void k_finish_record(DevParams P, Fields F) {
   k_finish_record_body(P, F, blockIdx.x);
+}
+
+// Zero normal pressure gradient on every wall: p_b = (4 p_1 - p_2)/3 along each wall normal the
+// node lies on (products on edges and corners); applied after a correction. With record, the last
+// of the nblocks blocks (a ticket: every block has read the halt flag by then) ends the step.
+__device__ __forceinline__ void k_pressure_walls_body(const DevParams& P, const Fields& F,
+                                                      int record, int nblocks, unsigned vbx) {
+  if (*F.halt) return;
+  const int N = P.N, ni = N - 2;
+  const int t = vbx * blockDim.x + threadIdx.x;
+  if (t < N * N * N - ni * ni * ni && F.rec->div_max > P.tol_div) {
+    int i, j, k;
+    boundary_node(t, N, i, j, k);
+    int ix[2], jy[2], kz[2];
+    double wx[2], wy[2], wz[2];
+    const int nx = wall_weights(i, N, ix, wx), ny = wall_weights(j, N, jy, wy),
+              nz = wall_weights(k, N, kz, wz);
+    double s = 0.0;
+    for (int c3 = 0; c3 < nz; ++c3) {
+      double s2 = 0.0;
+      for (int b = 0; b < ny; ++b) {
+        double s1 = 0.0;
+        for (int a = 0; a < nx; ++a) s1 += wx[a] * F.p[node32(ix[a], jy[b], kz[c3], N)];
+        s2 += wy[b] * s1;
+      }
+      s += wz[c3] * s2;
+    }
+    const int c = node32(i, j, k, N);
+    F.p[c] = s;
+    if (P.krylov_fp32) F.ps[c] = (float)s;
+  }
+  if (record) {
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(F.counter, 1u) == (unsigned)nblocks - 1) {
+      *F.counter = 0u;
+      k_finish_record_body(P, F, 0);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) k_pressure_walls(DevParams P, Fields F, int record,
+                                                             int nblocks) {
+  pdl_wait_and_release();
+  k_pressure_walls_body(P, F, record, nblocks, blockIdx.x);
 }
 
 __global__ void k_arm(int* halt, unsigned int* ring_pos, int* steady_stop, int stop) {

@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kTmaMaxThreads)
   const double* tot = grid_total<SumFF, M>(acc, F.red, F.counter, bid, nb);
   const bool bad = failed != 0;
   if (tot) {
-    if (PV) finish_pv(F, tot);
+    if (PV) finish_pv(F, tot, false);
     else finish_st(F, tot);
     // p/v: r p v r0 in, p v out; s/t: r v in, t out; the compact operators
     count_bytes(F, PV ? HOSC_K_BICG_PV : HOSC_K_BICG_ST,
