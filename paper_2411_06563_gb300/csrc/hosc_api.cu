@@ -76,6 +76,10 @@ struct Ctx {
   int tty = 0, tkz = 0, tstages = 3;       // bulk-copy stencil kernels (tty == 0: not used)
   int tkernels = 3;                        // which of them run (1 p/v, 2 s/t, 3 both)
   int xr_flat = 0;                         // x/r as one flat stream (k8_xr)
+  // the one-launch solve: the grid is small enough for it, the caller has chosen no launch shape, and
+  // the context is not a pool's member
+  bool coop_fits = false, shape_chosen = false, pooled = false;
+  int ckz = 0;
   alignas(64) unsigned char tmap_host[kTmaMaps * kTmaMapBytes];   // their tensor maps
   // a round of steps enqueued for a pool (hosc_pool.cu): level and length, records read back
   // asynchronously into h_ring / h_ring_pos, completion marked by round_ev
@@ -146,6 +150,8 @@ void apply_tiles(Ctx* c) {
   c->P.tstages = c->tstages;
   c->P.tkernels = c->tkernels;
   c->P.xr_flat = c->xr_flat;
+  c->P.coop = c->coop_fits && !c->shape_chosen && !c->pooled && c->prm.solver == 0;
+  c->P.ckz = c->ckz;
   c->P.lean = !c->merged && c->sx == 0 && c->tty == 0;
 }
 
@@ -195,7 +201,8 @@ DevParams device_params(const hosc_params& p, int have_prev, int phase) {
   d.have_prev = have_prev;
   d.max_lin_iter = p.max_lin_iter;
   d.krylov_fp32 = (p.precision == HOSC_MIXED);
-  if (!d.krylov_fp32) planar_shape(p.N, &d.pb, &d.pkz);
+  if (!d.krylov_fp32 && !(p.solver == 0 && solve_shape_planar(p.N, &d.pb, &d.pkz)))
+    planar_shape(p.N, &d.pb, &d.pkz);
   d.sweep_fp32 = (p.precision == HOSC_MIXED && phase == 0);
   d.h = 1.0 / (p.N - 1);
   d.h2 = d.h * d.h;
@@ -436,6 +443,13 @@ hosc_status solve_b2(Ctx* c, const DevParams& P) {
 // BiCGSTAB on the four systems; the host checks the done flags every few iterations.
 hosc_status solve_with(Ctx* c, const DevParams& P) {
   const Fields& F = c->F;
+  if (P.coop) {   // counted under the p/v class
+    prof_begin(c, HOSC_K_BICG_PV);
+    launch_solve(P, F, c->stream);
+    prof_end(c, HOSC_K_BICG_PV);
+    c->launches += 1;
+    return check_launch();
+  }
   if (P.krylov_fp32 && !P.lean) {
     launch_bicg_init(P, F, c->stream);
     c->launches += 1;
@@ -707,6 +721,11 @@ cudaError_t append_step(Ctx* c, cudaStream_t s0, cudaStream_t s1, int cur, int h
   launch_viscosity(P, F, cur, s0);
   launch_sources(P, F, cur, s0);
   launch_rhs(P, F, cur, s0);
+  if (P.coop) {
+    launch_solve(P, F, s0);
+    launch_update(P, F, cur, 1, s0);
+    return cudaSuccess;
+  }
   const int apart = first_apart(P) ? 1 : 0;
   if (apart) append_iteration(P, F, 0, true, s0);
   else launch_bicg_init(P, F, s0);
@@ -811,7 +830,8 @@ hosc_status fold_records(Ctx* c, unsigned n, hosc_info* info, bool* steady) {
     const long per = b2 ? 5 : (c->P.krylov_fp32 && c->P.merged ? 2 : 3);
     const long iters = b2 ? (most + 1) / 2 : most, apart = first_apart(c->P) ? 1 : 0;
     const long passes = std::max(1L, (iters - apart + 1) / 2);
-    c->launches += 3 + (1 - apart) + kUpdateLaunches + per * (apart + 2 * passes) + passes;
+    c->launches += 3 + kUpdateLaunches +
+                   (c->P.coop ? 1 : (1 - apart) + per * (apart + 2 * passes) + passes);
     if (r.status != HOSC_OK) {
       st = (hosc_status)r.status;
       break;
@@ -932,7 +952,16 @@ hosc_status make_ctx(const hosc_params* p, void* dev_ws, size_t bytes, void** ou
     hosc_destroy(c);
     return HOSC_ECUDA;
   }
-  default_tiles(p->N, &c->kblock, &c->kz);
+  // the launch shape of the one-launch solve is the default of the kernel-by-kernel one too, so that
+  // both give the same bits
+  if (p->precision == HOSC_MIXED) {
+    c->coop_fits = solve_shape_mixed(p->N, &c->kblock, &c->kz);
+    c->ckz = c->kz;
+  } else {
+    int b = 0, z = 0;
+    c->coop_fits = p->solver == 0 && solve_shape_planar(p->N, &b, &z);
+  }
+  if (!c->coop_fits || p->precision != HOSC_MIXED) default_tiles(p->N, &c->kblock, &c->kz);
   st = set_initial_state(c);
   if (st) {
     hosc_destroy(c);
@@ -963,6 +992,13 @@ long ctx_signature(void* ctx) {
                  ((long)c->merged << 52);
   return s ^ ((long)c->tty << 53) ^ ((long)c->tkz << 56) ^ ((long)c->xr_flat << 62) ^
          ((long)c->tstages << 45) ^ ((long)c->tkernels << 48);
+}
+
+void ctx_join_pool(void* ctx) {
+  Ctx* c = (Ctx*)ctx;
+  c->pooled = true;
+  apply_tiles(c);
+  drop_graphs(c);
 }
 
 // Start of a round of n steps from the current level (read back by ctx_collect_round).
@@ -1145,6 +1181,7 @@ size_t workspace_layout(int N, int bicgstab2, Fields* f, char* base) {
   F.eloc = (double*)take(3 * n3 * sizeof(double));
   // per-block partials: one row per block of any accepted launch shape
   F.red = (double*)take((size_t)red_rows((long)n3) * kRedSlots * sizeof(double));
+  F.exch = (ulonglong2*)take(kExchValues * sizeof(ulonglong2));
   F.counter = (unsigned int*)take(sizeof(unsigned int));
   F.ks = (KrylovScalars*)take(4 * sizeof(KrylovScalars));
   F.rec = (StepRecord*)take(sizeof(StepRecord));
@@ -1582,11 +1619,20 @@ hosc_status hosc_time_kernel(void* ctx, int kernel_id, int reps, double* ms_per_
   return HOSC_OK;
 }
 
+// A launch shape set by the caller: the solve runs kernel by kernel with it.
+static void choose_shape(Ctx* c) {
+  if (c->shape_chosen) return;
+  c->shape_chosen = true;
+  if (c->P.coop) drop_graphs(c);
+  apply_tiles(c);
+}
+
 hosc_status hosc_set_tiles(void* ctx, int kblock, int kz, int narrow) {
   Ctx* c = (Ctx*)ctx;
   if (!c) return HOSC_EINVAL;
   if (c->stage != 0) return HOSC_ESTATE;
   if (!tiles_valid(c, kblock, kz, narrow)) return HOSC_EINVAL;
+  choose_shape(c);
   if (kblock != c->kblock || kz != c->kz || narrow != c->narrow) {
     c->kblock = c->P.kblock = kblock;
     c->kz = c->P.kz = kz;
@@ -1602,6 +1648,7 @@ hosc_status hosc_set_stencil_tiles(void* ctx, int sx, int sy, int skz) {
   if (c->stage != 0) return HOSC_ESTATE;
   CU(cudaSetDevice(c->device));
   if (!stencil_tiles_valid(c, sx, sy, skz)) return HOSC_EINVAL;
+  choose_shape(c);
   if (sx == 0) sy = skz = 0;
   if (sx != c->sx || sy != c->sy || skz != c->skz || (sx > 0 && c->tty > 0)) {
     c->sx = sx;
@@ -1643,6 +1690,7 @@ hosc_status hosc_set_tma_tiles(void* ctx, int tty, int tkz, int stages, int kern
       return HOSC_ECUDA;
     }
   }
+  choose_shape(c);
   if (tty != c->tty || tkz != c->tkz || stages != c->tstages || kernels != c->tkernels ||
       (tty > 0 && c->sx > 0)) {
     c->tty = tty;
@@ -1660,6 +1708,7 @@ hosc_status hosc_set_xr_form(void* ctx, int flat) {
   Ctx* c = (Ctx*)ctx;
   if (!c || (flat != 0 && flat != 1)) return HOSC_EINVAL;
   if (c->stage != 0) return HOSC_ESTATE;
+  choose_shape(c);
   if (flat != c->xr_flat) {
     c->xr_flat = flat;
     apply_tiles(c);
@@ -1687,6 +1736,7 @@ hosc_status hosc_set_krylov_merged(void* ctx, int merged) {
   Ctx* c = (Ctx*)ctx;
   if (!c || (merged != 0 && merged != 1)) return HOSC_EINVAL;
   if (c->stage != 0) return HOSC_ESTATE;
+  choose_shape(c);
   if (merged != c->merged) {
     const int save = c->merged;
     c->merged = merged;
@@ -1730,6 +1780,16 @@ hosc_status hosc_autotune(void* ctx, int reps, int* kblock_out, int* kz_out, dou
   if (c->stage != 0) return HOSC_ESTATE;
   if (!c->P.krylov_fp32) return HOSC_EINVAL;
   CU(cudaSetDevice(c->device));
+  // where the one-launch solve runs it stays: the shapes found are those of the kernels beside it
+  struct KeepChoice {
+    Ctx* c;
+    bool chosen;
+    ~KeepChoice() {
+      c->shape_chosen = chosen;
+      apply_tiles(c);
+      drop_graphs(c);
+    }
+  } keep{c, c->shape_chosen};
   {   // the register kernels first
     hosc_status s0 = hosc_set_stencil_tiles(c, 0, 0, 0);
     if (!s0) s0 = hosc_set_tma_tiles(c, 0, 0, 3, 3);

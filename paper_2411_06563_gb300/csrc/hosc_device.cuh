@@ -198,25 +198,53 @@ __host__ __device__ constexpr int row_stride() {
   return M > 2 * kRedSlots ? 4 * kRedSlots : (M > kRedSlots ? 2 * kRedSlots : kRedSlots);
 }
 
+// Sum of nr rows of M slots in an order that does not depend on the block's size, so that every kernel
+// that forms the same rows gets the same bits: group g of G adds rows g, g + G, ... one after another
+// (four loads in flight), then the groups combine in a tree. load(row, slot); the totals are left in
+// tot (shared), valid for every thread. blockDim.x must be a multiple of 32.
+template <class T, int M, class Load>
+__device__ __forceinline__ void sum_rows(int nr, Load load, double* tot) {
+  constexpr int Mp = pow2_at_least(M);
+  constexpr int G = Mp <= 8 ? 64 : 512 / Mp;
+  __shared__ double s_g[Mp * G];
+  const int t = threadIdx.x, bd = blockDim.x, lane = t & 31, nw = bd >> 5;
+  for (int w = t; w < Mp * G; w += bd) {
+    const int m = w % Mp;
+    double acc = 0.0;
+    int r = m < M ? w / Mp : nr;   // the slots past the M values stay zero
+    for (; r + 3 * G < nr; r += 4 * G) {
+      const double a0 = load(r, m), a1 = load(r + G, m), a2 = load(r + 2 * G, m),
+                   a3 = load(r + 3 * G, m);
+      acc = T::add(T::add(T::add(T::add(acc, a0), a1), a2), a3);
+    }
+    for (; r < nr; r += G) acc = T::add(acc, load(r, m));
+    s_g[w] = acc;
+  }
+  __syncthreads();
+  for (int m = t >> 5; m < Mp; m += nw) {
+    double a = lane < G ? s_g[lane * Mp + m] : 0.0;
+    if (G > 32) a = T::add(a, s_g[(lane + 32) % G * Mp + m]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) a = T::add(a, T::shfl_xor(a, off));
+    if (lane == 0) tot[m] = a;
+  }
+  __syncthreads();
+}
+
 // Second half of a reduction over the grid, called by every block once its warp 0 has written the
 // block's values to rows of red: takes a ticket; the block that takes the last of `tickets` (no block
-// waits for another) sums the nr rows of M slots in a fixed order and returns the totals in shared
-// memory, valid for its every thread; the other blocks return null. The ticket counter is left at
-// zero for the next kernel. In the last block, with Mp the power of two >= M, thread t reads slot
-// t % Mp of rows t / Mp, t / Mp + blockDim/Mp, ... (consecutive threads read consecutive doubles;
-// four rows' loads in flight at a time). blockDim.x must be a multiple of 32, at most 32 kMaxWarps.
+// waits for another) sums the nr rows of M slots and returns the totals in shared memory, valid for
+// its every thread; the other blocks return null. The ticket counter is left at zero for the next
+// kernel.
 template <class T, int M>
 __device__ __forceinline__ const double* last_block_total(const double* red, unsigned int* counter,
-                                                          unsigned int nr_, unsigned int tickets) {
-  constexpr int Mp = pow2_at_least(M);
+                                                          unsigned int nr, unsigned int tickets) {
   constexpr long S = row_stride<M>();
-  __shared__ double s_d[kMaxWarps * Mp];
-  __shared__ double s_tot[Mp];
+  __shared__ double s_tot[pow2_at_least(M)];
   __shared__ int s_last;
-  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-  if (wid == 0) {
+  if (threadIdx.x < 32) {
     __syncwarp();
-    if (lane == 0) {
+    if (threadIdx.x == 0) {
       __threadfence();
       s_last = atomicAdd(counter, 1u) == tickets - 1;
     }
@@ -224,27 +252,8 @@ __device__ __forceinline__ const double* last_block_total(const double* red, uns
   __syncthreads();
   if (!s_last) return nullptr;
   __threadfence();
-  const int m = t % Mp, rstep = blockDim.x / Mp, nr = (int)nr_;
-  double acc = 0.0;
-  int r = m < M ? t / Mp : nr;   // lanes past the M values read nothing
-  for (; r + 3 * rstep < nr; r += 4 * rstep) {
-    const double a0 = __ldcg(red + r * S + m);
-    const double a1 = __ldcg(red + (r + rstep) * S + m);
-    const double a2 = __ldcg(red + (r + 2 * rstep) * S + m);
-    const double a3 = __ldcg(red + (r + 3 * rstep) * S + m);
-    acc = T::add(T::add(acc, T::add(a0, a1)), T::add(a2, a3));
-  }
-  for (; r < nr; r += rstep) acc = T::add(acc, __ldcg(red + r * S + m));
-#pragma unroll
-  for (int off = Mp; off < 32; off <<= 1) acc = T::add(acc, T::shfl_xor(acc, off));
-  if (lane < Mp) s_d[wid * Mp + lane] = acc;
-  __syncthreads();
-  if (wid == 0) {
-    const double tot = cross_warps<T, Mp>(s_d);
-    if (lane < Mp) s_tot[lane] = tot;
-    if (lane == 0) *counter = 0u;
-  }
-  __syncthreads();
+  if (threadIdx.x == 0) *counter = 0u;
+  sum_rows<T, M>((int)nr, [&](int r, int m) { return __ldcg(red + r * S + m); }, s_tot);
   return s_tot;
 }
 

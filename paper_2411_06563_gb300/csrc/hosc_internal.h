@@ -54,6 +54,8 @@ struct DevParams {
                      // columns, tkz planes per block; tty == 0: not used
   int tstages;       // their ring of shared-memory stages (3, 4, 6 or 8)
   int tkernels;      // which of them run: 1 p/v, 2 s/t, 3 both
+  int coop;          // the solve is one cooperative launch (hosc_solve.cu)
+  int ckz;           // its planes per block, mixed precision (FP64: pb and pkz)
   int lean;          // interleaved solve started by the right-hand sides' kernel: no initialisation,
                      // the first iteration reads r_0 and nothing else (register kernels, either x/r)
   int xr_flat;       // x/r as one flat grid-stride stream (k8_xr) instead of the column march
@@ -83,6 +85,8 @@ struct DevParams {
   double div_steady;   // max|div V| below this (div_steady, else tol_div) is steady
 };
 
+constexpr int kSolveRows = 152;      // most rows (blocks) of a system in the one-launch FP64 solve
+constexpr int kExchValues = 8192;   // 16-byte values of the exchange buffer
 constexpr int kRing = 256;   // step records kept on the device between host reads
 
 // BiCGSTAB scalars of one system, resident in device memory.
@@ -129,6 +133,7 @@ struct Fields {
   double* u0[4];
   double* r2[4];
   double* u2[4];
+  ulonglong2* exch;  // [kExchValues] exchanges of the one-launch solve, zero before it
   double* div;       // div V^{n+1}
   double* red;       // reduction partials [blocks][kRedSlots]
   unsigned int* counter;   // last-block ticket (reset by the last block)
@@ -234,6 +239,11 @@ void launch_b2(int kernel, const DevParams& P, const Fields& F, int cp, bool fir
                cudaStream_t s);
 // End of the body of the BiCGSTAB loop of a captured step: end of the loop when every system is done.
 void launch_loop_cond(const Fields& F, unsigned long long handle, cudaStream_t s);
+// The whole solve as one cooperative launch (P.coop): scalars started and exchange buffer zeroed by the
+// right-hand sides' kernel. The shapes it runs with on an N^3 grid; false when the grid is too large.
+void launch_solve(const DevParams& P, const Fields& F, cudaStream_t s);
+bool solve_shape_planar(int N, int* pb, int* pkz);
+bool solve_shape_mixed(int N, int* kblock, int* kz);
 // Mark all four systems as iterating (for timing the Krylov kernels in isolation).
 void launch_krylov_activate(const Fields& F, cudaStream_t s);
 // S6-S8: increments, theta walls, div V, pressure correction and walls, in mixed precision with the
@@ -283,6 +293,9 @@ size_t ctx_workspace(void* ctx);             // device bytes the context holds
 int ctx_N(void* ctx);
 cudaStream_t ctx_branch_stream(void* ctx);   // stream on which ctx_append_round captures
 long ctx_signature(void* ctx);               // changes when a captured round no longer applies
+// A member of a pool: its solves run kernel by kernel, beside those of the other members (a cooperative
+// grid takes the whole GPU).
+void ctx_join_pool(void* ctx);
 void ctx_begin_round(void* ctx, long n);
 hosc_status ctx_enqueue_round(void* ctx, int n);
 hosc_status ctx_append_round(void* ctx, int n);

@@ -106,10 +106,10 @@ template <int KIND>
 __device__ __forceinline__ void planar_finish(const DevParams& P, const Fields& F,
                                               const double* tot, bool first,
                                               const int (&done)[4]) {
-  if (KIND == PL_PV || KIND == PL_U1) finish_pv(F, tot, first);
-  if (KIND == PL_U2) finish_pv(F, tot, false);
-  if (KIND == PL_ST) finish_st(F, tot);
-  if (KIND == PL_XR) finish_xr(P, F, tot);
+  if (KIND == PL_PV || KIND == PL_U1) finish_pv(F.ks, tot, first);
+  if (KIND == PL_U2) finish_pv(F.ks, tot, false);
+  if (KIND == PL_ST) finish_st(F.ks, tot);
+  if (KIND == PL_XR) finish_xr(P, F.ks, tot);
   if (KIND == PL_R1 && threadIdx.x < 4) {
     KrylovScalars& k = F.ks[threadIdx.x];
     const double rho1 = tot[threadIdx.x];
@@ -214,7 +214,7 @@ __device__ __forceinline__ void planar_end(const DevParams& P, const Fields& F, 
     planar_finish<KIND>(P, F, tot, FIRST, done);
 }
 
-// The kernels that apply an operator. pp: parity of the iteration (BiCGSTAB) or cycle.
+// The planar kernels that apply an operator. pp: parity of the iteration (BiCGSTAB) or cycle.
 template <int KIND, int B, bool FIRST>
 __global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, int pp) {
   extern __shared__ double planes[];   // two planes of N + B + N values
@@ -242,8 +242,8 @@ __global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, i
     auto value = [&](int c) {
       const double x = X[c];
       if (plain) return x;
-      if (KIND == PL_PV) return x + beta * (Z[c] - q * Y[c]);
-      return x - q * Y[c];
+      if (KIND == PL_PV) return fma(beta, fma(-q, Y[c], Z[c]), x);
+      return fma(-q, Y[c], x);
     };
     const double* const* A = s < 3 ? F.Am : F.Ae;
     const double *a0 = A[0], *a1 = A[1], *a2 = A[2], *a3 = A[3], *a4 = A[4], *a5 = A[5], *a6 = A[6];
@@ -263,18 +263,18 @@ __global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, i
       __syncthreads();
       if (b.inner) {
         const double* o = pl + N + t;
-        const double y = a0[c] * mid + a1[c] * o[1] + a2[c] * o[-1] + a3[c] * o[N] +
-                         a4[c] * o[-N] + a5[c] * hi + a6[c] * lo;
+        const double y = planar_row(a0[c], a1[c], a2[c], a3[c], a4[c], a5[c], a6[c], mid, o[1], o[-1],
+                                    o[N], o[-N], hi, lo);
         if (KIND == PL_PV) {
           F.pk[1 - pp][s][c] = mid;
           F.vk[1 - pp][s][c] = y;
           const double r0 = rhs[c];
-          dot[0] += r0 * y;
-          if (FIRST) dot[L] += r0 * r0;
+          dot[0] = fma(r0, y, dot[0]);
+          if (FIRST) dot[L] = fma(r0, r0, dot[L]);
         } else if (KIND == PL_ST) {
           F.t[s][c] = y;
-          dot[0] += y * mid;
-          dot[L] += y * y;
+          dot[0] = fma(y, mid, dot[0]);
+          dot[L] = fma(y, y, dot[L]);
         } else if (KIND == PL_U1) {
           F.vk[0][s][c] = y;
           const double r0 = rhs[c];
@@ -336,12 +336,12 @@ __global__ void __launch_bounds__(B) k_planar_end(DevParams P, Fields F, int pp)
 #pragma unroll 2
       for (int k = b.k0; k < b.k1; ++k) {
         const int c = b.l + N2 * k;
-        const double sv = ro[c] - a * v[c];
-        x[c] = (FIRST ? 0.0 : x[c]) + a * p[c] + om * sv;
-        const double rn = sv - om * tv[c];
+        const double sv = fma(-a, v[c], ro[c]);
+        x[c] = fma(om, sv, fma(a, p[c], FIRST ? 0.0 : x[c]));
+        const double rn = fma(-om, tv[c], sv);
         r[c] = rn;
-        dot[0] += rhs[c] * rn;
-        dot[1] += rn * rn;
+        dot[0] = fma(rhs[c], rn, dot[0]);
+        dot[1] = fma(rn, rn, dot[1]);
       }
     } else {
       const double g1 = F.ks[s].g1, g2 = F.ks[s].g2;
@@ -624,7 +624,7 @@ __device__ __forceinline__ Op4 staged_op(const float4* sq, const StageLayout& L,
   Op4 op;
   op.m = sq[L.op_m() + t];
   op.e = sq[L.op_e() + t];
-  op.l12 = ((const float*)(sq + L.op_l()))[t] * (1.f / 12.f);
+  op.l12 = __fmul_rn(((const float*)(sq + L.op_l()))[t], 1.f / 12.f);
   return op;
 }
 
@@ -677,7 +677,7 @@ __global__ void __launch_bounds__(256) k5_pv(DevParams P, Fields F, int pp) {
   const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
   const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
   if (const double* tot = grid_total<SumFF, 4>(acc, F.red, F.counter, bid, nb)) {
-    finish_pv(F, tot, false);
+    finish_pv(F.ks, tot, false);
     count_bytes(F, HOSC_K_BICG_PV, bytes4(P, 6.0 + op_words(ene)));
   }
 }
@@ -728,7 +728,7 @@ __global__ void __launch_bounds__(256) k5_st(DevParams P, Fields F, int pp) {
   const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
   const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
   if (const double* tot = grid_total<SumFF, 8>(acc, F.red, F.counter, bid, nb)) {
-    finish_st(F, tot);
+    finish_st(F.ks, tot);
     count_bytes(F, HOSC_K_BICG_ST, bytes4(P, 3.0 + op_words(ene)));
   }
 }
@@ -864,7 +864,7 @@ __global__ void __launch_bounds__(256) k8_xr(DevParams P, Fields F, int pp) {
     ff_dot4(acc + 4, rn, rn);
   }
   if (const double* tot = grid_total<SumFF, 8>(acc, F.red, F.counter, blockIdx.x, gridDim.x)) {
-    finish_xr(P, F, tot);
+    finish_xr(P, F.ks, tot);
     // r v p x t r0 in, x r out
     count_bytes(F, HOSC_K_BICG_XR, bytes4(P, FIRST ? 6.0 : 8.0));
   }

@@ -29,7 +29,7 @@ struct FF {
 
 __device__ __forceinline__ FF ff_prod(float a, float b) {
   FF r;
-  r.hi = a * b;
+  r.hi = __fmul_rn(a, b);     // never fused into a sum
   r.lo = fmaf(a, b, -r.hi);   // exact rounding error of the product
   return r;
 }
@@ -90,7 +90,7 @@ struct Op4 {
 __device__ __forceinline__ Op4 load_op(const Fields& F, int c, bool ene) {
   Op4 op;
   op.m = HOSC_LDG(F.kwm + c);
-  op.l12 = HOSC_LDG(F.kL + c) * (1.f / 12.f);
+  op.l12 = __fmul_rn(HOSC_LDG(F.kL + c), 1.f / 12.f);
   op.e = ene ? HOSC_LDG(F.kwe + c) : make_float4(0.f, 0.f, 0.f, 0.f);
   return op;
 }
@@ -99,18 +99,25 @@ __device__ __forceinline__ float4 apply_op(const DevParams& P, const Op4& op, fl
                                            float4 xm, float4 yp, float4 ym, float4 zp,
                                            float4 zm) {
   // momentum weights of the six neighbours, shared by the u, v, w lanes
+  // (l12 is a product of its own in load_op and the staged forms: not fused into these)
   const float Sx = P.csf[0] + op.l12, Sy = P.csf[1] + op.l12, Sz = P.csf[2] + op.l12;
   const float4 m = op.m, e = op.e;
   const float a1 = Sx - m.x, a2 = Sx + m.x, a3 = Sy - m.y, a4 = Sy + m.y, a5 = Sz - m.z,
               a6 = Sz + m.z;
+  // one explicit order of the sums and fused multiply-adds, so that every kernel that applies the
+  // operator gets the same bits
+  auto row = [&](float c, float cp, float cm, float yp_, float ym_, float zp_, float zm_) {
+    return fmaf(a6, zm_, fmaf(a5, zp_, fmaf(a4, ym_, fmaf(a3, yp_, fmaf(a2, cm, fmaf(a1, cp,
+                __fmul_rn(m.w, c)))))));
+  };
   float4 y;
-  y.x = m.w * o.x + a1 * xp.x + a2 * xm.x + a3 * yp.x + a4 * ym.x + a5 * zp.x + a6 * zm.x;
-  y.y = m.w * o.y + a1 * xp.y + a2 * xm.y + a3 * yp.y + a4 * ym.y + a5 * zp.y + a6 * zm.y;
-  y.z = m.w * o.z + a1 * xp.z + a2 * xm.z + a3 * yp.z + a4 * ym.z + a5 * zp.z + a6 * zm.z;
+  y.x = row(o.x, xp.x, xm.x, yp.x, ym.x, zp.x, zm.x);
+  y.y = row(o.y, xp.y, xm.y, yp.y, ym.y, zp.y, zm.y);
+  y.z = row(o.z, xp.z, xm.z, yp.z, ym.z, zp.z, zm.z);
   const float c12 = 1.f / 12.f;
   const float ex = P.csf[0] + c12, ey = P.csf[1] + c12, ez = P.csf[2] + c12;
-  y.w = e.w * o.w + (ex - e.x) * xp.w + (ex + e.x) * xm.w + (ey - e.y) * yp.w +
-        (ey + e.y) * ym.w + (ez - e.z) * zp.w + (ez + e.z) * zm.w;
+  y.w = fmaf(ez + e.z, zm.w, fmaf(ez - e.z, zp.w, fmaf(ey + e.y, ym.w, fmaf(ey - e.y, yp.w,
+        fmaf(ex + e.x, xm.w, fmaf(ex - e.x, xp.w, __fmul_rn(e.w, o.w)))))));
   if (P.precond) {
     const float im = 1.f / m.w;
     y.x *= im;
@@ -119,6 +126,14 @@ __device__ __forceinline__ float4 apply_op(const DevParams& P, const Op4& op, fl
     y.w = e.w != 0.f ? y.w / e.w : 0.f;
   }
   return y;
+}
+
+// A row of the planar FP64 operator, in one explicit order for the same reason.
+__device__ __forceinline__ double planar_row(double a0, double a1, double a2, double a3, double a4,
+                                             double a5, double a6, double c, double xp, double xm,
+                                             double yp, double ym, double zp, double zm) {
+  return fma(a6, zm, fma(a5, zp, fma(a4, ym, fma(a3, yp, fma(a2, xm, fma(a1, xp,
+             __dmul_rn(a0, c)))))));
 }
 
 // Float4 words per interior node of the compact operators a launch reads: kwm and kL, and kwe
@@ -225,18 +240,15 @@ __device__ __forceinline__ void finish_init(const DevParams& P, const Fields& F,
   k.done = (norm == 0.0 || halt || (s == 3 && P.inner_pass)) ? 1 : 0;
 }
 
-// r_0 . v of each system (slots 0..3): alpha = rho / (r_0 . v). In the first iteration of a lean form
-// r_0 . r_0 too (4..7), which is rho; a system whose right-hand side is zero is then done.
-__device__ __forceinline__ void finish_pv(const Fields& F, const double* tot, bool first) {
-  if (threadIdx.x >= 4) return;
-  KrylovScalars& k = F.ks[threadIdx.x];
+// One system's scalars from r_0 . v = d: alpha = rho / d. In the first iteration of a lean form r_0 .
+// r_0 = rr too, which is rho; a system whose right-hand side is zero is then done.
+__device__ __forceinline__ void pv_scalars(KrylovScalars& k, double d, double rr, bool first) {
   const int done = k.done;
   double rho = k.rho;
-  const double d = tot[threadIdx.x];
   if (done) return;
   if (first) {
-    rho = tot[4 + threadIdx.x];
-    const double norm = sqrt(rho);
+    rho = rr;
+    const double norm = sqrt(rr);
     k.rho = rho;
     k.r0norm = norm;
     k.rnorm = norm;
@@ -253,24 +265,19 @@ __device__ __forceinline__ void finish_pv(const Fields& F, const double* tot, bo
   }
 }
 
-// t . s (slots 0..3) and t . t (4..7): omega = (t . s) / (t . t), 0 when t = 0.
-__device__ __forceinline__ void finish_st(const Fields& F, const double* tot) {
-  if (threadIdx.x >= 4) return;
-  KrylovScalars& k = F.ks[threadIdx.x];
-  if (k.done) return;
-  const double ts = tot[threadIdx.x], tt = tot[4 + threadIdx.x];
-  k.omega = tt > 0.0 ? ts / tt : 0.0;
+// omega = (t . s) / (t . t), 0 when t = 0.
+__device__ __forceinline__ void st_scalars(KrylovScalars& k, double ts, double tt) {
+  if (!k.done) k.omega = tt > 0.0 ? ts / tt : 0.0;
 }
 
-// r_0 . r (slots 0..3) and r . r (4..7): the convergence and breakdown tests, beta and rho of the
-// next iteration.
-__device__ __forceinline__ void finish_xr(const DevParams& P, const Fields& F, const double* tot) {
-  if (threadIdx.x >= 4) return;
-  KrylovScalars& k = F.ks[threadIdx.x];
+// r_0 . r = rho_new and r . r = rr: the convergence and breakdown tests, beta and rho of the next
+// iteration.
+__device__ __forceinline__ void xr_scalars(const DevParams& P, KrylovScalars& k, double rho_new,
+                                           double rr) {
   const int done = k.done, iters = k.iters + 1;
   const double rho = k.rho, alpha = k.alpha, omega = k.omega, r0norm = k.r0norm;
   if (done) return;
-  const double rho_new = tot[threadIdx.x], rnorm = sqrt(tot[4 + threadIdx.x]);
+  const double rnorm = sqrt(rr);
   k.rnorm = rnorm;
   k.iters = iters;
   if (rnorm <= P.tol_lin * r0norm) {
@@ -283,6 +290,18 @@ __device__ __forceinline__ void finish_xr(const DevParams& P, const Fields& F, c
     k.beta = (rho_new / rho) * (alpha / omega);
     k.rho = rho_new;
   }
+}
+
+// The same for the four systems at ks from the totals of a launch: slots 0..3 and 4..7.
+__device__ __forceinline__ void finish_pv(KrylovScalars* ks, const double* tot, bool first) {
+  const int s = threadIdx.x;
+  if (s < 4) pv_scalars(ks[s], tot[s], first ? tot[4 + s] : 0.0, first);
+}
+__device__ __forceinline__ void finish_st(KrylovScalars* ks, const double* tot) {
+  if (threadIdx.x < 4) st_scalars(ks[threadIdx.x], tot[threadIdx.x], tot[4 + threadIdx.x]);
+}
+__device__ __forceinline__ void finish_xr(const DevParams& P, KrylovScalars* ks, const double* tot) {
+  if (threadIdx.x < 4) xr_scalars(P, ks[threadIdx.x], tot[threadIdx.x], tot[4 + threadIdx.x]);
 }
 
 // Add a launch's algorithmic bytes (a thread that takes no part in the ends above).
@@ -379,7 +398,7 @@ __device__ __forceinline__ void k4_pv_body(const DevParams& P, const Fields& F, 
   }
   if (const double* tot =
           grid_total<SumFF, M>(acc, F.red, F.counter, block_id(vg), block_count(vg))) {
-    finish_pv(F, tot, FIRST);
+    finish_pv(F.ks, tot, FIRST);
     // r p v r0 in, p v out, the compact operators
     count_bytes(F, HOSC_K_BICG_PV, bytes4(P, (FIRST ? 3.0 : 6.0) + op_words(ene)));
   }
@@ -426,7 +445,7 @@ __device__ __forceinline__ void k4_st_body(const DevParams& P, const Fields& F, 
   }
   if (const double* tot =
           grid_total<SumFF, 8>(acc, F.red, F.counter, block_id(vg), block_count(vg))) {
-    finish_st(F, tot);
+    finish_st(F.ks, tot);
     // r v in, t out, the compact operators
     count_bytes(F, HOSC_K_BICG_ST, bytes4(P, 3.0 + op_words(ene)));
   }
@@ -471,7 +490,7 @@ __device__ __forceinline__ void k4_xr_body(const DevParams& P, const Fields& F, 
   const double* tot =
       grid_total<SumFF, 8>(acc, F.red, F.counter, block_id(vg), block_count(vg));
   if (!tot) return;
-  finish_xr(P, F, tot);
+  finish_xr(P, F.ks, tot);
   count_bytes(F, HOSC_K_BICG_XR, bytes4(P, FIRST ? 6.0 : 8.0));   // r v p x t r0 in, x r out
 }
 

@@ -2,9 +2,9 @@
 // any device allocation. The Krylov vectors, reduction partials and solver scalars live in one
 // file-scope device array of fixed size (HOSC_NOALLOC_MAX_N nodes per side), shared by every call
 // in the process; inputs and outputs are the caller's device arrays. The kernels are the ones of
-// the context path (hosc_krylov.cu), so the result equals the context's solve. The host checks
-// convergence every 4 to 16 iterations: it copies the four systems' solver scalars to the host and
-// synchronises the stream, so a call returns only once its solve has finished.
+// the context path (hosc_solve.cu, hosc_krylov.cu), so the result equals the context's solve. A call
+// copies the four systems' solver scalars to the host and synchronises the stream (once for the
+// one-launch solve, else every 4 to 16 iterations), so it returns only once its solve has finished.
 
 #include <cuda_runtime.h>
 #include <string.h>
@@ -35,6 +35,9 @@ static_assert(kOffCounter + sizeof(unsigned int) <= kOffHalt, "counter overlaps 
 static_assert(kOffHalt + sizeof(int) <= kOffBytes, "halt flag overlaps the byte counters");
 static_assert(kOffBytes + HOSC_K_COUNT * sizeof(double) <= kOffRed,
               "byte counters overlap the reduction partials");
+// The one-launch solve puts its exchanges where the other form has its partials.
+constexpr size_t kExchBytes = kControlBytes - kOffRed;
+static_assert(kExchBytes >= 16 * 4 * 4 * (size_t)kSolveRows, "exchanges exceed the control block");
 static_assert(kOffRed + kMaxBlocks * kRedSlots * sizeof(double) <= kControlBytes,
               "reduction partials exceed the control block");
 
@@ -106,11 +109,6 @@ extern "C" hosc_status hosc_bicgstab_noalloc(int N, const double* const* weights
     F.rhs[s] = const_cast<double*>(rhs[s]);
     F.x[s] = x[s];
   }
-  // Every call shares the scratch and finds the previous call's contents: the vectors must read
-  // zero on the walls and the ticket counter and halt flag must start at zero.
-  if (cudaMemsetAsync(base, 0, vec_used, sm) != cudaSuccess) return HOSC_ECUDA;
-  if (cudaMemsetAsync(ctl, 0, kOffRed, sm) != cudaSuccess) return HOSC_ECUDA;
-
   DevParams P;
   memset(&P, 0, sizeof(P));
   P.N = N;
@@ -119,31 +117,45 @@ extern "C" hosc_status hosc_bicgstab_noalloc(int N, const double* const* weights
   P.h = 1.0 / (N - 1);
   P.h2 = P.h * P.h;
   P.rhs_copied = 1;
-  planar_shape(N, &P.pb, &P.pkz);
-
   KrylovScalars ks[4];
-  launch_bicg_init(P, F, sm);
-  int pp = 0, it = 0, check = 4;
-  while (it < max_iter) {
-    const int chunk = (max_iter - it < check) ? max_iter - it : check;
-    for (int q = 0; q < chunk; ++q) {
-      const bool first = it + q == 0;
-      launch_bicg_pv(P, F, pp, first, sm);
-      launch_bicg_st(P, F, pp, first, sm);
-      launch_bicg_xr(P, F, pp, first, sm);
-      pp ^= 1;
+  auto read_scalars = [&]() {
+    return cudaMemcpyAsync(ks, F.ks, sizeof(ks), cudaMemcpyDeviceToHost, sm) == cudaSuccess &&
+           cudaStreamSynchronize(sm) == cudaSuccess;
+  };
+  // Every call shares the scratch and finds the previous call's contents.
+  if (solve_shape_planar(N, &P.pb, &P.pkz)) {
+    // one launch (every grid up to HOSC_NOALLOC_MAX_N where its blocks are resident): the solver's
+    // scalars, the halt flag and the exchanges start at zero
+    F.exch = (ulonglong2*)F.red;
+    if (cudaMemsetAsync(ctl, 0, kControlBytes, sm) != cudaSuccess) return HOSC_ECUDA;
+    launch_solve(P, F, sm);
+    if (cudaGetLastError() != cudaSuccess || !read_scalars()) return HOSC_ECUDA;
+  } else {
+    // the vectors must read zero on the walls, the ticket counter and halt flag start at zero
+    if (cudaMemsetAsync(base, 0, vec_used, sm) != cudaSuccess) return HOSC_ECUDA;
+    if (cudaMemsetAsync(ctl, 0, kOffRed, sm) != cudaSuccess) return HOSC_ECUDA;
+    planar_shape(N, &P.pb, &P.pkz);
+    launch_bicg_init(P, F, sm);
+    int pp = 0, it = 0, check = 4;
+    while (it < max_iter) {
+      const int chunk = (max_iter - it < check) ? max_iter - it : check;
+      for (int q = 0; q < chunk; ++q) {
+        const bool first = it + q == 0;
+        launch_bicg_pv(P, F, pp, first, sm);
+        launch_bicg_st(P, F, pp, first, sm);
+        launch_bicg_xr(P, F, pp, first, sm);
+        pp ^= 1;
+      }
+      it += chunk;
+      if (cudaGetLastError() != cudaSuccess || !read_scalars()) return HOSC_ECUDA;
+      if (ks[0].done && ks[1].done && ks[2].done && ks[3].done) break;
+      if (check < 16) check *= 2;
     }
-    it += chunk;
-    if (cudaGetLastError() != cudaSuccess) return HOSC_ECUDA;
-    if (cudaMemcpyAsync(ks, F.ks, sizeof(ks), cudaMemcpyDeviceToHost, sm) != cudaSuccess ||
-        cudaStreamSynchronize(sm) != cudaSuccess)
-      return HOSC_ECUDA;
-    if (ks[0].done && ks[1].done && ks[2].done && ks[3].done) break;
-    if (check < 16) check *= 2;
   }
   st = HOSC_OK;
   for (int s = 0; s < 4; ++s) {
     if (iters_out) iters_out[s] = ks[s].iters;
+    if (ks[s].status == HOSC_ECUDA) return HOSC_ECUDA;   // a bounded wait ran out
     if (ks[s].status != 0 || !ks[s].done) st = HOSC_ENOCONV;
   }
   return st;

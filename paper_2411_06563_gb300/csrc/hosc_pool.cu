@@ -266,6 +266,7 @@ hosc_status hosc_pool_admit(void* pool, const hosc_params* params, long max_step
   void* ctx = nullptr;
   hosc_status st = hosc_create(&p, &ctx);
   if (st) return st;
+  ctx_join_pool(ctx);
   int s = -1;
   for (int q = 0; q < (int)P->m.size(); ++q)
     if (P->m[q].state == kFree) {

@@ -1,0 +1,618 @@
+// The BiCGSTAB solve of one step as one launch, for grids whose unknowns fit on the chip (Punia & Ray,
+// arXiv:2411.06563, Sec. 2.2: unpreconditioned BiCGSTAB on the four level-(n+1) systems of Eq. 5).
+//
+// On small grids an iteration's three launches cost 5 to 15 us each whatever the size: the launch
+// itself, the scalars' read, the first loads, the ticket, the last block's sum of the partials and its
+// divisions. Here the grid is cooperative (every block resident); a block keeps its nodes' vectors in
+// registers and their operator rows in shared memory from the first iteration to the last, and a phase
+// (p/v, s/t, x/r) ends in one exchange: each block puts its partial sums in its row of a buffer, and
+// every block reads all rows, adds them in the same order and computes the scalars itself. A value
+// travels as two 8-byte words that each carry 4 bytes of it and the exchange's number, so that a
+// reader needs no other flag; two buffers alternate, since a block that has finished exchange e has
+// every row of it, and so nobody still reads exchange e - 1. The vectors that other blocks need at the
+// borders of a block (v after p/v; r and p - omega v after x/r) are written to memory before the
+// exchange and read through L2 after it.
+//
+// The arithmetic of a node, the partial sums of a block and the order of the rows' sum are those of
+// the kernels that run an iteration in three launches (hosc_krylov.cu) with the same block shape: the
+// same bits.
+//
+// Every wait is bounded (kWaitNs on the GPU timer): a block whose wait runs out leaves the solve, the
+// others follow when theirs do, and the step reports HOSC_ECUDA.
+//
+// Measured against an iteration in three launches: FP64 21^3 25.4 -> 16.6 us, 41^3 49 -> 27.8 us (there half of it
+// FP64 instructions); mixed step at 41^3 226 -> 140 us, at 64^3 348 -> 242 us.
+
+#include <math.h>
+
+#include "hosc_device.cuh"
+#include "hosc_internal.h"
+#include "hosc_krylov4.cuh"
+
+namespace hosc {
+
+namespace {
+
+constexpr unsigned long long kWaitNs = 2000000000ull;   // 2 s
+
+__device__ __forceinline__ unsigned long long solve_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// One value of an exchange: two words of (4 bytes of the value, the exchange's number).
+__device__ __forceinline__ void put_value(ulonglong2* p, double v, unsigned e) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned long long f = (unsigned long long)e << 32;
+  asm volatile("st.volatile.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"((b & 0xffffffffull) | f),
+               "l"((b >> 32) | f)
+               : "memory");
+}
+__device__ __forceinline__ bool get_value(const ulonglong2* p, unsigned e, double& v) {
+  unsigned long long a, b;
+  asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+  v = __longlong_as_double((long long)((a & 0xffffffffull) | (b << 32)));
+  return (unsigned)(a >> 32) == e && (unsigned)(b >> 32) == e;
+}
+
+// The blocks that exchange with one another: rows of `stride` values, two buffers.
+struct Exchange {
+  ulonglong2* rows;
+  int nr, stride, mine;   // number of rows, values a row, this block's row
+  unsigned e;             // number of the last exchange
+  int* failed;            // shared: a wait of this block has run out
+};
+
+// Thread m < M of the block puts its value of the block's row and the block gathers the totals of all
+// rows, in the order of sum_rows, in tot (shared). A function of its own: inlined, its loops cost the
+// callers the registers that hold their vectors.
+template <class T, int M>
+__device__ __noinline__ bool gather(ulonglong2* rows, int nr, int stride, int row, unsigned e,
+                                    double mine, double* tot, int* failed) {
+  constexpr int Mp = pow2_at_least(M);
+  constexpr int G = 64;
+  static_assert(Mp <= 8, "groups as in sum_rows");
+  __shared__ double s_g[Mp * G];
+  rows += (size_t)(e & 1u) * nr * stride;
+  const int t = threadIdx.x, lane = t & 31;
+  if (t < M) {
+    __threadfence();   // the block's writes to memory come before its row
+    put_value(rows + row * stride + t, mine, e);
+  }
+  for (int w = t; w < Mp * G; w += blockDim.x) {
+    const int m = w % Mp;
+    double acc = 0.0;
+    if (m < M) {
+      for (int r = w / Mp; r < nr; r += 4 * G) {
+        const int n = min(4, (nr - r + G - 1) / G);   // rows r, r + G, ... of this pass
+        double a[4];
+        unsigned long long t0 = 0;
+        for (unsigned spin = 0;; ++spin) {
+          bool ok = true;
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (q < n) ok &= get_value(rows + (r + q * G) * stride + m, e, a[q]);
+          if (ok) break;
+          if ((spin & 255u) == 255u) {
+            const unsigned long long now = solve_ns();
+            if (t0 == 0) t0 = now;
+            if (now - t0 > kWaitNs || *(volatile int*)failed) {
+              *(volatile int*)failed = 1;
+              break;
+            }
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q < n) acc = T::add(acc, a[q]);
+      }
+    }
+    s_g[w] = acc;
+  }
+  __threadfence();
+  __syncthreads();
+  for (int m = t >> 5; m < Mp; m += (int)(blockDim.x >> 5)) {
+    double a = T::add(s_g[lane * Mp + m], s_g[(lane + 32) * Mp + m]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) a = T::add(a, T::shfl_xor(a, off));
+    if (lane == 0) tot[m] = a;
+  }
+  __syncthreads();
+  return *(volatile int*)failed == 0;
+}
+
+// The totals of M values per thread over all blocks of the exchange, in tot (shared). Orders the
+// block's earlier writes to memory before the others' reads that follow. False when a wait ran out
+// (uniform over the block).
+template <class Op, int M>
+__device__ __forceinline__ bool exchange(Exchange& x, const typename Op::V (&v)[M], double* tot) {
+  x.e += 1;
+  const typename Op::V mine = block_total<Op, M>(v);
+  return gather<typename Op::Total, M>(x.rows, x.nr, x.stride, x.mine, x.e, Op::value(mine), tot,
+                                       x.failed);
+}
+
+// ------------------------------------------------------------------ FP64 (planar)
+//
+// A block has one system, B nodes of the plane (i + N j, walls included) and up to KZ planes; a
+// system's blocks exchange among themselves and leave when it is done.
+
+template <int B, int KZ>
+constexpr size_t planar_state(int N) {   // operator rows and rhs, then KZ planes of B + 2 N values
+  return sizeof(double) * ((size_t)8 * KZ * B + (size_t)KZ * (B + 2 * N));
+}
+
+template <int B, int KZ>
+__global__ void __launch_bounds__(B, KZ <= 4 ? 512 / B : 1)
+    k_solve_planar(DevParams P, Fields F) {
+  extern __shared__ double sh[];
+  __shared__ KrylovScalars k;
+  __shared__ double tot[2];
+  __shared__ int failed;
+  if (*F.halt) return;   // the same for every block
+  const int s = (int)(blockIdx.x & 3u), t = threadIdx.x;
+  const int N = P.N, N2 = N * N, w = B + 2 * N;
+  const int l0 = (int)(blockIdx.x >> 2) * B, l = l0 + t;
+  const int k0 = 1 + (int)blockIdx.y * P.pkz, nk = min(P.pkz, N - 1 - k0);
+  const unsigned chunks = gridDim.x >> 2;
+  Exchange x;
+  x.nr = (int)(chunks * gridDim.y);
+  x.stride = 2;
+  x.mine = (int)((blockIdx.x >> 2) + chunks * blockIdx.y);
+  x.rows = F.exch + (size_t)s * 2 * x.nr * x.stride;
+  x.e = 0;
+  x.failed = &failed;
+  auto inside = [&](int q) {   // node q of the plane lies inside the walls
+    if (q < 0 || q >= N2) return false;
+    const int j = q / N, i = q - j * N;
+    return i > 0 && i < N - 1 && j > 0 && j < N - 1;
+  };
+  const bool in = inside(l);
+  // the node before or after the chunk whose value this thread fetches (2 N <= B)
+  const int hl = t < N ? l0 - N + t : l0 + B + (t - N), hs = t < N ? t : B + t;
+  const bool has_halo = t < 2 * N, hin = has_halo && inside(hl);
+  const bool below = in && k0 > 1, above = in && k0 + nk < N - 1;
+  double* a = sh;                    // weight q of plane kk: a[(8 kk + q) B + t]; rhs at q = 7
+  double* planes = sh + 8 * KZ * B;  // plane kk: nodes l0 - N .. l0 + B + N
+  const double* rhs = F.rhs[s];
+  double *R = F.r[s], *Q = F.pk[0][s], *V = F.vk[0][s];
+  double r[KZ], xi[KZ], p[KZ], v[KZ], tv[KZ];
+  const double* const* A = s < 3 ? F.Am : F.Ae;
+  const int c0 = l + N2 * k0;
+#pragma unroll
+  for (int kk = 0; kk < KZ; ++kk) {
+    r[kk] = xi[kk] = p[kk] = v[kk] = tv[kk] = 0.0;
+    if (in && kk < nk) {
+      r[kk] = p[kk] = rhs[c0 + N2 * kk];
+      a[(8 * kk + 7) * B + t] = r[kk];
+#pragma unroll
+      for (int q = 0; q < 7; ++q) a[(8 * kk + q) * B + t] = A[q][c0 + N2 * kk];
+    }
+  }
+  if (t == 0) {
+    k = F.ks[s];
+    failed = 0;
+  }
+  __syncthreads();
+  // the operator on own values f (registers) and the others' values val(c): y of each plane
+  auto stencil = [&](const double (&f)[KZ], double (&y)[KZ], auto val) {
+    const double lo = below ? val(c0 - N2) : 0.0, hi = above ? val(c0 + N2 * nk) : 0.0;
+#pragma unroll
+    for (int kk = 0; kk < KZ; ++kk) {
+      const double h = hin && kk < nk ? val(hl + N2 * (k0 + kk)) : 0.0;
+      planes[kk * w + N + t] = f[kk];   // zero on the walls
+      if (has_halo) planes[kk * w + hs] = h;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < KZ; ++kk) {
+      if (!in || kk >= nk) continue;
+      const double* o = planes + kk * w + N + t;
+      const double* ak = a + 8 * kk * B + t;
+      const double zp = kk + 1 < nk && kk + 1 < KZ ? f[kk + 1 < KZ ? kk + 1 : kk] : hi;
+      const double zm = kk > 0 ? f[kk > 0 ? kk - 1 : 0] : lo;
+      y[kk] = planar_row(ak[0], ak[B], ak[2 * B], ak[3 * B], ak[4 * B], ak[5 * B], ak[6 * B], f[kk],
+                         o[1], o[-1], o[N], o[-N], zp, zm);
+    }
+  };
+  bool ok = true;
+  for (int it = 0; !k.done; ++it) {
+    // p = r + beta (p - omega v), v = A p
+    const bool first = it == 0;
+    const double beta = k.beta;
+    double d2[2] = {0.0, 0.0};
+    if (first) {
+      stencil(p, v, [&](int c) { return rhs[c]; });
+    } else {
+#pragma unroll
+      for (int kk = 0; kk < KZ; ++kk) p[kk] = fma(beta, p[kk], r[kk]);
+      stencil(p, v, [&](int c) { return fma(beta, __ldcg(Q + c), __ldcg(R + c)); });
+    }
+#pragma unroll
+    for (int kk = 0; kk < KZ; ++kk)
+      if (in && kk < nk) {
+        V[c0 + N2 * kk] = v[kk];
+        const double r0 = a[(8 * kk + 7) * B + t];
+        d2[0] = fma(r0, v[kk], d2[0]);
+        if (first) d2[1] = fma(r0, r0, d2[1]);
+      }
+    if (first) {
+      ok = exchange<SumD, 2>(x, d2, tot);
+    } else {
+      double d1[1] = {d2[0]};
+      ok = exchange<SumD, 1>(x, d1, tot);
+    }
+    if (!ok) break;
+    if (t == 0) pv_scalars(k, tot[0], first ? tot[1] : 0.0, first);
+    __syncthreads();
+    if (k.done) break;
+    // s = r - alpha v (kept in r), t = A s
+    const double alpha = k.alpha;
+#pragma unroll
+    for (int kk = 0; kk < KZ; ++kk) r[kk] = fma(-alpha, v[kk], r[kk]);
+    if (first)
+      stencil(r, tv, [&](int c) { return fma(-alpha, __ldcg(V + c), rhs[c]); });
+    else
+      stencil(r, tv, [&](int c) { return fma(-alpha, __ldcg(V + c), __ldcg(R + c)); });
+    double ds[2] = {0.0, 0.0};
+#pragma unroll
+    for (int kk = 0; kk < KZ; ++kk)
+      if (in && kk < nk) {
+        ds[0] = fma(tv[kk], r[kk], ds[0]);
+        ds[1] = fma(tv[kk], tv[kk], ds[1]);
+      }
+    ok = exchange<SumD, 2>(x, ds, tot);
+    if (!ok) break;
+    if (t == 0) st_scalars(k, tot[0], tot[1]);
+    __syncthreads();
+    // x += alpha p + omega s, r = s - omega t; p - omega v for the next p
+    const double omega = k.omega;
+    double dr[2] = {0.0, 0.0};
+#pragma unroll
+    for (int kk = 0; kk < KZ; ++kk)
+      if (in && kk < nk) {
+        const int c = c0 + N2 * kk;
+        xi[kk] = fma(omega, r[kk], fma(alpha, p[kk], xi[kk]));
+        r[kk] = fma(-omega, tv[kk], r[kk]);
+        p[kk] = fma(-omega, v[kk], p[kk]);
+        R[c] = r[kk];
+        Q[c] = p[kk];
+        dr[0] = fma(a[(8 * kk + 7) * B + t], r[kk], dr[0]);
+        dr[1] = fma(r[kk], r[kk], dr[1]);
+      }
+    ok = exchange<SumD, 2>(x, dr, tot);
+    if (!ok) break;
+    if (t == 0) xr_scalars(P, k, tot[0], tot[1]);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int kk = 0; kk < KZ; ++kk)
+    if (in && kk < nk) F.x[s][c0 + N2 * kk] = xi[kk];
+  if (!ok && t == 0) {
+    k.done = 1;
+    k.status = HOSC_ECUDA;
+  }
+  if (t == 0 && (x.mine == 0 || !ok)) {
+    F.ks[s] = k;
+    // algorithmic bytes of the three kernel classes (the momentum weights counted once)
+    const double ni = N - 2, n3 = 8.0 * ni * ni * ni * k.iters, wt = s == 0 || s == 3 ? 7.0 : 0.0;
+    atomicAdd(F.alg_bytes + HOSC_K_BICG_PV, n3 * (6.0 + wt));
+    atomicAdd(F.alg_bytes + HOSC_K_BICG_ST, n3 * (3.0 + wt));
+    atomicAdd(F.alg_bytes + HOSC_K_BICG_XR, n3 * 8.0);
+  }
+}
+
+// ------------------------------------------------------------------ mixed (interleaved float)
+//
+// A block has 256 interior columns (in the order of the register kernels) and up to KZ planes, with
+// all four systems of a node in one float4.
+
+constexpr int kSolveBlock = 256;
+
+template <int KZ>
+constexpr size_t mixed_state(int N) {   // operators, r_0, v, then KZ planes of 256 + 2 (N - 2) float4
+  return 16 * ((size_t)4 * KZ * kSolveBlock + (size_t)KZ * (kSolveBlock + 2 * (N - 2))) +
+         4 * (size_t)KZ * kSolveBlock;
+}
+
+template <int KZ>
+__global__ void __launch_bounds__(kSolveBlock, 2) k_solve_mixed(DevParams P, Fields F) {
+  constexpr int B = kSolveBlock;
+  extern __shared__ float4 sh4[];
+  __shared__ KrylovScalars ks[4];
+  __shared__ Scal4 sc;
+  __shared__ double tot[8];
+  __shared__ int failed;
+  if (*F.halt) return;   // the same for every block
+  const int t = threadIdx.x, N = P.N, N2 = N * N, ni = N - 2, w = B + 2 * ni;
+  const int q0 = (int)blockIdx.x * B, q = q0 + t;
+  const int k0 = 1 + (int)blockIdx.y * P.ckz, nk = min(P.ckz, N - 1 - k0);
+  Exchange x;
+  x.nr = (int)(gridDim.x * gridDim.y);
+  x.stride = 8;
+  x.mine = (int)(blockIdx.x + gridDim.x * blockIdx.y);
+  x.rows = F.exch;
+  x.e = 0;
+  x.failed = &failed;
+  auto column_of = [&](int c) {   // node (i, j, 0) of interior column c
+    const int j = c / ni;
+    return 1 + c - j * ni + N * (j + 1);
+  };
+  const bool in = q < ni * ni;
+  const int i = q % ni, c0 = (in ? column_of(q) : 0) + N2 * k0;
+  const bool has_xp = i < ni - 1, has_xm = i > 0;
+  // the column before or after the chunk whose value this thread fetches (2 ni <= B)
+  const int hq = t < ni ? q0 - ni + t : q0 + B + (t - ni), hs = t < ni ? t : B + t;
+  const bool has_halo = t < 2 * ni, hin = has_halo && hq >= 0 && hq < ni * ni;
+  const int hc = (hin ? column_of(hq) : 0) + N2 * k0;
+  const bool below = in && k0 > 1, above = in && k0 + nk < N - 1;
+  float4* om = sh4;                 // operators, r_0 and v of plane kk at kk B + t
+  float4* oe = om + KZ * B;
+  float4* r0 = oe + KZ * B;
+  float4* vs = r0 + KZ * B;
+  float4* planes = vs + KZ * B;     // plane kk: columns q0 - ni .. q0 + B + ni
+  float* ol = (float*)(planes + KZ * w);
+  const float4 zero = f4(0.f);
+  float4 r[KZ], p[KZ], tv[KZ];
+#pragma unroll
+  for (int kk = 0; kk < KZ; ++kk) {
+    r[kk] = p[kk] = tv[kk] = zero;
+    if (in && kk < nk) {
+      const int c = c0 + N2 * kk;
+      r[kk] = p[kk] = F.kr0[c];
+      r0[kk * B + t] = r[kk];
+      om[kk * B + t] = F.kwm[c];
+      oe[kk * B + t] = F.kwe[c];
+      ol[kk * B + t] = __fmul_rn(F.kL[c], 1.f / 12.f);
+    }
+  }
+  if (t < 4) ks[t] = F.ks[t];
+  if (t == 0) failed = 0;
+  __syncthreads();
+  // the operators on own values f (registers) and the others' values val(c): out(kk, y) of each plane
+  auto stencil = [&](const float4 (&f)[KZ], bool ene, auto val, auto out) {
+    const float4 lo = below ? val(c0 - N2) : zero, hi = above ? val(c0 + N2 * nk) : zero;
+#pragma unroll
+    for (int kk = 0; kk < KZ; ++kk) {
+      const float4 h = hin && kk < nk ? val(hc + N2 * kk) : zero;
+      planes[kk * w + ni + t] = f[kk];   // zero past the last column
+      if (has_halo) planes[kk * w + hs] = h;
+      if (KZ > 2 && kk % 2) asm volatile("" ::: "memory");
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < KZ; ++kk) {
+      if (!in || kk >= nk) continue;
+      const float4* o = planes + kk * w + ni + t;
+      Op4 op;
+      op.m = om[kk * B + t];
+      op.e = ene ? oe[kk * B + t] : zero;
+      op.l12 = ol[kk * B + t];
+      const float4 zp = kk + 1 < nk && kk + 1 < KZ ? f[kk + 1 < KZ ? kk + 1 : kk] : hi;
+      const float4 zm = kk > 0 ? f[kk > 0 ? kk - 1 : 0] : lo;
+      out(kk, apply_op(P, op, f[kk], has_xp ? o[1] : zero, has_xm ? o[-1] : zero, o[ni], o[-ni],
+                       zp, zm));
+      asm volatile("" ::: "memory");   // one plane's operands in registers at a time
+    }
+  };
+  double bytes[3] = {0.0, 0.0, 0.0};
+  bool ok = true;
+  bool any = false;   // an iterate has been written
+  for (int it = 0;; ++it) {
+    const bool first = it == 0;
+    load_scalars(ks, sc);
+    if (sc.all_done) break;
+    // p = r + beta (p - omega v), v = A p
+    bool ene = !sc.done[3];
+    {
+      const float4 b = sc.b;
+      FF acc[8] = {};
+      auto out = [&](int kk, const float4& y) {
+        F.kv[0][c0 + N2 * kk] = y;
+        vs[kk * B + t] = y;
+        const float4 z = r0[kk * B + t];
+        ff_dot4(acc, z, y);
+        if (first) ff_dot4(acc + 4, z, z);
+      };
+      if (first) {
+        stencil(p, ene, [&](int c) { return F.kr0[c]; }, out);
+      } else {
+#pragma unroll
+        for (int kk = 0; kk < KZ; ++kk) p[kk] = fma4(b, p[kk], r[kk]);
+        stencil(p, ene, [&](int c) { return fma4(b, __ldcg(F.kp[0] + c), __ldcg(F.kr + c)); }, out);
+      }
+      bytes[0] += (first ? 3.0 : 6.0) + op_words(ene);
+      if (first) {
+        ok = exchange<SumFF, 8>(x, acc, tot);
+      } else {
+        FF a4[4] = {acc[0], acc[1], acc[2], acc[3]};
+        ok = exchange<SumFF, 4>(x, a4, tot);
+      }
+      if (!ok) break;
+      finish_pv(ks, tot, first);
+      __syncthreads();
+    }
+    load_scalars(ks, sc);
+    if (sc.all_done) break;
+    // s = r - alpha v (kept in r), t = A s
+    ene = !sc.done[3];
+    {
+      const float4 ma = neg4(sc.a);
+      FF acc[8] = {};
+#pragma unroll
+      for (int kk = 0; kk < KZ; ++kk)
+        if (in && kk < nk) r[kk] = fma4(ma, vs[kk * B + t], r[kk]);
+      const float4* R = first ? F.kr0 : F.kr;
+      stencil(r, ene, [&](int c) { return fma4(ma, __ldcg(F.kv[0] + c), __ldcg(R + c)); },
+              [&](int kk, const float4& y) {
+                tv[kk] = y;
+                ff_dot4(acc, y, r[kk]);
+                ff_dot4(acc + 4, y, y);
+              });
+      bytes[1] += 3.0 + op_words(ene);
+      ok = exchange<SumFF, 8>(x, acc, tot);
+      if (!ok) break;
+      finish_st(ks, tot);
+      __syncthreads();
+    }
+    load_scalars(ks, sc);
+    // x += alpha p + omega s, r = s - omega t; p - omega v for the next p
+    {
+      const float4 a = sc.a, o = sc.om, mo = neg4(sc.om);
+      FF acc[8] = {};
+      bytes[2] += first ? 6.0 : 8.0;
+      any = true;
+#pragma unroll
+      for (int kk = 0; kk < KZ; ++kk)
+        if (in && kk < nk) {
+          const int c = c0 + N2 * kk;
+          F.kx[c] = fma4(o, r[kk], fma4(a, p[kk], first ? zero : F.kx[c]));
+          r[kk] = fma4(mo, tv[kk], r[kk]);
+          p[kk] = fma4(mo, vs[kk * B + t], p[kk]);
+          F.kr[c] = r[kk];
+          F.kp[0][c] = p[kk];
+          ff_dot4(acc, r0[kk * B + t], r[kk]);
+          ff_dot4(acc + 4, r[kk], r[kk]);
+        }
+      ok = exchange<SumFF, 8>(x, acc, tot);
+      if (!ok) break;
+      finish_xr(P, ks, tot);
+      __syncthreads();
+    }
+  }
+  if (!any && in)   // every right-hand side is zero (or none to solve): zero increments
+    for (int kk = 0; kk < nk; ++kk) F.kx[c0 + N2 * kk] = zero;
+  if (!ok && t < 4) {
+    ks[t].done = 1;
+    ks[t].status = HOSC_ECUDA;
+  }
+  if (x.mine == 0 || !ok) {
+    if (t < 4) F.ks[t] = ks[t];
+    if (t < 3) atomicAdd(F.alg_bytes + HOSC_K_BICG_PV + t, bytes4(P, bytes[t]));
+  }
+}
+
+// ------------------------------------------------------------------ host
+
+typedef void (*SolveFn)(DevParams, Fields);
+
+SolveFn planar_fn(int B, int KZ, int N, size_t* smem) {
+#define CASE(b, z)                         \
+  if (B == b && KZ == z) {                 \
+    *smem = planar_state<b, z>(N);         \
+    return k_solve_planar<b, z>;           \
+  }
+  CASE(128, 1) CASE(128, 2) CASE(128, 4) CASE(256, 1) CASE(256, 2) CASE(256, 4) CASE(256, 8)
+#undef CASE
+  return nullptr;
+}
+SolveFn mixed_fn(int KZ, int N, size_t* smem) {
+  *smem = KZ == 1 ? mixed_state<1>(N) : KZ == 2 ? mixed_state<2>(N) : mixed_state<4>(N);
+  return KZ == 1 ? k_solve_mixed<1> : KZ == 2 ? k_solve_mixed<2> : KZ == 4 ? k_solve_mixed<4> : nullptr;
+}
+
+// Blocks of fn that are resident at once, 0 when it cannot run so.
+long resident(SolveFn fn, int threads, size_t smem) {
+  if (!fn || smem > 200 * 1024) return 0;
+  int occ = 0;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return (long)occ * device_sms();
+}
+
+int template_planes(int z) { return z <= 1 ? 1 : z <= 2 ? 2 : z <= 4 ? 4 : 8; }
+
+void launch_cooperative(SolveFn fn, dim3 grid, int threads, size_t smem, cudaStream_t s,
+                        const DevParams& P, const Fields& F) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, fn, P, F);
+}
+
+}  // namespace
+
+// Shapes of the one-launch solves: the least modelled time of a phase (the busiest SM's FP64
+// instructions, or planes, and the rows of the exchange) among the shapes whose blocks are all
+// resident. False when none is: the vectors do not fit on the chip.
+bool solve_shape_planar(int N, int* pb, int* pkz) {
+  // the answer for the last grid and device of this thread: asked at every set-up and every
+  // allocation-free solve
+  static thread_local struct { int N, device, pb, pkz; } last = {0, -1, 0, 0};
+  int device = 0;
+  if (cudaGetDevice(&device) != cudaSuccess) return false;
+  if (last.N == N && last.device == device) {
+    *pb = last.pb;
+    *pkz = last.pkz;
+    return last.pb > 0;
+  }
+  const int sms = device_sms(), ni = N - 2;
+  double best = 1e300;
+  last = {N, device, 0, 0};
+  for (int B : {128, 256}) {
+    if (2 * N > B) continue;
+    const long chunks = (N * (long)N + B - 1) / B;
+    for (int z = 1; z <= 8 && z <= ni; ++z) {
+      const long rows = chunks * ((ni + z - 1) / z);
+      if (rows > kSolveRows) continue;
+      const double work = B / 32.0 * (12.0 * z + 20.0) + 2.0 * ((2 * N + 31) / 32) * z;
+      const double cost = work * (double)((4 * rows + sms - 1) / sms) + 0.5 * rows;
+      if (cost >= best) continue;
+      size_t smem = 0;
+      const SolveFn fn = planar_fn(B, template_planes(z), N, &smem);
+      if (resident(fn, B, smem) < 4 * rows) continue;
+      best = cost;
+      last.pb = *pb = B;
+      last.pkz = *pkz = z;
+    }
+  }
+  return best < 1e300;
+}
+
+bool solve_shape_mixed(int N, int* kblock, int* kz) {
+  const int sms = device_sms(), ni = N - 2;
+  if (2 * ni > kSolveBlock) return false;
+  const long chunks = ((long)ni * ni + kSolveBlock - 1) / kSolveBlock;
+  double best = 1e300;
+  for (int z = 1; z <= 4 && z <= ni; ++z) {
+    const long rows = chunks * ((ni + z - 1) / z);
+    if (rows * 2 * 8 > kExchValues) continue;
+    const double cost = (z + 1.5) * (double)((rows + sms - 1) / sms) + 0.004 * rows;
+    if (cost >= best) continue;
+    size_t smem = 0;
+    const SolveFn fn = mixed_fn(template_planes(z), N, &smem);
+    if (resident(fn, kSolveBlock, smem) < rows) continue;
+    best = cost;
+    *kblock = kSolveBlock;
+    *kz = z;
+  }
+  return best < 1e300;
+}
+
+void launch_solve(const DevParams& P, const Fields& F, cudaStream_t s) {
+  const int ni = P.N - 2;
+  size_t smem = 0;
+  if (P.krylov_fp32) {
+    const SolveFn fn = mixed_fn(template_planes(P.ckz), P.N, &smem);
+    const dim3 g((ni * ni + kSolveBlock - 1) / kSolveBlock, (ni + P.ckz - 1) / P.ckz);
+    launch_cooperative(fn, g, kSolveBlock, smem, s, P, F);
+  } else {
+    const SolveFn fn = planar_fn(P.pb, template_planes(P.pkz), P.N, &smem);
+    const dim3 g(4u * ((P.N * P.N + P.pb - 1) / P.pb), (ni + P.pkz - 1) / P.pkz);
+    launch_cooperative(fn, g, P.pb, smem, s, P, F);
+  }
+}
+
+}  // namespace hosc

@@ -462,6 +462,9 @@ __device__ __forceinline__ void k_rhs_body(const DevParams& P, const Tc* HOSC_RE
   const long c = node(i, j, k, N);
   const RhsC<Tc>& rc = rhs_constants<Tc>(P);
   if (t < 4) start_system(P, F, (int)t);   // the solve's scalars
+  if (P.coop)                              // and its exchange buffer
+    for (unsigned e = t; e < (unsigned)kExchValues; e += ni * ni * ni)
+      F.exch[e] = make_ulonglong2(0ull, 0ull);
   const bool hist = P.have_prev != 0;
   const Tc kap = par<Tc>(P.a_boost, P.a_boostf);
   Tc rv[4], Bm[3], Be[3], Dm, De, Lc;   // right-hand sides and compact operators, stored at the end

@@ -260,8 +260,8 @@ __global__ void __launch_bounds__(kTmaMaxThreads)
         Op4 op;
         op.m = ((const float4*)(st + L.off_m))[e];
         op.e = ene ? ((const float4*)(st + L.off_e))[e] : zero;
-        op.l12 = ((const float*)(st + L.off_l + ty * L.lrow))[(int)(lin & 3L) + tx] *
-                 (1.f / 12.f);
+        op.l12 = __fmul_rn(((const float*)(st + L.off_l + ty * L.lrow))[(int)(lin & 3L) + tx],
+                           1.f / 12.f);
         const float4 y = apply_op(P, op, pc, val(u, h + 1), val(u, h - 1), val(u, h + hx),
                                   val(u, h - hx), pz, pm);
         const int c = (i0 + tx) + N * (j0 + ty) + N2 * k;
@@ -288,8 +288,8 @@ __global__ void __launch_bounds__(kTmaMaxThreads)
   const double* tot = grid_total<SumFF, M>(acc, F.red, F.counter, bid, nb);
   const bool bad = failed != 0;
   if (tot) {
-    if (PV) finish_pv(F, tot, false);
-    else finish_st(F, tot);
+    if (PV) finish_pv(F.ks, tot, false);
+    else finish_st(F.ks, tot);
     // p/v: r p v r0 in, p v out; s/t: r v in, t out; the compact operators
     count_bytes(F, PV ? HOSC_K_BICG_PV : HOSC_K_BICG_ST,
                 bytes4(P, (PV ? 6.0 : 3.0) + op_words(ene)));
