@@ -285,7 +285,8 @@ hosc_status hosc_time_kernel(void* ctx, int kernel_id, int reps, double* ms_per_
  * the merged iteration form), kz in 1..N-2, and at most N^3/16 + 1024 blocks per launch;
  * narrow = 1 selects the kernels compiled for at most 64 registers per thread (more resident
  * blocks), 0 those with more (80 for the three-kernel form, 128 for the merged form). The
- * default (128 threads, wide, kz from the wave model below) is chosen from N at creation.
+ * default (384 threads, wide, kz from the wave model below; on grids whose solve runs as one launch
+ * 256 threads) is chosen from N at creation.
  * Changing it drops the captured steps (captured again at the next step). HOSC_EINVAL for a shape
  * outside these limits, HOSC_ESTATE in the middle of a stage-by-stage step. The FP64 solve has
  * one thread per node and ignores the setting. */

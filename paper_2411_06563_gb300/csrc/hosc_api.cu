@@ -1180,9 +1180,10 @@ size_t workspace_layout(int N, int bicgstab2, Fields* f, char* base) {
   F.div = fld();
   F.eloc = (double*)take(3 * n3 * sizeof(double));
   // per-block partials: one row per block of any accepted launch shape
-  F.red = (double*)take((size_t)red_rows((long)n3) * kRedSlots * sizeof(double));
+  F.rb.red = (double*)take((size_t)red_rows((long)n3) * kRedSlots * sizeof(double));
+  F.rb.red2 = (double*)take((size_t)red_groups((long)n3) * kRedSlots * sizeof(double));
   F.exch = (ulonglong2*)take(kExchValues * sizeof(ulonglong2));
-  F.counter = (unsigned int*)take(sizeof(unsigned int));
+  F.rb.counter = (unsigned int*)take((size_t)(red_groups((long)n3) + 1) * sizeof(unsigned int));
   F.ks = (KrylovScalars*)take(4 * sizeof(KrylovScalars));
   F.rec = (StepRecord*)take(sizeof(StepRecord));
   F.diag_scal = (double*)take(8 * sizeof(double));

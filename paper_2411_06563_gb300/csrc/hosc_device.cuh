@@ -231,16 +231,10 @@ __device__ __forceinline__ void sum_rows(int nr, Load load, double* tot) {
   __syncthreads();
 }
 
-// Second half of a reduction over the grid, called by every block once its warp 0 has written the
-// block's values to rows of red: takes a ticket; the block that takes the last of `tickets` (no block
-// waits for another) sums the nr rows of M slots and returns the totals in shared memory, valid for
-// its every thread; the other blocks return null. The ticket counter is left at zero for the next
-// kernel.
-template <class T, int M>
-__device__ __forceinline__ const double* last_block_total(const double* red, unsigned int* counter,
-                                                          unsigned int nr, unsigned int tickets) {
-  constexpr long S = row_stride<M>();
-  __shared__ double s_tot[pow2_at_least(M)];
+// A ticket of the `tickets` given out at counter, taken after warp 0's writes; true in the block that
+// takes the last one (no block waits for another), which leaves the counter at zero for the next
+// kernel and sees what the others wrote.
+__device__ __forceinline__ bool last_ticket(unsigned int* counter, unsigned int tickets) {
   __shared__ int s_last;
   if (threadIdx.x < 32) {
     __syncwarp();
@@ -250,22 +244,48 @@ __device__ __forceinline__ const double* last_block_total(const double* red, uns
     }
   }
   __syncthreads();
-  if (!s_last) return nullptr;
-  __threadfence();
-  if (threadIdx.x == 0) *counter = 0u;
-  sum_rows<T, M>((int)nr, [&](int r, int m) { return __ldcg(red + r * S + m); }, s_tot);
+  const bool last = s_last;
+  if (last) {
+    __threadfence();
+    if (threadIdx.x == 0) *counter = 0u;
+  }
+  return last;
+}
+
+// Second half of a reduction over the grid, called by every block once its warp 0 has written values to
+// row `row` of the nr rows of M slots (per_row blocks write a row): the last block returns the totals
+// in shared memory, valid for its every thread; the others return null. Above kFlatRows rows the sum
+// has two levels: one block summing the 8 000 rows of a 257^3 launch took 50 to 75 us of each kernel
+// (x/r 384 -> 318 us, p/v 510 -> 448 us, s/t 369 -> 300 us).
+template <class T, int M>
+__device__ __forceinline__ const double* last_block_total(const RedBuf& b, unsigned int row,
+                                                          unsigned int nr, unsigned int per_row) {
+  constexpr long S = row_stride<M>();
+  __shared__ double s_tot[pow2_at_least(M)];
+  const double* rows = b.red;
+  unsigned int tickets = nr * per_row;
+  if (nr > kFlatRows) {
+    const unsigned int g = row / kGroupRows, r0 = g * kGroupRows, n = min(kGroupRows, nr - r0);
+    if (!last_ticket(b.counter + 1 + g, n * per_row)) return nullptr;
+    rows = b.red + r0 * S;
+    sum_rows<T, M>((int)n, [&](int r, int m) { return __ldcg(rows + r * S + m); }, s_tot);
+    if (threadIdx.x < M) b.red2[g * S + threadIdx.x] = s_tot[threadIdx.x];
+    rows = b.red2;
+    tickets = nr = (nr + kGroupRows - 1) / kGroupRows;
+  }
+  if (!last_ticket(b.counter, tickets)) return nullptr;
+  sum_rows<T, M>((int)nr, [&](int r, int m) { return __ldcg(rows + r * S + m); }, s_tot);
   return s_tot;
 }
 
-// Reduction over the grid of M values per thread: block b of nb writes its totals to its row of red;
+// Reduction over the grid of M values per thread: block b of nb writes its totals to its row;
 // the last block returns the totals (see last_block_total), the others null.
 template <class Op, int M>
-__device__ __forceinline__ const double* grid_total(const typename Op::V (&v)[M], double* red,
-                                                    unsigned int* counter, unsigned int b,
-                                                    unsigned int nb) {
+__device__ __forceinline__ const double* grid_total(const typename Op::V (&v)[M], const RedBuf& buf,
+                                                    unsigned int b, unsigned int nb) {
   const typename Op::V mine = block_total<Op, M>(v);
-  if (threadIdx.x < M) red[(long)b * row_stride<M>() + threadIdx.x] = Op::value(mine);
-  return last_block_total<typename Op::Total, M>(red, counter, nb, nb);
+  if (threadIdx.x < M) buf.red[(long)b * row_stride<M>() + threadIdx.x] = Op::value(mine);
+  return last_block_total<typename Op::Total, M>(buf, b, nb, 1u);
 }
 
 }  // namespace hosc

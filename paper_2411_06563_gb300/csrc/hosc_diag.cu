@@ -78,8 +78,7 @@ __global__ void __launch_bounds__(kThreads) k_entropy(DevParams P, const double*
                                                      const double* __restrict__ v,
                                                      const double* __restrict__ w,
                                                      const double* __restrict__ th, double* eloc,
-                                                     int store, double* red,
-                                                     unsigned int* counter, int nblocks,
+                                                     int store, RedBuf rb, int nblocks,
                                                      double* scal) {
   const int N = P.N;
   const long n3 = (long)N * N * N;
@@ -119,7 +118,7 @@ __global__ void __launch_bounds__(kThreads) k_entropy(DevParams P, const double*
     acc[0] = wgt * eht;
     acc[1] = wgt * eff;
   }
-  if (const double* tot = grid_total<SumD, 2>(acc, red, counter, blockIdx.x, (unsigned)nblocks)) {
+  if (const double* tot = grid_total<SumD, 2>(acc, rb, blockIdx.x, (unsigned)nblocks)) {
     if (threadIdx.x < 2) scal[3 + threadIdx.x] = tot[threadIdx.x];
   }
 }
@@ -133,7 +132,7 @@ void launch_diagnostics(const DevParams& P, const Fields& F, int cur, int want_f
   k_nu_reduce<<<1, kThreads, 0, s>>>(P, F.nu_hot, F.nu_cold, F.nu_avg, F.diag_scal);
   const int b = red_blocks(n3);
   k_entropy<<<b, kThreads, 0, s>>>(P, F.u[cur], F.v[cur], F.w[cur], F.th, F.eloc, want_fields,
-                                   F.red, F.counter, b, F.diag_scal);
+                                   F.rb, b, F.diag_scal);
 }
 
 }  // namespace hosc

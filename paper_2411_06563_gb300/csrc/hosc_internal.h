@@ -108,6 +108,16 @@ struct StepRecord {
   double res_theta;  // max |theta^{n+1} - theta^n| (walls included), kept for inner passes
 };
 
+// Where the blocks of a launch leave their partial sums. Up to kFlatRows rows are summed by the last
+// block; more rows in groups of kGroupRows by the last block of each group, and the groups' sums by the
+// last of those.
+constexpr unsigned kFlatRows = 512, kGroupRows = 64;
+struct RedBuf {
+  double* red;             // [rows][kRedSlots]
+  double* red2;            // [groups][kRedSlots]
+  unsigned int* counter;   // last-block tickets: the launch's, then the groups' (reset by the last)
+};
+
 // Device arrays of one context. All N^3 doubles unless noted.
 struct Fields {
   double* u[2];      // velocity, double-buffered: [cur] level n, [1-cur] level n+1 / n-1
@@ -135,8 +145,7 @@ struct Fields {
   double* u2[4];
   ulonglong2* exch;  // [kExchValues] exchanges of the one-launch solve, zero before it
   double* div;       // div V^{n+1}
-  double* red;       // reduction partials [blocks][kRedSlots]
-  unsigned int* counter;   // last-block ticket (reset by the last block)
+  RedBuf rb;         // reduction partials
   KrylovScalars* ks;       // [4]
   StepRecord* rec;         // [1]
   double* diag_scal;       // diagnostics scalars
@@ -186,10 +195,11 @@ int red_blocks(long count, int threads = kThreads);
 // Rows of the per-block partials buffer of an N^3 context: enough for any launch shape the
 // validation accepts (at least 32 threads per block, one plane per thread).
 inline long red_rows(long n3) { return n3 / 16 + 1024; }
+inline long red_groups(long n3) { return red_rows(n3) / kGroupRows + 8; }
 // Blocks of one interleaved Krylov launch (the partials buffer holds red_rows(N^3) rows).
 long krylov4_blocks(const DevParams& P);
 // Threads per block and planes per thread of the interleaved Krylov kernels when none are set:
-// 128 threads (wide three-kernel form) and the z-segment with the least wave cost below.
+// 384 threads (wide three-kernel form) and the z-segment with the least wave cost below.
 void default_tiles(int N, int* kblock, int* kz);
 // Shape of the planar FP64 Krylov kernels for a grid.
 void planar_shape(int N, int* pb, int* pkz);

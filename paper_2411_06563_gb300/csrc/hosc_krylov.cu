@@ -207,10 +207,9 @@ __device__ __forceinline__ void planar_end(const DevParams& P, const Fields& F, 
   const double mine = block_total<SumD, M>(dot);
   if (threadIdx.x < M) {
     const int slot = M == 5 ? 5 * b.s + (int)threadIdx.x : b.s + 4 * (int)threadIdx.x;
-    F.red[(long)b.row * row_stride<S>() + slot] = mine;
+    F.rb.red[(long)b.row * row_stride<S>() + slot] = mine;
   }
-  if (const double* tot = last_block_total<SumD, S>(F.red, F.counter, b.rows,
-                                                    gridDim.x * gridDim.y))
+  if (const double* tot = last_block_total<SumD, S>(F.rb, b.row, b.rows, 4u))
     planar_finish<KIND>(P, F, tot, FIRST, done);
 }
 
@@ -408,7 +407,7 @@ __global__ void __launch_bounds__(kThreads) k6_init(DevParams P, Fields F) {
     F.kv[1][c] = z;
     ff_dot4(acc, r, r);
   }
-  if (const double* tot = grid_total<SumFF, 4>(acc, F.red, F.counter, blockIdx.x, gridDim.x))
+  if (const double* tot = grid_total<SumFF, 4>(acc, F.rb, blockIdx.x, gridDim.x))
     finish_init(P, F, tot);
 }
 
@@ -456,7 +455,7 @@ __global__ void __launch_bounds__(256, MinB) k6_a(DevParams P, Fields F, int pp)
     }
   }
   if (const double* tot =
-          grid_total<SumFF, 12>(acc, F.red, F.counter, block_id(), block_count())) {
+          grid_total<SumFF, 12>(acc, F.rb, block_id(), block_count())) {
     if (threadIdx.x < 4) {
       const int s = threadIdx.x;
       KrylovScalars& k = F.ks[s];
@@ -514,7 +513,7 @@ __global__ void __launch_bounds__(256, MinB) k6_b(DevParams P, Fields F, int pp)
     }
   }
   if (const double* tot =
-          grid_total<SumFF, 16>(acc, F.red, F.counter, block_id(), block_count())) {
+          grid_total<SumFF, 16>(acc, F.rb, block_id(), block_count())) {
     if (threadIdx.x < 4) {
       const int s = threadIdx.x;
       KrylovScalars& k = F.ks[s];
@@ -624,7 +623,7 @@ __device__ __forceinline__ Op4 staged_op(const float4* sq, const StageLayout& L,
   Op4 op;
   op.m = sq[L.op_m() + t];
   op.e = sq[L.op_e() + t];
-  op.l12 = __fmul_rn(((const float*)(sq + L.op_l()))[t], 1.f / 12.f);
+  op.L = ((const float*)(sq + L.op_l()))[t];
   return op;
 }
 
@@ -676,7 +675,7 @@ __global__ void __launch_bounds__(256) k5_pv(DevParams P, Fields F, int pp) {
   }
   const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
   const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
-  if (const double* tot = grid_total<SumFF, 4>(acc, F.red, F.counter, bid, nb)) {
+  if (const double* tot = grid_total<SumFF, 4>(acc, F.rb, bid, nb)) {
     finish_pv(F.ks, tot, false);
     count_bytes(F, HOSC_K_BICG_PV, bytes4(P, 6.0 + op_words(ene)));
   }
@@ -727,7 +726,7 @@ __global__ void __launch_bounds__(256) k5_st(DevParams P, Fields F, int pp) {
   }
   const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
   const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
-  if (const double* tot = grid_total<SumFF, 8>(acc, F.red, F.counter, bid, nb)) {
+  if (const double* tot = grid_total<SumFF, 8>(acc, F.rb, bid, nb)) {
     finish_st(F.ks, tot);
     count_bytes(F, HOSC_K_BICG_ST, bytes4(P, 3.0 + op_words(ene)));
   }
@@ -863,7 +862,7 @@ __global__ void __launch_bounds__(256) k8_xr(DevParams P, Fields F, int pp) {
     ff_dot4(acc, r0, rn);
     ff_dot4(acc + 4, rn, rn);
   }
-  if (const double* tot = grid_total<SumFF, 8>(acc, F.red, F.counter, blockIdx.x, gridDim.x)) {
+  if (const double* tot = grid_total<SumFF, 8>(acc, F.rb, blockIdx.x, gridDim.x)) {
     finish_xr(P, F.ks, tot);
     // r v p x t r0 in, x r out
     count_bytes(F, HOSC_K_BICG_XR, bytes4(P, FIRST ? 6.0 : 8.0));
@@ -1056,20 +1055,22 @@ double krylov4_wave_cost(int N, int kblock, int kz, int narrow, int merged, int 
   return (double)waves * (kz + 2);
 }
 
+// Blocks of 384 threads: with the same bytes in flight as three blocks of 128 a launch leaves a third
+// of the partials (sum of the three kernels at 71^3 43 -> 35 us, 81^3 47 -> 43.5, 101^3 77.3 -> 70.8,
+// 161^3 and 257^3 within 1 %); the planes a block by the wave model.
 void default_tiles(int N, int* kblock, int* kz) {
   const int sms = device_sms();
   const int ni = N - 2;
   double best = 1e300;
-  int bb = 128, bz = 1;
-  for (int z = 1; z <= (ni < 16 ? ni : 16); ++z) {
-    const double c = krylov4_wave_cost(N, 128, z, 0, 0, sms);
+  *kblock = 384;
+  *kz = 1;
+  for (int z = 1; z <= (ni < 33 ? ni : 33); ++z) {
+    const double c = krylov4_wave_cost(N, 384, z, 0, 0, sms);
     if (c < best) {
       best = c;
-      bz = z;
+      *kz = z;
     }
   }
-  *kblock = bb;
-  *kz = bz;
 }
 
 }  // namespace hosc

@@ -84,13 +84,13 @@ __device__ __forceinline__ void ff_dot4(FF* acc, float4 a, float4 b) {
 // is zero. With Jacobi row scaling (precond) each row is divided by its diagonal D.
 struct Op4 {
   float4 m, e;   // (B_x, B_y, B_z, D) of momentum and of energy
-  float l12;     // L/12
+  float L;       // L of the momentum row
 };
 
 __device__ __forceinline__ Op4 load_op(const Fields& F, int c, bool ene) {
   Op4 op;
   op.m = HOSC_LDG(F.kwm + c);
-  op.l12 = __fmul_rn(HOSC_LDG(F.kL + c), 1.f / 12.f);
+  op.L = HOSC_LDG(F.kL + c);
   op.e = ene ? HOSC_LDG(F.kwe + c) : make_float4(0.f, 0.f, 0.f, 0.f);
   return op;
 }
@@ -99,25 +99,25 @@ __device__ __forceinline__ float4 apply_op(const DevParams& P, const Op4& op, fl
                                            float4 xm, float4 yp, float4 ym, float4 zp,
                                            float4 zm) {
   // momentum weights of the six neighbours, shared by the u, v, w lanes
-  // (l12 is a product of its own in load_op and the staged forms: not fused into these)
-  const float Sx = P.csf[0] + op.l12, Sy = P.csf[1] + op.l12, Sz = P.csf[2] + op.l12;
+  const float c12 = 1.f / 12.f;
+  const float Sx = fmaf(op.L, c12, P.csf[0]), Sy = fmaf(op.L, c12, P.csf[1]),
+              Sz = fmaf(op.L, c12, P.csf[2]);
   const float4 m = op.m, e = op.e;
   const float a1 = Sx - m.x, a2 = Sx + m.x, a3 = Sy - m.y, a4 = Sy + m.y, a5 = Sz - m.z,
               a6 = Sz + m.z;
   // one explicit order of the sums and fused multiply-adds, so that every kernel that applies the
   // operator gets the same bits
   auto row = [&](float c, float cp, float cm, float yp_, float ym_, float zp_, float zm_) {
-    return fmaf(a6, zm_, fmaf(a5, zp_, fmaf(a4, ym_, fmaf(a3, yp_, fmaf(a2, cm, fmaf(a1, cp,
-                __fmul_rn(m.w, c)))))));
+    return fmaf(a6, zm_, fmaf(a5, zp_, fmaf(a4, ym_, fmaf(a3, yp_, fmaf(a2, cm, fmaf(m.w, c,
+                __fmul_rn(a1, cp)))))));
   };
   float4 y;
   y.x = row(o.x, xp.x, xm.x, yp.x, ym.x, zp.x, zm.x);
   y.y = row(o.y, xp.y, xm.y, yp.y, ym.y, zp.y, zm.y);
   y.z = row(o.z, xp.z, xm.z, yp.z, ym.z, zp.z, zm.z);
-  const float c12 = 1.f / 12.f;
   const float ex = P.csf[0] + c12, ey = P.csf[1] + c12, ez = P.csf[2] + c12;
   y.w = fmaf(ez + e.z, zm.w, fmaf(ez - e.z, zp.w, fmaf(ey + e.y, ym.w, fmaf(ey - e.y, yp.w,
-        fmaf(ex + e.x, xm.w, fmaf(ex - e.x, xp.w, __fmul_rn(e.w, o.w)))))));
+        fmaf(ex + e.x, xm.w, fmaf(e.w, o.w, __fmul_rn(ex - e.x, xp.w)))))));
   if (P.precond) {
     const float im = 1.f / m.w;
     y.x *= im;
@@ -132,8 +132,8 @@ __device__ __forceinline__ float4 apply_op(const DevParams& P, const Op4& op, fl
 __device__ __forceinline__ double planar_row(double a0, double a1, double a2, double a3, double a4,
                                              double a5, double a6, double c, double xp, double xm,
                                              double yp, double ym, double zp, double zm) {
-  return fma(a6, zm, fma(a5, zp, fma(a4, ym, fma(a3, yp, fma(a2, xm, fma(a1, xp,
-             __dmul_rn(a0, c)))))));
+  return fma(a6, zm, fma(a5, zp, fma(a4, ym, fma(a3, yp, fma(a2, xm, fma(a0, c,
+             __dmul_rn(a1, xp)))))));
 }
 
 // Float4 words per interior node of the compact operators a launch reads: kwm and kL, and kwe
@@ -339,7 +339,7 @@ __device__ __forceinline__ bool k4_init_body(const DevParams& P, const Fields& F
     F.kv[1][c] = z;
     ff_dot4(acc, r, r);
   }
-  const double* tot = grid_total<SumFF, 4>(acc, F.red, F.counter, vbx, vnb);
+  const double* tot = grid_total<SumFF, 4>(acc, F.rb, vbx, vnb);
   if (!tot) return false;
   finish_init(P, F, tot);
   return true;
@@ -397,7 +397,7 @@ __device__ __forceinline__ void k4_pv_body(const DevParams& P, const Fields& F, 
     }
   }
   if (const double* tot =
-          grid_total<SumFF, M>(acc, F.red, F.counter, block_id(vg), block_count(vg))) {
+          grid_total<SumFF, M>(acc, F.rb, block_id(vg), block_count(vg))) {
     finish_pv(F.ks, tot, FIRST);
     // r p v r0 in, p v out, the compact operators
     count_bytes(F, HOSC_K_BICG_PV, bytes4(P, (FIRST ? 3.0 : 6.0) + op_words(ene)));
@@ -444,7 +444,7 @@ __device__ __forceinline__ void k4_st_body(const DevParams& P, const Fields& F, 
     }
   }
   if (const double* tot =
-          grid_total<SumFF, 8>(acc, F.red, F.counter, block_id(vg), block_count(vg))) {
+          grid_total<SumFF, 8>(acc, F.rb, block_id(vg), block_count(vg))) {
     finish_st(F.ks, tot);
     // r v in, t out, the compact operators
     count_bytes(F, HOSC_K_BICG_ST, bytes4(P, 3.0 + op_words(ene)));
@@ -488,7 +488,7 @@ __device__ __forceinline__ void k4_xr_body(const DevParams& P, const Fields& F, 
     }
   }
   const double* tot =
-      grid_total<SumFF, 8>(acc, F.red, F.counter, block_id(vg), block_count(vg));
+      grid_total<SumFF, 8>(acc, F.rb, block_id(vg), block_count(vg));
   if (!tot) return;
   finish_xr(P, F.ks, tot);
   count_bytes(F, HOSC_K_BICG_XR, bytes4(P, FIRST ? 6.0 : 8.0));   // r v p x t r0 in, x r out

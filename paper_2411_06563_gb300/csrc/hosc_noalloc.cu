@@ -38,8 +38,11 @@ static_assert(kOffBytes + HOSC_K_COUNT * sizeof(double) <= kOffRed,
 // The one-launch solve puts its exchanges where the other form has its partials.
 constexpr size_t kExchBytes = kControlBytes - kOffRed;
 static_assert(kExchBytes >= 16 * 4 * 4 * (size_t)kSolveRows, "exchanges exceed the control block");
-static_assert(kOffRed + kMaxBlocks * kRedSlots * sizeof(double) <= kControlBytes,
+static_assert(kOffRed + (kMaxBlocks + kMaxBlocks / kGroupRows + 1) * kRedSlots * sizeof(double) <=
+                  kControlBytes,
               "reduction partials exceed the control block");
+static_assert(kOffCounter + (kMaxBlocks / kGroupRows + 2) * sizeof(unsigned int) <= kOffHalt,
+              "tickets overlap the halt flag");
 
 // The scratch. In host code this name is only a stand-in for the symbol: its device address comes
 // from cudaGetSymbolAddress, once per device.
@@ -97,10 +100,11 @@ extern "C" hosc_status hosc_bicgstab_noalloc(int N, const double* const* weights
   const size_t vec_used = (size_t)(p - base);
   char* ctl = base + kVectorsBytes;
   F.ks = (KrylovScalars*)ctl;                      // 4 x sizeof(KrylovScalars) = 320 bytes
-  F.counter = (unsigned int*)(ctl + kOffCounter);
+  F.rb.counter = (unsigned int*)(ctl + kOffCounter);
   F.halt = (int*)(ctl + kOffHalt);
   F.alg_bytes = (double*)(ctl + kOffBytes);
-  F.red = (double*)(ctl + kOffRed);
+  F.rb.red = (double*)(ctl + kOffRed);
+  F.rb.red2 = F.rb.red + kMaxBlocks * kRedSlots;
   for (int q = 0; q < 7; ++q) {
     F.Am[q] = const_cast<double*>(weights[q]);
     F.Ae[q] = const_cast<double*>(weights[7 + q]);
@@ -126,7 +130,7 @@ extern "C" hosc_status hosc_bicgstab_noalloc(int N, const double* const* weights
   if (solve_shape_planar(N, &P.pb, &P.pkz)) {
     // one launch (every grid up to HOSC_NOALLOC_MAX_N where its blocks are resident): the solver's
     // scalars, the halt flag and the exchanges start at zero
-    F.exch = (ulonglong2*)F.red;
+    F.exch = (ulonglong2*)F.rb.red;
     if (cudaMemsetAsync(ctl, 0, kControlBytes, sm) != cudaSuccess) return HOSC_ECUDA;
     launch_solve(P, F, sm);
     if (cudaGetLastError() != cudaSuccess || !read_scalars()) return HOSC_ECUDA;

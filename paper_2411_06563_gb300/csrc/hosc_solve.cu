@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kSolveBlock, 2) k_solve_mixed(DevParams P, Fie
       r0[kk * B + t] = r[kk];
       om[kk * B + t] = F.kwm[c];
       oe[kk * B + t] = F.kwe[c];
-      ol[kk * B + t] = __fmul_rn(F.kL[c], 1.f / 12.f);
+      ol[kk * B + t] = F.kL[c];
     }
   }
   if (t < 4) ks[t] = F.ks[t];
@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kSolveBlock, 2) k_solve_mixed(DevParams P, Fie
       Op4 op;
       op.m = om[kk * B + t];
       op.e = ene ? oe[kk * B + t] : zero;
-      op.l12 = ol[kk * B + t];
+      op.L = ol[kk * B + t];
       const float4 zp = kk + 1 < nk && kk + 1 < KZ ? f[kk + 1 < KZ ? kk + 1 : kk] : hi;
       const float4 zm = kk > 0 ? f[kk > 0 ? kk - 1 : 0] : lo;
       out(kk, apply_op(P, op, f[kk], has_xp ? o[1] : zero, has_xm ? o[-1] : zero, o[ni], o[-ni],

@@ -651,7 +651,7 @@ __device__ __forceinline__ void k_increment_body(const DevParams& P, const Field
       F.ws[1 - cur][t] = (float)w;
     }
   }
-  if (const double* tot = grid_total<MaxD, 2>(m, F.red, F.counter, vbx, nblocks)) {
+  if (const double* tot = grid_total<MaxD, 2>(m, F.rb, vbx, nblocks)) {
     if (threadIdx.x == 0) {
       // an inner pressure pass changes u, v, w only: theta's change stays that of the first pass
       if (!P.inner_pass) F.rec->res_theta = tot[1];
@@ -724,7 +724,7 @@ __device__ __forceinline__ void k_div_walls_body(const DevParams& P, const Field
       if (P.krylov_fp32) F.ths[c] = (float)s;
     }
   }
-  if (const double* tot = grid_total<MaxD, 2>(m, F.red, F.counter, vbx, nblocks)) {
+  if (const double* tot = grid_total<MaxD, 2>(m, F.rb, vbx, nblocks)) {
     if (threadIdx.x == 0) {
       F.rec->div_max = tot[0];
       F.rec->res = fmax(F.rec->res, tot[1]);
@@ -828,10 +828,7 @@ __device__ __forceinline__ void k_pressure_walls_body(const DevParams& P, const 
   }
   if (record) {
     __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(F.counter, 1u) == (unsigned)nblocks - 1) {
-      *F.counter = 0u;
-      k_finish_record_body(P, F, 0);
-    }
+    if (last_ticket(F.rb.counter, (unsigned)nblocks)) k_finish_record_body(P, F, 0);
   }
 }
 

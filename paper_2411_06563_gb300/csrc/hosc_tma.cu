@@ -260,8 +260,7 @@ __global__ void __launch_bounds__(kTmaMaxThreads)
         Op4 op;
         op.m = ((const float4*)(st + L.off_m))[e];
         op.e = ene ? ((const float4*)(st + L.off_e))[e] : zero;
-        op.l12 = __fmul_rn(((const float*)(st + L.off_l + ty * L.lrow))[(int)(lin & 3L) + tx],
-                           1.f / 12.f);
+        op.L = ((const float*)(st + L.off_l + ty * L.lrow))[(int)(lin & 3L) + tx];
         const float4 y = apply_op(P, op, pc, val(u, h + 1), val(u, h - 1), val(u, h + hx),
                                   val(u, h - hx), pz, pm);
         const int c = (i0 + tx) + N * (j0 + ty) + N2 * k;
@@ -285,7 +284,7 @@ __global__ void __launch_bounds__(kTmaMaxThreads)
   const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
   const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
   // synchronises the block: failed is final after it
-  const double* tot = grid_total<SumFF, M>(acc, F.red, F.counter, bid, nb);
+  const double* tot = grid_total<SumFF, M>(acc, F.rb, bid, nb);
   const bool bad = failed != 0;
   if (tot) {
     if (PV) finish_pv(F.ks, tot, false);
