@@ -80,6 +80,8 @@ struct Ctx {
   // the context is not a pool's member
   bool coop_fits = false, shape_chosen = false, pooled = false;
   int ckz = 0;
+  bool plane_fits = false;                 // shared-plane kernels
+  int ptx = 1, pty = 1, plz = 1;
   alignas(64) unsigned char tmap_host[kTmaMaps * kTmaMapBytes];   // their tensor maps
   // a round of steps enqueued for a pool (hosc_pool.cu): level and length, records read back
   // asynchronously into h_ring / h_ring_pos, completion marked by round_ev
@@ -152,6 +154,11 @@ void apply_tiles(Ctx* c) {
   c->P.xr_flat = c->xr_flat;
   c->P.coop = c->coop_fits && !c->shape_chosen && !c->pooled && c->prm.solver == 0;
   c->P.ckz = c->ckz;
+  // the shared-plane kernels unless the caller has chosen a shape of the others
+  c->P.plane = c->plane_fits && !c->shape_chosen && !c->merged && c->sx == 0 && c->tty == 0;
+  c->P.ptx = c->ptx;
+  c->P.pty = c->pty;
+  c->P.plz = c->plz;
   c->P.lean = !c->merged && c->sx == 0 && c->tty == 0;
 }
 
@@ -961,6 +968,8 @@ hosc_status make_ctx(const hosc_params* p, void* dev_ws, size_t bytes, void** ou
     int b = 0, z = 0;
     c->coop_fits = p->solver == 0 && solve_shape_planar(p->N, &b, &z);
   }
+  c->plane_fits =
+      p->precision == HOSC_MIXED && plane_shape(p->N, &c->ptx, &c->pty, &c->plz);
   if (!c->coop_fits || p->precision != HOSC_MIXED) default_tiles(p->N, &c->kblock, &c->kz);
   st = set_initial_state(c);
   if (st) {
@@ -1624,7 +1633,7 @@ hosc_status hosc_time_kernel(void* ctx, int kernel_id, int reps, double* ms_per_
 static void choose_shape(Ctx* c) {
   if (c->shape_chosen) return;
   c->shape_chosen = true;
-  if (c->P.coop) drop_graphs(c);
+  if (c->P.coop || c->P.plane) drop_graphs(c);
   apply_tiles(c);
 }
 
@@ -1791,6 +1800,8 @@ hosc_status hosc_autotune(void* ctx, int reps, int* kblock_out, int* kz_out, dou
       drop_graphs(c);
     }
   } keep{c, c->shape_chosen};
+  const bool plane0 = c->P.plane != 0;   // the default p/v and s/t of this grid: timed at the end
+  if (!c->plane_fits && !c->coop_fits) keep.chosen = true;
   {   // the register kernels first
     hosc_status s0 = hosc_set_stencil_tiles(c, 0, 0, 0);
     if (!s0) s0 = hosc_set_tma_tiles(c, 0, 0, 3, 3);
@@ -2031,6 +2042,30 @@ hosc_status hosc_autotune(void* ctx, int reps, int* kblock_out, int* kz_out, dou
     st = hosc_set_xr_form(c, use_flat ? 1 : 0);
     if (st) return st;
     best += (use_flat ? flat : col) - (save ? flat : col);
+  }
+  if (plane0) {   // p/v and s/t as shared-plane kernels against the ones found
+    double found = 0.0, plane = 0.0;
+    for (int form = 0; form < 2 && !st; ++form) {
+      c->P.plane = form;
+      const int tty = c->P.tty, sx = c->P.sx;
+      if (form) c->P.tty = c->P.sx = 0;
+      for (int kid = HOSC_K_BICG_PV; kid <= HOSC_K_BICG_ST && !st; ++kid) {
+        double ms = 0.0;
+        st = time_class(c, kid, 4 * reps, &ms);
+        (form ? plane : found) += ms;
+      }
+      c->P.tty = tty;
+      c->P.sx = sx;
+    }
+    apply_tiles(c);
+    if (st) return st;
+    keep.chosen = plane > found;
+    if (!keep.chosen) {
+      st = hosc_set_tma_tiles(c, 0, 0, 3, 3);
+      if (!st) st = hosc_set_stencil_tiles(c, 0, 0, 0);
+      if (st) return st;
+      best += plane - found;
+    }
   }
   if (kblock_out) *kblock_out = best_b;
   if (kz_out) *kz_out = best_z;

@@ -202,12 +202,29 @@ __host__ __device__ constexpr int row_stride() {
 // that forms the same rows gets the same bits: group g of G adds rows g, g + G, ... one after another
 // (four loads in flight), then the groups combine in a tree. load(row, slot); the totals are left in
 // tot (shared), valid for every thread. blockDim.x must be a multiple of 32.
+template <int Mp>
+constexpr int row_groups() { return Mp <= 8 ? 64 : 512 / Mp; }
+
+// The totals of M slots over the groups of s_g[group * Mp + slot] into tot, a warp a slot.
+template <class T, int M>
+__device__ __forceinline__ void sum_groups(const double* s_g, double* tot) {
+  constexpr int Mp = pow2_at_least(M), G = row_groups<Mp>();
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int m = threadIdx.x >> 5; m < M; m += nw) {
+    double a = lane < G ? s_g[lane * Mp + m] : 0.0;
+    if (G > 32) a = T::add(a, s_g[(lane + 32) % G * Mp + m]);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) a = T::add(a, T::shfl_xor(a, off));
+    if (lane == 0) tot[m] = a;
+  }
+}
+
 template <class T, int M, class Load>
 __device__ __forceinline__ void sum_rows(int nr, Load load, double* tot) {
   constexpr int Mp = pow2_at_least(M);
-  constexpr int G = Mp <= 8 ? 64 : 512 / Mp;
+  constexpr int G = row_groups<Mp>();
   __shared__ double s_g[Mp * G];
-  const int t = threadIdx.x, bd = blockDim.x, lane = t & 31, nw = bd >> 5;
+  const int t = threadIdx.x, bd = blockDim.x;
   for (int w = t; w < Mp * G; w += bd) {
     const int m = w % Mp;
     double acc = 0.0;
@@ -221,13 +238,7 @@ __device__ __forceinline__ void sum_rows(int nr, Load load, double* tot) {
     s_g[w] = acc;
   }
   __syncthreads();
-  for (int m = t >> 5; m < Mp; m += nw) {
-    double a = lane < G ? s_g[lane * Mp + m] : 0.0;
-    if (G > 32) a = T::add(a, s_g[(lane + 32) % G * Mp + m]);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) a = T::add(a, T::shfl_xor(a, off));
-    if (lane == 0) tot[m] = a;
-  }
+  sum_groups<T, M>(s_g, tot);
   __syncthreads();
 }
 

@@ -56,6 +56,8 @@ struct DevParams {
   int tkernels;      // which of them run: 1 p/v, 2 s/t, 3 both
   int coop;          // the solve is one cooperative launch (hosc_solve.cu)
   int ckz;           // its planes per block, mixed precision (FP64: pb and pkz)
+  int plane;         // p/v and s/t as shared-plane kernels: tile of ptx * pty columns, plz planes
+  int ptx, pty, plz;
   int lean;          // interleaved solve started by the right-hand sides' kernel: no initialisation,
                      // the first iteration reads r_0 and nothing else (register kernels, either x/r)
   int xr_flat;       // x/r as one flat grid-stride stream (k8_xr) instead of the column march
@@ -201,6 +203,9 @@ long krylov4_blocks(const DevParams& P);
 // Threads per block and planes per thread of the interleaved Krylov kernels when none are set:
 // 384 threads (wide three-kernel form) and the z-segment with the least wave cost below.
 void default_tiles(int N, int* kblock, int* kz);
+// Shape of the shared-plane kernels for a grid; false where the register kernels run.
+constexpr int kPlaneMinN = 104;
+bool plane_shape(int N, int* ptx, int* pty, int* plz);
 // Shape of the planar FP64 Krylov kernels for a grid.
 void planar_shape(int N, int* pb, int* pkz);
 // Waves of resident blocks a launch shape needs on this GPU times the planes each block streams
@@ -249,7 +254,7 @@ void launch_b2(int kernel, const DevParams& P, const Fields& F, int cp, bool fir
                cudaStream_t s);
 // End of the body of the BiCGSTAB loop of a captured step: end of the loop when every system is done.
 void launch_loop_cond(const Fields& F, unsigned long long handle, cudaStream_t s);
-// The whole solve as one cooperative launch (P.coop): scalars started and exchange buffer zeroed by the
+// The whole solve as one cooperative launch (P.coop): exchange buffer zeroed by the sources, scalars started by the
 // right-hand sides' kernel. The shapes it runs with on an N^3 grid; false when the grid is too large.
 void launch_solve(const DevParams& P, const Fields& F, cudaStream_t s);
 bool solve_shape_planar(int N, int* pb, int* pkz);

@@ -536,6 +536,138 @@ __global__ void __launch_bounds__(256, MinB) k6_b(DevParams P, Fields F, int pp)
   }
 }
 
+// ------------------------------------------------------- shared-plane stencil kernels
+//
+// p/v and s/t of the three-kernel form, the default above the grids of the one-launch solve. A block
+// has a tile of ptx * pty interior columns (one thread each) and pkz planes. The vector that the
+// operator is applied to (r + beta (p - omega v), r - alpha v) is evaluated once at each node of the tile
+// and of the ring around it and put in shared memory (two planes, one barrier a plane); the planes above
+// and below stay in registers. A thread then reads 3 vectors (2 for s/t) and its operator row a plane
+// where the register kernels read 21 (14) and the row; and the loads of the next plane are issued before
+// the barrier, so that a plane's arithmetic covers them (the register kernels wait for a plane's 19
+// dependent loads: 24 warps an SM at half of the copy bandwidth). Walls are read as the zeros they hold.
+// Same arithmetic of a node as the register kernels. Measured, alone, register -> shared plane: s/t
+// 301 -> 262 us at 257^3, 81.5 -> 71.5 at 161^3, 44.4 -> 42.4 at 129^3, 19.9 -> 22.4 at 101^3; p/v 450 -> 439,
+// 121 -> 117.5, 69.1 -> 67.1, 36.9 -> 35.3 (step at 101^3 891 against 883 us, 81^3 561 against 587): used
+// from kPlaneMinN up, where a launch is several waves of blocks.
+
+constexpr int kPlaneThreads = 384;
+
+template <bool PV, bool FIRST>
+__global__ void __launch_bounds__(kPlaneThreads, 2) k_plane(DevParams P, Fields F, int pp) {
+  constexpr int M = PV && !FIRST ? 4 : 8;
+  extern __shared__ float4 plane_sh[];
+  __shared__ Scal4 sc;
+  pdl_wait_and_release();
+  load_scalars(F.ks, sc);
+  if (sc.all_done) return;   // uniform over the grid
+  const bool ene = !sc.done[3];
+  const int N = P.N, N2 = N * N, tx = P.ptx, ty = P.pty, w = tx + 2, t = threadIdx.x;
+  const int i0 = 1 + (int)blockIdx.x * tx, j0 = 1 + (int)blockIdx.y * ty;
+  const int k0 = 1 + (int)blockIdx.z * P.plz, k1 = min(k0 + P.plz, N - 1);
+  const int np = 1 - pp;
+  const float4 b = sc.b, mom = neg4(sc.om), ma = neg4(sc.a);
+  const float4* __restrict__ R = FIRST ? F.kr0 : F.kr;
+  const float4* __restrict__ Y = PV ? F.kp[pp] : F.kv[np];
+  const float4* __restrict__ Z = F.kv[pp];
+  struct Raw {
+    float4 r, y, z;
+  };
+  auto load = [&](int c) {
+    Raw a;
+    a.r = __ldg(R + c);
+    if (!(PV && FIRST)) a.y = __ldg(Y + c);
+    if (PV && !FIRST) a.z = __ldg(Z + c);
+    return a;
+  };
+  auto value = [&](const Raw& a) {
+    if (PV && FIRST) return a.r;
+    if (PV) return fma4(b, fma4(mom, a.z, a.y), a.r);
+    return fma4(ma, a.y, a.r);
+  };
+  // this thread's column, and its node of the ring (the tile's 2 (tx + ty) neighbours)
+  const int cy = t / tx, cx = t - cy * tx;
+  const bool in = t < tx * ty && i0 + cx <= N - 2 && j0 + cy <= N - 2;
+  const int c0 = in ? i0 + cx + N * (j0 + cy) : 0, h = (cy + 1) * w + cx + 1;
+  int rx = 0, ry = 0;
+  if (t < tx) rx = t + 1;
+  else if (t < 2 * tx) rx = t - tx + 1, ry = ty + 1;
+  else if (t < 2 * tx + ty) ry = t - 2 * tx + 1;
+  else rx = tx + 1, ry = t - 2 * tx - ty + 1;
+  const int gi = i0 - 1 + rx, gj = j0 - 1 + ry;
+  const bool ring = t < 2 * (tx + ty), rin = ring && gi <= N - 1 && gj <= N - 1;
+  const int rc = rin ? gi + N * gj : 0, hr = ry * w + rx;
+  const float4 zero = f4(0.f);
+  Raw own = {zero, zero, zero}, rim = {zero, zero, zero};
+  float4 pm = zero, pc = zero, q = zero;
+  Op4 op = {zero, zero, 0.f};
+  if (in) {
+    pm = value(load(c0 + N2 * (k0 - 1)));
+    pc = value(load(c0 + N2 * k0));
+    own = load(c0 + N2 * (k0 + 1));
+    op = load_op(F, c0 + N2 * k0, ene);
+    if (PV && !FIRST) q = __ldg(F.kr0 + c0 + N2 * k0);
+  }
+  if (rin) rim = load(rc + N2 * k0);
+  FF acc[M] = {};
+  for (int k = k0; k < k1; ++k) {
+    float4* s = plane_sh + (k & 1) * w * (ty + 2);
+    const bool more = k + 1 < k1;
+    if (t < tx * ty) s[h] = pc;   // zero past the interior
+    if (ring) s[hr] = rin ? value(rim) : zero;
+    const float4 pz = in ? value(own) : zero;
+    const Op4 o = op;
+    const float4 z = q;
+    if (more && in) {   // the next plane's operands, in flight over this plane's arithmetic
+      const int cn = c0 + N2 * (k + 1);
+      own = load(cn + N2);
+      op = load_op(F, cn, ene);
+      if (PV && !FIRST) q = __ldg(F.kr0 + cn);
+    }
+    if (more && rin) rim = load(rc + N2 * (k + 1));
+    __syncthreads();
+    if (in) {
+      const int c = c0 + N2 * k;
+      const float4 y = apply_op(P, o, pc, s[h + 1], s[h - 1], s[h + w], s[h - w], pz, pm);
+      if (PV) {
+        F.kp[np][c] = pc;
+        F.kv[np][c] = y;
+        ff_dot4(acc, FIRST ? pc : z, y);
+        if (FIRST) ff_dot4(acc + M - 4, pc, pc);
+      } else {
+        F.kt[c] = y;
+        ff_dot4(acc, y, pc);
+        ff_dot4(acc + M - 4, y, y);
+      }
+    }
+    pm = pc;
+    pc = pz;
+  }
+  const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+  const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
+  if (const double* tot = grid_total<SumFF, M>(acc, F.rb, bid, nb)) {
+    if (PV) {
+      finish_pv(F.ks, tot, FIRST);
+      count_bytes(F, HOSC_K_BICG_PV, bytes4(P, (FIRST ? 3.0 : 6.0) + op_words(ene)));
+    } else {
+      finish_st(F.ks, tot);
+      count_bytes(F, HOSC_K_BICG_ST, bytes4(P, 3.0 + op_words(ene)));
+    }
+  }
+}
+
+dim3 plane_grid(const DevParams& P) {
+  const int ni = P.N - 2;
+  return dim3((ni + P.ptx - 1) / P.ptx, (ni + P.pty - 1) / P.pty, (ni + P.plz - 1) / P.plz);
+}
+
+template <bool PV>
+void launch_plane(const DevParams& P, const Fields& F, int pp, bool first, cudaStream_t s) {
+  const size_t smem = 2 * sizeof(float4) * (size_t)(P.ptx + 2) * (P.pty + 2);
+  if (first) launch_pdl(k_plane<PV, true>, plane_grid(P), kPlaneThreads, smem, s, P, F, pp);
+  else launch_pdl(k_plane<PV, false>, plane_grid(P), kPlaneThreads, smem, s, P, F, pp);
+}
+
 // ------------------------------------------------------- staged stencil kernels (cp.async)
 //
 // The p/v and s/t kernels again, with their reads staged through shared memory. A block owns a
@@ -913,6 +1045,8 @@ void launch_bicg_pv(const DevParams& P, const Fields& F, int pp, bool first, cud
     launch_tma_pv(P, F, pp, s);
   } else if (P.sx > 0) {
     k5_pv<<<grid5(P), P.sx * P.sy, staged_smem_bytes(P.sx, P.sy, true), s>>>(P, F, pp);
+  } else if (P.plane) {
+    launch_plane<true>(P, F, pp, first, s);
   } else if (first && P.lean) {
     if (P.narrow) launch_pdl(k4_pv<4, true>, grid4(P), P.kblock, 0, s, P, F, pp);
     else launch_pdl(k4_pv<2, true>, grid4(P), P.kblock, 0, s, P, F, pp);
@@ -931,6 +1065,8 @@ void launch_bicg_st(const DevParams& P, const Fields& F, int pp, bool first, cud
     launch_tma_st(P, F, pp, s);
   } else if (P.sx > 0) {
     k5_st<<<grid5(P), P.sx * P.sy, staged_smem_bytes(P.sx, P.sy, false), s>>>(P, F, pp);
+  } else if (P.plane) {
+    launch_plane<false>(P, F, pp, first, s);
   } else {
     const int f = first && P.lean;
     if (P.narrow) launch_pdl(k4_st<4>, grid4(P), P.kblock, 0, s, P, F, pp, f);
@@ -1055,6 +1191,37 @@ double krylov4_wave_cost(int N, int kblock, int kz, int narrow, int merged, int 
   return (double)waves * (kz + 2);
 }
 
+// Tile and planes of the shared-plane kernels: the least modelled time, waves of the two resident blocks
+// an SM times the planes a block streams times the nodes it reads a plane (tile and ring), among tiles
+// that cut the interior evenly and fit a block's threads.
+bool plane_shape(int N, int* ptx, int* pty, int* plz) {
+  if (N < kPlaneMinN) return false;
+  const int sms = device_sms(), ni = N - 2;
+  double best = 1e300;
+  *ptx = *pty = *plz = 1;
+  for (int nx = 1; nx <= ni; ++nx) {
+    const int tx = (ni + nx - 1) / nx;
+    if (tx > 128) continue;
+    if (tx < 16 && nx > 1) break;
+    int ty = kPlaneThreads / tx < ni ? kPlaneThreads / tx : ni;
+    const int ny = (ni + ty - 1) / ty;
+    ty = (ni + ny - 1) / ny;
+    if (2 * (tx + ty) > kPlaneThreads) continue;
+    for (int z = 1; z <= ni && z <= 64; ++z) {
+      const long blocks = (long)((ni + tx - 1) / tx) * ny * ((ni + z - 1) / z);
+      const double waves = (double)((blocks + 2 * sms - 1) / (2 * sms));
+      const double cost = waves * (z + 2) * (kPlaneThreads + 2.0 * (tx + ty));
+      if (cost < best) {
+        best = cost;
+        *ptx = tx;
+        *pty = ty;
+        *plz = z;
+      }
+    }
+  }
+  return best < 1e300;
+}
+
 // Blocks of 384 threads: with the same bytes in flight as three blocks of 128 a launch leaves a third
 // of the partials (sum of the three kernels at 71^3 43 -> 35 us, 81^3 47 -> 43.5, 101^3 77.3 -> 70.8,
 // 161^3 and 257^3 within 1 %); the planes a block by the wave model.
@@ -1064,8 +1231,10 @@ void default_tiles(int N, int* kblock, int* kz) {
   double best = 1e300;
   *kblock = 384;
   *kz = 1;
+  const long slots = (long)krylov4_occupancy(384, 0, 0) * sms, chunks = ((long)ni * ni + 383) / 384;
   for (int z = 1; z <= (ni < 33 ? ni : 33); ++z) {
-    const double c = krylov4_wave_cost(N, 384, z, 0, 0, sms);
+    const long items = chunks * ((ni + z - 1) / z);
+    const double c = (double)((items + slots - 1) / slots) * (z + 2);
     if (c < best) {
       best = c;
       *kz = z;

@@ -183,6 +183,7 @@ struct Scal4 {
 // The first warp reads the four systems' scalars, one lane a system.
 __device__ __forceinline__ void load_scalars(const KrylovScalars* ks, Scal4& sc) {
   if (threadIdx.x < 32) {
+    __syncwarp();
     const int s = threadIdx.x;
     int d = 1;
     if (s < 4) {

@@ -359,6 +359,7 @@ void round_member_shape(RoundMember* M) {
   M->P.merged = 0;
   M->P.sx = M->P.sy = M->P.skz = 0;
   M->P.lean = 1;
+  M->P.plane = M->P.coop = 0;
   M->kx = (int)((ni * ni + kRoundThreads - 1) / kRoundThreads);
   M->ky = (int)((ni + M->P.kz - 1) / M->P.kz);
 }

@@ -41,6 +41,8 @@ __device__ __forceinline__ unsigned long long solve_ns() {
   return t;
 }
 
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
 // One value of an exchange: two words of (4 bytes of the value, the exchange's number).
 __device__ __forceinline__ void put_value(ulonglong2* p, double v, unsigned e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v);
@@ -71,13 +73,12 @@ template <class T, int M>
 __device__ __noinline__ bool gather(ulonglong2* rows, int nr, int stride, int row, unsigned e,
                                     double mine, double* tot, int* failed) {
   constexpr int Mp = pow2_at_least(M);
-  constexpr int G = 64;
-  static_assert(Mp <= 8, "groups as in sum_rows");
+  constexpr int G = row_groups<Mp>();
   __shared__ double s_g[Mp * G];
   rows += (size_t)(e & 1u) * nr * stride;
-  const int t = threadIdx.x, lane = t & 31;
+  const int t = threadIdx.x;
   if (t < M) {
-    __threadfence();   // the block's writes to memory come before its row
+    fence_gpu();   // the block's writes to memory come before its row
     put_value(rows + row * stride + t, mine, e);
   }
   for (int w = t; w < Mp * G; w += blockDim.x) {
@@ -110,14 +111,9 @@ __device__ __noinline__ bool gather(ulonglong2* rows, int nr, int stride, int ro
     }
     s_g[w] = acc;
   }
-  __threadfence();
+  fence_gpu();   // the others' writes that came before their rows
   __syncthreads();
-  for (int m = t >> 5; m < Mp; m += (int)(blockDim.x >> 5)) {
-    double a = T::add(s_g[lane * Mp + m], s_g[(lane + 32) * Mp + m]);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) a = T::add(a, T::shfl_xor(a, off));
-    if (lane == 0) tot[m] = a;
-  }
+  sum_groups<T, M>(s_g, tot);
   __syncthreads();
   return *(volatile int*)failed == 0;
 }
@@ -431,7 +427,6 @@ __global__ void __launch_bounds__(kSolveBlock, 2) k_solve_mixed(DevParams P, Fie
       }
       if (!ok) break;
       finish_pv(ks, tot, first);
-      __syncthreads();
     }
     load_scalars(ks, sc);
     if (sc.all_done) break;
@@ -454,7 +449,6 @@ __global__ void __launch_bounds__(kSolveBlock, 2) k_solve_mixed(DevParams P, Fie
       ok = exchange<SumFF, 8>(x, acc, tot);
       if (!ok) break;
       finish_st(ks, tot);
-      __syncthreads();
     }
     load_scalars(ks, sc);
     // x += alpha p + omega s, r = s - omega t; p - omega v for the next p
@@ -478,7 +472,6 @@ __global__ void __launch_bounds__(kSolveBlock, 2) k_solve_mixed(DevParams P, Fie
       ok = exchange<SumFF, 8>(x, acc, tot);
       if (!ok) break;
       finish_xr(P, ks, tot);
-      __syncthreads();
     }
   }
   if (!any && in)   // every right-hand side is zero (or none to solve): zero increments
@@ -582,6 +575,15 @@ bool solve_shape_planar(int N, int* pb, int* pkz) {
 }
 
 bool solve_shape_mixed(int N, int* kblock, int* kz) {
+  static thread_local struct { int N, device, kblock, kz; } last = {0, -1, 0, 0};
+  int device = 0;
+  if (cudaGetDevice(&device) != cudaSuccess) return false;
+  if (last.N == N && last.device == device) {
+    *kblock = last.kblock;
+    *kz = last.kz;
+    return last.kz > 0;
+  }
+  last = {N, device, 0, 0};
   const int sms = device_sms(), ni = N - 2;
   if (2 * ni > kSolveBlock) return false;
   const long chunks = ((long)ni * ni + kSolveBlock - 1) / kSolveBlock;
@@ -595,8 +597,8 @@ bool solve_shape_mixed(int N, int* kblock, int* kz) {
     const SolveFn fn = mixed_fn(template_planes(z), N, &smem);
     if (resident(fn, kSolveBlock, smem) < rows) continue;
     best = cost;
-    *kblock = kSolveBlock;
-    *kz = z;
+    last.kblock = *kblock = kSolveBlock;
+    last.kz = *kz = z;
   }
   return best < 1e300;
 }

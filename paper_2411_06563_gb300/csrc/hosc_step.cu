@@ -54,15 +54,16 @@ void launch_viscosity(const DevParams& P, const Fields& F, int cur, cudaStream_t
 }
 
 void launch_sources(const DevParams& P, const Fields& F, int cur, cudaStream_t s) {
+  ulonglong2* exch = P.coop ? F.exch : nullptr;
   const SweepGrid g = sweep_grid(P);
   if (P.sweep_fp32)
     launch_pdl(k_sources<float>, g.nb, g.threads, 0, s, P, F.us[cur], F.vs[cur], F.ws[cur], F.ths,
                F.ps, reinterpret_cast<const float*>(F.eta), reinterpret_cast<float*>(F.Eu[cur]),
                reinterpret_cast<float*>(F.Ev[cur]), reinterpret_cast<float*>(F.Ew[cur]), F.halt,
-               g.nbi);
+               g.nbi, exch);
   else
     launch_pdl(k_sources<double>, g.nb, g.threads, 0, s, P, F.u[cur], F.v[cur], F.w[cur], F.th, F.p,
-               F.eta, F.Eu[cur], F.Ev[cur], F.Ew[cur], F.halt, g.nbi);
+               F.eta, F.Eu[cur], F.Ev[cur], F.Ew[cur], F.halt, g.nbi, exch);
 }
 
 template <class Tc, class Ts>
