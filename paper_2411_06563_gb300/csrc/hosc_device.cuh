@@ -165,8 +165,8 @@ __device__ __forceinline__ typename Op::V cross_warps(const typename Op::V* s) {
   const int lane = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
   typename Op::V r = Op::zero();
   for (int w = lane / Mp; w < nw; w += 32 / Mp) r = Op::add(r, s[w * Mp + lane % Mp]);
-#pragma unroll
-  for (int off = Mp; off < 32; off <<= 1) r = Op::add(r, Op::shfl_xor(r, off));
+  const int used = min(32, nw * Mp);   // the lanes past it hold zeros
+  for (int off = Mp; off < used; off <<= 1) r = Op::add(r, Op::shfl_xor(r, off));
   return r;
 }
 

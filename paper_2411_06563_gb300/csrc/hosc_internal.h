@@ -46,7 +46,7 @@ struct DevParams {
                      // form, kblock <= 256)
   int merged;        // interleaved solve: two kernels per BiCGSTAB iteration (the x, r update
                      // folded into the next p, v kernel) instead of three
-  int pb, pkz;       // planar FP64 Krylov kernels: threads per block (128, 256, 512), planes per block
+  int pb, pkz;       // planar FP64 Krylov kernels: threads per block, planes per block
   int rhs_copied;    // planar solve: the first residual is a copy of rhs (whose walls may hold anything)
   int sx, sy, skz;   // staged stencil kernels (p/v and s/t): tile of sx * sy interior columns,
                      // skz planes per block; sx == 0 selects the register kernels instead
@@ -87,6 +87,7 @@ struct DevParams {
   double div_steady;   // max|div V| below this (div_steady, else tol_div) is steady
 };
 
+constexpr int kPlanarMost = 512;    // most threads a block of the planar kernels (a multiple of 32)
 constexpr int kSolveRows = 152;      // most rows (blocks) of a system in the one-launch FP64 solve
 constexpr int kExchValues = 8192;   // 16-byte values of the exchange buffer
 constexpr int kRing = 256;   // step records kept on the device between host reads

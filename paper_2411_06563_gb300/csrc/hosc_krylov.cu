@@ -214,8 +214,8 @@ __device__ __forceinline__ void planar_end(const DevParams& P, const Fields& F, 
 }
 
 // The planar kernels that apply an operator. pp: parity of the iteration (BiCGSTAB) or cycle.
-template <int KIND, int B, bool FIRST>
-__global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, int pp) {
+template <int KIND, bool FIRST>
+__global__ void __launch_bounds__(kPlanarMost, 2) k_planar(DevParams P, Fields F, int pp) {
   extern __shared__ double planes[];   // two planes of N + B + N values
   pdl_wait_and_release();
   Planar b;
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, i
   constexpr int L = pl_dots(KIND, FIRST) - 1;
   double dot[L + 1] = {};
   if (b.live) {   // the same for the whole block
-    const int s = b.s, N = P.N, N2 = N * N, t = threadIdx.x, w = B + 2 * N;
+    const int s = b.s, N = P.N, N2 = N * N, t = threadIdx.x, B = blockDim.x, w = B + 2 * N;
     const double alpha = F.ks[s].alpha, beta = F.ks[s].beta, omega = F.ks[s].omega;
     const double* rhs = F.rhs[s];
     // the vector that the operator is applied to: X - q Y (p/v: X + beta (Z - omega Y))
@@ -259,11 +259,16 @@ __global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, i
         pl[h < N ? h : B + h] = hl >= 0 && hl < N2 ? value(hl + N2 * k) : 0.0;
       }
       const double hi = mine ? value(c + N2) : 0.0;
+      // the weights' loads in flight with the halo's, before the barrier: p/v and s/t at 91^3 together
+      // 159.4 -> 154.8 us
+      double e0 = 0.0, e1 = 0.0, e2 = 0.0, e3 = 0.0, e4 = 0.0, e5 = 0.0, e6 = 0.0;
+      if (b.inner) {
+        e0 = a0[c], e1 = a1[c], e2 = a2[c], e3 = a3[c], e4 = a4[c], e5 = a5[c], e6 = a6[c];
+      }
       __syncthreads();
       if (b.inner) {
         const double* o = pl + N + t;
-        const double y = planar_row(a0[c], a1[c], a2[c], a3[c], a4[c], a5[c], a6[c], mid, o[1], o[-1],
-                                    o[N], o[-N], hi, lo);
+        const double y = planar_row(e0, e1, e2, e3, e4, e5, e6, mid, o[1], o[-1], o[N], o[-N], hi, lo);
         if (KIND == PL_PV) {
           F.pk[1 - pp][s][c] = mid;
           F.vk[1 - pp][s][c] = y;
@@ -316,8 +321,8 @@ __global__ void __launch_bounds__(B, 1024 / B) k_planar(DevParams P, Fields F, i
 }
 
 // The pointwise ends: x/r (s = r - alpha v; x += alpha p + omega s; r = s - omega t; r0.r, r.r) and MR.
-template <int KIND, int B, bool FIRST>
-__global__ void __launch_bounds__(B) k_planar_end(DevParams P, Fields F, int pp) {
+template <int KIND, bool FIRST>
+__global__ void __launch_bounds__(kPlanarMost) k_planar_end(DevParams P, Fields F, int pp) {
   pdl_wait_and_release();
   Planar b;
   int done[4];
@@ -1015,18 +1020,13 @@ int xr_flat_blocks() {
 }
 
 
-template <int KIND, int B, bool FIRST>
-void launch_planar_b(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
-  if constexpr (KIND >= PL_XR)
-    launch_pdl(k_planar_end<KIND, B, FIRST>, planar_grid(P), B, 0, s, P, F, pp);
-  else   // two planes of N + B + N doubles: 41 KB at N = 1025
-    launch_pdl(k_planar<KIND, B, FIRST>, planar_grid(P), B, 16 * (size_t)(B + 2 * P.N), s, P, F, pp);
-}
 template <int KIND, bool FIRST>
 void launch_planar_f(const DevParams& P, const Fields& F, int pp, cudaStream_t s) {
-  if (P.pb == 128) launch_planar_b<KIND, 128, FIRST>(P, F, pp, s);
-  else if (P.pb == 256) launch_planar_b<KIND, 256, FIRST>(P, F, pp, s);
-  else launch_planar_b<KIND, 512, FIRST>(P, F, pp, s);
+  if constexpr (KIND >= PL_XR)
+    launch_pdl(k_planar_end<KIND, FIRST>, planar_grid(P), P.pb, 0, s, P, F, pp);
+  else   // two planes of N + pb + N doubles: 41 KB at N = 1025
+    launch_pdl(k_planar<KIND, FIRST>, planar_grid(P), P.pb, 16 * (size_t)(P.pb + 2 * P.N), s, P, F,
+               pp);
 }
 template <int KIND>
 void launch_planar(const DevParams& P, const Fields& F, int pp, bool first,

@@ -20,8 +20,10 @@
 // Every wait is bounded (kWaitNs on the GPU timer): a block whose wait runs out leaves the solve, the
 // others follow when theirs do, and the step reports HOSC_ECUDA.
 //
-// Measured against an iteration in three launches: FP64 21^3 25.4 -> 16.6 us, 41^3 49 -> 27.8 us (there half of it
-// FP64 instructions); mixed step at 41^3 226 -> 140 us, at 64^3 348 -> 242 us.
+// Measured against an iteration in three launches: FP64 21^3 25.4 -> 12.5 us, 31^3 35 -> 18.8 us, 41^3
+// 49 -> 24.9 us (there half of it FP64 instructions); mixed step at 41^3 226 -> 142 us, at 64^3
+// 348 -> 244 us. An iteration at 21^3 spends about 3 x 1.2 us on the exchanges' trip through L2, 3 x 0.5 us
+// on the writes before them becoming visible, 1.5 us on divisions; the rest is FP64 work and barriers.
 
 #include <math.h>
 
@@ -51,9 +53,11 @@ __device__ __forceinline__ void put_value(ulonglong2* p, double v, unsigned e) {
                "l"((b >> 32) | f)
                : "memory");
 }
+// An acquire: what the writer wrote before its row is visible to this thread, and to the block after its
+// next barrier.
 __device__ __forceinline__ bool get_value(const ulonglong2* p, unsigned e, double& v) {
   unsigned long long a, b;
-  asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+  asm volatile("ld.acquire.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
   v = __longlong_as_double((long long)((a & 0xffffffffull) | (b << 32)));
   return (unsigned)(a >> 32) == e && (unsigned)(b >> 32) == e;
 }
@@ -111,7 +115,6 @@ __device__ __noinline__ bool gather(ulonglong2* rows, int nr, int stride, int ro
     }
     s_g[w] = acc;
   }
-  fence_gpu();   // the others' writes that came before their rows
   __syncthreads();
   sum_groups<T, M>(s_g, tot);
   __syncthreads();
@@ -129,18 +132,45 @@ __device__ __forceinline__ bool exchange(Exchange& x, const typename Op::V (&v)[
                                        x.failed);
 }
 
+// xr_scalars for S systems at ks, its three serial chains side by side: the two quotients of beta in two
+// groups of S lanes (one division's time), the square root and the tests in another warp.
+template <int S>
+__device__ __forceinline__ void split_xr_scalars(const DevParams& P, KrylovScalars* ks,
+                                                 const double* tot) {
+  const int t = threadIdx.x, s = t % S;
+  if (t < 2 * S) {
+    const bool lo = t < S;
+    const double q = (lo ? tot[s] : ks[s].alpha) / (lo ? ks[s].rho : ks[s].omega);
+    const double q2 = __shfl_down_sync((1u << (2 * S)) - 1u, q, S);
+    if (lo) {   // not read where the system is done
+      ks[s].beta = q * q2;
+      ks[s].rho = tot[s];
+    }
+  } else if (t >= 32 && t < 32 + S && !ks[s].done) {
+    const double rnorm = sqrt(tot[S + s]);
+    const int iters = ks[s].iters + 1;
+    ks[s].rnorm = rnorm;
+    ks[s].iters = iters;
+    const bool conv = rnorm <= P.tol_lin * ks[s].r0norm;
+    if (conv || !isfinite(rnorm) || iters >= P.max_lin_iter || tot[s] == 0.0 || ks[s].omega == 0.0) {
+      ks[s].done = 1;
+      ks[s].status = conv ? 0 : HOSC_ENOCONV;
+    }
+  }
+}
+
 // ------------------------------------------------------------------ FP64 (planar)
 //
-// A block has one system, B nodes of the plane (i + N j, walls included) and up to KZ planes; a
-// system's blocks exchange among themselves and leave when it is done.
+// A block has one system, as many consecutive nodes of the plane (i + N j, walls included) as threads
+// and up to KZ planes; a system's blocks exchange among themselves and leave when it is done.
 
-template <int B, int KZ>
-constexpr size_t planar_state(int N) {   // operator rows and rhs, then KZ planes of B + 2 N values
+template <int KZ>
+size_t planar_state(int N, int B) {   // operator rows and rhs, then KZ planes of B + 2 N values
   return sizeof(double) * ((size_t)8 * KZ * B + (size_t)KZ * (B + 2 * N));
 }
 
-template <int B, int KZ>
-__global__ void __launch_bounds__(B, KZ <= 4 ? 512 / B : 1)
+template <int KZ>
+__global__ void __launch_bounds__(KZ <= 4 ? kPlanarMost : kPlanarMost / 2)
     k_solve_planar(DevParams P, Fields F) {
   extern __shared__ double sh[];
   __shared__ KrylovScalars k;
@@ -148,7 +178,7 @@ __global__ void __launch_bounds__(B, KZ <= 4 ? 512 / B : 1)
   __shared__ int failed;
   if (*F.halt) return;   // the same for every block
   const int s = (int)(blockIdx.x & 3u), t = threadIdx.x;
-  const int N = P.N, N2 = N * N, w = B + 2 * N;
+  const int N = P.N, N2 = N * N, B = blockDim.x, w = B + 2 * N;
   const int l0 = (int)(blockIdx.x >> 2) * B, l = l0 + t;
   const int k0 = 1 + (int)blockIdx.y * P.pkz, nk = min(P.pkz, N - 1 - k0);
   const unsigned chunks = gridDim.x >> 2;
@@ -279,7 +309,7 @@ __global__ void __launch_bounds__(B, KZ <= 4 ? 512 / B : 1)
       }
     ok = exchange<SumD, 2>(x, dr, tot);
     if (!ok) break;
-    if (t == 0) xr_scalars(P, k, tot[0], tot[1]);
+    split_xr_scalars<1>(P, &k, tot);
     __syncthreads();
   }
 #pragma unroll
@@ -471,8 +501,9 @@ __global__ void __launch_bounds__(kSolveBlock, 2) k_solve_mixed(DevParams P, Fie
         }
       ok = exchange<SumFF, 8>(x, acc, tot);
       if (!ok) break;
-      finish_xr(P, ks, tot);
+      split_xr_scalars<4>(P, ks, tot);
     }
+    __syncthreads();   // two warps write the scalars
   }
   if (!any && in)   // every right-hand side is zero (or none to solve): zero increments
     for (int kk = 0; kk < nk; ++kk) F.kx[c0 + N2 * kk] = zero;
@@ -490,15 +521,17 @@ __global__ void __launch_bounds__(kSolveBlock, 2) k_solve_mixed(DevParams P, Fie
 
 typedef void (*SolveFn)(DevParams, Fields);
 
-SolveFn planar_fn(int B, int KZ, int N, size_t* smem) {
-#define CASE(b, z)                         \
-  if (B == b && KZ == z) {                 \
-    *smem = planar_state<b, z>(N);         \
-    return k_solve_planar<b, z>;           \
-  }
-  CASE(128, 1) CASE(128, 2) CASE(128, 4) CASE(256, 1) CASE(256, 2) CASE(256, 4) CASE(256, 8)
-#undef CASE
-  return nullptr;
+int template_planes(int z) { return z <= 1 ? 1 : z <= 2 ? 2 : z <= 4 ? 4 : 8; }
+
+SolveFn planar_fn(int B, int z, int N, size_t* smem) {
+  const int KZ = template_planes(z);
+  *smem = KZ == 1 ? planar_state<1>(N, B) : KZ == 2 ? planar_state<2>(N, B)
+          : KZ == 4 ? planar_state<4>(N, B) : planar_state<8>(N, B);
+  // eight planes: registers for 256 threads; fewer than 160 leave the FP64 pipe idle (31^3 with 128: 20.7
+  // us an iteration, with 160 18.8)
+  if (KZ > 4 && (B > kPlanarMost / 2 || B < 160)) return nullptr;
+  return KZ == 1 ? k_solve_planar<1> : KZ == 2 ? k_solve_planar<2>
+         : KZ == 4 ? k_solve_planar<4> : k_solve_planar<8>;
 }
 SolveFn mixed_fn(int KZ, int N, size_t* smem) {
   *smem = KZ == 1 ? mixed_state<1>(N) : KZ == 2 ? mixed_state<2>(N) : mixed_state<4>(N);
@@ -518,8 +551,6 @@ long resident(SolveFn fn, int threads, size_t smem) {
   return (long)occ * device_sms();
 }
 
-int template_planes(int z) { return z <= 1 ? 1 : z <= 2 ? 2 : z <= 4 ? 4 : 8; }
-
 void launch_cooperative(SolveFn fn, dim3 grid, int threads, size_t smem, cudaStream_t s,
                         const DevParams& P, const Fields& F) {
   cudaLaunchConfig_t cfg = {};
@@ -537,9 +568,15 @@ void launch_cooperative(SolveFn fn, dim3 grid, int threads, size_t smem, cudaStr
 
 }  // namespace
 
-// Shapes of the one-launch solves: the least modelled time of a phase (the busiest SM's FP64
-// instructions, or planes, and the rows of the exchange) among the shapes whose blocks are all
-// resident. False when none is: the vectors do not fit on the chip.
+// Shapes of the one-launch solves: the least modelled time of an iteration among the shapes whose
+// blocks are all resident. False when none is: the vectors do not fit on the chip.
+//
+// FP64: microseconds of the busiest SM's FP64 instructions and of the exchange's rows, and what a form
+// of KZ planes costs beside them (one plane: both neighbours of every node come from memory; more than
+// two: registers). Fitted to every shape from 64 to 512 threads at 9^3 to 41^3; the chosen shape is
+// the fastest there or within 0.8 us of it. 21^3 (128, 3) -> (160, 2): 14.4 -> 12.5 us an iteration,
+// 25^3 (128, 4) -> (224, 2): 16.8 -> 13.8, 37^3 (256, 5) -> (352, 4): 23.1 -> 21.4. Mixed precision:
+// planes of the busiest SM and rows.
 bool solve_shape_planar(int N, int* pb, int* pkz) {
   // the answer for the last grid and device of this thread: asked at every set-up and every
   // allocation-free solve
@@ -554,17 +591,19 @@ bool solve_shape_planar(int N, int* pb, int* pkz) {
   const int sms = device_sms(), ni = N - 2;
   double best = 1e300;
   last = {N, device, 0, 0};
-  for (int B : {128, 256}) {
+  for (int B = 64; B <= kPlanarMost; B += 32) {
     if (2 * N > B) continue;
     const long chunks = (N * (long)N + B - 1) / B;
     for (int z = 1; z <= 8 && z <= ni; ++z) {
       const long rows = chunks * ((ni + z - 1) / z);
       if (rows > kSolveRows) continue;
+      const int KZ = template_planes(z);
       const double work = B / 32.0 * (12.0 * z + 20.0) + 2.0 * ((2 * N + 31) / 32) * z;
-      const double cost = work * (double)((4 * rows + sms - 1) / sms) + 0.5 * rows;
+      const double cost = 0.0094 * work * (double)((4 * rows + sms - 1) / sms) + 0.06 * rows +
+                          (KZ == 1 ? 0.7 : KZ == 2 ? 0.0 : KZ == 4 ? 1.2 : 1.6);
       if (cost >= best) continue;
       size_t smem = 0;
-      const SolveFn fn = planar_fn(B, template_planes(z), N, &smem);
+      const SolveFn fn = planar_fn(B, z, N, &smem);
       if (resident(fn, B, smem) < 4 * rows) continue;
       best = cost;
       last.pb = *pb = B;
@@ -611,7 +650,7 @@ void launch_solve(const DevParams& P, const Fields& F, cudaStream_t s) {
     const dim3 g((ni * ni + kSolveBlock - 1) / kSolveBlock, (ni + P.ckz - 1) / P.ckz);
     launch_cooperative(fn, g, kSolveBlock, smem, s, P, F);
   } else {
-    const SolveFn fn = planar_fn(P.pb, template_planes(P.pkz), P.N, &smem);
+    const SolveFn fn = planar_fn(P.pb, P.pkz, P.N, &smem);
     const dim3 g(4u * ((P.N * P.N + P.pb - 1) / P.pb), (ni + P.pkz - 1) / P.pkz);
     launch_cooperative(fn, g, P.pb, smem, s, P, F);
   }
