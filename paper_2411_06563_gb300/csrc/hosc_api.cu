@@ -857,10 +857,7 @@ hosc_status graph_steps(Ctx* c, long nsteps, bool stop_steady, hosc_info* info, 
   long done = 0;
   while (done < nsteps) {
     const long batch = (nsteps - done) < kRing ? (nsteps - done) : kRing;
-    const int stop = stop_steady ? 1 : 0;
-    CU(cudaMemsetAsync(F.halt, 0, sizeof(int), c->stream));
-    CU(cudaMemsetAsync(F.ring_pos, 0, sizeof(unsigned), c->stream));
-    CU(cudaMemcpyAsync(F.steady_stop, &stop, sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    launch_arm(F, stop_steady ? 1 : 0, c->stream);
     const int cur0 = c->cur, prev0 = c->P.have_prev, phase0 = c->phase;
     int cur = cur0, hp = prev0;
     if (c->P.sweep_fp32 && !c->shadow_valid) {   // float state copies for the first FP32 sweep
@@ -886,14 +883,16 @@ hosc_status graph_steps(Ctx* c, long nsteps, bool stop_steady, hosc_info* info, 
       cur ^= 1;
       hp = c->prm.use_history ? 1 : 0;
     }
-    unsigned n = 0;
-    CU(cudaMemcpyAsync(&n, F.ring_pos, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
-    CU(cudaStreamSynchronize(c->stream));
-    if (n > (unsigned)batch) n = (unsigned)batch;
-    CU(cudaMemcpyAsync(c->h_ring, F.ring, n * sizeof(StepRecord), cudaMemcpyDeviceToHost,
+    // the records of all the batch's steps, whether they ran or not, in one wait: a wait for their
+    // number first, copies from and to pageable memory and two memsets cost 11 us of a
+    // one-step call (21^3: 237 -> 226 us)
+    CU(cudaMemcpyAsync(c->h_ring_pos, F.ring_pos, sizeof(unsigned), cudaMemcpyDeviceToHost,
+                       c->stream));
+    CU(cudaMemcpyAsync(c->h_ring, F.ring, batch * sizeof(StepRecord), cudaMemcpyDeviceToHost,
                        c->stream));
     CU(cudaMemcpyAsync(c->h_rec, F.rec, sizeof(StepRecord), cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
+    const unsigned n = std::min(*c->h_ring_pos, (unsigned)batch);
     // the state advanced by the n steps that ran
     c->cur = cur0 ^ (int)(n & 1u);
     if (n > 0) c->P.have_prev = c->prm.use_history ? 1 : 0;
