@@ -152,7 +152,7 @@ void apply_tiles(Ctx* c) {
   c->P.tstages = c->tstages;
   c->P.tkernels = c->tkernels;
   c->P.xr_flat = c->xr_flat;
-  c->P.coop = c->coop_fits && !c->shape_chosen && !c->pooled && c->prm.solver == 0;
+  c->P.coop = c->coop_fits && !c->shape_chosen && !c->pooled;
   c->P.ckz = c->ckz;
   // the shared-plane kernels unless the caller has chosen a shape of the others
   c->P.plane = c->plane_fits && !c->shape_chosen && !c->merged && c->sx == 0 && c->tty == 0;
@@ -208,7 +208,7 @@ DevParams device_params(const hosc_params& p, int have_prev, int phase) {
   d.have_prev = have_prev;
   d.max_lin_iter = p.max_lin_iter;
   d.krylov_fp32 = (p.precision == HOSC_MIXED);
-  if (!d.krylov_fp32 && !(p.solver == 0 && solve_shape_planar(p.N, &d.pb, &d.pkz)))
+  if (!d.krylov_fp32 && !solve_shape_planar(p.N, p.solver, &d.pb, &d.pkz))
     planar_shape(p.N, &d.pb, &d.pkz);
   d.sweep_fp32 = (p.precision == HOSC_MIXED && phase == 0);
   d.h = 1.0 / (p.N - 1);
@@ -965,7 +965,7 @@ hosc_status make_ctx(const hosc_params* p, void* dev_ws, size_t bytes, void** ou
     c->ckz = c->kz;
   } else {
     int b = 0, z = 0;
-    c->coop_fits = p->solver == 0 && solve_shape_planar(p->N, &b, &z);
+    c->coop_fits = solve_shape_planar(p->N, p->solver, &b, &z);
   }
   c->plane_fits =
       p->precision == HOSC_MIXED && plane_shape(p->N, &c->ptx, &c->pty, &c->plz);

@@ -206,9 +206,9 @@ template <int Mp>
 constexpr int row_groups() { return Mp <= 8 ? 64 : 512 / Mp; }
 
 // The totals of M slots over the groups of s_g[group * Mp + slot] into tot, a warp a slot.
-template <class T, int M>
+template <class T, int M, int G = row_groups<pow2_at_least(M)>()>
 __device__ __forceinline__ void sum_groups(const double* s_g, double* tot) {
-  constexpr int Mp = pow2_at_least(M), G = row_groups<Mp>();
+  constexpr int Mp = pow2_at_least(M);
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int m = threadIdx.x >> 5; m < M; m += nw) {
     double a = lane < G ? s_g[lane * Mp + m] : 0.0;

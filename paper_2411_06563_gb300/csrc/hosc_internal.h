@@ -88,7 +88,7 @@ struct DevParams {
 };
 
 constexpr int kPlanarMost = 512;    // most threads a block of the planar kernels (a multiple of 32)
-constexpr int kSolveRows = 152;      // most rows (blocks) of a system in the one-launch FP64 solve
+constexpr int kSolveRows = 152;      // most rows (blocks) of a system in the one-launch FP64 solves
 constexpr int kExchValues = 8192;   // 16-byte values of the exchange buffer
 constexpr int kRing = 256;   // step records kept on the device between host reads
 
@@ -258,7 +258,7 @@ void launch_loop_cond(const Fields& F, unsigned long long handle, cudaStream_t s
 // The whole solve as one cooperative launch (P.coop): exchange buffer zeroed by the sources, scalars started by the
 // right-hand sides' kernel. The shapes it runs with on an N^3 grid; false when the grid is too large.
 void launch_solve(const DevParams& P, const Fields& F, cudaStream_t s);
-bool solve_shape_planar(int N, int* pb, int* pkz);
+bool solve_shape_planar(int N, int solver, int* pb, int* pkz);
 bool solve_shape_mixed(int N, int* kblock, int* kz);
 // Mark all four systems as iterating (for timing the Krylov kernels in isolation).
 void launch_krylov_activate(const Fields& F, cudaStream_t s);

@@ -96,11 +96,6 @@ constexpr int pl_slots(int kind, bool first) {
   return kind == PL_R2 ? 20 : 4 * pl_dots(kind, first);
 }
 
-__device__ __forceinline__ void b2_fail(KrylovScalars& k) {
-  k.done = 1;
-  k.status = HOSC_ENOCONV;
-}
-
 // The scalars that a launch of this kind leaves, and its algorithmic bytes.
 template <int KIND>
 __device__ __forceinline__ void planar_finish(const DevParams& P, const Fields& F,
@@ -110,53 +105,10 @@ __device__ __forceinline__ void planar_finish(const DevParams& P, const Fields& 
   if (KIND == PL_U2) finish_pv(F.ks, tot, false);
   if (KIND == PL_ST) finish_st(F.ks, tot);
   if (KIND == PL_XR) finish_xr(P, F.ks, tot);
-  if (KIND == PL_R1 && threadIdx.x < 4) {
-    KrylovScalars& k = F.ks[threadIdx.x];
-    const double rho1 = tot[threadIdx.x];
-    if (!k.done) {
-      if (k.rho == 0.0 || !isfinite(rho1)) {
-        b2_fail(k);
-      } else {
-        k.beta = k.alpha * rho1 / k.rho;
-        k.rho = rho1;
-      }
-    }
-  }
-  if (KIND == PL_R2 && threadIdx.x < 4) {
-    KrylovScalars& k = F.ks[threadIdx.x];
-    const double* d = tot + 5 * threadIdx.x;   // r1.r1, r1.r2, r2.r2, r0.r1, r0.r2
-    const double sig1 = d[0];
-    const double tau = sig1 > 0.0 ? d[1] / sig1 : 0.0;
-    const double sig2 = d[2] - tau * d[1];   // |r_2 - tau r_1|^2
-    if (!k.done) {
-      if (!(sig1 > 0.0) || !(sig2 > 0.0) || !isfinite(sig2)) {
-        b2_fail(k);
-      } else {
-        const double gp1 = d[3] / sig1, g2 = (d[4] - tau * d[3]) / sig2;
-        k.g2 = g2;
-        k.g1 = gp1 - tau * g2;
-        k.omega = g2;
-      }
-    }
-  }
-  if (KIND == PL_MR && threadIdx.x < 4) {
-    KrylovScalars& k = F.ks[threadIdx.x];
-    if (!k.done) {
-      const double rho1 = tot[threadIdx.x], rnorm = sqrt(tot[4 + threadIdx.x]);
-      k.rnorm = rnorm;
-      k.iters += 2;
-      const double rho0 = -k.omega * k.rho;
-      if (rnorm <= P.tol_lin * k.r0norm) {
-        k.done = 1;
-        k.status = 0;
-      } else if (!isfinite(rnorm) || k.iters >= P.max_lin_iter || rho0 == 0.0) {
-        b2_fail(k);
-      } else {
-        k.beta = k.alpha * rho1 / rho0;
-        k.rho = rho1;
-      }
-    }
-  }
+  const int q = threadIdx.x;
+  if (KIND == PL_R1 && q < 4) b2_r1_scalars(F.ks[q], tot[q]);
+  if (KIND == PL_R2 && q < 4) b2_r2_scalars(F.ks[q], tot + 5 * q);
+  if (KIND == PL_MR && q < 4) b2_mr_scalars(P, F.ks[q], tot[q], tot[4 + q]);
   constexpr int cls = KIND == PL_PV || KIND == PL_U1 || KIND == PL_U2 ? HOSC_K_BICG_PV
                       : KIND >= PL_XR                                 ? HOSC_K_BICG_XR
                                                                       : HOSC_K_BICG_ST;
@@ -282,33 +234,33 @@ __global__ void __launch_bounds__(kPlanarMost, 2) k_planar(DevParams P, Fields F
         } else if (KIND == PL_U1) {
           F.vk[0][s][c] = y;
           const double r0 = rhs[c];
-          dot[0] += r0 * y;
-          if (FIRST) dot[L] += r0 * r0;
+          dot[0] = fma(r0, y, dot[0]);
+          if (FIRST) dot[L] = fma(r0, r0, dot[L]);
         } else if (KIND == PL_R1) {
           (pp ? F.r[s] : F.t[s])[c] = mid;
           F.pk[0][s][c] = y;
-          const double r0 = X[c], u0 = FIRST ? r0 : r0 - beta * F.u0[s][c];
+          const double r0 = X[c], u0 = FIRST ? r0 : fma(-beta, F.u0[s][c], r0);
           F.u0[s][c] = u0;
-          F.x[s][c] = FIRST ? alpha * u0 : F.x[s][c] + alpha * u0;
-          dot[0] += rhs[c] * y;
+          F.x[s][c] = fma(alpha, u0, FIRST ? 0.0 : F.x[s][c]);
+          dot[0] = fma(rhs[c], y, dot[0]);
         } else if (KIND == PL_U2) {
           const double* r0 = pp ? F.r[s] : F.t[s];   // written by R1
-          F.u0[s][c] = r0[c] - beta * F.u0[s][c];
+          F.u0[s][c] = fma(-beta, F.u0[s][c], r0[c]);
           F.vk[1][s][c] = mid;
           F.u2[s][c] = y;
-          dot[0] += rhs[c] * y;
+          dot[0] = fma(rhs[c], y, dot[0]);
         } else {
           double* r0 = pp ? F.r[s] : F.t[s];
-          const double r0c = r0[c] - alpha * F.vk[1][s][c];
+          const double r0c = fma(-alpha, F.vk[1][s][c], r0[c]);
           r0[c] = r0c;
           F.pk[1][s][c] = mid;
           F.r2[s][c] = y;
-          F.x[s][c] += alpha * F.u0[s][c];
-          dot[0] += mid * mid;   // L = 4 here
-          dot[L / 4] += mid * y;
-          dot[L / 2] += y * y;
-          dot[3 * L / 4] += r0c * mid;
-          dot[L] += r0c * y;
+          F.x[s][c] = fma(alpha, F.u0[s][c], F.x[s][c]);
+          dot[0] = fma(mid, mid, dot[0]);   // L = 4 here
+          dot[L / 4] = fma(mid, y, dot[L / 4]);
+          dot[L / 2] = fma(y, y, dot[L / 2]);
+          dot[3 * L / 4] = fma(r0c, mid, dot[3 * L / 4]);
+          dot[L] = fma(r0c, y, dot[L]);
         }
       }
       lo = mid;
@@ -355,12 +307,12 @@ __global__ void __launch_bounds__(kPlanarMost) k_planar_end(DevParams P, Fields 
       for (int k = b.k0; k < b.k1; ++k) {
         const int c = b.l + N2 * k;
         const double r0c = r0[c], r1c = r1[c];
-        x[c] += g1 * r0c + g2 * r1c;
-        const double rn = r0c - g1 * r1c - g2 * r2[c];
+        x[c] = fma(g2, r1c, fma(g1, r0c, x[c]));
+        const double rn = fma(-g2, r2[c], fma(-g1, r1c, r0c));
         r0[c] = rn;
-        u0[c] -= g1 * u1[c] + g2 * u2[c];
-        dot[0] += rhs[c] * rn;
-        dot[1] += rn * rn;
+        u0[c] = fma(-g2, u2[c], fma(-g1, u1[c], u0[c]));
+        dot[0] = fma(rhs[c], rn, dot[0]);
+        dot[1] = fma(rn, rn, dot[1]);
       }
     }
   } else if (KIND == PL_XR && FIRST && b.inner) {

@@ -293,6 +293,56 @@ __device__ __forceinline__ void xr_scalars(const DevParams& P, KrylovScalars& k,
   }
 }
 
+// BiCGSTAB(2): rho_1 = rt.r_1 and beta after R1.
+__device__ __forceinline__ void b2_fail(KrylovScalars& k) {
+  k.done = 1;
+  k.status = HOSC_ENOCONV;
+}
+__device__ __forceinline__ void b2_r1_scalars(KrylovScalars& k, double rho1) {
+  if (k.done) return;
+  if (k.rho == 0.0 || !isfinite(rho1)) {
+    b2_fail(k);
+  } else {
+    k.beta = k.alpha * rho1 / k.rho;
+    k.rho = rho1;
+  }
+}
+
+// The minimal-residual coefficients from d = r_1.r_1, r_1.r_2, r_2.r_2, r_0.r_1, r_0.r_2.
+__device__ __forceinline__ void b2_r2_scalars(KrylovScalars& k, const double* d) {
+  if (k.done) return;
+  const double sig1 = d[0];
+  const double tau = sig1 > 0.0 ? d[1] / sig1 : 0.0;
+  const double sig2 = d[2] - tau * d[1];   // |r_2 - tau r_1|^2
+  if (!(sig1 > 0.0) || !(sig2 > 0.0) || !isfinite(sig2)) {
+    b2_fail(k);
+  } else {
+    const double gp1 = d[3] / sig1, g2 = (d[4] - tau * d[3]) / sig2;
+    k.g2 = g2;
+    k.g1 = gp1 - tau * g2;
+    k.omega = g2;
+  }
+}
+
+// The end of a cycle from rho_1 = rt.r_0 and rr = r_0.r_0.
+__device__ __forceinline__ void b2_mr_scalars(const DevParams& P, KrylovScalars& k, double rho1,
+                                              double rr) {
+  if (k.done) return;
+  const double rnorm = sqrt(rr);
+  k.rnorm = rnorm;
+  k.iters += 2;
+  const double rho0 = -k.omega * k.rho;
+  if (rnorm <= P.tol_lin * k.r0norm) {
+    k.done = 1;
+    k.status = 0;
+  } else if (!isfinite(rnorm) || k.iters >= P.max_lin_iter || rho0 == 0.0) {
+    b2_fail(k);
+  } else {
+    k.beta = k.alpha * rho1 / rho0;
+    k.rho = rho1;
+  }
+}
+
 // The same for the four systems at ks from the totals of a launch: slots 0..3 and 4..7.
 __device__ __forceinline__ void finish_pv(KrylovScalars* ks, const double* tot, bool first) {
   const int s = threadIdx.x;

@@ -127,7 +127,7 @@ extern "C" hosc_status hosc_bicgstab_noalloc(int N, const double* const* weights
            cudaStreamSynchronize(sm) == cudaSuccess;
   };
   // Every call shares the scratch and finds the previous call's contents.
-  if (solve_shape_planar(N, &P.pb, &P.pkz)) {
+  if (solve_shape_planar(N, 0, &P.pb, &P.pkz)) {
     // one launch (every grid up to HOSC_NOALLOC_MAX_N where its blocks are resident): the solver's
     // scalars, the halt flag and the exchanges start at zero
     F.exch = (ulonglong2*)F.rb.red;

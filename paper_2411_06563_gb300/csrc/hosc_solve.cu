@@ -73,11 +73,10 @@ struct Exchange {
 // Thread m < M of the block puts its value of the block's row and the block gathers the totals of all
 // rows, in the order of sum_rows, in tot (shared). A function of its own: inlined, its loops cost the
 // callers the registers that hold their vectors.
-template <class T, int M>
+template <class T, int M, int G>
 __device__ __noinline__ bool gather(ulonglong2* rows, int nr, int stride, int row, unsigned e,
                                     double mine, double* tot, int* failed) {
   constexpr int Mp = pow2_at_least(M);
-  constexpr int G = row_groups<Mp>();
   __shared__ double s_g[Mp * G];
   rows += (size_t)(e & 1u) * nr * stride;
   const int t = threadIdx.x;
@@ -116,7 +115,7 @@ __device__ __noinline__ bool gather(ulonglong2* rows, int nr, int stride, int ro
     s_g[w] = acc;
   }
   __syncthreads();
-  sum_groups<T, M>(s_g, tot);
+  sum_groups<T, M, G>(s_g, tot);
   __syncthreads();
   return *(volatile int*)failed == 0;
 }
@@ -124,11 +123,11 @@ __device__ __noinline__ bool gather(ulonglong2* rows, int nr, int stride, int ro
 // The totals of M values per thread over all blocks of the exchange, in tot (shared). Orders the
 // block's earlier writes to memory before the others' reads that follow. False when a wait ran out
 // (uniform over the block).
-template <class Op, int M>
+template <class Op, int M, int G = row_groups<pow2_at_least(M)>()>
 __device__ __forceinline__ bool exchange(Exchange& x, const typename Op::V (&v)[M], double* tot) {
   x.e += 1;
   const typename Op::V mine = block_total<Op, M>(v);
-  return gather<typename Op::Total, M>(x.rows, x.nr, x.stride, x.mine, x.e, Op::value(mine), tot,
+  return gather<typename Op::Total, M, G>(x.rows, x.nr, x.stride, x.mine, x.e, Op::value(mine), tot,
                                        x.failed);
 }
 
@@ -169,6 +168,112 @@ size_t planar_state(int N, int B) {   // operator rows and rhs, then KZ planes o
   return sizeof(double) * ((size_t)8 * KZ * B + (size_t)KZ * (B + 2 * N));
 }
 
+// Most threads of the BiCGSTAB(2) form: seven vectors of KZ planes in registers.
+constexpr int b2_threads(int KZ) { return KZ <= 2 ? kPlanarMost : KZ == 4 ? 384 : 256; }
+
+static_assert(4 * 2 * 5 * kSolveRows <= kExchValues, "the rows of five values exceed the buffer");
+
+// A thread's nodes of its block's planes, with the operator rows, rhs and the planes in shared memory.
+template <int KZ>
+struct Slab {
+  int s, N, N2, B, w, t, c0, k0, nk, hs, hc;
+  bool in, has_halo, hin, below, above;
+  double* a;        // weight q of plane kk: a[(8 kk + q) B + t]; rhs at q = 7
+  double* planes;   // plane kk: nodes l0 - N .. l0 + B + N
+
+  __device__ __forceinline__ Slab(const DevParams& P, double* sh) {
+    s = (int)(blockIdx.x & 3u), t = threadIdx.x;
+    N = P.N, N2 = N * N, B = blockDim.x, w = B + 2 * N;
+    const int l0 = (int)(blockIdx.x >> 2) * B, l = l0 + t;
+    k0 = 1 + (int)blockIdx.y * P.pkz, nk = min(P.pkz, N - 1 - k0);
+    // the node before or after the chunk whose value this thread fetches (2 N <= B)
+    const int hl = t < N ? l0 - N + t : l0 + B + (t - N);
+    hs = t < N ? t : B + t;
+    in = inside(l);
+    has_halo = t < 2 * N, hin = has_halo && inside(hl);
+    below = in && k0 > 1, above = in && k0 + nk < N - 1;
+    c0 = l + N2 * k0, hc = hl + N2 * k0;
+    a = sh;
+    planes = sh + 8 * KZ * B;
+  }
+  __device__ __forceinline__ bool inside(int q) const {   // node q of the plane lies inside the walls
+    if (q < 0 || q >= N2) return false;
+    const int j = q / N, i = q - j * N;
+    return i > 0 && i < N - 1 && j > 0 && j < N - 1;
+  }
+  __device__ __forceinline__ Exchange rows(const Fields& F, int stride, int* failed) const {
+    const unsigned chunks = gridDim.x >> 2;
+    Exchange x;
+    x.nr = (int)(chunks * gridDim.y);
+    x.stride = stride;
+    x.mine = (int)((blockIdx.x >> 2) + chunks * blockIdx.y);
+    x.rows = F.exch + (size_t)s * 2 * x.nr * x.stride;
+    x.e = 0;
+    x.failed = failed;
+    return x;
+  }
+  __device__ __forceinline__ bool mine(int kk) const { return in && kk < nk; }
+  __device__ __forceinline__ int c(int kk) const { return c0 + N2 * kk; }
+  __device__ __forceinline__ double r0(int kk) const { return a[(8 * kk + 7) * B + t]; }
+  // rhs into r (zero elsewhere), operator rows and rhs into shared memory
+  __device__ __forceinline__ void load(const Fields& F, double (&r)[KZ]) {
+    const double* rhs = F.rhs[s];
+    const double* const* A = s < 3 ? F.Am : F.Ae;
+#pragma unroll
+    for (int kk = 0; kk < KZ; ++kk) {
+      r[kk] = 0.0;
+      if (mine(kk)) {
+        r[kk] = rhs[c(kk)];
+        a[(8 * kk + 7) * B + t] = r[kk];
+#pragma unroll
+        for (int q = 0; q < 7; ++q) a[(8 * kk + q) * B + t] = A[q][c(kk)];
+      }
+    }
+  }
+  // the operator on own values f (registers) and the others' values val(c): y of each plane
+  template <class Val>
+  __device__ __forceinline__ void apply(const double (&f)[KZ], double (&y)[KZ], Val val) const {
+    const double lo = below ? val(c0 - N2) : 0.0, hi = above ? val(c0 + N2 * nk) : 0.0;
+#pragma unroll
+    for (int kk = 0; kk < KZ; ++kk) {
+      const double h = hin && kk < nk ? val(hc + N2 * kk) : 0.0;
+      planes[kk * w + N + t] = f[kk];   // zero on the walls
+      if (has_halo) planes[kk * w + hs] = h;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < KZ; ++kk) {
+      if (!mine(kk)) continue;
+      const double* o = planes + kk * w + N + t;
+      const double* ak = a + 8 * kk * B + t;
+      const double zp = kk + 1 < nk && kk + 1 < KZ ? f[kk + 1 < KZ ? kk + 1 : kk] : hi;
+      const double zm = kk > 0 ? f[kk > 0 ? kk - 1 : 0] : lo;
+      y[kk] = planar_row(ak[0], ak[B], ak[2 * B], ak[3 * B], ak[4 * B], ak[5 * B], ak[6 * B], f[kk],
+                         o[1], o[-1], o[N], o[-N], zp, zm);
+    }
+  }
+  // the end of a solve: the increments, the scalars and the algorithmic bytes, from the words an
+  // iteration of the three kernel classes (pvw, stw: of weights, the momentum ones counted once)
+  __device__ __forceinline__ void store(const Fields& F, const double (&xi)[KZ], KrylovScalars& k,
+                                        bool ok, bool first_row, double iters, double pv, double pvw,
+                                        double st, double stw, double xr) const {
+#pragma unroll
+    for (int kk = 0; kk < KZ; ++kk)
+      if (mine(kk)) F.x[s][c(kk)] = xi[kk];
+    if (!ok && t == 0) {
+      k.done = 1;
+      k.status = HOSC_ECUDA;
+    }
+    if (t == 0 && (first_row || !ok)) {
+      F.ks[s] = k;
+      const double ni = N - 2, n3 = 8.0 * ni * ni * ni * iters, wt = s == 0 || s == 3 ? 1.0 : 0.0;
+      atomicAdd(F.alg_bytes + HOSC_K_BICG_PV, n3 * (pv + wt * pvw));
+      atomicAdd(F.alg_bytes + HOSC_K_BICG_ST, n3 * (st + wt * stw));
+      atomicAdd(F.alg_bytes + HOSC_K_BICG_XR, n3 * xr);
+    }
+  }
+};
+
 template <int KZ>
 __global__ void __launch_bounds__(KZ <= 4 ? kPlanarMost : kPlanarMost / 2)
     k_solve_planar(DevParams P, Fields F) {
@@ -177,71 +282,23 @@ __global__ void __launch_bounds__(KZ <= 4 ? kPlanarMost : kPlanarMost / 2)
   __shared__ double tot[2];
   __shared__ int failed;
   if (*F.halt) return;   // the same for every block
-  const int s = (int)(blockIdx.x & 3u), t = threadIdx.x;
-  const int N = P.N, N2 = N * N, B = blockDim.x, w = B + 2 * N;
-  const int l0 = (int)(blockIdx.x >> 2) * B, l = l0 + t;
-  const int k0 = 1 + (int)blockIdx.y * P.pkz, nk = min(P.pkz, N - 1 - k0);
-  const unsigned chunks = gridDim.x >> 2;
-  Exchange x;
-  x.nr = (int)(chunks * gridDim.y);
-  x.stride = 2;
-  x.mine = (int)((blockIdx.x >> 2) + chunks * blockIdx.y);
-  x.rows = F.exch + (size_t)s * 2 * x.nr * x.stride;
-  x.e = 0;
-  x.failed = &failed;
-  auto inside = [&](int q) {   // node q of the plane lies inside the walls
-    if (q < 0 || q >= N2) return false;
-    const int j = q / N, i = q - j * N;
-    return i > 0 && i < N - 1 && j > 0 && j < N - 1;
-  };
-  const bool in = inside(l);
-  // the node before or after the chunk whose value this thread fetches (2 N <= B)
-  const int hl = t < N ? l0 - N + t : l0 + B + (t - N), hs = t < N ? t : B + t;
-  const bool has_halo = t < 2 * N, hin = has_halo && inside(hl);
-  const bool below = in && k0 > 1, above = in && k0 + nk < N - 1;
-  double* a = sh;                    // weight q of plane kk: a[(8 kk + q) B + t]; rhs at q = 7
-  double* planes = sh + 8 * KZ * B;  // plane kk: nodes l0 - N .. l0 + B + N
+  Slab<KZ> b(P, sh);
+  Exchange x = b.rows(F, 2, &failed);
+  const int t = b.t, s = b.s;
   const double* rhs = F.rhs[s];
   double *R = F.r[s], *Q = F.pk[0][s], *V = F.vk[0][s];
   double r[KZ], xi[KZ], p[KZ], v[KZ], tv[KZ];
-  const double* const* A = s < 3 ? F.Am : F.Ae;
-  const int c0 = l + N2 * k0;
+  b.load(F, r);
 #pragma unroll
   for (int kk = 0; kk < KZ; ++kk) {
-    r[kk] = xi[kk] = p[kk] = v[kk] = tv[kk] = 0.0;
-    if (in && kk < nk) {
-      r[kk] = p[kk] = rhs[c0 + N2 * kk];
-      a[(8 * kk + 7) * B + t] = r[kk];
-#pragma unroll
-      for (int q = 0; q < 7; ++q) a[(8 * kk + q) * B + t] = A[q][c0 + N2 * kk];
-    }
+    p[kk] = r[kk];
+    xi[kk] = v[kk] = tv[kk] = 0.0;
   }
   if (t == 0) {
     k = F.ks[s];
     failed = 0;
   }
   __syncthreads();
-  // the operator on own values f (registers) and the others' values val(c): y of each plane
-  auto stencil = [&](const double (&f)[KZ], double (&y)[KZ], auto val) {
-    const double lo = below ? val(c0 - N2) : 0.0, hi = above ? val(c0 + N2 * nk) : 0.0;
-#pragma unroll
-    for (int kk = 0; kk < KZ; ++kk) {
-      const double h = hin && kk < nk ? val(hl + N2 * (k0 + kk)) : 0.0;
-      planes[kk * w + N + t] = f[kk];   // zero on the walls
-      if (has_halo) planes[kk * w + hs] = h;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < KZ; ++kk) {
-      if (!in || kk >= nk) continue;
-      const double* o = planes + kk * w + N + t;
-      const double* ak = a + 8 * kk * B + t;
-      const double zp = kk + 1 < nk && kk + 1 < KZ ? f[kk + 1 < KZ ? kk + 1 : kk] : hi;
-      const double zm = kk > 0 ? f[kk > 0 ? kk - 1 : 0] : lo;
-      y[kk] = planar_row(ak[0], ak[B], ak[2 * B], ak[3 * B], ak[4 * B], ak[5 * B], ak[6 * B], f[kk],
-                         o[1], o[-1], o[N], o[-N], zp, zm);
-    }
-  };
   bool ok = true;
   for (int it = 0; !k.done; ++it) {
     // p = r + beta (p - omega v), v = A p
@@ -249,17 +306,17 @@ __global__ void __launch_bounds__(KZ <= 4 ? kPlanarMost : kPlanarMost / 2)
     const double beta = k.beta;
     double d2[2] = {0.0, 0.0};
     if (first) {
-      stencil(p, v, [&](int c) { return rhs[c]; });
+      b.apply(p, v, [&](int c) { return rhs[c]; });
     } else {
 #pragma unroll
       for (int kk = 0; kk < KZ; ++kk) p[kk] = fma(beta, p[kk], r[kk]);
-      stencil(p, v, [&](int c) { return fma(beta, __ldcg(Q + c), __ldcg(R + c)); });
+      b.apply(p, v, [&](int c) { return fma(beta, __ldcg(Q + c), __ldcg(R + c)); });
     }
 #pragma unroll
     for (int kk = 0; kk < KZ; ++kk)
-      if (in && kk < nk) {
-        V[c0 + N2 * kk] = v[kk];
-        const double r0 = a[(8 * kk + 7) * B + t];
+      if (b.mine(kk)) {
+        V[b.c(kk)] = v[kk];
+        const double r0 = b.r0(kk);
         d2[0] = fma(r0, v[kk], d2[0]);
         if (first) d2[1] = fma(r0, r0, d2[1]);
       }
@@ -278,13 +335,13 @@ __global__ void __launch_bounds__(KZ <= 4 ? kPlanarMost : kPlanarMost / 2)
 #pragma unroll
     for (int kk = 0; kk < KZ; ++kk) r[kk] = fma(-alpha, v[kk], r[kk]);
     if (first)
-      stencil(r, tv, [&](int c) { return fma(-alpha, __ldcg(V + c), rhs[c]); });
+      b.apply(r, tv, [&](int c) { return fma(-alpha, __ldcg(V + c), rhs[c]); });
     else
-      stencil(r, tv, [&](int c) { return fma(-alpha, __ldcg(V + c), __ldcg(R + c)); });
+      b.apply(r, tv, [&](int c) { return fma(-alpha, __ldcg(V + c), __ldcg(R + c)); });
     double ds[2] = {0.0, 0.0};
 #pragma unroll
     for (int kk = 0; kk < KZ; ++kk)
-      if (in && kk < nk) {
+      if (b.mine(kk)) {
         ds[0] = fma(tv[kk], r[kk], ds[0]);
         ds[1] = fma(tv[kk], tv[kk], ds[1]);
       }
@@ -297,14 +354,14 @@ __global__ void __launch_bounds__(KZ <= 4 ? kPlanarMost : kPlanarMost / 2)
     double dr[2] = {0.0, 0.0};
 #pragma unroll
     for (int kk = 0; kk < KZ; ++kk)
-      if (in && kk < nk) {
-        const int c = c0 + N2 * kk;
+      if (b.mine(kk)) {
+        const int c = b.c(kk);
         xi[kk] = fma(omega, r[kk], fma(alpha, p[kk], xi[kk]));
         r[kk] = fma(-omega, tv[kk], r[kk]);
         p[kk] = fma(-omega, v[kk], p[kk]);
         R[c] = r[kk];
         Q[c] = p[kk];
-        dr[0] = fma(a[(8 * kk + 7) * B + t], r[kk], dr[0]);
+        dr[0] = fma(b.r0(kk), r[kk], dr[0]);
         dr[1] = fma(r[kk], r[kk], dr[1]);
       }
     ok = exchange<SumD, 2>(x, dr, tot);
@@ -312,21 +369,161 @@ __global__ void __launch_bounds__(KZ <= 4 ? kPlanarMost : kPlanarMost / 2)
     split_xr_scalars<1>(P, &k, tot);
     __syncthreads();
   }
+  b.store(F, xi, k, ok, x.mine == 0, k.iters, 6.0, 7.0, 3.0, 7.0, 8.0);
+}
+
+// BiCGSTAB(2): the five phases of a cycle (see the kernels of hosc_krylov.cu, whose arithmetic this is). A
+// neighbour's value is r_0 - beta u_0 in U1, r_0 - alpha u_1 in R1, r_1 - beta u_1 in U2 and r_1 -
+// alpha u_2 in R2, so that r_0 and u_0 are written after MR, u_1 after U1, r_1 after R1, u_2 after U2.
+// A 34^3 box (9 cycles' iterations a step): 467 us a step with five launches a cycle, 352 so.
+template <int KZ>
+__global__ void __launch_bounds__(b2_threads(KZ)) k_solve_b2(DevParams P, Fields F) {
+  extern __shared__ double sh[];
+  __shared__ KrylovScalars k;
+  __shared__ double tot[5];
+  __shared__ int failed;
+  if (*F.halt) return;   // the same for every block
+  Slab<KZ> b(P, sh);
+  Exchange x = b.rows(F, 5, &failed);
+  const int t = b.t, s = b.s;
+  const double* rhs = F.rhs[s];
+  double *R0 = F.r[s], *R1 = F.pk[0][s], *U0 = F.u0[s], *U1 = F.vk[0][s], *U2 = F.u2[s];
+  double r0[KZ], r1[KZ], r2[KZ], u0[KZ], u1[KZ], u2[KZ], xi[KZ];
+  b.load(F, r0);
 #pragma unroll
-  for (int kk = 0; kk < KZ; ++kk)
-    if (in && kk < nk) F.x[s][c0 + N2 * kk] = xi[kk];
-  if (!ok && t == 0) {
-    k.done = 1;
-    k.status = HOSC_ECUDA;
+  for (int kk = 0; kk < KZ; ++kk) {
+    u0[kk] = r0[kk];
+    r1[kk] = r2[kk] = u1[kk] = u2[kk] = xi[kk] = 0.0;
   }
-  if (t == 0 && (x.mine == 0 || !ok)) {
-    F.ks[s] = k;
-    // algorithmic bytes of the three kernel classes (the momentum weights counted once)
-    const double ni = N - 2, n3 = 8.0 * ni * ni * ni * k.iters, wt = s == 0 || s == 3 ? 7.0 : 0.0;
-    atomicAdd(F.alg_bytes + HOSC_K_BICG_PV, n3 * (6.0 + wt));
-    atomicAdd(F.alg_bytes + HOSC_K_BICG_ST, n3 * (3.0 + wt));
-    atomicAdd(F.alg_bytes + HOSC_K_BICG_XR, n3 * 8.0);
+  if (t == 0) {
+    k = F.ks[s];
+    failed = 0;
   }
+  __syncthreads();
+  bool ok = true;
+  for (int it = 0; !k.done; ++it) {
+    const bool first = it == 0;
+    {   // U1: u_0 = r_0 - beta u_0, u_1 = A u_0
+      const double beta = k.beta;
+      double d2[2] = {0.0, 0.0};
+      if (first) {
+        b.apply(u0, u1, [&](int c) { return rhs[c]; });
+      } else {
+#pragma unroll
+        for (int kk = 0; kk < KZ; ++kk) u0[kk] = fma(-beta, u0[kk], r0[kk]);
+        b.apply(u0, u1, [&](int c) { return fma(-beta, __ldcg(U0 + c), __ldcg(R0 + c)); });
+      }
+#pragma unroll
+      for (int kk = 0; kk < KZ; ++kk)
+        if (b.mine(kk)) {
+          U1[b.c(kk)] = u1[kk];
+          const double rt = b.r0(kk);
+          d2[0] = fma(rt, u1[kk], d2[0]);
+          if (first) d2[1] = fma(rt, rt, d2[1]);
+        }
+      if (first) {
+        ok = exchange<SumD, 2>(x, d2, tot);
+      } else {
+        double d1[1] = {d2[0]};
+        ok = exchange<SumD, 1>(x, d1, tot);
+      }
+      if (!ok) break;
+      if (t == 0) pv_scalars(k, tot[0], first ? tot[1] : 0.0, first);
+      __syncthreads();
+      if (k.done) break;
+    }
+    {   // R1: r_0 -= alpha u_1, r_1 = A r_0; x += alpha u_0
+      const double alpha = k.alpha;
+      double d1[1] = {0.0};
+#pragma unroll
+      for (int kk = 0; kk < KZ; ++kk) {
+        r0[kk] = fma(-alpha, u1[kk], r0[kk]);
+        xi[kk] = fma(alpha, u0[kk], xi[kk]);
+      }
+      if (first)
+        b.apply(r0, r1, [&](int c) { return fma(-alpha, __ldcg(U1 + c), rhs[c]); });
+      else
+        b.apply(r0, r1, [&](int c) { return fma(-alpha, __ldcg(U1 + c), __ldcg(R0 + c)); });
+#pragma unroll
+      for (int kk = 0; kk < KZ; ++kk)
+        if (b.mine(kk)) {
+          R1[b.c(kk)] = r1[kk];
+          d1[0] = fma(b.r0(kk), r1[kk], d1[0]);
+        }
+      ok = exchange<SumD, 1>(x, d1, tot);
+      if (!ok) break;
+      if (t == 0) b2_r1_scalars(k, tot[0]);
+      __syncthreads();
+      if (k.done) break;
+    }
+    {   // U2: u_0 = r_0 - beta u_0, u_1 = r_1 - beta u_1, u_2 = A u_1
+      const double beta = k.beta;
+      double d1[1] = {0.0};
+#pragma unroll
+      for (int kk = 0; kk < KZ; ++kk) {
+        u0[kk] = fma(-beta, u0[kk], r0[kk]);
+        u1[kk] = fma(-beta, u1[kk], r1[kk]);
+      }
+      b.apply(u1, u2, [&](int c) { return fma(-beta, __ldcg(U1 + c), __ldcg(R1 + c)); });
+#pragma unroll
+      for (int kk = 0; kk < KZ; ++kk)
+        if (b.mine(kk)) {
+          U2[b.c(kk)] = u2[kk];
+          d1[0] = fma(b.r0(kk), u2[kk], d1[0]);
+        }
+      ok = exchange<SumD, 1>(x, d1, tot);
+      if (!ok) break;
+      if (t == 0) pv_scalars(k, tot[0], 0.0, false);
+      __syncthreads();
+      if (k.done) break;
+    }
+    {   // R2: r_0 -= alpha u_1, r_1 -= alpha u_2, r_2 = A r_1; x += alpha u_0
+      const double alpha = k.alpha;
+      double d[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int kk = 0; kk < KZ; ++kk) {
+        r0[kk] = fma(-alpha, u1[kk], r0[kk]);
+        r1[kk] = fma(-alpha, u2[kk], r1[kk]);
+        xi[kk] = fma(alpha, u0[kk], xi[kk]);
+      }
+      b.apply(r1, r2, [&](int c) { return fma(-alpha, __ldcg(U2 + c), __ldcg(R1 + c)); });
+#pragma unroll
+      for (int kk = 0; kk < KZ; ++kk)
+        if (b.mine(kk)) {
+          d[0] = fma(r1[kk], r1[kk], d[0]);
+          d[1] = fma(r1[kk], r2[kk], d[1]);
+          d[2] = fma(r2[kk], r2[kk], d[2]);
+          d[3] = fma(r0[kk], r1[kk], d[3]);
+          d[4] = fma(r0[kk], r2[kk], d[4]);
+        }
+      // the rows of the kernel have 20 slots: 16 groups
+      ok = exchange<SumD, 5, row_groups<32>()>(x, d, tot);
+      if (!ok) break;
+      if (t == 0) b2_r2_scalars(k, tot);
+      __syncthreads();
+      if (k.done) break;
+    }
+    {   // MR
+      const double g1 = k.g1, g2 = k.g2;
+      double dr[2] = {0.0, 0.0};
+#pragma unroll
+      for (int kk = 0; kk < KZ; ++kk)
+        if (b.mine(kk)) {
+          xi[kk] = fma(g2, r1[kk], fma(g1, r0[kk], xi[kk]));
+          r0[kk] = fma(-g2, r2[kk], fma(-g1, r1[kk], r0[kk]));
+          u0[kk] = fma(-g2, u2[kk], fma(-g1, u1[kk], u0[kk]));
+          R0[b.c(kk)] = r0[kk];
+          U0[b.c(kk)] = u0[kk];
+          dr[0] = fma(b.r0(kk), r0[kk], dr[0]);
+          dr[1] = fma(r0[kk], r0[kk], dr[1]);
+        }
+      ok = exchange<SumD, 2>(x, dr, tot);
+      if (!ok) break;
+      if (t == 0) b2_mr_scalars(P, k, tot[0], tot[1]);
+      __syncthreads();
+    }
+  }
+  b.store(F, xi, k, ok, x.mine == 0, 0.5 * k.iters, 12.0, 14.0, 19.0, 14.0, 11.0);
 }
 
 // ------------------------------------------------------------------ mixed (interleaved float)
@@ -523,10 +720,15 @@ typedef void (*SolveFn)(DevParams, Fields);
 
 int template_planes(int z) { return z <= 1 ? 1 : z <= 2 ? 2 : z <= 4 ? 4 : 8; }
 
-SolveFn planar_fn(int B, int z, int N, size_t* smem) {
+SolveFn planar_fn(int solver, int B, int z, int N, size_t* smem) {
   const int KZ = template_planes(z);
   *smem = KZ == 1 ? planar_state<1>(N, B) : KZ == 2 ? planar_state<2>(N, B)
           : KZ == 4 ? planar_state<4>(N, B) : planar_state<8>(N, B);
+  if (solver == 1) {
+    if (B > b2_threads(KZ)) return nullptr;
+    return KZ == 1 ? k_solve_b2<1> : KZ == 2 ? k_solve_b2<2>
+           : KZ == 4 ? k_solve_b2<4> : k_solve_b2<8>;
+  }
   // eight planes: registers for 256 threads; fewer than 160 leave the FP64 pipe idle (31^3 with 128: 20.7
   // us an iteration, with 160 18.8)
   if (KZ > 4 && (B > kPlanarMost / 2 || B < 160)) return nullptr;
@@ -577,10 +779,11 @@ void launch_cooperative(SolveFn fn, dim3 grid, int threads, size_t smem, cudaStr
 // the fastest there or within 0.8 us of it. 21^3 (128, 3) -> (160, 2): 14.4 -> 12.5 us an iteration,
 // 25^3 (128, 4) -> (224, 2): 16.8 -> 13.8, 37^3 (256, 5) -> (352, 4): 23.1 -> 21.4. Mixed precision:
 // planes of the busiest SM and rows.
-bool solve_shape_planar(int N, int* pb, int* pkz) {
+bool solve_shape_planar(int N, int solver, int* pb, int* pkz) {
   // the answer for the last grid and device of this thread: asked at every set-up and every
   // allocation-free solve
-  static thread_local struct { int N, device, pb, pkz; } last = {0, -1, 0, 0};
+  static thread_local struct Last { int N, device, pb, pkz; } of[2] = {{0, -1, 0, 0}, {0, -1, 0, 0}};
+  Last& last = of[solver];
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess) return false;
   if (last.N == N && last.device == device) {
@@ -603,7 +806,7 @@ bool solve_shape_planar(int N, int* pb, int* pkz) {
                           (KZ == 1 ? 0.7 : KZ == 2 ? 0.0 : KZ == 4 ? 1.2 : 1.6);
       if (cost >= best) continue;
       size_t smem = 0;
-      const SolveFn fn = planar_fn(B, z, N, &smem);
+      const SolveFn fn = planar_fn(solver, B, z, N, &smem);
       if (resident(fn, B, smem) < 4 * rows) continue;
       best = cost;
       last.pb = *pb = B;
@@ -650,7 +853,7 @@ void launch_solve(const DevParams& P, const Fields& F, cudaStream_t s) {
     const dim3 g((ni * ni + kSolveBlock - 1) / kSolveBlock, (ni + P.ckz - 1) / P.ckz);
     launch_cooperative(fn, g, kSolveBlock, smem, s, P, F);
   } else {
-    const SolveFn fn = planar_fn(P.pb, P.pkz, P.N, &smem);
+    const SolveFn fn = planar_fn(P.solver, P.pb, P.pkz, P.N, &smem);
     const dim3 g(4u * ((P.N * P.N + P.pb - 1) / P.pb), (ni + P.pkz - 1) / P.pkz);
     launch_cooperative(fn, g, P.pb, smem, s, P, F);
   }
