@@ -20,12 +20,14 @@
 // Every wait is bounded (kWaitNs on the GPU timer): a block whose wait runs out leaves the solve, the
 // others follow when theirs do, and the step reports HOSC_ECUDA.
 //
-// Measured against an iteration in three launches: FP64 21^3 25.4 -> 12.5 us, 31^3 35 -> 18.8 us, 41^3
-// 49 -> 24.9 us (there half of it FP64 instructions); mixed step at 41^3 226 -> 142 us, at 64^3
-// 348 -> 244 us. An iteration at 21^3 spends about 3 x 1.2 us on the exchanges' trip through L2, 3 x 0.5 us
+// Measured against an iteration in three launches: FP64 21^3 25.4 -> 12.1 us, 31^3 35 -> 18.1 us, 41^3
+// 49 -> 24.2 us (there half of it FP64 instructions); mixed step at 41^3 226 -> 133 us, at 64^3
+// 348 -> 232 us. An iteration at 21^3 spends about 3 x 1.2 us on the exchanges' trip through L2, 3 x 0.5 us
 // on the writes before them becoming visible, 1.5 us on divisions; the rest is FP64 work and barriers.
 
 #include <math.h>
+
+#include <type_traits>
 
 #include "hosc_device.cuh"
 #include "hosc_internal.h"
@@ -71,9 +73,11 @@ struct Exchange {
 };
 
 // Thread m < M of the block puts its value of the block's row and the block gathers the totals of all
-// rows, in the order of sum_rows, in tot (shared). A function of its own: inlined, its loops cost the
-// callers the registers that hold their vectors.
-template <class T, int M, int G>
+// rows, in the order of sum_rows, in tot (shared), K rows of a sum in flight. A function of its own:
+// inlined, its loops cost the callers the registers that hold their vectors; what it uses itself they
+// have to keep clear of all the same, so K is small (a step with K = 4, 2 and 1: 21^3 FP64 351, 331 and
+// 327 us, 64^3 mixed 244, 232 and 236; two sums side by side, eight in flight: 398 and 286).
+template <class T, int M, int G, int K>
 __device__ __noinline__ bool gather(ulonglong2* rows, int nr, int stride, int row, unsigned e,
                                     double mine, double* tot, int* failed) {
   constexpr int Mp = pow2_at_least(M);
@@ -88,14 +92,14 @@ __device__ __noinline__ bool gather(ulonglong2* rows, int nr, int stride, int ro
     const int m = w % Mp;
     double acc = 0.0;
     if (m < M) {
-      for (int r = w / Mp; r < nr; r += 4 * G) {
-        const int n = min(4, (nr - r + G - 1) / G);   // rows r, r + G, ... of this pass
-        double a[4];
+      for (int r = w / Mp; r < nr; r += K * G) {
+        const int n = min(K, (nr - r + G - 1) / G);   // rows r, r + G, ... of this pass
+        double a[K];
         unsigned long long t0 = 0;
         for (unsigned spin = 0;; ++spin) {
           bool ok = true;
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
+          for (int q = 0; q < K; ++q)
             if (q < n) ok &= get_value(rows + (r + q * G) * stride + m, e, a[q]);
           if (ok) break;
           if ((spin & 255u) == 255u) {
@@ -108,7 +112,7 @@ __device__ __noinline__ bool gather(ulonglong2* rows, int nr, int stride, int ro
           }
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+        for (int q = 0; q < K; ++q)
           if (q < n) acc = T::add(acc, a[q]);
       }
     }
@@ -127,7 +131,9 @@ template <class Op, int M, int G = row_groups<pow2_at_least(M)>()>
 __device__ __forceinline__ bool exchange(Exchange& x, const typename Op::V (&v)[M], double* tot) {
   x.e += 1;
   const typename Op::V mine = block_total<Op, M>(v);
-  return gather<typename Op::Total, M, G>(x.rows, x.nr, x.stride, x.mine, x.e, Op::value(mine), tot,
+    // the FP64 shapes mostly have no more rows than groups, the mixed ones up to four times as many
+  constexpr int K = std::is_same<Op, typename Op::Total>::value ? 1 : 2;
+  return gather<typename Op::Total, M, G, K>(x.rows, x.nr, x.stride, x.mine, x.e, Op::value(mine), tot,
                                        x.failed);
 }
 
@@ -375,7 +381,7 @@ __global__ void __launch_bounds__(KZ <= 4 ? kPlanarMost : kPlanarMost / 2)
 // BiCGSTAB(2): the five phases of a cycle (see the kernels of hosc_krylov.cu, whose arithmetic this is). A
 // neighbour's value is r_0 - beta u_0 in U1, r_0 - alpha u_1 in R1, r_1 - beta u_1 in U2 and r_1 -
 // alpha u_2 in R2, so that r_0 and u_0 are written after MR, u_1 after U1, r_1 after R1, u_2 after U2.
-// A 34^3 box (9 cycles' iterations a step): 467 us a step with five launches a cycle, 352 so.
+// A 34^3 box (9 cycles' iterations a step): 467 us a step with five launches a cycle, 308 so.
 template <int KZ>
 __global__ void __launch_bounds__(b2_threads(KZ)) k_solve_b2(DevParams P, Fields F) {
   extern __shared__ double sh[];
