@@ -54,13 +54,11 @@ WORKLOADS = {
 # _kernel_shape gives it); any other configuration, or a kernel changed since its capture,
 # reports null.
 NCU_TRAFFIC = {
-    # profiles/k4_pv_cavity101_mixed.md, "In-step DRAM traffic" (40 launches each)
-    ("cavity101", "k_bicg_pv", ("register", 256, 9, 0)): 105.0e6,
-    ("cavity101", "k_bicg_pv", ("register", 384, 9, 0)): 104.7e6,
-    # profiles/k7_pv_bulk_copy_cavity101_mixed.md (50 in-step launches each)
-    ("cavity101", "k_bicg_pv", ("bulk-copy", 2, 33, 6)): 96.2e6,
-    ("cavity101", "k_bicg_st", ("register", 384, 9, 0)): 57.3e6,
-    ("cavity101", "k_bicg_xr", ("flat",)): 98.7e6,
+    # profiles/in_step_dram_cavity101_mixed.md (33 to 66 launches each)
+    ("cavity101", "k_bicg_pv", ("register", 384, 9, 0)): 98.3e6,
+    ("cavity101", "k_bicg_pv", ("bulk-copy", 4, 19, 4)): 96.6e6,
+    ("cavity101", "k_bicg_st", ("register", 384, 9, 0)): 56.3e6,
+    ("cavity101", "k_bicg_xr", ("register", 384, 9, 0)): 95.5e6,
 }
 
 

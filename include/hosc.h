@@ -261,7 +261,9 @@ hosc_status hosc_get_params(void* ctx, hosc_params* out);
  * records per launch). enable(on != 0) resets the accumulators; read returns, for one kernel
  * class, the summed event milliseconds, the launch count and the algorithmic bytes those launches
  * moved (each array element read or written once per launch, counting only the systems still
- * iterating). The algorithmic-byte counters run whether or not timing is on. Outputs may be NULL. */
+ * iterating). A solve that runs as one launch is timed and counted as one launch of the p/v class,
+ * its bytes under the three classes. The algorithmic-byte counters run whether or not timing is on.
+ * Outputs may be NULL. */
 hosc_status hosc_profile_enable(void* ctx, int on);
 hosc_status hosc_profile_read(void* ctx, int kernel_id, double* total_ms, long* launches,
                               double* alg_bytes);
@@ -286,8 +288,12 @@ hosc_status hosc_time_kernel(void* ctx, int kernel_id, int reps, double* ms_per_
  * narrow = 1 selects the kernels compiled for at most 64 registers per thread (more resident
  * blocks), 0 those with more (80 for the three-kernel form, 128 for the merged form). The
  * default (384 threads, wide, kz from the wave model below; on grids whose solve runs as one launch
- * 256 threads) is chosen from N at creation.
- * Changing it drops the captured steps (captured again at the next step). HOSC_EINVAL for a shape
+ * 256 threads) is chosen from N at creation. On grids whose vectors fit on the chip (mixed precision
+ * up to about 68^3, FP64 up to about 42^3) the solve is one cooperative launch until a shape is set
+ * here or by one of the calls below, and from 104^3 up p/v and s/t share planes in shared memory until
+ * then; a call that sets a shape selects the kernels it describes, also with the default values. The
+ * one-launch solve with the default shape and its kernel-by-kernel form give the same bits.
+ * Changing the shape drops the captured steps (captured again at the next step). HOSC_EINVAL for a shape
  * outside these limits, HOSC_ESTATE in the middle of a stage-by-stage step. The FP64 solve has
  * one thread per node and ignores the setting. */
 hosc_status hosc_set_tiles(void* ctx, int kblock, int kz, int narrow);
@@ -345,7 +351,9 @@ int hosc_get_krylov_merged(void* ctx);
  * {64, 96, 128, 160, 192, 256, 320, 384} and kz in 1..33 whose modelled cost (waves of
  * resident blocks on this GPU, from the kernels' occupancy, times kz + 2 planes streamed per
  * block) is within 1.5x of the least, for both register budgets (narrow 0 and 1), time the
- * four fastest again with 4 reps launches each and keep the fastest; then time the other
+ * four fastest again with 4 reps launches each and keep the fastest (on grids whose solve is one
+ * launch that form stays, and from 104^3 up the shared-plane kernels stay where they are the faster);
+ * then time the other
  * iteration form (hosc_set_krylov_merged)
  * at that shape and keep the faster; with the three-kernel form, then time the
  * staged p/v and s/t kernels (hosc_set_stencil_tiles) for tiles sx in {8, 16, ..., 64},
@@ -378,9 +386,10 @@ long hosc_kernel_launches(void* ctx);
  * pool sized at start-up) already owns the device memory, so that a cudaMalloc beside it would
  * fail or fragment the pool, and solvers that run under a fixed device-memory budget decided
  * before the first step. The paper has no counterpart; this is an interface of this library.
- * The call is synchronous: every 4 to 16 iterations it copies the four systems' solver scalars to
- * a host array and waits for the stream (cudaStreamSynchronize) to test convergence, and it
- * returns once the solve has finished.
+ * The call is synchronous: the solve is one cooperative launch that stops by itself, after which the
+ * four systems' solver scalars are copied to a host array and the stream is waited for
+ * (cudaStreamSynchronize). Where the device cannot hold that launch's blocks at once it runs kernel by
+ * kernel and reads the scalars every 4 to 16 iterations.
  *
  * Solves A_mom x_s = rhs_s for s = u, v, w and A_ene x_theta = rhs_theta with the same kernels as
  * hosc_step (FP64 BiCGSTAB from x = 0, stop when ||r|| <= tol ||r_0||), on the interior nodes of
@@ -396,7 +405,8 @@ long hosc_kernel_launches(void* ctx);
  * current: make that first call before any stream capture. All calls share the array and it keeps
  * the last call's contents (each call clears what must start at zero), so calls that overlap on
  * the GPU race: serialise them (one stream, or wait between calls). Returns HOSC_ENOCONV if a
- * system did not converge within max_iter, HOSC_ECUDA on a CUDA error. */
+ * system did not converge within max_iter, HOSC_ECUDA on a CUDA error or when a wait of one block for
+ * another ran past its 2 s. */
 #define HOSC_NOALLOC_MAX_N 41
 hosc_status hosc_bicgstab_noalloc(int N, const double* const* weights, const double* const* rhs,
                                   double* const* x, double tol, int max_iter, int* iters_out,

@@ -59,8 +59,8 @@ __global__ void k_loop_cond(const KrylovScalars* ks, cudaGraphConditionalHandle 
 // times the SMs; the three momentum blocks of a chunk are neighbours in the grid, so their weights
 // come from L2. A block's partial goes to its row's slot of its system; the last block of the launch
 // sums all rows. The shape (B, pkz) has the least modelled load of the busiest SM (planar_shape).
-// Measured, alone: p/v 137 -> 84.7 us, s/t 117 -> 75.9, x/r 74.5 -> 46.4 at 91^3; 14.4 -> 7.4, 14.2 ->
-// 7.5, 12.3 -> 7.6 at 21^3.
+// Measured, alone: p/v 137 -> 82.1 us, s/t 117 -> 71.6, x/r 74.5 -> 45.7 at 91^3; 14.4 -> 8.6, 14.2 ->
+// 7.4, 12.3 -> 9.3 at 21^3.
 //
 // BiCGSTAB (solver = 0): p/v, s/t, x/r. BiCGSTAB(2) (Sleijpen and Fokkema's BiCGSTAB(ell) with
 // ell = 2; shadow residual rt = r_0 = rhs), one cycle in five kernels:
