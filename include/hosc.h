@@ -352,9 +352,8 @@ int hosc_get_krylov_merged(void* ctx);
  * resident blocks on this GPU, from the kernels' occupancy, times kz + 2 planes streamed per
  * block) is within 1.5x of the least, for both register budgets (narrow 0 and 1), time the
  * four fastest again with 4 reps launches each and keep the fastest (on grids whose solve is one
- * launch that form stays, and from 104^3 up the shared-plane kernels stay where they are the faster);
- * then time the other
- * iteration form (hosc_set_krylov_merged)
+ * launch that form stays and this ends the search; from 104^3 up the shared-plane kernels stay where they
+ * are the faster); then time the other iteration form (hosc_set_krylov_merged)
  * at that shape and keep the faster; with the three-kernel form, then time the
  * staged p/v and s/t kernels (hosc_set_stencil_tiles) for tiles sx in {8, 16, ..., 64},
  * sy in {4, 8} and skz in 1..33 within 1.5x of their least modelled cost, and the bulk-copy

@@ -1789,7 +1789,6 @@ hosc_status hosc_autotune(void* ctx, int reps, int* kblock_out, int* kz_out, dou
   if (c->stage != 0) return HOSC_ESTATE;
   if (!c->P.krylov_fp32) return HOSC_EINVAL;
   CU(cudaSetDevice(c->device));
-  // where the one-launch solve runs it stays: the shapes found are those of the kernels beside it
   struct KeepChoice {
     Ctx* c;
     bool chosen;
@@ -1800,6 +1799,7 @@ hosc_status hosc_autotune(void* ctx, int reps, int* kblock_out, int* kz_out, dou
     }
   } keep{c, c->shape_chosen};
   const bool plane0 = c->P.plane != 0;   // the default p/v and s/t of this grid: timed at the end
+  const bool one_launch = c->P.coop != 0;   // it stays, with the register shape found beside it
   if (!c->plane_fits && !c->coop_fits) keep.chosen = true;
   {   // the register kernels first
     hosc_status s0 = hosc_set_stencil_tiles(c, 0, 0, 0);
@@ -1869,7 +1869,7 @@ hosc_status hosc_autotune(void* ctx, int reps, int* kblock_out, int* kz_out, dou
   st = hosc_set_tiles(c, best_b, best_z, best_n);
   if (st) return st;
   // The other iteration form (two or three kernels) at the shape found.
-  {
+  if (!one_launch) {
     const int other = 1 - c->merged;
     c->merged = other;
     apply_tiles(c);
@@ -1890,7 +1890,8 @@ hosc_status hosc_autotune(void* ctx, int reps, int* kblock_out, int* kz_out, dou
       best = tot;
     }
   }
-  if (c->merged) {   // the staged kernels implement the three-kernel form only
+  // the staged kernels implement the three-kernel form only
+  if (c->merged || one_launch) {
     st = hosc_set_stencil_tiles(c, 0, 0, 0);
     if (!st) st = hosc_set_tma_tiles(c, 0, 0, 3, 3);
     if (!st) st = hosc_set_xr_form(c, 0);
