@@ -572,7 +572,8 @@ hosc_status run_stage(Ctx* c, int stage) {
       }
       prof_end(c, HOSC_K_UPDATE);
       if (st) return st;
-      if (c->P.krylov_fp32) c->shadow_valid = true;   // the update writes the float copies too
+      // the update writes the float copies of what it writes: valid copies stay valid, and copies that
+      // were not made before the step (FP64 sweeps do not read them) are not complete after it
       // increments: x4 + u, v, w, theta read, u, v, w, theta written; div: V read, div written;
       // pressure: p, div read, p written
       c->host_bytes[HOSC_K_UPDATE] += 8.0 * (n3 * 12 + ni3 * 4 + ni3 * 3);
@@ -1117,7 +1118,9 @@ hosc_status ctx_collect_round(void* ctx, bool wait, hosc_info* info, bool* stead
   c->cur = c->round_cur0 ^ (int)(n & 1u);
   if (n > 0) {
     c->P.have_prev = c->prm.use_history ? 1 : 0;
-    c->shadow_valid = true;
+    // a round of FP32 sweeps starts from complete float copies; one of FP64 sweeps leaves them as valid
+    // as they were
+    if (c->P.sweep_fp32) c->shadow_valid = true;
   }
   bool st_steady = false;
   hosc_status st = fold_records(c, n, info, &st_steady);
