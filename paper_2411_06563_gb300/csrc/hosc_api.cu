@@ -721,7 +721,8 @@ bool first_apart(const DevParams& P) { return !P.krylov_fp32 || P.lean; }
 // (the forms without one: the initialisation), then a conditional WHILE node whose body (captured on
 // s1) runs two iterations (the ping-pong buffers return to their parity) and sets the condition on the
 // device, then the update kernels. Nothing in the step waits on the host. cur and
-// have_prev are those of the step's level n.
+// have_prev are those of the step's level n. A refused launch does not end a capture by itself: the step
+// without it would run, so the launches' error is returned (a caller clears older errors first).
 cudaError_t append_step(Ctx* c, cudaStream_t s0, cudaStream_t s1, int cur, int have_prev) {
   DevParams P = c->P;
   P.have_prev = have_prev;
@@ -732,7 +733,7 @@ cudaError_t append_step(Ctx* c, cudaStream_t s0, cudaStream_t s1, int cur, int h
   if (P.coop) {
     launch_solve(P, F, s0);
     launch_update(P, F, cur, 1, s0);
-    return cudaSuccess;
+    return cudaGetLastError();
   }
   const int apart = first_apart(P) ? 1 : 0;
   if (apart) append_iteration(P, F, 0, true, s0);
@@ -766,13 +767,15 @@ cudaError_t append_step(Ctx* c, cudaStream_t s0, cudaStream_t s1, int cur, int h
     }
   }
   launch_update(P, F, cur, 1, s0);
-  return e;
+  const cudaError_t el = cudaGetLastError();
+  return e == cudaSuccess ? el : e;
 }
 
 // Capture one step at the context's current level into an executable graph.
 hosc_status capture_step(Ctx* c, cudaGraphExec_t* out) {
   cudaStream_t s0 = c->cap[0], s1 = c->cap[1];
   cudaGraph_t g = nullptr;
+  cudaGetLastError();
   CU(cudaGraphCreate(&g, 0));
   cudaError_t e = cudaStreamBeginCaptureToGraph(s0, g, nullptr, nullptr, 0,
                                                 cudaStreamCaptureModeThreadLocal);
@@ -858,6 +861,7 @@ hosc_status graph_steps(Ctx* c, long nsteps, bool stop_steady, hosc_info* info, 
   long done = 0;
   while (done < nsteps) {
     const long batch = (nsteps - done) < kRing ? (nsteps - done) : kRing;
+    cudaGetLastError();   // of earlier calls
     launch_arm(F, stop_steady ? 1 : 0, c->stream);
     const int cur0 = c->cur, prev0 = c->P.have_prev, phase0 = c->phase;
     int cur = cur0, hp = prev0;
@@ -865,6 +869,11 @@ hosc_status graph_steps(Ctx* c, long nsteps, bool stop_steady, hosc_info* info, 
       launch_shadow(c->P, F, cur0, prev0, c->stream);
       c->launches += 1;
       c->shadow_valid = true;
+    }
+    hosc_status armed = check_launch();
+    if (armed) {
+      c->shadow_valid = false;
+      return armed;
     }
     for (long q = 0; q < batch; ++q) {
       cudaGraphExec_t& ge = c->graph[phase0][cur][hp];
@@ -1027,11 +1036,17 @@ hosc_status ctx_enqueue_round(void* ctx, int n) {
   CU(cudaSetDevice(c->device));
   const Fields& F = c->F;
   ctx_begin_round(c, n);
+  cudaGetLastError();   // of earlier calls
   launch_arm(F, 1, c->stream);
   if (c->P.sweep_fp32 && !c->shadow_valid) {
     launch_shadow(c->P, F, c->cur, c->P.have_prev, c->stream);
     c->launches += 1;
     c->shadow_valid = true;
+  }
+  const hosc_status armed = check_launch();
+  if (armed) {
+    c->shadow_valid = false;
+    return armed;
   }
   int cur = c->cur, hp = c->P.have_prev;
   for (int q = 0; q < n; ++q) {

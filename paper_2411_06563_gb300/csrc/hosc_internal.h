@@ -99,6 +99,14 @@ struct KrylovScalars {
   int done, iters, status, pad;
 };
 
+// Outcome of a system at the end of a step. HOSC_ECUDA when a bounded wait inside a Krylov kernel ran
+// out, or when the solve never ended: a launch of it did not run, and the increments are not this
+// step's. (The merged form, run by the host, may stop at its last iteration with the system still open.)
+__host__ __device__ inline int system_status(const KrylovScalars& k, int merged) {
+  if (k.status == HOSC_ECUDA || (!k.done && (!merged || k.r0norm == 0.0))) return HOSC_ECUDA;
+  return k.status != 0 ? HOSC_ENOCONV : HOSC_OK;
+}
+
 // What one step reports, resident in device memory (one small D2H copy per host call).
 struct StepRecord {
   double res;        // max |chi^{n+1} - chi^n|

@@ -88,6 +88,7 @@ void drop_exec(Pool* P) {
 hosc_status capture_round(Pool* P) {
   const auto t0 = std::chrono::steady_clock::now();
   drop_exec(P);
+  cudaGetLastError();   // of earlier calls
   PCU(cudaStreamBeginCapture(P->stream, cudaStreamCaptureModeThreadLocal));
   hosc_status st = HOSC_OK;
   cudaError_t e = cudaEventRecord(P->fork, P->stream);

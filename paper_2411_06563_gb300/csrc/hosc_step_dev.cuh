@@ -779,9 +779,8 @@ __device__ __forceinline__ void k_finish_record_body(const DevParams& P, const F
   for (int s = 0; s < 4; ++s) {
     r->iters[s] = F.ks[s].iters;
     r->lin_status[s] = F.ks[s].status;
-    // HOSC_ECUDA: a bounded wait inside a Krylov kernel ran out; anything else: no convergence
-    if (F.ks[s].status == HOSC_ECUDA) st = HOSC_ECUDA;
-    else if (F.ks[s].status != 0 && st != HOSC_ECUDA) st = HOSC_ENOCONV;
+    const int q_st = system_status(F.ks[s], P.merged);
+    if (q_st != HOSC_OK && st != HOSC_ECUDA) st = q_st;
     const double q = F.ks[s].r0norm > 0.0 ? F.ks[s].rnorm / F.ks[s].r0norm : 0.0;
     lres = fmax(lres, isfinite(q) ? q : INFINITY);
   }

@@ -1,0 +1,147 @@
+"""The host code that chooses, captures and launches the kernels, on a device played on the host
+(fake_device.cpp): which kernels a call leads to, and what becomes of a launch that is refused."""
+
+import ctypes
+import os
+import shutil
+import subprocess
+
+import pytest
+
+from paper_2411_06563_gb300 import hosc as H
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2411_06563_gb300", "csrc")
+FP64, MIXED = H.HOSC_FP64, H.HOSC_MIXED
+
+
+@pytest.fixture(scope="module")
+def fake_path(tmp_path_factory):
+    if shutil.which("g++") is None or not os.path.isdir("/usr/local/cuda/include"):
+        pytest.skip("no C++ compiler or CUDA headers")
+    out = str(tmp_path_factory.mktemp("fake") / "libhosc_fake.so")
+    subprocess.run(["g++", "-x", "c++", "-std=c++17", "-O1", "-fPIC", "-shared", "-I",
+                    "/usr/local/cuda/include", "-I", os.path.join(ROOT, "include"), "-I", CSRC,
+                    os.path.join(CSRC, "hosc_api.cu"), os.path.join(CSRC, "hosc_pool.cu"),
+                    os.path.join(ROOT, "tests", "fake_device.cpp"), "-Wl,-Bsymbolic", "-o", out],
+                   check=True, timeout=300)
+    return out
+
+
+class Fake:
+    def __init__(self, lib):
+        self.lib = lib
+        lib.fake_log.restype = ctypes.c_char_p
+        lib.fake_cost.argtypes = [ctypes.c_char_p, ctypes.c_double]
+
+    def log(self):
+        return self.lib.fake_log().decode().split("\n")[:-1]
+
+    def clear(self):
+        self.lib.fake_clear()
+
+    def refuse(self, name, launches=-1):
+        self.lib.fake_refuse(name.encode(), launches)
+
+    def cost(self, name, ms):
+        self.lib.fake_cost(name.encode(), ms)
+
+
+@pytest.fixture()
+def fake(fake_path, monkeypatch):
+    monkeypatch.setattr(H, "LIB_PATH", fake_path)
+    monkeypatch.setattr(H, "_lib", None)
+    H.lib().fake_reset()
+    return Fake(H.lib())
+
+
+def _params(N, precision, **kw):
+    p = H.hosc_default_params(N, 1e4, 1.0, 0.75)
+    p.precision = precision
+    p.use_history = 0
+    for k, v in kw.items():
+        setattr(p, k, v)
+    return p
+
+
+# ------------------------------------------------------------------ refused launches
+
+# one launch (FP64, mixed, BiCGSTAB(2)), planar and register kernels in the loop
+STEPS = [(21, FP64, 0, "arm viscosity sources rhs solve update"),
+         (30, MIXED, 0, "arm shadow viscosity sources rhs solve update"),
+         (21, FP64, 1, "solve update"),
+         (50, FP64, 0, "arm viscosity sources rhs pv st xr loop update"),
+         (50, FP64, 1, "b2 loop update"),
+         (75, MIXED, 0, "arm shadow viscosity sources rhs pv st xr loop update")]
+
+
+@pytest.mark.parametrize("N,precision,solver,name",
+                         [(N, pr, so, n) for N, pr, so, names in STEPS for n in names.split()])
+def test_a_refused_launch_fails_the_step(fake, N, precision, solver, name):
+    """No step is reported that ran without one of its launches; the next call, launched kernel by
+    kernel where the capture failed, is whole again."""
+    with H.Cavity(_params(N, precision, solver=solver)) as cav:
+        fake.refuse(name, 1)
+        st, info = H.hosc_step(cav.h, 2)
+        assert st == H.HOSC_ECUDA and info.steps == 0
+        fake.clear()
+        st, info = H.hosc_step(cav.h, 2)
+        assert st == H.HOSC_OK and info.steps == 2
+        ran = [line.split()[0] for line in fake.log()]
+        assert "update" in ran
+        for q in ("viscosity", "sources", "rhs"):
+            assert ran.count(q) == 2
+        if precision == MIXED and name in ("arm", "shadow"):
+            assert "shadow" in ran   # the float copies that the refused call did not make
+
+
+@pytest.mark.parametrize("mode", [H.HOSC_POOL_STREAMS, H.HOSC_POOL_GRAPH])
+@pytest.mark.parametrize("name", ["arm", "pv", "update"])
+def test_a_refused_launch_fails_the_round(fake, mode, name):
+    p = _params(30, MIXED)
+    st, pool = H.hosc_pool_create(H.hosc_workspace_bytes(p) + 1, 2, mode, 0)
+    assert st == 0 and H.hosc_pool_admit(pool, p, 100)[0] == 0
+    fake.refuse(name, 1)
+    assert H.hosc_pool_run(pool, 1)[0] == H.HOSC_ECUDA
+    H.hosc_pool_destroy(pool)
+
+
+def test_an_older_error_is_not_the_steps(fake):
+    """An error that an earlier call left behind does not fail a step that ran."""
+    with H.Cavity(_params(21, FP64)) as cav, H.Cavity(_params(21, FP64)) as other:
+        fake.refuse("diagnostics", 1)
+        fake.refuse("finish", 1)
+        assert H.hosc_diagnostics(other.h, 21)[0] == H.HOSC_ECUDA
+        assert H.hosc_step(cav.h, 1)[0] == H.HOSC_OK
+
+
+def test_outcome_of_a_system(tmp_path):
+    """A system whose solve did not end is no success (one left open by the host's last iteration of
+    the merged form is, as its residual tells)."""
+    src = tmp_path / "outcome.cpp"
+    src.write_text(r"""
+#include <cuda_runtime.h>
+#include <stdio.h>
+#include <string.h>
+#include "hosc.h"
+#include "hosc_internal.h"
+int main() {
+  struct { int done, status; double r0; int merged; } c[] = {
+      {1, 0, 1, 0}, {1, 0, 0, 0}, {1, HOSC_ENOCONV, 1, 0}, {1, HOSC_ECUDA, 1, 0}, {0, 0, 0, 0},
+      {0, 0, 1, 0}, {0, 0, 1, 1}, {0, 0, 0, 1}};
+  for (auto& q : c) {
+    hosc::KrylovScalars k;
+    memset(&k, 0, sizeof(k));
+    k.done = q.done, k.status = q.status, k.r0norm = q.r0;
+    printf("%d ", hosc::system_status(k, q.merged));
+  }
+}
+""")
+    exe = str(tmp_path / "outcome")
+    subprocess.run(["g++", "-std=c++17", "-I", "/usr/local/cuda/include", "-I",
+                    os.path.join(ROOT, "include"), "-I", CSRC, str(src), "-o", exe], check=True,
+                   timeout=120)
+    out = [int(v) for v in subprocess.run([exe], check=True, capture_output=True, text=True,
+                                          timeout=60).stdout.split()]
+    OK, NO, EC = H.HOSC_OK, H.HOSC_ENOCONV, H.HOSC_ECUDA
+    assert out == [OK, OK, NO, EC, EC, EC, OK, EC]
