@@ -340,8 +340,9 @@ int hosc_get_xr_form(void* ctx);
  * folding the x, r update of iteration i-1 into the p, v kernel of iteration i and obtaining
  * r_0.r_{i+1} for beta from r_0.s and r_0.t of the s, t kernel (the same method; the
  * convergence test sees the true residual one kernel later); 0 (the default) runs the three
- * kernels p/v, s/t, x/r. HOSC_EINVAL for another value or when the current launch shape does not suit the form,
- * HOSC_ESTATE mid-step. Drops the captured steps. hosc_get_krylov_merged returns the current
+ * kernels p/v, s/t, x/r. A default block of more than 256 threads gives way to one of 128 while the
+ * form is merged. HOSC_EINVAL for another value or when the launch shape set by hosc_set_tiles (or found
+ * by the autotuner) does not suit the form, which changes nothing; HOSC_ESTATE mid-step. Drops the captured steps. hosc_get_krylov_merged returns the current
  * form (-1 for a NULL context). */
 hosc_status hosc_set_krylov_merged(void* ctx, int merged);
 int hosc_get_krylov_merged(void* ctx);

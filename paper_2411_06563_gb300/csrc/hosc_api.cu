@@ -79,6 +79,8 @@ struct Ctx {
   // the one-launch solve: the grid is small enough for it, the caller has chosen no launch shape, and
   // the context is not a pool's member
   bool coop_fits = false, shape_chosen = false, pooled = false;
+  bool tiles_set = false;   // kblock, kz and narrow are the caller's (or the autotuner's)
+  int wide_b = 0, wide_z = 0;   // the default that gave way to the merged form (0: none did)
   int ckz = 0;
   bool plane_fits = false;                 // shared-plane kernels
   int ptx = 1, pty = 1, plz = 1;
@@ -176,8 +178,25 @@ bool stencil_tiles_valid(const Ctx* c, int sx, int sy, int skz) {
          staged_wave_cost(c->prm.N, sx, sy, skz, device_sms()) < 1e299;
 }
 
+constexpr int kMergedMost = 256;   // threads a block of the merged form's kernels at most
+
+// A shape for the merged form: 128 threads, planes by the wave model.
+void merged_tiles(int N, int* kblock, int* kz) {
+  const int sms = device_sms();
+  double best = INFINITY;
+  *kblock = 128;
+  *kz = 1;
+  for (int z = 1; z <= std::min(N - 2, 16); ++z) {
+    const double cost = krylov4_wave_cost(N, *kblock, z, 0, 0, sms);
+    if (cost < best) {
+      best = cost;
+      *kz = z;
+    }
+  }
+}
+
 bool tiles_valid(const Ctx* c, int kblock, int kz, int narrow) {
-  if (kblock < 64 || kblock > ((narrow || c->P.merged) ? 256 : 384) || kblock % 32 != 0)
+  if (kblock < 64 || kblock > ((narrow || c->P.merged) ? kMergedMost : 384) || kblock % 32 != 0)
     return false;
   if (narrow != 0 && narrow != 1) return false;
   if (kz < 1 || kz > c->prm.N - 2) return false;
@@ -1660,6 +1679,7 @@ hosc_status hosc_set_tiles(void* ctx, int kblock, int kz, int narrow) {
   if (c->stage != 0) return HOSC_ESTATE;
   if (!tiles_valid(c, kblock, kz, narrow)) return HOSC_EINVAL;
   choose_shape(c);
+  c->tiles_set = true;
   if (kblock != c->kblock || kz != c->kz || narrow != c->narrow) {
     c->kblock = c->P.kblock = kblock;
     c->kz = c->P.kz = kz;
@@ -1763,18 +1783,28 @@ hosc_status hosc_set_krylov_merged(void* ctx, int merged) {
   Ctx* c = (Ctx*)ctx;
   if (!c || (merged != 0 && merged != 1)) return HOSC_EINVAL;
   if (c->stage != 0) return HOSC_ESTATE;
-  choose_shape(c);
   if (merged != c->merged) {
-    const int save = c->merged;
+    const int save_b = c->kblock, save_z = c->kz;
+    // a default block that the merged form does not take (384 threads) gives way to one that it does,
+    // and comes back with the three kernels; a block that was set stays and may be refused
+    if (merged && !c->tiles_set && c->kblock > kMergedMost)
+      merged_tiles(c->prm.N, &c->kblock, &c->kz);
+    else if (!merged && !c->tiles_set && c->wide_b)
+      c->kblock = c->wide_b, c->kz = c->wide_z;
     c->merged = merged;
     apply_tiles(c);
     if (!tiles_valid(c, c->kblock, c->kz, c->narrow)) {
-      c->merged = save;
+      c->merged = 1 - merged;
+      c->kblock = save_b;
+      c->kz = save_z;
       apply_tiles(c);
       return HOSC_EINVAL;
     }
+    c->wide_b = merged && c->kblock != save_b ? save_b : 0;
+    c->wide_z = save_z;
     drop_graphs(c);
   }
+  choose_shape(c);
   return HOSC_OK;
 }
 

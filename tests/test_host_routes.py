@@ -145,3 +145,29 @@ int main() {
                                           timeout=60).stdout.split()]
     OK, NO, EC = H.HOSC_OK, H.HOSC_ENOCONV, H.HOSC_ECUDA
     assert out == [OK, OK, NO, EC, EC, EC, OK, EC]
+
+
+# ------------------------------------------------------------------ launch shapes
+
+def _step_forms(fake, cav):
+    """The Krylov form of each launch of one step: 'pv register 384x8', ..."""
+    fake.clear()
+    assert H.hosc_step(cav.h, 1)[0] == 0
+    return sorted({" ".join(line.split()[:2]) for line in fake.log()
+                   if line.split()[0] in ("solve", "pv", "init")})
+
+
+@pytest.mark.parametrize("N", [30, 69, 75, 104])
+def test_merged_form_of_a_new_context(fake, N):
+    """The merged form is taken at the default shape, whatever that is, and the default is back with
+    the three-kernel form."""
+    with H.Cavity(_params(N, MIXED)) as cav:
+        default = H.hosc_get_tiles(cav.h)
+        assert H.hosc_set_krylov_merged(cav.h, 1) == 0 and H.hosc_get_krylov_merged(cav.h) == 1
+        assert H.hosc_get_tiles(cav.h)[1] <= 256
+        assert _step_forms(fake, cav) == ["init merged", "pv merged"]
+        assert H.hosc_set_krylov_merged(cav.h, 0) == 0
+        assert H.hosc_get_tiles(cav.h) == default
+        assert H.hosc_set_tiles(cav.h, 384, 1) == 0
+        assert H.hosc_set_krylov_merged(cav.h, 1) == H.HOSC_EINVAL   # the caller's shape stays
+        assert H.hosc_get_tiles(cav.h)[1:] == (384, 1, 0) and H.hosc_get_krylov_merged(cav.h) == 0
