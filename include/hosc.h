@@ -288,14 +288,16 @@ hosc_status hosc_time_kernel(void* ctx, int kernel_id, int reps, double* ms_per_
  * narrow = 1 selects the kernels compiled for at most 64 registers per thread (more resident
  * blocks), 0 those with more (80 for the three-kernel form, 128 for the merged form). The
  * default (384 threads, wide, kz from the wave model below; on grids whose solve runs as one launch
- * 256 threads) is chosen from N at creation. On grids whose vectors fit on the chip (mixed precision
- * up to about 68^3, FP64 up to about 42^3) the solve is one cooperative launch until a shape is set
- * here or by one of the calls below, and from 104^3 up p/v and s/t share planes in shared memory until
- * then; a call that sets a shape selects the kernels it describes, also with the default values. The
- * one-launch solve with the default shape and its kernel-by-kernel form give the same bits.
+ * 256 threads) is chosen from N at creation. On mixed grids whose vectors fit on the chip (up to about
+ * 68^3) the solve is one cooperative launch, and from 104^3 up p/v and s/t share planes in shared memory,
+ * until tiles are set here (also the default ones) or one of the calls below selects another form than
+ * its default; a call that leaves its form at the default changes nothing, and undoing a selection of
+ * those calls brings the default kernels back (tiles, once set, stay set). The one-launch solve with the
+ * default shape and its kernel-by-kernel form give the same bits.
  * Changing the shape drops the captured steps (captured again at the next step). HOSC_EINVAL for a shape
- * outside these limits, HOSC_ESTATE in the middle of a stage-by-stage step. The FP64 solve has
- * one thread per node and ignores the setting. */
+ * outside these limits, HOSC_ESTATE in the middle of a stage-by-stage step. The FP64 kernels have
+ * shapes of their own, one launch up to about 42^3, and take no setting: the call is accepted without
+ * effect on them. */
 hosc_status hosc_set_tiles(void* ctx, int kblock, int kz, int narrow);
 hosc_status hosc_get_tiles(void* ctx, int* kblock, int* kz, int* narrow);
 
@@ -303,7 +305,7 @@ hosc_status hosc_get_tiles(void* ctx, int* kblock, int* kz, int* narrow);
  * staged through shared memory by cp.async, several planes ahead): a block owns sx * sy interior
  * columns (one thread each; sx * sy a multiple of 32 in 32..256) and skz consecutive planes
  * (1..N-2). sx == 0
- * selects the register kernels of hosc_set_tiles for p/v and s/t (the default). HOSC_EINVAL for
+ * selects none of these (the default; see hosc_set_tiles for what runs then). HOSC_EINVAL for
  * a shape that does not fit (shared memory above 200 KB per block, too many blocks),
  * HOSC_ESTATE in the middle of a stage-by-stage step. Changing it drops the captured steps. */
 hosc_status hosc_set_stencil_tiles(void* ctx, int sx, int sy, int skz);
@@ -315,7 +317,7 @@ hosc_status hosc_get_stencil_tiles(void* ctx, int* sx, int* sy, int* skz);
  * computed; one producer thread, mbarrier completion), so that the bytes in flight do not
  * depend on registers or resident warps. A block owns tty rows of the
  * plane's interior columns (whole rows up to 126 columns; wider planes are cut into equal
- * pieces) and tkz consecutive planes (1..N-2). tty == 0 selects the register kernels (the
+ * pieces) and tkz consecutive planes (1..N-2). tty == 0 selects none of these (the
  * default; tkz and stages are then ignored); setting tiles here clears hosc_set_stencil_tiles
  * and the reverse. HOSC_EINVAL for a
  * shape that does not fit (at most 512 threads and 200 KB of shared memory per block, too many

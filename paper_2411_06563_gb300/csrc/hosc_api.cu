@@ -76,9 +76,8 @@ struct Ctx {
   int tty = 0, tkz = 0, tstages = 3;       // bulk-copy stencil kernels (tty == 0: not used)
   int tkernels = 3;                        // which of them run (1 p/v, 2 s/t, 3 both)
   int xr_flat = 0;                         // x/r as one flat stream (k8_xr)
-  // the one-launch solve: the grid is small enough for it, the caller has chosen no launch shape, and
-  // the context is not a pool's member
-  bool coop_fits = false, shape_chosen = false, pooled = false;
+  // the one-launch solve: the grid is small enough for it, and the context is not a pool's member
+  bool coop_fits = false, pooled = false;
   bool tiles_set = false;   // kblock, kz and narrow are the caller's (or the autotuner's)
   int wide_b = 0, wide_z = 0;   // the default that gave way to the merged form (0: none did)
   int ckz = 0;
@@ -154,10 +153,14 @@ void apply_tiles(Ctx* c) {
   c->P.tstages = c->tstages;
   c->P.tkernels = c->tkernels;
   c->P.xr_flat = c->xr_flat;
-  c->P.coop = c->coop_fits && !c->shape_chosen && !c->pooled;
+  // The default forms, one launch and shared planes, give way to what the caller selects: tiles, or a
+  // form other than the default of one of the mixed-precision kernels. A call that leaves each of those
+  // at its default leaves them on, and undoing the selection brings them back. FP64 kernels take no
+  // shape: the one-launch solve stays whatever is set.
+  const bool set = c->tiles_set || c->merged || c->sx > 0 || c->tty > 0;
+  c->P.coop = c->coop_fits && !c->pooled && !(c->P.krylov_fp32 && (set || c->xr_flat));
   c->P.ckz = c->ckz;
-  // the shared-plane kernels unless the caller has chosen a shape of the others
-  c->P.plane = c->plane_fits && !c->shape_chosen && !c->merged && c->sx == 0 && c->tty == 0;
+  c->P.plane = c->plane_fits && !set;
   c->P.ptx = c->ptx;
   c->P.pty = c->pty;
   c->P.plz = c->plz;
@@ -1665,12 +1668,11 @@ hosc_status hosc_time_kernel(void* ctx, int kernel_id, int reps, double* ms_per_
   return HOSC_OK;
 }
 
-// A launch shape set by the caller: the solve runs kernel by kernel with it.
-static void choose_shape(Ctx* c) {
-  if (c->shape_chosen) return;
-  c->shape_chosen = true;
-  if (c->P.coop || c->P.plane) drop_graphs(c);
+// After a change of a selection: drop the captured steps, which hold the old kernels and shapes.
+static void reshape(Ctx* c, bool changed) {
+  const int coop = c->P.coop, plane = c->P.plane;
   apply_tiles(c);
+  if (changed || coop != c->P.coop || plane != c->P.plane) drop_graphs(c);
 }
 
 hosc_status hosc_set_tiles(void* ctx, int kblock, int kz, int narrow) {
@@ -1678,14 +1680,12 @@ hosc_status hosc_set_tiles(void* ctx, int kblock, int kz, int narrow) {
   if (!c) return HOSC_EINVAL;
   if (c->stage != 0) return HOSC_ESTATE;
   if (!tiles_valid(c, kblock, kz, narrow)) return HOSC_EINVAL;
-  choose_shape(c);
+  const bool changed = kblock != c->kblock || kz != c->kz || narrow != c->narrow;
+  c->kblock = kblock;
+  c->kz = kz;
+  c->narrow = narrow;
   c->tiles_set = true;
-  if (kblock != c->kblock || kz != c->kz || narrow != c->narrow) {
-    c->kblock = c->P.kblock = kblock;
-    c->kz = c->P.kz = kz;
-    c->narrow = c->P.narrow = narrow;
-    drop_graphs(c);   // the captured steps hold the old launch shapes
-  }
+  reshape(c, changed);
   return HOSC_OK;
 }
 
@@ -1695,7 +1695,6 @@ hosc_status hosc_set_stencil_tiles(void* ctx, int sx, int sy, int skz) {
   if (c->stage != 0) return HOSC_ESTATE;
   CU(cudaSetDevice(c->device));
   if (!stencil_tiles_valid(c, sx, sy, skz)) return HOSC_EINVAL;
-  choose_shape(c);
   if (sx == 0) sy = skz = 0;
   if (sx != c->sx || sy != c->sy || skz != c->skz || (sx > 0 && c->tty > 0)) {
     c->sx = sx;
@@ -1706,8 +1705,7 @@ hosc_status hosc_set_stencil_tiles(void* ctx, int sx, int sy, int skz) {
       c->tstages = 3;
       c->tkernels = 3;
     }
-    apply_tiles(c);
-    drop_graphs(c);
+    reshape(c, true);
   }
   return HOSC_OK;
 }
@@ -1737,7 +1735,6 @@ hosc_status hosc_set_tma_tiles(void* ctx, int tty, int tkz, int stages, int kern
       return HOSC_ECUDA;
     }
   }
-  choose_shape(c);
   if (tty != c->tty || tkz != c->tkz || stages != c->tstages || kernels != c->tkernels ||
       (tty > 0 && c->sx > 0)) {
     c->tty = tty;
@@ -1745,8 +1742,7 @@ hosc_status hosc_set_tma_tiles(void* ctx, int tty, int tkz, int stages, int kern
     c->tstages = stages;
     c->tkernels = kernels;
     if (tty > 0) c->sx = c->sy = c->skz = 0;
-    apply_tiles(c);
-    drop_graphs(c);
+    reshape(c, true);
   }
   return HOSC_OK;
 }
@@ -1755,11 +1751,9 @@ hosc_status hosc_set_xr_form(void* ctx, int flat) {
   Ctx* c = (Ctx*)ctx;
   if (!c || (flat != 0 && flat != 1)) return HOSC_EINVAL;
   if (c->stage != 0) return HOSC_ESTATE;
-  choose_shape(c);
   if (flat != c->xr_flat) {
     c->xr_flat = flat;
-    apply_tiles(c);
-    drop_graphs(c);
+    reshape(c, true);
   }
   return HOSC_OK;
 }
@@ -1804,7 +1798,6 @@ hosc_status hosc_set_krylov_merged(void* ctx, int merged) {
     c->wide_z = save_z;
     drop_graphs(c);
   }
-  choose_shape(c);
   return HOSC_OK;
 }
 
@@ -1837,18 +1830,19 @@ hosc_status hosc_autotune(void* ctx, int reps, int* kblock_out, int* kz_out, dou
   if (c->stage != 0) return HOSC_ESTATE;
   if (!c->P.krylov_fp32) return HOSC_EINVAL;
   CU(cudaSetDevice(c->device));
-  struct KeepChoice {
+  const bool plane0 = c->P.plane != 0;   // the default p/v and s/t of this grid: timed at the end
+  const bool one_launch = c->P.coop != 0;   // it stays, with the register shape found beside it
+  struct Pin {   // the search times the kernels of set shapes; what it ends with stays set, or not
     Ctx* c;
-    bool chosen;
-    ~KeepChoice() {
-      c->shape_chosen = chosen;
+    bool set;
+    ~Pin() {
+      c->tiles_set = set;
       apply_tiles(c);
       drop_graphs(c);
     }
-  } keep{c, c->shape_chosen};
-  const bool plane0 = c->P.plane != 0;   // the default p/v and s/t of this grid: timed at the end
-  const bool one_launch = c->P.coop != 0;   // it stays, with the register shape found beside it
-  if (!c->plane_fits && !c->coop_fits) keep.chosen = true;
+  } pin{c, !plane0 && !one_launch};
+  c->tiles_set = true;
+  apply_tiles(c);
   {   // the register kernels first
     hosc_status s0 = hosc_set_stencil_tiles(c, 0, 0, 0);
     if (!s0) s0 = hosc_set_tma_tiles(c, 0, 0, 3, 3);
@@ -2107,8 +2101,8 @@ hosc_status hosc_autotune(void* ctx, int reps, int* kblock_out, int* kz_out, dou
     }
     apply_tiles(c);
     if (st) return st;
-    keep.chosen = plane > found;
-    if (!keep.chosen) {
+    pin.set = plane > found;
+    if (!pin.set) {
       st = hosc_set_tma_tiles(c, 0, 0, 3, 3);
       if (!st) st = hosc_set_stencil_tiles(c, 0, 0, 0);
       if (st) return st;

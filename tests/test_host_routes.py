@@ -171,3 +171,40 @@ def test_merged_form_of_a_new_context(fake, N):
         assert H.hosc_set_tiles(cav.h, 384, 1) == 0
         assert H.hosc_set_krylov_merged(cav.h, 1) == H.HOSC_EINVAL   # the caller's shape stays
         assert H.hosc_get_tiles(cav.h)[1:] == (384, 1, 0) and H.hosc_get_krylov_merged(cav.h) == 0
+
+
+# a call of each kind that selects nothing
+IDLE = [("hosc_set_xr_form", (0,)), ("hosc_set_stencil_tiles", (0, 0, 0)),
+        ("hosc_set_tma_tiles", (0, 0, 3, 3)), ("hosc_set_krylov_merged", (0,))]
+# one that selects a form, and the one that undoes it
+SELECT = [("hosc_set_xr_form", (1,), (0,)), ("hosc_set_stencil_tiles", (16, 2, 5), (0, 0, 0)),
+          ("hosc_set_krylov_merged", (1,), (0,))]
+
+
+@pytest.mark.parametrize("N,precision,default", [(21, FP64, "solve one_launch"),
+                                                 (30, MIXED, "solve one_launch"),
+                                                 (75, MIXED, "pv register"),
+                                                 (104, MIXED, "pv plane")])
+def test_calls_that_select_nothing_keep_the_default_kernels(fake, N, precision, default):
+    with H.Cavity(_params(N, precision)) as cav:
+        assert _step_forms(fake, cav) == [default]
+        for name, args in IDLE:
+            assert getattr(H, name)(cav.h, *args) == 0
+            assert _step_forms(fake, cav) == [default], name
+        assert H.hosc_set_xr_form(cav.h, 2) == H.HOSC_EINVAL
+        assert H.hosc_set_tiles(cav.h, 100, 1) == H.HOSC_EINVAL
+        assert _step_forms(fake, cav) == [default]
+        for name, on, off in SELECT:
+            assert getattr(H, name)(cav.h, *on) == 0
+            forms = _step_forms(fake, cav)
+            if precision == FP64:
+                assert forms == [default], name   # FP64 kernels take no setting
+            elif name == "hosc_set_xr_form":
+                assert forms == [default.replace("solve one_launch", "pv register")]
+            else:
+                assert default not in forms, name
+            assert getattr(H, name)(cav.h, *off) == 0
+            assert _step_forms(fake, cav) == [default], name
+        _, b, z, narrow = H.hosc_get_tiles(cav.h)
+        assert H.hosc_set_tiles(cav.h, b, z, narrow) == 0
+        assert _step_forms(fake, cav) == [default if precision == FP64 else "pv register"]
