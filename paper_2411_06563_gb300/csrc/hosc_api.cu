@@ -56,6 +56,7 @@ struct Ctx {
   cudaGraphExec_t graph[2][2][2] = {};
   cudaStream_t cap[2] = {nullptr, nullptr};   // private streams used only for capture
   bool graphs_ok = true;                      // capture or instantiation failed once: stay off
+  long shape_version = 0;                     // launch shapes and forms so far (drop_graphs)
   StepRecord* h_ring = nullptr;
   long launches = 0;
   KrylovScalars* h_ks = nullptr;
@@ -823,7 +824,9 @@ bool graphs_usable(Ctx* c) {
   return c->graphs_ok && !c->prof_on && c->stage == 0 && c->prm.inner_max == 0;
 }
 
+// The captured steps no longer apply, nor does a round that a pool has captured.
 void drop_graphs(Ctx* c) {
+  c->shape_version += 1;
   for (auto& a : c->graph)
     for (auto& b : a)
       for (auto& g : b)
@@ -1023,15 +1026,34 @@ size_t ctx_workspace(void* ctx) { return ((Ctx*)ctx)->ws_bytes; }
 int ctx_N(void* ctx) { return ((Ctx*)ctx)->prm.N; }
 cudaStream_t ctx_branch_stream(void* ctx) { return ((Ctx*)ctx)->cap[0]; }
 
-// What a captured round assumes about the context: level parity, history, phase, launch shape.
+// What a captured round assumes about the context: level parity, history, phase, launch shape and form.
 long ctx_signature(void* ctx) {
   const Ctx* c = (const Ctx*)ctx;
-  const long s = (long)c->cur | ((long)c->P.have_prev << 1) | ((long)c->phase << 2) |
-                 ((long)c->kblock << 3) | ((long)c->kz << 13) | ((long)c->narrow << 23) |
-                 ((long)c->sx << 24) | ((long)c->sy << 32) | ((long)c->skz << 42) |
-                 ((long)c->merged << 52);
-  return s ^ ((long)c->tty << 53) ^ ((long)c->tkz << 56) ^ ((long)c->xr_flat << 62) ^
-         ((long)c->tstages << 45) ^ ((long)c->tkernels << 48);
+  return (long)c->cur | ((long)c->P.have_prev << 1) | ((long)c->phase << 2) | (c->shape_version << 3);
+}
+
+LaunchShape ctx_shape(void* ctx) {
+  const Ctx* c = (const Ctx*)ctx;
+  return {c->kblock, c->kz, c->narrow, c->tiles_set, c->merged, c->sx, c->sy, c->skz,
+          c->tty, c->tkz, c->tstages, c->tkernels, c->xr_flat};
+}
+
+// The tiles first: the merged form does not take every default block.
+hosc_status ctx_set_shape(void* ctx, const LaunchShape& t) {
+  Ctx* c = (Ctx*)ctx;
+  const LaunchShape now = ctx_shape(ctx);
+  if (memcmp(&now, &t, sizeof(t)) == 0) return HOSC_OK;
+  hosc_status st = hosc_set_krylov_merged(ctx, 0);
+  if (!st) st = hosc_set_tiles(ctx, t.kblock, t.kz, t.narrow);
+  if (!st) st = hosc_set_krylov_merged(ctx, t.merged);
+  if (!st) st = hosc_set_stencil_tiles(ctx, t.sx, t.sy, t.skz);
+  if (!st) st = hosc_set_tma_tiles(ctx, t.tty, t.tkz, t.stages, t.kernels);
+  if (!st) st = hosc_set_xr_form(ctx, t.xr_flat);
+  if (st) return st;
+  c->tiles_set = t.set != 0;
+  apply_tiles(c);
+  drop_graphs(c);
+  return HOSC_OK;
 }
 
 void ctx_join_pool(void* ctx) {

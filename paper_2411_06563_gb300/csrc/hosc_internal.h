@@ -317,6 +317,13 @@ size_t ctx_workspace(void* ctx);             // device bytes the context holds
 int ctx_N(void* ctx);
 cudaStream_t ctx_branch_stream(void* ctx);   // stream on which ctx_append_round captures
 long ctx_signature(void* ctx);               // changes when a captured round no longer applies
+// What hosc_set_tiles and the calls beside it select, whole: a member's shape goes to the others of its
+// size. set == 0: the default forms (shared planes) stay, with these tiles for the kernels beside them.
+struct LaunchShape {
+  int kblock, kz, narrow, set, merged, sx, sy, skz, tty, tkz, stages, kernels, xr_flat;
+};
+LaunchShape ctx_shape(void* ctx);
+hosc_status ctx_set_shape(void* ctx, const LaunchShape& shape);
 // A member of a pool: its solves run kernel by kernel, beside those of the other members (a cooperative
 // grid takes the whole GPU).
 void ctx_join_pool(void* ctx);

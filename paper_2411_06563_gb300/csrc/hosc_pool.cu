@@ -20,7 +20,6 @@
 #include <stdio.h>
 #include <string.h>
 
-#include <array>
 #include <chrono>
 #include <map>
 #include <new>
@@ -68,9 +67,7 @@ struct Pool {
   cudaEvent_t fork = nullptr;
   cudaGraphExec_t exec = nullptr;
   bool dirty = true;                          // membership changed since the capture
-  // tuned launch shapes per N: kblock, kz, narrow, sx, sy, skz, tty, tkz, merged, x/r form,
-  // ring stages and kernels of the bulk-copy kernels
-  std::map<int, std::array<int, 12>> tiles;
+  std::map<int, LaunchShape> tiles;           // tuned launch shapes and forms per N
   long rounds = 0, captures = 0;
   double capture_ms = 0.0;
   RoundState* rs = nullptr;                   // persistent mode: the round kernel's tables
@@ -126,15 +123,6 @@ bool needs_capture(const Pool* P) {
   return false;
 }
 
-hosc_status apply_shape(void* ctx, const std::array<int, 12>& t) {
-  hosc_status st = hosc_set_krylov_merged(ctx, t[8]);
-  if (!st) st = hosc_set_tiles(ctx, t[0], t[1], t[2]);
-  if (!st) st = hosc_set_stencil_tiles(ctx, t[3], t[4], t[5]);
-  if (!st) st = hosc_set_tma_tiles(ctx, t[6], t[7], t[10], t[11]);
-  if (!st) st = hosc_set_xr_form(ctx, t[9]);
-  return st;
-}
-
 // After a member's round: complete it (steady, failed, out of steps) or tune its launch shape.
 hosc_status settle(Pool* P, int slot, hosc_status st, bool steady, const hosc_info& ri,
                    int* done, int cap, int* ndone) {
@@ -179,16 +167,10 @@ hosc_status settle(Pool* P, int slot, hosc_status st, bool steady, const hosc_in
       auto it = P->tiles.find(q.N);
       if (it == P->tiles.end()) {
         hosc_status ts = hosc_autotune(q.ctx, 3, nullptr, nullptr, nullptr);
-        std::array<int, 12> t = {};
-        if (!ts) ts = hosc_get_tiles(q.ctx, &t[0], &t[1], &t[2]);
-        if (!ts) ts = hosc_get_stencil_tiles(q.ctx, &t[3], &t[4], &t[5]);
-        if (!ts) ts = hosc_get_tma_tiles(q.ctx, &t[6], &t[7], &t[10], &t[11]);
-        if (!ts) t[8] = hosc_get_krylov_merged(q.ctx);
-        if (!ts) t[9] = hosc_get_xr_form(q.ctx);
         if (ts) return ts;
-        P->tiles[q.N] = t;
+        P->tiles[q.N] = ctx_shape(q.ctx);
       } else {
-        hosc_status ts = apply_shape(q.ctx, it->second);
+        hosc_status ts = ctx_set_shape(q.ctx, it->second);
         if (ts) return ts;
       }
     }
@@ -296,7 +278,7 @@ hosc_status hosc_pool_admit(void* pool, const hosc_params* params, long max_step
   P->dirty = true;
   if (p.precision == HOSC_MIXED) {
     auto it = P->tiles.find(p.N);
-    if (it != P->tiles.end()) apply_shape(ctx, it->second);
+    if (it != P->tiles.end()) ctx_set_shape(ctx, it->second);
   }
   *slot = s;
   return HOSC_OK;

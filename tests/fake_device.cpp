@@ -62,7 +62,8 @@ void launch(cudaStream_t s, const std::string& name, const std::string& detail,
   }
   run(s, [=]() {
     g_log += name + (detail.empty() ? "" : " " + detail) + "\n";
-    auto c = g_cost.find(detail.empty() ? name : name + " " + detail.substr(0, detail.find(' ')));
+    auto c = g_cost.find(name + " " + detail.substr(0, detail.find(' ')));
+    if (c == g_cost.end()) c = g_cost.find(name);
     g_now += c == g_cost.end() ? 1.0 : c->second;
     if (effect) effect();
   });
@@ -277,7 +278,7 @@ void launch_bicg_init(const DevParams& P, const Fields& F, cudaStream_t s) {
 void launch_bicg_pv(const DevParams& P, const Fields&, int, bool, cudaStream_t s) { launch(s, "pv", krylov(P)); }
 void launch_bicg_st(const DevParams& P, const Fields&, int, bool, cudaStream_t s) { launch(s, "st", krylov(P)); }
 void launch_bicg_xr(const DevParams& P, const Fields& F, int, bool, cudaStream_t s) {
-  launch(s, "xr", krylov(P), [=]() { end_of_solve(F); });
+  launch(s, P.xr_flat ? "xr_flat" : "xr", krylov(P), [=]() { end_of_solve(F); });
 }
 void launch_b2(int k, const DevParams& P, const Fields& F, int, bool, cudaStream_t s) {
   launch(s, "b2", krylov(P), [=]() { if (k == 4) end_of_solve(F); });

@@ -208,3 +208,60 @@ def test_calls_that_select_nothing_keep_the_default_kernels(fake, N, precision, 
         _, b, z, narrow = H.hosc_get_tiles(cav.h)
         assert H.hosc_set_tiles(cav.h, b, z, narrow) == 0
         assert _step_forms(fake, cav) == [default if precision == FP64 else "pv register"]
+
+
+# ------------------------------------------------------------------ shapes in a pool
+
+def _round_forms(fake, pool):
+    """p/v lines of one round, with their counts."""
+    fake.clear()
+    assert H.hosc_pool_run(pool, 1)[0] == 0
+    pv = [line for line in fake.log() if line.startswith("pv ")]
+    return {q: pv.count(q) for q in pv}
+
+
+def _pool(N, members, mode, **kw):
+    p = _params(N, MIXED, **kw)
+    st, pool = H.hosc_pool_create(4 * H.hosc_workspace_bytes(p), 2, mode, 1)
+    assert st == 0
+    slots = [H.hosc_pool_admit(pool, p, 1000) for _ in range(members)]
+    assert all(s[0] == 0 for s in slots)
+    return p, pool, [s[1] for s in slots]
+
+
+@pytest.mark.parametrize("mode", [H.HOSC_POOL_STREAMS, H.HOSC_POOL_GRAPH])
+@pytest.mark.parametrize("N,best,flat", [(104, "plane", False), (104, "register", False),
+                                         (104, "staged", False), (75, "merged", False),
+                                         (75, "register", True), (104, "plane", True),
+                                         (30, "staged", False)])
+def test_a_tuned_form_reaches_every_member(fake, mode, N, best, flat):
+    """The member that a size is tuned on, one that was there and one admitted later run, round after
+    round, the form and the tiles that the search found the fastest."""
+    for kind in ("pv", "st"):
+        fake.cost("%s %s" % (kind, best), 0.125)
+    if flat:
+        fake.cost("xr_flat", 0.125)
+    p, pool, slots = _pool(N, 2, mode)
+    _round_forms(fake, pool)
+    one = _round_forms(fake, pool)
+    assert len(one) == 1, one
+    (line, count), = one.items()
+    assert line.split()[1] == best and (line.endswith(" flat") == flat), line
+    assert H.hosc_pool_admit(pool, p, 1000)[0] == 0
+    for _ in range(2):
+        more = _round_forms(fake, pool)
+        assert list(more) == [line] and more[line] == count * 3 // 2
+    H.hosc_pool_destroy(pool)
+
+
+def test_a_captured_round_follows_the_form(fake):
+    """A form that changes without its tiles makes the pool capture its round again."""
+    p, pool, slots = _pool(104, 1, H.HOSC_POOL_GRAPH)
+    H.hosc_pool_destroy(pool)
+    st, pool = H.hosc_pool_create(4 * H.hosc_workspace_bytes(p), 2, H.HOSC_POOL_GRAPH, 0)
+    assert st == 0 and H.hosc_pool_admit(pool, p, 1000)[0] == 0
+    ctx = H.hosc_pool_result(pool, 0)[4]
+    assert {q.split()[1] for q in _round_forms(fake, pool)} == {"plane"}
+    assert H.hosc_set_tiles(ctx, *H.hosc_get_tiles(ctx)[1:]) == 0
+    assert {q.split()[1] for q in _round_forms(fake, pool)} == {"register"}
+    H.hosc_pool_destroy(pool)
