@@ -1932,7 +1932,22 @@ hosc_status hosc_autotune(void* ctx, int reps, int* kblock_out, int* kz_out, dou
   if (st) return st;
   st = hosc_set_tiles(c, best_b, best_z, best_n);
   if (st) return st;
-  // The other iteration form (two or three kernels) at the shape found.
+  // p/v and s/t as shared-plane kernels (form 1) or as what the context has selected (form 0).
+  auto time_pair = [&](int form, double* ms) {
+    c->P.plane = form;
+    if (form) c->P.tty = c->P.sx = 0;
+    hosc_status q = HOSC_OK;
+    *ms = 0.0;
+    for (int kid = HOSC_K_BICG_PV; kid <= HOSC_K_BICG_ST && !q; ++kid) {
+      double one = 0.0;
+      q = time_class(c, kid, 4 * reps, &one);
+      *ms += one;
+    }
+    apply_tiles(c);
+    return q;
+  };
+  // The other iteration form (two or three kernels) at the shape found; the merged one has to be faster
+  // than the shared planes too, which end the search otherwise.
   if (!one_launch) {
     const int other = 1 - c->merged;
     c->merged = other;
@@ -1948,7 +1963,15 @@ hosc_status hosc_autotune(void* ctx, int reps, int* kblock_out, int* kz_out, dou
     c->merged = 1 - other;
     apply_tiles(c);
     if (st) return st;
-    if (ok && tot < best) {
+    double plane = INFINITY;
+    if (ok && tot < best && plane0) {
+      double xr = 0.0;
+      st = time_pair(1, &plane);
+      if (!st) st = time_class(c, HOSC_K_BICG_XR, 4 * reps, &xr);
+      if (st) return st;
+      plane += xr;
+    }
+    if (ok && tot < best && tot < plane) {
       st = hosc_set_krylov_merged(c, other);
       if (st) return st;
       best = tot;
@@ -2109,19 +2132,8 @@ hosc_status hosc_autotune(void* ctx, int reps, int* kblock_out, int* kz_out, dou
   }
   if (plane0) {   // p/v and s/t as shared-plane kernels against the ones found
     double found = 0.0, plane = 0.0;
-    for (int form = 0; form < 2 && !st; ++form) {
-      c->P.plane = form;
-      const int tty = c->P.tty, sx = c->P.sx;
-      if (form) c->P.tty = c->P.sx = 0;
-      for (int kid = HOSC_K_BICG_PV; kid <= HOSC_K_BICG_ST && !st; ++kid) {
-        double ms = 0.0;
-        st = time_class(c, kid, 4 * reps, &ms);
-        (form ? plane : found) += ms;
-      }
-      c->P.tty = tty;
-      c->P.sx = sx;
-    }
-    apply_tiles(c);
+    st = time_pair(0, &found);
+    if (!st) st = time_pair(1, &plane);
     if (st) return st;
     pin.set = plane > found;
     if (!pin.set) {

@@ -62,7 +62,8 @@ void launch(cudaStream_t s, const std::string& name, const std::string& detail,
   }
   run(s, [=]() {
     g_log += name + (detail.empty() ? "" : " " + detail) + "\n";
-    auto c = g_cost.find(name + " " + detail.substr(0, detail.find(' ')));
+    auto c = g_cost.find(name + " " + detail);
+    if (c == g_cost.end()) c = g_cost.find(name + " " + detail.substr(0, detail.find(' ')));
     if (c == g_cost.end()) c = g_cost.find(name);
     g_now += c == g_cost.end() ? 1.0 : c->second;
     if (effect) effect();

@@ -254,6 +254,21 @@ def test_a_tuned_form_reaches_every_member(fake, mode, N, best, flat):
     H.hosc_pool_destroy(pool)
 
 
+@pytest.mark.parametrize("merged,plane,expect", [(0.5, 0.125, "plane"), (0.125, 0.5, "merged"),
+                                                 (0.75, 2.0, "merged"), (2.0, 2.0, "register")])
+def test_the_search_keeps_the_faster_of_merged_form_and_shared_planes(fake, merged, plane, expect):
+    for kind in ("pv", "st"):
+        fake.cost("%s merged" % kind, merged)
+        fake.cost("%s plane" % kind, plane)
+        fake.cost("%s staged" % kind, 4.0)
+        for z in range(1, 34):   # a block that the merged form takes is the fastest
+            fake.cost("%s register 256x%d" % (kind, z), 0.9)
+    with H.Cavity(_params(104, MIXED)) as cav:
+        assert cav.step(1)["call_status"] == 0
+        assert H.hosc_autotune(cav.h, 2)[0] == 0
+        assert [q.split()[1] for q in _step_forms(fake, cav) if q.startswith("pv")] == [expect]
+
+
 def test_a_captured_round_follows_the_form(fake):
     """A form that changes without its tiles makes the pool capture its round again."""
     p, pool, slots = _pool(104, 1, H.HOSC_POOL_GRAPH)
