@@ -280,8 +280,11 @@ DevParams device_params(const hosc_params& p, int have_prev, int phase) {
   d.eta_exp = 0.5 * (p.n - 1.0);
   {
     const double m = d.eta_exp != 0.0 ? rint(1.0 / fabs(d.eta_exp)) : 0.0;
-    // equal to the rounding of n - 1: the power then differs by less than its last place
-    if (m >= 2.0 && m <= 64.0 && fabs(fabs(d.eta_exp) * m - 1.0) < 1e-15) d.eta_root = (int)m;
+    const double e = fma(fabs(d.eta_exp), m, -1.0);   // exact
+    if (m >= 2.0 && m <= 64.0 && fabs(e) < 1e-15) {
+      d.eta_root = (int)m;
+      d.eta_res = (float)(-e * 0.69314718055994531);
+    }
   }
   d.dtf = (float)p.dt;
   d.Prf = (float)p.Pr;

@@ -71,7 +71,8 @@ struct DevParams {
   float csf[3];      // -dt/(2 h_d^2): the dt part of the symmetric weights of the compact operators
   RhsC<double> rc;
   RhsC<float> rcf;
-  int eta_root;      // m when (n - 1)/2 = -1/m or 1/m for an integer m in 2..64, else 0
+  int eta_root;      // m when (n - 1)/2 is -1/m or 1/m to rounding for an integer m in 2..64, else 0
+  float eta_res;     // (1 - m |(n - 1)/2|) ln 2
   double eta_exp;    // (n - 1)/2, the exponent of the regularised viscosity
   // float copies of the scalars the float sweeps use (converted once on the host)
   float dtf, Prf, Raf, theta_reff, I2_epsf, eta_expf, a_limitf, a_boostf;

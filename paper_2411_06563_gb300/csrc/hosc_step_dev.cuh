@@ -164,21 +164,26 @@ __device__ __forceinline__ void sweep_node(int N, unsigned vbx, unsigned nbi, Fn
 
 // ------------------------------------------------------------------------------------ S1
 
-// x^(-1/m) for an integer m in 2..64: a float estimate y of 1e-6 and one third-order step of
-// Newton's iteration on y^-m = x, y (1 - r)^(-1/m) to r^2 with r = 1 - x y^m (the r^3 term is below
-// 1e-16 of y); y^m by squaring. Largest error found against 200-bit arithmetic over 20 000 x in
-// [1e-12, 1e12]: 0.75 units in the last place (m = 8), 0.79 (m = 64); about 15 FP64 instructions
-// against some 130 of pow().
-__device__ __forceinline__ double inverse_root(double x, int m) {
-  const float a = 1.0f / (float)m;
-  const double y = (double)exp2f(-a * log2f((float)x));
+// x^(-(1 - e)/m) for an integer m in 2..64 and an e of rounding size: a float estimate y of 1e-6 and one
+// third-order step of Newton's iteration on y^-m = x^(1 - e), y (1 - r)^(-1/m) to r^2 with r = x^e - x y^m
+// (the r^3 term is below 1e-16 of y); y^m by squaring. Largest error found against 200-bit arithmetic
+// over 20 000 x in [1e-12, 1e12] with e = 0: 0.75 units in the last place (m = 8), 0.79 (m = 64); about
+// 15 FP64 instructions against some 130 of pow(). A rounded n leaves an e (n = 1 + 2/3 missed the power
+// by 14 units at 1e18 without it): x^e = 1 + e ln x to first order, e ln x = e2 log2(x) below 1e-13, is
+// put together on the integer units (as an FP64 sum it cost the sweep 3.5 % at 101^3).
+__device__ __forceinline__ double inverse_root(double x, int m, float e2) {
+  const float a = 1.0f / (float)m, lx = log2f((float)x);
+  const double y = (double)exp2f(-a * lx);
   double p = 1.0, b = y;
   for (int e = m;;) {   // m is the same for every thread
     if (e & 1) p *= b;
     if ((e >>= 1) == 0) break;
     b *= b;
   }
-  const double r = fma(-x, p, 1.0);
+  const float d = e2 * lx;
+  // 1 + d: doubles lie 2^-52 apart above 1 and 2^-53 below
+  const long long k = __float2int_rn(d * (d < 0.0f ? 9007199254740992.0f : 4503599627370496.0f));
+  const double r = fma(-x, p, __longlong_as_double(0x3ff0000000000000LL + k));
   const float c2 = 0.5f * a * (1.0f + a);
   return fma(y, r * fma((double)c2, r, 1.0 / (double)m), y);
 }
@@ -216,7 +221,7 @@ __device__ __forceinline__ void k_viscosity_body(const DevParams& P, const T* HO
     const T x = I2 + par<T>(P.I2_eps, P.I2_epsf);
     if constexpr (sizeof(T) == sizeof(double)) {
       if (P.eta_root && x >= 1e-30 && x <= 1e30) {
-        const double z = inverse_root(x, P.eta_root);
+        const double z = inverse_root(x, P.eta_root, P.eta_res);
         const bool thin = P.eta_exp < 0.0;   // the same for every thread
         eta[t] = thin ? z : 1.0 / z;
         L[t] = thin ? 1.0 / (P.Pr * z) : P.iPr * z;
