@@ -227,7 +227,13 @@ void hosc_destroy(void* ctx);
 hosc_status hosc_reset(void* ctx);
 
 /* Take nsteps >= 1 pseudo-time steps. Enqueues the work and waits for it once at the end.
- * Stops early at the first step whose status is not HOSC_OK and returns that status. */
+ * Stops early at the first step whose status is not HOSC_OK and returns that status.
+ * Where the solve is one launch (see hosc_set_tiles) its blocks wait for one another, and the launch starts
+ * when all of them fit on the GPU at once: a step waits for other kernels that hold SMs, however long,
+ * also where some SMs are free, and contexts on different streams take turns in the solve. A kernel that
+ * keeps SMs until it sees this step's result therefore stops it for good: set tiles (mixed precision) or
+ * use a pool, whose members solve kernel by kernel, beside such a kernel. Once started, a wait of one block
+ * for another that runs past 2 s ends the step with HOSC_ECUDA. */
 hosc_status hosc_step(void* ctx, int nsteps, hosc_info* out);
 
 /* Step until max|chi^{n+1}-chi^n| / dt < tol_steady and max|div V| < div_steady (tol_div when
