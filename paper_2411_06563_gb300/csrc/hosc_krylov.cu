@@ -900,7 +900,9 @@ void launch_bicg_init(const DevParams& P, const Fields& F, cudaStream_t s) {
 // vector is zero there: the workspace is zeroed at creation and no kernel writes other wall entries
 // than these zeros), in a grid-stride loop that
 // issues the loads of U nodes before their arithmetic, so that a thread keeps 6 U float4 loads in
-// flight. Same arithmetic and float-float partials as k4_xr; one block partial per block.
+// flight. Same arithmetic and float-float partials as k4_xr; one block partial per block. With a scalar
+// beyond float or not finite (a solve that fails) 0 times it is no zero: the walls are then left out, one
+// node at a time, since later solves read them.
 template <int U, bool FIRST>
 __global__ void __launch_bounds__(256) k8_xr(DevParams P, Fields F, int pp) {
   __shared__ Scal4 sc;
@@ -917,9 +919,13 @@ __global__ void __launch_bounds__(256) k8_xr(DevParams P, Fields F, int pp) {
   float4* __restrict__ R = F.kr;
   const unsigned N2 = (unsigned)P.N * (unsigned)P.N, hi = N2 * (unsigned)(P.N - 1);
   const unsigned stride = gridDim.x * blockDim.x;
+  auto finite = [](float4 q) {
+    return isfinite(q.x) && isfinite(q.y) && isfinite(q.z) && isfinite(q.w);
+  };
+  const bool wild = !finite(a) || !finite(om);   // the same for every thread
   FF acc[8] = {};
   unsigned c = N2 + blockIdx.x * blockDim.x + threadIdx.x;
-  for (; c + (U - 1) * stride < hi; c += U * stride) {
+  for (; !wild && c + (U - 1) * stride < hi; c += U * stride) {
     float4 r[U], v[U], p[U], t[U], r0[U], x[U];
 #pragma unroll
     for (int q = 0; q < U; ++q) {
@@ -943,6 +949,10 @@ __global__ void __launch_bounds__(256) k8_xr(DevParams P, Fields F, int pp) {
     }
   }
   for (; c < hi; c += stride) {
+    if (wild) {
+      const unsigned N = P.N, i = c % N, j = c / N % N;
+      if (i == 0 || i == N - 1 || j == 0 || j == N - 1) continue;
+    }
     const float4 r0 = __ldg(R0 + c);
     const float4 sv = fma4(ma, __ldg(V + c), FIRST ? r0 : R[c]);
     X[c] = fma4(om, sv, fma4(a, __ldg(Pv + c), FIRST ? f4(0.f) : X[c]));
