@@ -88,6 +88,7 @@ struct DevParams {
   double div_steady;   // max|div V| below this (div_steady, else tol_div) is steady
 };
 
+constexpr int kPlanarLeast = 128;   // least and
 constexpr int kPlanarMost = 512;    // most threads a block of the planar kernels (a multiple of 32)
 constexpr int kSolveRows = 152;      // most rows (blocks) of a system in the one-launch FP64 solves
 constexpr int kExchValues = 8192;   // 16-byte values of the exchange buffer

@@ -862,7 +862,7 @@ void planar_shape(int N, int* pb, int* pkz) {
   double best = 1e300;
   *pb = 512;
   *pkz = ni;
-  for (int B : {128, 256, 512}) {
+  for (int B = kPlanarLeast; B <= kPlanarMost; B *= 2) {
     const long chunks = (N * (long)N + B - 1) / B;
     for (int z = 1; z <= ni; ++z) {
       const long rows = chunks * ((ni + z - 1) / z);

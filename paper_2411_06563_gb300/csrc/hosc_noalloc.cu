@@ -24,7 +24,10 @@ constexpr size_t kVecBytes = kMaxNodes * sizeof(double);
 constexpr size_t kAlignB = 256;
 // 6 vectors (r, p x2, v x2, t) for each of the 4 systems, then the small control block.
 constexpr size_t kVectorsBytes = 24 * ((kVecBytes + kAlignB - 1) / kAlignB * kAlignB);
-constexpr size_t kMaxBlocks = 1024;   // rows of partials: red_rows / 4 and below for every N
+// Rows of partials, kernel by kernel: chunks of kPlanarLeast nodes or more, a plane or more.
+constexpr size_t kMaxBlocks = 1024;
+static_assert((kMaxN * kMaxN + kPlanarLeast - 1) / kPlanarLeast * (kMaxN - 2) <= (int)kMaxBlocks,
+              "a shape of planar_shape may have more rows than the control block");
 constexpr size_t kControlBytes = 64 * 1024 + kMaxBlocks * kRedSlots * sizeof(double);
 constexpr size_t kScratchBytes = kVectorsBytes + kControlBytes;
 // Offsets of the control block: solver scalars at 0, ticket counter at 512, halt flag at 768,
