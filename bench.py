@@ -56,7 +56,15 @@ WORKLOADS = {
 NCU_TRAFFIC = {
     # profiles/in_step_dram_cavity101_mixed.md (33 to 66 launches each)
     ("cavity101", "k_bicg_pv", ("register", 384, 9, 0)): 98.3e6,
-    ("cavity101", "k_bicg_pv", ("bulk-copy", 4, 19, 4)): 96.6e6,
+    # (the bulk-copy shapes between which the autotuner picks)
+    ("cavity101", "k_bicg_pv", ("bulk-copy", 4, 17, 4)): 97.0e6,
+    ("cavity101", "k_bicg_pv", ("bulk-copy", 4, 18, 4)): 95.8e6,
+    ("cavity101", "k_bicg_pv", ("bulk-copy", 4, 19, 4)): 96.1e6,
+    ("cavity101", "k_bicg_pv", ("bulk-copy", 4, 20, 4)): 96.2e6,
+    ("cavity101", "k_bicg_pv", ("bulk-copy", 3, 25, 4)): 96.0e6,
+    ("cavity101", "k_bicg_pv", ("bulk-copy", 3, 26, 4)): 96.0e6,
+    ("cavity101", "k_bicg_pv", ("bulk-copy", 3, 27, 4)): 95.5e6,
+    ("cavity101", "k_bicg_pv", ("bulk-copy", 3, 28, 4)): 94.8e6,
     ("cavity101", "k_bicg_st", ("register", 384, 9, 0)): 56.3e6,
     ("cavity101", "k_bicg_xr", ("register", 384, 9, 0)): 95.5e6,
 }

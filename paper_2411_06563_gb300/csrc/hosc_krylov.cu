@@ -507,6 +507,9 @@ __global__ void __launch_bounds__(256, MinB) k6_b(DevParams P, Fields F, int pp)
 // 301 -> 262 us at 257^3, 81.5 -> 71.5 at 161^3, 44.4 -> 42.4 at 129^3, 19.9 -> 22.4 at 101^3; p/v 450 -> 439,
 // 121 -> 117.5, 69.1 -> 67.1, 36.9 -> 35.3 (step at 101^3 891 against 883 us, 81^3 561 against 587): used
 // from kPlaneMinN up, where a launch is several waves of blocks.
+// The p/v form holds the next plane's three vectors, operator row, r_0 and ring node beside its own
+// plane in 80 registers and spills (120 bytes stored and 84 loaded a thread; s/t 32 and 32), which is why it
+// gains 2-3 % where s/t gains 13 %.
 
 constexpr int kPlaneThreads = 384;
 

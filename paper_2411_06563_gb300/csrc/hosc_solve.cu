@@ -18,7 +18,11 @@
 // same bits.
 //
 // Every wait is bounded (kWaitNs on the GPU timer): a block whose wait runs out leaves the solve, the
-// others follow when theirs do, and the step reports HOSC_ECUDA.
+// others follow when theirs do, and the step reports HOSC_ECUDA. No wait runs while some blocks cannot
+// start: a cooperative grid starts whole, after other kernels have left it the room.
+//
+// Spills (-Xptxas -v): 32 bytes stored and 44 loaded a thread in k_solve_planar<1> (held to 64 registers),
+// 22 and 12 in k_solve_mixed<4>, none in the other forms.
 //
 // Measured against an iteration in three launches: FP64 21^3 25.4 -> 12.1 us, 31^3 35 -> 18.1 us, 41^3
 // 49 -> 24.2 us (there half of it FP64 instructions); mixed step at 41^3 226 -> 133 us, at 64^3
@@ -47,7 +51,8 @@ __device__ __forceinline__ unsigned long long solve_ns() {
 
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
-// One value of an exchange: two words of (4 bytes of the value, the exchange's number).
+// One value of an exchange: two words of (4 bytes of the value, the exchange's number): data and flag in
+// one store, as the low-latency protocols of collective libraries send it.
 __device__ __forceinline__ void put_value(ulonglong2* p, double v, unsigned e) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v);
   const unsigned long long f = (unsigned long long)e << 32;
